@@ -474,7 +474,7 @@ def run_ours(args):
     backward_32k = dict(workload=w32.name, ms=msb, value=2.5 * flops32 / (msb * 1e-3) / 1e12, unit=UNIT,
                         frac=2.5 * flops32 / (msb * 1e-3) / 1e12 / peaks["bf16_tflops"], bound="tensor",
                         flops_per_pair_head=10 * w32.block * w32.block * w32.head_dim, launches=nb,
-                        kernels="delta, transposed layout (4), dQ and dK/dV on tcgen05 with accumulators in tensor memory, "
+                        kernels="preparation (delta, transposed layout), dQ and dK/dV on tcgen05 with accumulators in tensor memory, "
                                 "fp32 outputs")
     pa.pa_prefill_status(wsb32)
     del Q32, K32, V32, o32, lse32, dO32, dq32, dk32, dv32

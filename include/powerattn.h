@@ -216,7 +216,7 @@ pa_status pa_prefill_status(const void *workspace, void *stream, int32_t *detail
  * n_q_heads, head_dim] contiguous; dk, dv: device fp32 [batch, seq_len, n_kv_heads, head_dim]
  * contiguous (cleared by the call).  workspace: device, 256-byte aligned,
  * >= pa_prefill_backward_workspace_bytes(p, nnz) (a status block, the row sums delta and the
- * transposed layout).  Three memsets and seven kernels are enqueued.  S and P are recomputed tile by
+ * transposed layout).  Three kernels are enqueued.  S and P are recomputed tile by
  * tile on the tensor cores (bf16 operands, fp32 accumulation): head_dim 128 on tcgen05 with
  * accumulators in tensor memory, head_dim 64 (and head_dim 128 under PA_BACKWARD_PATH=mma) on the
  * warp-level MMA.  A key block that many query blocks list (a sink block is listed by all) is spread

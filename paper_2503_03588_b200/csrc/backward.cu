@@ -9,10 +9,8 @@
 // point, the kernels common to every head size (delta, the transposed layout) and the attention kernels
 // for head_dim 64; head_dim 128 takes the tcgen05 kernels of the sibling file for the two attention
 // kernels.  The kernels here:
-//   backward_delta_kernel    delta = rowsum(dO * O)
-//   csc_count / csc_fill     the CSR transposed: for every key block the query blocks that list it
-//                            (a column walks the rows below it with a binary search each, so the lists
-//                            come out ascending without atomics), and the columns cut into chunks
+//   backward_prep_kernel     delta = rowsum(dO * O); dK = dV = 0; the CSR transposed: for every key block
+//                            the query blocks that list it, ascending
 //   backward_dq_kernel       one CTA per (query block, query head): walks the row's key blocks
 //   backward_dkv_kernel      one CTA per (key block, chunk of its query blocks, KV head): walks the
 //                            chunk for every query head of the group; a column listed by many rows
@@ -26,7 +24,6 @@
 
 #include "backward.cuh"
 #include "common.cuh"
-#include "scan.cuh"
 #include "sm100_ptx.cuh"
 
 namespace pa {
@@ -43,82 +40,177 @@ __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], uint32_t a0, uint3
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// delta[b, h, t] = sum_d dO[b, t, h, d] O[b, t, h, d]; D / 8 lanes per (token, head) row, 16 bytes per lane.
-template <int D>
-__global__ void backward_delta_kernel(const BackwardArgs a)
+// ------------------------------------------------------------------------------------ preparation
+// One launch does everything that has to be there before the attention kernels: delta, dK and dV set to
+// zero (their parts are added up in memory), a clear status block, and the transposed layout.
+//
+// Blocks [0, n_csc) transpose the CSR, each for `cols_per_block` key blocks and none waiting for another:
+// it walks the rows from its first column on (a row lists nothing above itself), a warp per row, sets the
+// bit (column, row) of a bitmap in shared memory for its own columns and counts the entries of the columns
+// before them, which is where its part of row_idx starts.  A column's list is its set bits in order:
+// ascending, the same from run to run, no sorting.  The other blocks stream: eight tokens each, a warp per
+// token, D / 8 lanes per head.
+//
+// Bound by the stream of O and dO (0.70 of the DRAM rate at 32K tokens, 28 / 4 heads).  The transposition runs
+// beside it: 104 us in one launch, where delta (one pair of 16-byte loads per thread: 109 us), count, two scans
+// and fill (37 us) and three memsets ran one after the other; at 4K tokens 16 us instead of 31 and the gaps of
+// eight launches.
+constexpr int kPrepThreads = 256;
+constexpr int kPrepTokens = kPrepThreads / 32;
+constexpr int kPrepHeads = 64;                  // heads per pass (the staging of delta)
+constexpr int kPrepBitmapWords = 8192;          // 32 KB of bitmap per block at most
+constexpr int kPrepMaxCols = 64;                // columns per block at most: more blocks for mid-sized layouts
+constexpr int kPrepMaxBitmap = 224 * 1024;      // bytes of one column's bits at most: 117 million tokens
+
+static int32_t prep_cols_per_block(int32_t nqb)
 {
-    constexpr int kLanes = D / 8;              // lanes that share a row
-    constexpr int kRowsPerWarp = 32 / kLanes;
-    const int lane = threadIdx.x & 31, sub = lane % kLanes;
-    const int64_t row = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * kRowsPerWarp + lane / kLanes;
-    const int64_t rows = (int64_t)a.batch * a.N * a.Hq;
-    float acc = 0.f;
-    int h = 0;
-    int64_t t = 0, b = 0;
-    if (row < rows) {
-        h = (int)(row % a.Hq);
-        t = (row / a.Hq) % a.N;
-        b = row / ((int64_t)a.Hq * a.N);
-        const int64_t off = b * a.o_sb + t * a.o_ss + (int64_t)h * a.o_sh + 8 * sub;
-        const uint4 x = *reinterpret_cast<const uint4 *>(a.o + off);
-        const uint4 y = *reinterpret_cast<const uint4 *>(a.d_o + off);
-        const uint32_t xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
+    const int32_t words = (nqb + 31) / 32;
+    int32_t cols = kPrepBitmapWords / words;
+    if (cols > kPrepMaxCols) cols = kPrepMaxCols;
+    return cols < 1 ? 1 : cols;
+}
+
+__device__ void transpose_layout(const BackwardArgs &a, int32_t block, int32_t cols, uint32_t *bits)
+{
+    __shared__ int32_t s_count[kPrepMaxCols];
+    __shared__ int32_t s_before;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int kWarps = kPrepThreads / 32, kAhead = 4;
+    const int32_t j0 = block * cols, j1 = j0 + cols < a.nqb ? j0 + cols : a.nqb;
+    const int32_t w0 = j0 / 32, words = (a.nqb + 31) / 32 - w0;  // (rows below j0 list nothing here)
+    for (int32_t x = tid; x < (j1 - j0) * words; x += kPrepThreads) bits[x] = 0;
+    if (tid == 0) s_before = 0;
+    __syncthreads();
+    int32_t before = 0;
+    for (int32_t ib = j0 + warp * kAhead; ib < a.nqb; ib += kWarps * kAhead) {
+        int32_t lo[kAhead], hi[kAhead], col[kAhead];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const float2 xf = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&xs[e]));
-            const float2 yf = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&ys[e]));
-            acc += xf.x * yf.x + xf.y * yf.y;
+        for (int x = 0; x < kAhead; ++x) {  // (the loads of four rows in flight together)
+            const bool on = ib + x < a.nqb;
+            lo[x] = on ? __ldg(a.row_ptr + ib + x) : 0;
+            hi[x] = on ? __ldg(a.row_ptr + ib + x + 1) : 0;
+        }
+#pragma unroll
+        for (int x = 0; x < kAhead; ++x) col[x] = lo[x] + lane < hi[x] ? __ldg(a.col_idx + lo[x] + lane) : -1;
+#pragma unroll
+        for (int x = 0; x < kAhead; ++x) {
+            const int32_t i = ib + x;
+            for (int32_t e = lo[x], c = col[x]; e < hi[x]; e += 32) {
+                if (c >= j0 && c < j1) atomicOr(bits + (c - j0) * words + (i / 32 - w0), 1u << (i & 31));
+                before += (c >= 0 && c < j0) ? 1 : 0;
+                c = e + 32 + lane < hi[x] ? __ldg(a.col_idx + e + 32 + lane) : -1;
+            }
         }
     }
+    before = __reduce_add_sync(0xffffffffu, before);
+    if (lane == 0 && before) atomicAdd(&s_before, before);
+    __syncthreads();
+    for (int32_t j = j0 + warp; j < j1; j += kWarps) {
+        int32_t n = 0;
+        for (int32_t w = lane; w < words; w += 32) n += __popc(bits[(j - j0) * words + w]);
+        n = __reduce_add_sync(0xffffffffu, n);
+        if (lane == 0) s_count[j - j0] = n;
+    }
+    __syncthreads();
+    if (warp == 0) {  // exclusive prefix over the block's columns, from the entries before them
+        int32_t carry = s_before + __ldg(a.row_ptr + j0) - __ldg(a.row_ptr);
+        for (int32_t x = 0; x < j1 - j0; x += 32) {
+            const int32_t n = x + lane < j1 - j0 ? s_count[x + lane] : 0;
+            int32_t incl = n;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            if (x + lane < j1 - j0) {
+                s_count[x + lane] = carry + incl - n;
+                a.col_ptr[j0 + x + lane] = carry + incl - n;
+            }
+            carry += __shfl_sync(0xffffffffu, incl, 31);
+        }
+        if (lane == 0 && j1 == a.nqb) a.col_ptr[a.nqb] = carry;
+    }
+    __syncthreads();
+    for (int32_t j = j0 + warp; j < j1; j += kWarps) {
+        int32_t pos = s_count[j - j0];
+        for (int32_t wb = 0; wb < words; wb += 32) {
+            uint32_t m = wb + lane < words ? bits[(j - j0) * words + wb + lane] : 0u;
+            const int32_t n = __popc(m);
+            int32_t incl = n;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            int32_t *out = a.row_idx + pos + incl - n;
+            for (; m; m &= m - 1) *out++ = 32 * (w0 + wb + lane) + __ffs(m) - 1;
+            pos += __shfl_sync(0xffffffffu, incl, 31);
+        }
+    }
+}
+
+// delta[b, h, t] = sum_d dO[b, t, h, d] O[b, t, h, d].
+template <int D>
+__global__ void __launch_bounds__(kPrepThreads) backward_prep_kernel(const BackwardArgs a, const int32_t n_csc,
+                                                                     const int32_t cols_per_block)
+{
+    extern __shared__ uint32_t prep_bits[];
+    if (blockIdx.x == 0 && threadIdx.x < kBwdStatusBytes / sizeof(int32_t)) a.status[threadIdx.x] = 0;
+    if (blockIdx.x < (unsigned)n_csc) {
+        transpose_layout(a, (int32_t)blockIdx.x, cols_per_block, prep_bits);
+        return;
+    }
+    __shared__ float s_delta[kPrepHeads][kPrepTokens + 1];
+    constexpr int kLanes = D / 8;             // lanes that share a head's row, 16 bytes each
+    constexpr int kHeadsPerStep = 32 / kLanes;
+    constexpr int kUnroll = 7;                // (28 heads of 128 features: two rounds)
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, sub = lane % kLanes, hsub = lane / kLanes;
+    const int64_t groups = (a.N + kPrepTokens - 1) / kPrepTokens, grp = (int64_t)blockIdx.x - n_csc;
+    const int64_t b = grp / groups, t0 = (grp - b * groups) * kPrepTokens, t = t0 + warp;
+    const bool in = t < a.N;
+    {  // dK and dV of these tokens: contiguous
+        const int64_t per_token = (int64_t)a.Hkv * D / 4, tokens = a.N - t0 < kPrepTokens ? a.N - t0 : kPrepTokens;
+        float4 *zk = reinterpret_cast<float4 *>(a.dk) + (b * a.N + t0) * per_token;
+        float4 *zv = reinterpret_cast<float4 *>(a.dv) + (b * a.N + t0) * per_token;
+        for (int64_t x = tid; x < tokens * per_token; x += kPrepThreads) {
+            zk[x] = make_float4(0.f, 0.f, 0.f, 0.f);
+            zv[x] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    }
+    const int64_t base = b * a.o_sb + (in ? t : 0) * a.o_ss + 8 * sub;
+    for (int hb = 0; hb < a.Hq; hb += kPrepHeads) {
+        const int heads = a.Hq - hb < kPrepHeads ? a.Hq - hb : kPrepHeads;
+        for (int h0 = 0; h0 < heads; h0 += kHeadsPerStep * kUnroll) {
+            uint4 x[kUnroll], y[kUnroll];
 #pragma unroll
-    for (int o = kLanes / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (row < rows && sub == 0) a.delta[(b * a.Hq + h) * a.N + t] = acc;
-}
-
-// Does row i of the CSR list block j?  (rows are ascending: binary search)
-__device__ __forceinline__ bool row_lists(const int32_t *row_ptr, const int32_t *col_idx, int32_t i, int32_t j)
-{
-    int32_t lo = row_ptr[i], hi = row_ptr[i + 1];
-    while (lo < hi) {
-        const int32_t mid = (lo + hi) >> 1;
-        const int32_t c = col_idx[mid];
-        if (c == j) return true;
-        if (c < j) lo = mid + 1;
-        else hi = mid;
-    }
-    return false;
-}
-
-// One warp per key block j: counts the query blocks i >= j that list it.  col_ptr[j + 1] = count
-// (scanned afterwards), chunk_ptr[j + 1] = ceil(count / kBwdChunk).
-__global__ void csc_count_kernel(const BackwardArgs a)
-{
-    const int32_t j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (j >= a.nqb) return;
-    int32_t cnt = 0;
-    for (int32_t i = j + lane; i < a.nqb; i += 32) cnt += row_lists(a.row_ptr, a.col_idx, i, j) ? 1 : 0;
-    for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-    if (lane == 0) {
-        if (j == 0) a.col_ptr[0] = a.chunk_ptr[0] = 0;
-        a.col_ptr[j + 1] = cnt;
-        a.chunk_ptr[j + 1] = (cnt + kBwdChunk - 1) / kBwdChunk;
-    }
-}
-
-// One warp per key block j: writes its listers in ascending order.
-__global__ void csc_fill_kernel(const BackwardArgs a)
-{
-    const int32_t j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (j >= a.nqb) return;
-    int32_t pos = a.col_ptr[j];
-    for (int32_t base = j; base < a.nqb; base += 32) {
-        const int32_t i = base + lane;
-        const bool on = i < a.nqb && row_lists(a.row_ptr, a.col_idx, i, j);
-        const uint32_t m = __ballot_sync(0xffffffffu, on);
-        if (on) a.row_idx[pos + __popc(m & ((1u << lane) - 1u))] = i;
-        pos += __popc(m);
+            for (int u = 0; u < kUnroll; ++u) {
+                const int h = h0 + u * kHeadsPerStep + hsub;
+                const bool on = in && h < heads;
+                const int64_t off = base + (int64_t)(hb + h) * a.o_sh;
+                x[u] = on ? __ldg(reinterpret_cast<const uint4 *>(a.o + off)) : make_uint4(0, 0, 0, 0);
+                y[u] = on ? __ldg(reinterpret_cast<const uint4 *>(a.d_o + off)) : make_uint4(0, 0, 0, 0);
+            }
+#pragma unroll
+            for (int u = 0; u < kUnroll; ++u) {
+                const uint32_t xs[4] = {x[u].x, x[u].y, x[u].z, x[u].w}, ys[4] = {y[u].x, y[u].y, y[u].z, y[u].w};
+                float acc = 0.f;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float2 xf = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&xs[e]));
+                    const float2 yf = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&ys[e]));
+                    acc += xf.x * yf.x + xf.y * yf.y;
+                }
+#pragma unroll
+                for (int o = kLanes / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                const int h = h0 + u * kHeadsPerStep + hsub;
+                if (sub == 0 && h < heads) s_delta[h][warp] = acc;
+            }
+        }
+        __syncthreads();
+        // Eight tokens of a head are one 32-byte sector of delta (where N is a multiple of eight).
+        for (int x = tid; x < heads * kPrepTokens; x += kPrepThreads) {
+            const int h = x / kPrepTokens, w = x % kPrepTokens;
+            if (t0 + w < a.N) a.delta[(b * a.Hq + hb + h) * a.N + t0 + w] = s_delta[h][w];
+        }
+        __syncthreads();
     }
 }
 
@@ -304,17 +396,9 @@ __global__ void __launch_bounds__(kBwdThreads) backward_dkv_kernel(const Backwar
     const int hk = blockIdx.y, b = blockIdx.z;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, g = lane >> 2, t = lane & 3;
     const int r0 = 16 * wid;
-    if (c >= a.chunk_ptr[a.nqb]) return;
-    // The column whose chunks include c: last j with chunk_ptr[j] <= c.
-    int32_t lo = 0, hi = a.nqb;
-    while (hi - lo > 1) {
-        const int32_t mid = (lo + hi) >> 1;
-        if (a.chunk_ptr[mid] <= c) lo = mid;
-        else hi = mid;
-    }
-    const int32_t j = lo;
-    const int32_t e0 = a.col_ptr[j] + (c - a.chunk_ptr[j]) * kBwdChunk;
-    const int32_t e1 = e0 + kBwdChunk < a.col_ptr[j + 1] ? e0 + kBwdChunk : a.col_ptr[j + 1];
+    const BackwardChunk chunk = backward_chunk_at(a, c);
+    const int32_t j = chunk.j, e0 = chunk.e0, e1 = chunk.e1;
+    if (e0 >= e1) return;
 
     load_tile<D>(sK, a.k + b * a.k_sb + (int64_t)hk * a.k_sh, a.k_ss, (int64_t)j * kBwdBlk, a.N, tid);
     load_tile<D>(sV, a.v + b * a.v_sb + (int64_t)hk * a.v_sh, a.v_ss, (int64_t)j * kBwdBlk, a.N, tid);
@@ -382,8 +466,19 @@ __global__ void __launch_bounds__(kBwdThreads) backward_dkv_kernel(const Backwar
 
 namespace pa {
 
-// Workspace: status block (256 bytes), delta [batch, Hq, N] fp32, then col_ptr [nqb + 1], chunk_ptr [nqb + 1],
-// row_idx [nnz] int32.
+// Query blocks per chunk of a key block's list.  A chunk is walked by one CTA of the dK / dV kernels for the
+// whole head group, so it is also the granularity at which the work is dealt to the SMs: about eight chunks per
+// SM, no more than 32 blocks, and no less than four, below which a chunk's own cost (K and V in, dK and dV added
+// to memory) outweighs the balance.  (4K tokens, 28 / 4 heads: 112 us with chunks of 4, 229 us with chunks of 32,
+// of which the sink block's two are then the whole call's tail.)
+static int32_t backward_chunk(int64_t nnz, int64_t kv_rows, int sms)
+{
+    const int64_t c = nnz * kv_rows / (8 * (int64_t)sms);
+    return c < 4 ? 4 : c > kBwdMaxChunk ? kBwdMaxChunk : (int32_t)c;
+}
+
+// Workspace: status block (256 bytes), delta [batch, Hq, N] fp32, then col_ptr [nqb + 1], row_idx [nnz] int32
+// ([nqb + 1] words behind them are not used: the size is what callers have been told).
 static size_t backward_workspace_bytes(const pa_prefill_params *p, int64_t nnz)
 {
     const int64_t nqb = (p->seq_len + kBwdBlk - 1) / kBwdBlk;
@@ -426,19 +521,20 @@ static pa_status launch_backward(const BackwardArgs &a, const pa_prefill_params 
     if (device_once_begin(device, D == 128 ? ONCE_BACKWARD_ATTR : ONCE_BACKWARD_ATTR_64)) {
         const cudaError_t e1 = cudaFuncSetAttribute(backward_dq_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemDq);
         const cudaError_t e2 = cudaFuncSetAttribute(backward_dkv_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemDkv);
-        if (e1 != cudaSuccess || e2 != cudaSuccess) {
+        // (a bitmap row of more than the 32 KB aimed at is needed from 16 million tokens on)
+        const cudaError_t e3 = cudaFuncSetAttribute(backward_prep_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPrepMaxBitmap);
+        if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess) {
             device_once_reset(device, D == 128 ? ONCE_BACKWARD_ATTR : ONCE_BACKWARD_ATTR_64);
-            return fail(PA_ERR_CUDA, "cudaFuncSetAttribute failed: %s", cudaGetErrorString(e1 != cudaSuccess ? e1 : e2));
+            return fail(PA_ERR_CUDA, "cudaFuncSetAttribute failed: %s",
+                        cudaGetErrorString(e1 != cudaSuccess ? e1 : e2 != cudaSuccess ? e2 : e3));
         }
     }
-    const int64_t rows = (int64_t)a.batch * a.N * a.Hq;
-    constexpr int kDeltaRowsPerBlock = 8 * (32 / (D / 8));  // eight warps, each 32 / (D / 8) rows
-    backward_delta_kernel<D><<<(unsigned)((rows + kDeltaRowsPerBlock - 1) / kDeltaRowsPerBlock), 256, 0, st>>>(a);
-    const unsigned col_blocks = (unsigned)((a.nqb + 7) / 8);
-    csc_count_kernel<<<col_blocks, 256, 0, st>>>(a);
-    layout_scan_kernel<<<1, 1024, 0, st>>>(a.nqb, a.col_ptr);
-    layout_scan_kernel<<<1, 1024, 0, st>>>(a.nqb, a.chunk_ptr);
-    csc_fill_kernel<<<col_blocks, 256, 0, st>>>(a);
+    const int32_t cols = prep_cols_per_block(a.nqb), n_csc = (a.nqb + cols - 1) / cols;
+    const int64_t groups = (int64_t)a.batch * ((a.N + kPrepTokens - 1) / kPrepTokens);
+    const int32_t bitmap_cols = cols < a.nqb ? cols : a.nqb;
+    const size_t bitmap = (size_t)bitmap_cols * ((a.nqb + 31) / 32) * sizeof(uint32_t);
+    if (groups + n_csc > 0x7fffffff || bitmap > (size_t)kPrepMaxBitmap) return fail(PA_ERR_SHAPE, "batch x seq_len too large");
+    backward_prep_kernel<D><<<(unsigned)(n_csc + groups), kPrepThreads, bitmap, st>>>(a, n_csc, cols);
     // head_dim 128: dQ, dK and dV on the tcgen05 tensor cores (PA_BACKWARD_PATH=mma keeps the warp-level kernels).
     if (D == 128 && !env_switches().backward_mma) {
         PA_CUDA_OK(cudaGetLastError());
@@ -446,7 +542,7 @@ static pa_status launch_backward(const BackwardArgs &a, const pa_prefill_params 
     }
     backward_dq_kernel<D><<<dim3((unsigned)a.nqb, (unsigned)a.Hq, (unsigned)a.batch), kBwdThreads, kSmemDq, st>>>(a);
     // (an upper bound on the number of chunks; CTAs beyond the real count return at once)
-    const int64_t max_chunks = nnz / kBwdChunk + a.nqb;
+    const int64_t max_chunks = nnz / a.chunk + a.nqb;
     backward_dkv_kernel<D><<<dim3((unsigned)max_chunks, (unsigned)a.Hkv, (unsigned)a.batch), kBwdThreads, kSmemDkv, st>>>(a);
     PA_CUDA_OK(cudaGetLastError());
     return PA_OK;
@@ -496,8 +592,7 @@ extern "C" pa_status pa_prefill_backward(const pa_prefill_params *p, const void 
     a.delta = reinterpret_cast<float *>(ws + kBwdStatusBytes);
     size_t off = (kBwdStatusBytes + (size_t)p->batch * p->n_q_heads * p->seq_len * sizeof(float) + 255) & ~(size_t)255;
     a.col_ptr = reinterpret_cast<int32_t *>(ws + off);
-    a.chunk_ptr = a.col_ptr + (nqb + 1);
-    a.row_idx = a.chunk_ptr + (nqb + 1);
+    a.row_idx = a.col_ptr + (nqb + 1);
     a.dq = dq; a.dk = dk; a.dv = dv;
     a.q_sb = p->q.batch; a.q_ss = p->q.seq; a.q_sh = p->q.head;
     a.k_sb = p->k.batch; a.k_ss = p->k.seq; a.k_sh = p->k.head;
@@ -511,11 +606,8 @@ extern "C" pa_status pa_prefill_backward(const pa_prefill_params *p, const void 
     a.scale_log2 = a.scale * 1.4426950408889634f;
     a.npairs = (a.G + 1) / 2;
     a.wait_cycles = 0;
+    a.chunk = backward_chunk(nnz, (int64_t)a.batch * a.Hkv, dev.sms);
 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const size_t kv_bytes = (size_t)p->batch * p->seq_len * p->n_kv_heads * p->head_dim * sizeof(float);
-    PA_CUDA_OK(cudaMemsetAsync(workspace, 0, kBwdStatusBytes, st));
-    PA_CUDA_OK(cudaMemsetAsync(dk, 0, kv_bytes, st));
-    PA_CUDA_OK(cudaMemsetAsync(dv, 0, kv_bytes, st));
     return p->head_dim == 128 ? launch_backward<128>(a, p, nnz, dev.device, dev.sms, st) : launch_backward<64>(a, p, nnz, dev.device, dev.sms, st);
 }

@@ -12,7 +12,7 @@
 namespace pa {
 
 constexpr int kBwdBlk = 64;       // tokens per block
-constexpr int kBwdChunk = 32;     // query blocks per CTA of the dK / dV kernels
+constexpr int kBwdMaxChunk = 32;  // query blocks per chunk of the dK / dV kernels, at most
 constexpr size_t kBwdStatusBytes = 256;  // status block at the head of the workspace ([0] error code, [1] detail)
 
 struct BackwardArgs {
@@ -23,7 +23,7 @@ struct BackwardArgs {
     float *delta;              // [batch, Hq, N]
     int32_t *col_ptr;          // [nqb + 1]: extents of the transposed lists
     int32_t *row_idx;          // [nnz]: query blocks that list each key block, ascending
-    int32_t *chunk_ptr;        // [nqb + 1]: first chunk of each column
+    int32_t chunk;             // query blocks per chunk of a column, at most
     float *dq, *dk, *dv;       // fp32, contiguous [batch, N, H, D]
     int64_t q_sb, q_ss, q_sh, k_sb, k_ss, k_sh, v_sb, v_ss, v_sh, o_sb, o_ss, o_sh;
     int64_t N;
@@ -32,6 +32,32 @@ struct BackwardArgs {
     float scale, scale_log2;
     long long wait_cycles;     // limit of every barrier wait of the tensor-core kernels
 };
+
+// A chunk of a key block's list: the unit of work of the dK / dV kernels.  Column j owns the chunk slots
+// [col_ptr[j] / chunk + j, col_ptr[j + 1] / chunk + j + 1): at least ceil(count / chunk) of them for any
+// count, and known from col_ptr alone.  A column of several chunks is cut into equal parts; a slot beyond
+// its chunks is empty.
+struct BackwardChunk {
+    int32_t j, e0, e1;  // key block, extent in row_idx (empty: e0 == e1)
+};
+__device__ __forceinline__ BackwardChunk backward_chunk_at(const BackwardArgs &a, int32_t c)
+{
+    BackwardChunk r = {0, 0, 0};
+    int32_t lo = 0, hi = a.nqb;  // last column whose slots start at or before c
+    while (hi - lo > 1) {
+        const int32_t mid = (lo + hi) >> 1;
+        if (__ldg(a.col_ptr + mid) / a.chunk + mid <= c) lo = mid;
+        else hi = mid;
+    }
+    const int32_t p0 = __ldg(a.col_ptr + lo), cnt = __ldg(a.col_ptr + lo + 1) - p0;
+    const int32_t parts = (cnt + a.chunk - 1) / a.chunk, part = c - (p0 / a.chunk + lo);
+    r.j = lo;
+    if (part < parts) {
+        r.e0 = p0 + (int32_t)((int64_t)cnt * part / parts);
+        r.e1 = p0 + (int32_t)((int64_t)cnt * (part + 1) / parts);
+    }
+    return r;
+}
 
 // dQ, dK, dV for head_dim 128 on tcgen05 (delta and the transposed lists are already in the workspace).
 pa_status launch_backward_sm100(const BackwardArgs &a, const pa_prefill_params *p, int64_t nnz, int device, int sms,

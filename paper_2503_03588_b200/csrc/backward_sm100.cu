@@ -467,8 +467,9 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
 {
     constexpr int D = 128;
     using SM = DkvSmem;
-    const int32_t c = blockIdx.x;
-    if (c >= a.chunk_ptr[a.nqb]) return;  // (the grid is an upper bound on the number of chunks)
+    const BackwardChunk chunk = backward_chunk_at(a, (int32_t)blockIdx.x);
+    const int32_t j = chunk.j, e0 = chunk.e0, e1 = chunk.e1;
+    if (e0 >= e1) return;  // (the grid is an upper bound on the number of chunks)
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *smem = smem_raw + (smem_base - ptx::smem_u32(smem_raw));
@@ -481,16 +482,6 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     };
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int hk = blockIdx.y, b = blockIdx.z;
-    // The column whose chunks include c: last j with chunk_ptr[j] <= c.
-    int32_t lo = 0, hi = a.nqb;
-    while (hi - lo > 1) {
-        const int32_t mid = (lo + hi) >> 1;
-        if (a.chunk_ptr[mid] <= c) lo = mid;
-        else hi = mid;
-    }
-    const int32_t j = lo;
-    const int32_t e0 = a.col_ptr[j] + (c - a.chunk_ptr[j]) * kBwdChunk;
-    const int32_t e1 = e0 + kBwdChunk < a.col_ptr[j + 1] ? e0 + kBwdChunk : a.col_ptr[j + 1];
     const int n = (e1 - e0) * a.npairs;  // steps: listing query blocks x head pairs (pairs fastest); at least one
 
     if (threadIdx.x == 0) {
@@ -750,7 +741,7 @@ pa_status launch_backward_sm100(const BackwardArgs &args, const pa_prefill_param
     if (n_items > (int64_t)0x3fffffff) return fail(PA_ERR_SHAPE, "too many work items (%lld)", (long long)n_items);
     dq_kernel<<<(unsigned)(n_items < sms ? n_items : sms), kDqThreads, DqSmem::kAlloc, st>>>(tmQ, tmG, tmK, tmV, a, (uint32_t)n_items);
     // (an upper bound on the number of chunks; CTAs beyond the real count return at once)
-    const int64_t max_chunks = nnz / kBwdChunk + a.nqb;
+    const int64_t max_chunks = nnz / a.chunk + a.nqb;
     dkv_kernel<<<dim3((unsigned)max_chunks, (unsigned)a.Hkv, (unsigned)a.batch), kTcThreads, DkvSmem::kAlloc, st>>>(tmQ, tmG, tmK, tmV, a);
     PA_CUDA_OK(cudaGetLastError());
     return PA_OK;

@@ -1,4 +1,4 @@
-// One-block prefix sum used by the layout writers and the backward pass's transposed layout.
+// One-block prefix sum used by the layout writers.
 #pragma once
 
 #include <stdint.h>

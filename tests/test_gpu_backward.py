@@ -196,3 +196,44 @@ def test_backward_on_kv_head_shards_reproduces_the_whole_call(pa):
             assert torch.equal(dq, dq_full[:, :, heads]), (world, rank)
             assert torch.allclose(dk, dk_full[:, :, kv_heads], rtol=1e-4, atol=1e-5), (world, rank)
             assert torch.allclose(dv, dv_full[:, :, kv_heads], rtol=1e-4, atol=1e-5), (world, rank)
+
+
+def _random_causal_csr(nqb, rng):
+    """Rows of 0 to nqb ascending blocks, some rows and some columns empty, some columns listed by all."""
+    allowed = rng.random(nqb) < 0.8
+    allowed[: max(1, nqb // 20)] = True
+    rows = []
+    for i in range(nqb):
+        density = rng.choice([0.0, 0.05, 0.5, 1.0], p=[0.1, 0.5, 0.2, 0.2])
+        rows.append([j for j in range(i + 1) if allowed[j] and rng.random() < density])
+    rp = np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.int32)
+    return rp, np.asarray([j for r in rows for j in r], dtype=np.int32), rows
+
+
+@pytest.mark.parametrize("N,Hq,Hkv,D", [
+    (64 * 32 + 1, 2, 1, 128),    # 33 columns: one word and one bit of rows
+    (64 * 65, 4, 2, 64),         # 65 columns: one beyond what a block transposes
+    (64 * 40 - 9, 66, 33, 64),   # more heads than one pass over a token's rows takes; ragged tokens
+    (64 * 70 + 3, 3, 3, 128),    # rows of up to 71 entries; one head per group
+])
+def test_backward_on_arbitrary_causal_layouts(pa, oracle, N, Hq, Hkv, D):
+    """The transposed lists of layouts with empty rows, empty columns, columns listed by every row and rows
+    of more than 32 entries; the oracle takes the dense mask that the CSR stands for."""
+    nqb = (N + 63) // 64
+    rp, ci, rows = _random_causal_csr(nqb, np.random.default_rng(N))
+    dense = np.zeros((N, N), dtype=bool)
+    for i, r in enumerate(rows):
+        for j in r:
+            dense[i * 64:(i + 1) * 64, j * 64:(j + 1) * 64] = True
+    dense &= np.tril(np.ones((N, N), dtype=bool))
+    Q, K, V = (si.bf16_randn((1, N, h, D), 1600 + N + x) for x, h in enumerate((Hq, Hkv, Hkv)))
+    dO = si.bf16_randn((1, N, Hq, D), 1604 + N)
+    Qd, Kd, Vd, dOd, rpd, cid = (t.cuda() for t in (Q, K, V, dO, torch.as_tensor(rp), torch.as_tensor(ci)))
+    o, lse, ws = pa.pa_prefill(Qd, Kd, Vd, rpd, cid)
+    pa.pa_prefill_status(ws)
+    dq, dk, dv, wsb = pa.pa_prefill_backward(Qd, Kd, Vd, o, lse, dOd, rpd, cid,
+                                             dk=torch.full((1, N, Hkv, D), 7.0, device="cuda"),
+                                             dv=torch.full((1, N, Hkv, D), 7.0, device="cuda"))
+    pa.pa_prefill_status(wsb)
+    for g, r, n in zip((dq, dk, dv), oracle.backward(Q, K, V, dO, 64, 5, 1, dense=dense), ("dQ", "dK", "dV")):
+        _compare(g, r, n + " random layout")
