@@ -535,12 +535,14 @@ static pa_status launch_backward(const BackwardArgs &a, const pa_prefill_params 
     const size_t bitmap = (size_t)bitmap_cols * ((a.nqb + 31) / 32) * sizeof(uint32_t);
     if (groups + n_csc > 0x7fffffff || bitmap > (size_t)kPrepMaxBitmap) return fail(PA_ERR_SHAPE, "batch x seq_len too large");
     backward_prep_kernel<D><<<(unsigned)(n_csc + groups), kPrepThreads, bitmap, st>>>(a, n_csc, cols);
-    // head_dim 128: dQ, dK and dV on the tcgen05 tensor cores (PA_BACKWARD_PATH=mma keeps the warp-level kernels).
-    if (D == 128 && !env_switches().backward_mma) {
-        PA_CUDA_OK(cudaGetLastError());
-        return launch_backward_sm100(a, p, nnz, device, sms, st);
+    // dQ, and for head_dim 128 dK and dV, on the tcgen05 tensor cores (PA_BACKWARD_PATH=mma: on the warp-level kernels).
+    const bool mma = env_switches().backward_mma != 0;
+    PA_CUDA_OK(cudaGetLastError());
+    if (!mma) {
+        pa_status s = launch_backward_sm100(a, p, nnz, device, sms, st);
+        if (s != PA_OK || D == 128) return s;
     }
-    backward_dq_kernel<D><<<dim3((unsigned)a.nqb, (unsigned)a.Hq, (unsigned)a.batch), kBwdThreads, kSmemDq, st>>>(a);
+    if (mma) backward_dq_kernel<D><<<dim3((unsigned)a.nqb, (unsigned)a.Hq, (unsigned)a.batch), kBwdThreads, kSmemDq, st>>>(a);
     // (an upper bound on the number of chunks; CTAs beyond the real count return at once)
     const int64_t max_chunks = nnz / a.chunk + a.nqb;
     backward_dkv_kernel<D><<<dim3((unsigned)max_chunks, (unsigned)a.Hkv, (unsigned)a.batch), kBwdThreads, kSmemDkv, st>>>(a);

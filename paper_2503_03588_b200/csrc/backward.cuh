@@ -14,6 +14,7 @@ namespace pa {
 constexpr int kBwdBlk = 64;       // tokens per block
 constexpr int kBwdMaxChunk = 32;  // query blocks per chunk of the dK / dV kernels, at most
 constexpr size_t kBwdStatusBytes = 256;  // status block at the head of the workspace ([0] error code, [1] detail)
+constexpr int kBwdDqCounter = 16, kBwdDkvCounter = 24;  // words of the status block: items drawn by the tcgen05 kernels
 
 struct BackwardArgs {
     const __nv_bfloat16 *q, *k, *v, *o, *d_o;
@@ -59,7 +60,7 @@ __device__ __forceinline__ BackwardChunk backward_chunk_at(const BackwardArgs &a
     return r;
 }
 
-// dQ, dK, dV for head_dim 128 on tcgen05 (delta and the transposed lists are already in the workspace).
+// On tcgen05: dQ, and for head_dim 128 dK and dV (delta and the transposed lists are already in the workspace).
 pa_status launch_backward_sm100(const BackwardArgs &a, const pa_prefill_params *p, int64_t nnz, int device, int sms,
                                 cudaStream_t st);
 

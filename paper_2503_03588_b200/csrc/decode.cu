@@ -1063,9 +1063,9 @@ static pa_status launch_decode(const DecodeShape &p, const void *q, const void *
         CUtensorMap tmK, tmV;
         const bool paged = table != nullptr;
         TensorMapKey kk = {k_cache, paged ? (int64_t)kDecBlock : p.max_len, p.k.seq, p.k.head, p.k.batch, dev.device,
-                           p.head_dim, p.n_kv_heads, paged ? n_pages : p.batch, 1, kDecBlock};
+                           p.head_dim, p.n_kv_heads, paged ? n_pages : p.batch, 1, kDecBlock, 0};
         TensorMapKey kv = {v_cache, paged ? (int64_t)kDecBlock : p.max_len, p.v.seq, p.v.head, p.v.batch, dev.device,
-                           p.head_dim, p.n_kv_heads, paged ? n_pages : p.batch, 1, kDecBlock};
+                           p.head_dim, p.n_kv_heads, paged ? n_pages : p.batch, 1, kDecBlock, 0};
         if (pa_status s = get_tensor_map(kk, "k_cache", &tmK)) return s;
         if (pa_status s = get_tensor_map(kv, "v_cache", &tmV)) return s;
 

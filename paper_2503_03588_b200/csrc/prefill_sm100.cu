@@ -904,7 +904,7 @@ static pa_status launch_prefill(const pa_prefill_params *p, const void *q, const
     auto map_of = [&](const void *base, int heads, const pa_strides &st, int box_heads, const char *what, CUtensorMap *m) {
         // (packed sequences: one "batch" entry of total_tokens tokens)
         const TensorMapKey key = {base, varlen ? total_tokens : p->seq_len, st.seq, st.head, varlen ? 0 : st.batch, dev.device, D,
-                                  heads, varlen ? 1 : p->batch, box_heads, kBlk};
+                                  heads, varlen ? 1 : p->batch, box_heads, kBlk, 0};
         return get_tensor_map(key, what, m);
     };
     if (pa_status s = map_of(q, p->n_q_heads, p->q, 2, "q", &tmQ)) return s;
