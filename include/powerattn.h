@@ -218,8 +218,7 @@ pa_status pa_prefill_status(const void *workspace, void *stream, int32_t *detail
  * >= pa_prefill_backward_workspace_bytes(p, nnz) (a status block, the row sums delta and the
  * transposed layout).  Three kernels are enqueued.  S and P are recomputed tile by
  * tile on the tensor cores (bf16 operands, fp32 accumulation): on tcgen05 with accumulators
- * in tensor memory, dK and dV of head_dim 64 (and everything under PA_BACKWARD_PATH=mma) on the
- * warp-level MMA.  A key block that many query blocks list (a sink block is listed by all) is spread
+ * in tensor memory (under PA_BACKWARD_PATH=mma: on the warp-level MMA).  A key block that many query blocks list (a sink block is listed by all) is spread
  * over several CTAs that add their parts with fp32 atomics, so dk and dv of such blocks may differ
  * in the last bits from run to run.
  * Errors: as pa_prefill.  The tcgen05 kernels bound their barrier waits like the prefill kernel;

@@ -6,9 +6,8 @@
 //     dS_ij = P_ij (<dO_i, v_j> - delta_i)       dQ_i = scale sum_j dS_ij k_j
 //                                                dK_j = scale sum_i dS_ij q_i
 // (dK and dV also sum over the query heads that share the KV head).  This file holds the entry
-// point, the kernels common to every head size (delta, the transposed layout) and the attention kernels
-// for head_dim 64; head_dim 128 takes the tcgen05 kernels of the sibling file for the two attention
-// kernels.  The kernels here:
+// point, the preparation kernel (delta, the transposed layout) and attention kernels on the warp-level MMA;
+// the tcgen05 kernels of the sibling file are the ones that run unless PA_BACKWARD_PATH=mma asks for these.  The kernels here:
 //   backward_prep_kernel     delta = rowsum(dO * O); dK = dV = 0; the CSR transposed: for every key block
 //                            the query blocks that list it, ascending
 //   backward_dq_kernel       one CTA per (query block, query head): walks the row's key blocks
@@ -42,7 +41,7 @@ __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], uint32_t a0, uint3
 
 // ------------------------------------------------------------------------------------ preparation
 // One launch does everything that has to be there before the attention kernels: delta, dK and dV set to
-// zero (their parts are added up in memory), a clear status block, and the transposed layout.
+// zero (where most of them are added up in memory), a clear status block, and the transposed layout.
 //
 // Blocks [0, n_csc) transpose the CSR, each for `cols_per_block` key blocks and none waiting for another:
 // it walks the rows from its first column on (a row lists nothing above itself), a warp per row, sets the
@@ -166,7 +165,7 @@ __global__ void __launch_bounds__(kPrepThreads) backward_prep_kernel(const Backw
     const int64_t groups = (a.N + kPrepTokens - 1) / kPrepTokens, grp = (int64_t)blockIdx.x - n_csc;
     const int64_t b = grp / groups, t0 = (grp - b * groups) * kPrepTokens, t = t0 + warp;
     const bool in = t < a.N;
-    {  // dK and dV of these tokens: contiguous
+    if (a.prezero) {  // dK and dV of these tokens: contiguous
         const int64_t per_token = (int64_t)a.Hkv * D / 4, tokens = a.N - t0 < kPrepTokens ? a.N - t0 : kPrepTokens;
         float4 *zk = reinterpret_cast<float4 *>(a.dk) + (b * a.N + t0) * per_token;
         float4 *zv = reinterpret_cast<float4 *>(a.dv) + (b * a.N + t0) * per_token;
@@ -515,7 +514,7 @@ static pa_status check_backward(const pa_prefill_params *p, int64_t nnz)
 
 template <int D>
 static pa_status launch_backward(const BackwardArgs &a, const pa_prefill_params *p, int64_t nnz, int device, int sms,
-                                 cudaStream_t st)
+                                 bool mma, cudaStream_t st)
 {
     constexpr int kSmemDq = 4 * BwdTile<D>::kBytes, kSmemDkv = 4 * BwdTile<D>::kBytes + 2 * kBwdBlk * 4;
     if (device_once_begin(device, D == 128 ? ONCE_BACKWARD_ATTR : ONCE_BACKWARD_ATTR_64)) {
@@ -535,14 +534,10 @@ static pa_status launch_backward(const BackwardArgs &a, const pa_prefill_params 
     const size_t bitmap = (size_t)bitmap_cols * ((a.nqb + 31) / 32) * sizeof(uint32_t);
     if (groups + n_csc > 0x7fffffff || bitmap > (size_t)kPrepMaxBitmap) return fail(PA_ERR_SHAPE, "batch x seq_len too large");
     backward_prep_kernel<D><<<(unsigned)(n_csc + groups), kPrepThreads, bitmap, st>>>(a, n_csc, cols);
-    // dQ, and for head_dim 128 dK and dV, on the tcgen05 tensor cores (PA_BACKWARD_PATH=mma: on the warp-level kernels).
-    const bool mma = env_switches().backward_mma != 0;
     PA_CUDA_OK(cudaGetLastError());
-    if (!mma) {
-        pa_status s = launch_backward_sm100(a, p, nnz, device, sms, st);
-        if (s != PA_OK || D == 128) return s;
-    }
-    if (mma) backward_dq_kernel<D><<<dim3((unsigned)a.nqb, (unsigned)a.Hq, (unsigned)a.batch), kBwdThreads, kSmemDq, st>>>(a);
+    // dQ, dK and dV on the tcgen05 tensor cores (PA_BACKWARD_PATH=mma: on the warp-level kernels).
+    if (!mma) return launch_backward_sm100(a, p, nnz, device, sms, st);
+    backward_dq_kernel<D><<<dim3((unsigned)a.nqb, (unsigned)a.Hq, (unsigned)a.batch), kBwdThreads, kSmemDq, st>>>(a);
     // (an upper bound on the number of chunks; CTAs beyond the real count return at once)
     const int64_t max_chunks = nnz / a.chunk + a.nqb;
     backward_dkv_kernel<D><<<dim3((unsigned)max_chunks, (unsigned)a.Hkv, (unsigned)a.batch), kBwdThreads, kSmemDkv, st>>>(a);
@@ -609,7 +604,13 @@ extern "C" pa_status pa_prefill_backward(const pa_prefill_params *p, const void 
     a.npairs = (a.G + 1) / 2;
     a.wait_cycles = 0;
     a.chunk = backward_chunk(nnz, (int64_t)a.batch * a.Hkv, dev.sms);
+    // dK and dV are cleared by the preparation where most key blocks are added up from several chunks (small
+    // problems, small chunks); with chunks of full size the tcgen05 kernels write all but a few columns once and
+    // clear those.
+    const bool mma = env_switches().backward_mma != 0;
+    a.prezero = mma || a.chunk < kBwdMaxChunk;
 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    return p->head_dim == 128 ? launch_backward<128>(a, p, nnz, dev.device, dev.sms, st) : launch_backward<64>(a, p, nnz, dev.device, dev.sms, st);
+    return p->head_dim == 128 ? launch_backward<128>(a, p, nnz, dev.device, dev.sms, mma, st)
+                              : launch_backward<64>(a, p, nnz, dev.device, dev.sms, mma, st);
 }

@@ -30,6 +30,7 @@ struct BackwardArgs {
     int64_t N;
     int32_t nqb, batch, Hq, Hkv, G;
     int32_t npairs;            // head pairs per KV group: ceil(G / 2)
+    int32_t prezero;           // dK and dV are cleared by the preparation (else: where needed, by the dQ kernel)
     float scale, scale_log2;
     long long wait_cycles;     // limit of every barrier wait of the tensor-core kernels
 };
@@ -40,10 +41,11 @@ struct BackwardArgs {
 // its chunks is empty.
 struct BackwardChunk {
     int32_t j, e0, e1;  // key block, extent in row_idx (empty: e0 == e1)
+    int32_t parts;      // chunks of the column
 };
 __device__ __forceinline__ BackwardChunk backward_chunk_at(const BackwardArgs &a, int32_t c)
 {
-    BackwardChunk r = {0, 0, 0};
+    BackwardChunk r = {0, 0, 0, 0};
     int32_t lo = 0, hi = a.nqb;  // last column whose slots start at or before c
     while (hi - lo > 1) {
         const int32_t mid = (lo + hi) >> 1;
@@ -53,6 +55,7 @@ __device__ __forceinline__ BackwardChunk backward_chunk_at(const BackwardArgs &a
     const int32_t p0 = __ldg(a.col_ptr + lo), cnt = __ldg(a.col_ptr + lo + 1) - p0;
     const int32_t parts = (cnt + a.chunk - 1) / a.chunk, part = c - (p0 / a.chunk + lo);
     r.j = lo;
+    r.parts = parts;
     if (part < parts) {
         r.e0 = p0 + (int32_t)((int64_t)cnt * part / parts);
         r.e1 = p0 + (int32_t)((int64_t)cnt * (part + 1) / parts);
@@ -60,7 +63,7 @@ __device__ __forceinline__ BackwardChunk backward_chunk_at(const BackwardArgs &a
     return r;
 }
 
-// On tcgen05: dQ, and for head_dim 128 dK and dV (delta and the transposed lists are already in the workspace).
+// dQ, dK and dV on tcgen05 (delta and the transposed lists are already in the workspace).
 pa_status launch_backward_sm100(const BackwardArgs &a, const pa_prefill_params *p, int64_t nnz, int device, int sms,
                                 cudaStream_t st);
 

@@ -1,7 +1,7 @@
 // Backward pass of the block-sparse attention (derivatives of Eq. (1), Section 3.1, under the
 // key-block lists of Algorithm 1, Section 3.3) on the sm_100a tensor cores, head_dim 64 and 128.
 //
-// Two kernels (dK / dV: head_dim 128 only).  The dQ kernel's warps:
+// Two persistent kernels with the same skeleton:
 //   warp 0       TMA producer (bf16 tiles, 128-byte swizzle, into rings of shared-memory stages); it also draws
 //                the CTA's next work item from a counter in memory and hands it to the other warps through a
 //                small ring in shared memory
@@ -9,18 +9,16 @@
 //   warp 2       tensor-memory allocation, issuer of dP
 //   warp 3       issuer of the second products
 //   warps 4-19   four compute warpgroups
-//   warps 20-23  epilogue: the finished dQ out of tensor memory and out to global memory
-// The dK / dV kernel has the same warps 0-3 (without items: a CTA has one), and two compute warpgroups (warps
-// 4-11) which take alternate steps.
+//   warps 20-23  (dQ kernel) epilogue: the finished dQ out of tensor memory and out to global memory
 // A step is one query block and one (dK / dV kernel) or two (dQ kernel) of its key blocks for a pair of query
 // heads stacked on the 64 tokens of the query block: a 128-row tile, as in the forward kernel.  Per step the
 // tensor cores produce S = Q K^T and dP = dO V^T (fp32, tensor memory); the compute warps (thread = tile row =
-// TMEM lane) turn them into P = exp2(S scale log2e - LSE log2e) and dS = P (dP - delta), rounded
+// TMEM lane, 32 keys each) turn them into P = exp2(S scale log2e - LSE log2e) and dS = P (dP - delta), rounded
 // to bf16; the second products accumulate in tensor memory.
 //
 //   dq_kernel   an item is a (query block, head pair): walks the row's key blocks two at a time; dS goes back
 //               into tensor memory as the A operand of dQ += dS K (128 x D accumulator)
-//   dkv_kernel  one CTA per (chunk of a key block's listing query blocks, KV head): walks the chunk for every
+//   dkv_kernel  an item is a (chunk of a key block's listing query blocks, KV head): walks the chunk for every
 //               head pair of the group; P and dS go to shared memory as the B operands of dV^T += dO^T P and
 //               dK^T += Q^T dS (feature x key accumulators: the A operands are the dO and Q tiles read
 //               feature-major)
@@ -36,10 +34,10 @@
 #include "tensor_map.cuh"
 
 // Registers per thread by role.  A warpgroup asking for more than the pool holds would wait for ever: the dK / dV
-// kernel starts 384 threads x 168, the dQ kernel 768 x 80.
-#define PA_BWD_REG_CTRL 56
-#define PA_BWD_REG_COMP 216
-static_assert(4 * PA_BWD_REG_CTRL + 8 * PA_BWD_REG_COMP <= 12 * 168, "register split exceeds the CTA's registers");
+// kernel starts 640 threads x 96, the dQ kernel 768 x 80.
+#define PA_DKV_REG_CTRL 56
+#define PA_DKV_REG_COMP 104
+static_assert(4 * PA_DKV_REG_CTRL + 16 * PA_DKV_REG_COMP <= 20 * 96, "register split exceeds the CTA's registers");
 #define PA_DQ_REG_CTRL 48
 #define PA_DQ_REG_COMP 96
 #define PA_DQ_REG_EPI 48
@@ -47,7 +45,7 @@ static_assert(4 * PA_DQ_REG_CTRL + 16 * PA_DQ_REG_COMP + 4 * PA_DQ_REG_EPI <= 24
 
 namespace pa {
 
-constexpr int kTcThreads = 384;
+constexpr int kDkvThreads = 640;
 constexpr int kDqThreads = 768;
 constexpr int kCompWarps = 16;
 constexpr uint32_t kTcTmemCols = 512;
@@ -121,7 +119,7 @@ __device__ __forceinline__ float bwd_neg_lse2(float lse)
 // keys a thread, and the next step's products run beside the arithmetic.  Q and dO have one buffer each as well:
 // the next item's tiles arrive while the last step is computed and its dQ product runs.
 // Measured, 28 / 4 heads at 32K tokens: 586 us, where steps of one block with two S and dP buffers took 661; 64
-// features, 16 / 4 heads, 2 x 8K tokens: 109 us, where the warp-level MMA kernel took 218.
+// features, 16 / 4 heads, 2 x 8K tokens: 106 us, where the warp-level MMA kernel took 218.
 template <int D>
 struct DqCfg {
     static constexpr int kDH = D / 64;
@@ -466,6 +464,22 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
         const int row = quad * 32 + lane, qrow = row & 63;
         const uint32_t t_lane = tmem_base + ((uint32_t)(quad * 32) << 16);
         const uint32_t patch = smem_base + C::kOut + (uint32_t)quad * 8192u + (uint32_t)lane * 128u;
+        // Key blocks whose dK and dV are added up from several chunks, or that nobody lists, start from zero
+        // (where the preparation has not cleared everything).
+        if (!a.prezero)
+            for (int32_t j = blockIdx.x; j < a.nqb; j += gridDim.x) {
+                const int32_t cnt = __ldg(a.col_ptr + j + 1) - __ldg(a.col_ptr + j);
+                if (cnt > 0 && cnt <= a.chunk) continue;
+                const int64_t tok0 = (int64_t)j * kBwdBlk, toks = a.N - tok0 < kBwdBlk ? a.N - tok0 : kBwdBlk;
+                const int64_t words = toks * a.Hkv * (D / 4);
+                for (int32_t b = 0; b < a.batch; ++b) {
+                    const int64_t at = ((int64_t)b * a.N + tok0) * a.Hkv * (D / 4);
+                    for (int64_t x = row; x < words; x += 128) {
+                        reinterpret_cast<float4 *>(a.dk)[at + x] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        reinterpret_cast<float4 *>(a.dv)[at + x] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    }
+                }
+            }
         uint32_t kq = 0, np = 0;
         bool ok = true;
         for (uint32_t k = 0; ok; ++k) {
@@ -534,76 +548,120 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
 }
 
 // ------------------------------------------------------------------------------------- dK, dV
-struct DkvSmem {
-    static constexpr uint32_t kK = 0;                        // two halves of 64 keys x 128 B
-    static constexpr uint32_t kV = kK + 2 * kKeyTile;
-    static constexpr uint32_t kQG = kV + 2 * kKeyTile;       // stage: Q (two halves of 128 rows x 128 B), then dO
-    static constexpr uint32_t kStage = 4 * kRowTile;
-    static constexpr uint32_t kPD = kQG + 2 * kStage;        // buffer: P (128 rows x 64 keys), then dS
-    static constexpr uint32_t kBuf = 2 * kRowTile;
-    static constexpr uint32_t kBars = kPD + 2 * kBuf;
-    static constexpr uint32_t kAlloc = kBars + 512 + 1024;
+// Bound by how long a stage of Q and dO stays occupied: loaded, read by S and dP, and read again by the second
+// products once P and dS exist.  So everything that lengthens that round is cut or overlapped: Q and dO have
+// rings and barriers of their own (dO is free after dV, Q after dK), P is handed over before dS, which is computed
+// while dV runs, two warpgroups share a step (32 keys each) and two more work on the next one.  head_dim 128:
+// three Q stages, two of dO, one buffer for P and dS each.  head_dim 64: four stages, two P / dS buffers; a
+// stage's Q and dO tiles lie side by side and are read as ONE 128-row A operand [Q | dO]^T against B = [P | dS]
+// (N = 128): two quadrants of the product are dV^T and dK^T, the other two are not used, and the eight MMAs take
+// 512 clk where two products of 64 accumulator rows take 768.
+// Measured, 28 / 4 heads at 32K tokens: 848 us, where one CTA per chunk with two common Q + dO stages and two
+// warpgroups took 985; 64 features, 16 / 4 heads, 2 x 8K tokens: 177 us, where the warp-level MMA kernel took 306.
+template <int D>
+struct DkvCfg {
+    static constexpr int kDH = D / 64;
+    static constexpr int kQStages = D == 128 ? 3 : 4, kGStages = D == 128 ? 2 : 4, kPBufs = D == 128 ? 1 : 2;
+    static constexpr uint32_t kBlkTile = kDH * kKeyTile, kTile = kDH * kRowTile;
+    static constexpr uint32_t kK = 0, kV = kBlkTile;
+    static constexpr uint32_t kQ = 2 * kBlkTile;
+    static constexpr uint32_t kPitch = D == 128 ? kTile : 2 * kTile;  // from stage to stage
+    static constexpr uint32_t kG = D == 128 ? kQ + kQStages * kTile : kQ + kTile;
+    static constexpr uint32_t kPD = kQ + (kQStages + kGStages) * kTile;  // buffer: P (128 rows x 64 keys), then dS
+    static constexpr uint32_t kBars = kPD + kPBufs * 2 * kRowTile;
+    static constexpr uint32_t kAlloc = kBars + kBarArea + 1024;
     static_assert(kAlloc <= 227 * 1024, "shared memory budget");
-};
-enum : uint32_t {
-    KV_KV_FULL = 0,
-    KV_QG_FULL = 1, KV_QG_EMPTY = 3,  // [stage]
-    KV_SD_FULL = 5,                   // [buffer]: S and dP of a step are in tensor memory
-    KV_S_TAKEN = 7,                   // [buffer]: the group has them in registers
-    KV_PD_FULL = 9,                   // [buffer]: P and dS are in shared memory
-    KV_DONE = 11,
-    KV_BAR_COUNT = 12
+    enum : uint32_t {
+        KV_FULL, KV_EMPTY,
+        Q_FULL, Q_EMPTY = Q_FULL + kQStages,
+        G_FULL = Q_EMPTY + kQStages, G_EMPTY = G_FULL + kGStages,
+        S_FULL = G_EMPTY + kGStages, S_TAKEN = S_FULL + 2,     // [step parity]
+        DP_FULL = S_TAKEN + 2, DP_TAKEN = DP_FULL + 2,
+        P_FULL = DP_TAKEN + 2, DS_FULL = P_FULL + kPBufs,      // [P / dS buffer]
+        P_FREE = DS_FULL + kPBufs, DS_FREE = P_FREE + 2,       // [step parity]: that step's product has read it
+        ACC_FULL = DS_FREE + 2, ACC_FREE,                      // the item's dK^T and dV^T are complete / have been read
+        ITEM_FULL, ITEM_EMPTY = ITEM_FULL + kItemRing, COUNT = ITEM_EMPTY + kItemRing
+    };
+    static_assert(COUNT * 8 <= kBarBytes, "barrier area");
+    // Tensor memory columns: S at 128 b, dP at 128 b + 64 (b = step parity); accumulators at 256: dK^T, then dV^T
+    // (head_dim 128), or the product with [P | dS] (head_dim 64).
+    static constexpr uint32_t kColAcc = 256;
 };
 
-__global__ void __launch_bounds__(kTcThreads, 1)
+template <int D>
+__global__ void __launch_bounds__(kDkvThreads, 1)
 dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmG,
-           const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const BackwardArgs a)
+           const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const BackwardArgs a,
+           const uint32_t n_items)
 {
-    constexpr int D = 128;
-    using SM = DkvSmem;
-    const BackwardChunk chunk = backward_chunk_at(a, (int32_t)blockIdx.x);
-    const int32_t j = chunk.j, e0 = chunk.e0, e1 = chunk.e1;
-    if (e0 >= e1) return;  // (the grid is an upper bound on the number of chunks)
+    using C = DkvCfg<D>;
+    constexpr int DH = C::kDH;
+    constexpr uint32_t NQ = C::kQStages, NG = C::kGStages, NP = C::kPBufs;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *smem = smem_raw + (smem_base - ptx::smem_u32(smem_raw));
-    const uint32_t bars = smem_base + SM::kBars;
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + SM::kBars + KV_BAR_COUNT * 8);
-    volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + SM::kBars + KV_BAR_COUNT * 8 + 8);
+    const uint32_t bars = smem_base + C::kBars;
+    BwdTail *tail = reinterpret_cast<BwdTail *>(smem + C::kBars + kBarBytes);
+    volatile int *abort_flag = &tail->abort_flag;
     auto bar = [&](uint32_t idx) { return bars + idx * 8u; };
     auto wait_bar = [&](uint32_t b_, uint32_t parity, int code) {
         return ptx::mbar_wait_bounded(b_, parity, abort_flag, a.status, code, a.wait_cycles, (int)PA_ERR_TIMEOUT);
     };
+    auto wait_warp = [&](uint32_t b_, uint32_t parity, int code) {
+        return __all_sync(0xffffffffu, wait_bar(b_, parity, code)) != 0;
+    };
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int hk = blockIdx.y, b = blockIdx.z;
-    const int n = (e1 - e0) * a.npairs;  // steps: listing query blocks x head pairs (pairs fastest); at least one
+    auto read_item = [&](uint32_t k, BwdItem &w) {
+        if (!wait_warp(bar(C::ITEM_FULL + k % kItemRing), (k / kItemRing) & 1, 31)) return false;
+        w = tail->items[k % kItemRing];
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(bar(C::ITEM_EMPTY + k % kItemRing));
+        return true;
+    };
 
     if (threadIdx.x == 0) {
-        ptx::mbar_init(bar(KV_KV_FULL), 1);
-        for (int s = 0; s < 2; ++s) {
-            ptx::mbar_init(bar(KV_QG_FULL + s), 1);
-            ptx::mbar_init(bar(KV_QG_EMPTY + s), 1);
-            ptx::mbar_init(bar(KV_SD_FULL + s), 2);  // one commit from each of the S and dP issuers
-            ptx::mbar_init(bar(KV_S_TAKEN + s), 4);
-            ptx::mbar_init(bar(KV_PD_FULL + s), 4);
+        ptx::mbar_init(bar(C::KV_FULL), 1);
+        ptx::mbar_init(bar(C::KV_EMPTY), 2);  // one commit from each of the S and dP issuers
+        for (uint32_t s = 0; s < NQ; ++s) {
+            ptx::mbar_init(bar(C::Q_FULL + s), 1);
+            ptx::mbar_init(bar(C::Q_EMPTY + s), 1);
         }
-        ptx::mbar_init(bar(KV_DONE), 1);
-        *abort_flag = 0;
+        for (uint32_t s = 0; s < NG; ++s) {
+            ptx::mbar_init(bar(C::G_FULL + s), 1);
+            ptx::mbar_init(bar(C::G_EMPTY + s), 2);  // read by dP and by dV, in either order
+        }
+        for (int s = 0; s < 2; ++s) {
+            ptx::mbar_init(bar(C::S_FULL + s), 1);
+            ptx::mbar_init(bar(C::DP_FULL + s), 1);
+            ptx::mbar_init(bar(C::S_TAKEN + s), kCompWarps / 2);
+            ptx::mbar_init(bar(C::DP_TAKEN + s), kCompWarps / 2);
+            ptx::mbar_init(bar(C::P_FREE + s), 1);
+            ptx::mbar_init(bar(C::DS_FREE + s), 1);
+        }
+        for (uint32_t s = 0; s < NP; ++s) {
+            ptx::mbar_init(bar(C::P_FULL + s), kCompWarps / 2);
+            ptx::mbar_init(bar(C::DS_FULL + s), kCompWarps / 2);
+        }
+        ptx::mbar_init(bar(C::ACC_FULL), 1);
+        ptx::mbar_init(bar(C::ACC_FREE), kCompWarps);
+        for (uint32_t r = 0; r < kItemRing; ++r) {
+            ptx::mbar_init(bar(C::ITEM_FULL + r), 1);
+            ptx::mbar_init(bar(C::ITEM_EMPTY + r), kDkvThreads / 32 - 1);
+        }
+        tail->abort_flag = 0;
         ptx::fence_barrier_init();
         ptx::fence_proxy_async_smem();
     }
     if (warp == 2) {
-        ptx::tmem_alloc(ptx::smem_u32(tmem_slot), kTcTmemCols);
+        ptx::tmem_alloc(ptx::smem_u32(&tail->tmem), kTcTmemCols);
         ptx::tmem_relinquish();
     }
     ptx::tc_fence_before_sync();
     __syncthreads();
     ptx::tc_fence_after_sync();
-    const uint32_t tmem_base = *tmem_slot;
-    // Tensor memory columns: buffer b: S at 128 b, dP at 128 b + 64; dK^T at 256, dV^T at 320 (64 keys each).
-    constexpr uint32_t kColDk = 256, kColDv = 320;
+    const uint32_t tmem_base = tail->tmem;
 
-    if (warp < 4) ptx::setmaxnreg_dec<PA_BWD_REG_CTRL>();
+    if (warp < 4) ptx::setmaxnreg_dec<PA_DKV_REG_CTRL>();
     if (warp == 0) {
         // -------------------------------------------------------------- TMA producer
         if (lane == 0) {
@@ -611,24 +669,72 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             ptx::prefetch_tensormap(&tmG);
             ptx::prefetch_tensormap(&tmK);
             ptx::prefetch_tensormap(&tmV);
-            ptx::mbar_expect_tx(bar(KV_KV_FULL), 4 * kKeyTile);
-            for (int dh = 0; dh < 2; ++dh) {
-                ptx::tma_load_4d(smem_base + SM::kK + dh * kKeyTile, &tmK, bar(KV_KV_FULL), dh * 64, j * kBwdBlk, hk, b);
-                ptx::tma_load_4d(smem_base + SM::kV + dh * kKeyTile, &tmV, bar(KV_KV_FULL), dh * 64, j * kBwdBlk, hk, b);
-            }
-            int32_t i = 0;
-            for (int e = 0, hp = 0; e < n; ++e) {
-                if (hp == 0) i = __ldg(a.row_idx + e0 + e / a.npairs);
-                const uint32_t st = e & 1;
-                if (e >= 2 && !wait_bar(bar(KV_QG_EMPTY + st), ((e >> 1) - 1) & 1, 2)) break;
-                ptx::mbar_expect_tx(bar(KV_QG_FULL + st), SM::kStage);
-                const uint32_t dst = smem_base + SM::kQG + st * SM::kStage;
-                const int h0 = hk * a.G + 2 * hp;
-                for (int dh = 0; dh < 2; ++dh) {
-                    ptx::tma_load_4d(dst + dh * kRowTile, &tmQ, bar(KV_QG_FULL + st), dh * 64, i * kBwdBlk, h0, b);
-                    ptx::tma_load_4d(dst + 2 * kRowTile + dh * kRowTile, &tmG, bar(KV_QG_FULL + st), dh * 64, i * kBwdBlk, h0, b);
+            // Items: chunk slots in column order (the sink block's long column first), and within a slot the KV
+            // heads and batch entries; slots without work are passed over.
+            uint32_t it = blockIdx.x;
+            auto next_item = [&](BwdItem &w) {
+                w.n = -1;
+                const uint32_t per_slot = (uint32_t)(a.Hkv * a.batch);
+                while (it < n_items) {
+                    const uint32_t slot = it / per_slot, yz = it - slot * per_slot;
+                    const BackwardChunk ch = backward_chunk_at(a, (int32_t)slot);
+                    it = gridDim.x + (uint32_t)atomicAdd(a.status + kBwdDkvCounter, 1);
+                    if (ch.e0 >= ch.e1) continue;
+                    w.blk = ch.j;
+                    w.e0 = ch.e0;
+                    w.n = ch.e1 - ch.e0;
+                    w.parts = ch.parts;
+                    w.b = (int32_t)(yz / (uint32_t)a.Hkv);
+                    w.hk = (int32_t)(yz % (uint32_t)a.Hkv);
+                    return;
                 }
-                if (++hp == a.npairs) hp = 0;
+            };
+            auto publish = [&](uint32_t k, const BwdItem &w) {
+                const uint32_t r = k % kItemRing;
+                if (k >= kItemRing && !wait_bar(bar(C::ITEM_EMPTY + r), (k / kItemRing - 1) & 1, 32)) return false;
+                tail->items[r] = w;
+                ptx::mbar_arrive(bar(C::ITEM_FULL + r));
+                return true;
+            };
+            uint32_t c = 0;  // steps so far
+            BwdItem w, wn;
+            w.hp = w.pad = wn.hp = wn.pad = 0;
+            next_item(w);
+            bool ok = publish(0, w);
+            for (uint32_t k = 0; w.n >= 0 && ok; ++k) {
+                next_item(wn);
+                ok = publish(k + 1, wn);
+                if (!ok) break;
+                auto load_rows = [&](uint32_t dst, const CUtensorMap *tm, uint32_t full, uint32_t empty, uint32_t stages, int32_t i,
+                                     int h0, int code) {
+                    const uint32_t st = c % stages;
+                    if (c >= stages && !wait_bar(bar(empty + st), (c / stages - 1) & 1, code)) return false;
+                    ptx::mbar_expect_tx(bar(full + st), C::kTile);
+                    for (int dh = 0; dh < DH; ++dh)
+                        ptx::tma_load_4d(smem_base + dst + st * C::kPitch + dh * kRowTile, tm, bar(full + st), dh * 64,
+                                         i * kBwdBlk, h0, w.b);
+                    return true;
+                };
+                int32_t i = __ldg(a.row_idx + w.e0);
+                for (int x = 0; x < w.n && ok; ++x) {
+                    const int32_t in = x + 1 < w.n ? __ldg(a.row_idx + w.e0 + x + 1) : 0;
+                    for (int hp = 0; hp < a.npairs && ok; ++hp, ++c) {
+                        const int h0 = w.hk * a.G + 2 * hp;
+                        ok = load_rows(C::kQ, &tmQ, C::Q_FULL, C::Q_EMPTY, NQ, i, h0, 33);
+                        if (ok && x == 0 && hp == 0) {
+                            ok = k == 0 || wait_bar(bar(C::KV_EMPTY), (k - 1) & 1, 34);
+                            if (!ok) break;
+                            ptx::mbar_expect_tx(bar(C::KV_FULL), 2 * C::kBlkTile);
+                            for (int dh = 0; dh < DH; ++dh) {
+                                ptx::tma_load_4d(smem_base + C::kK + dh * kKeyTile, &tmK, bar(C::KV_FULL), dh * 64, w.blk * kBwdBlk, w.hk, w.b);
+                                ptx::tma_load_4d(smem_base + C::kV + dh * kKeyTile, &tmV, bar(C::KV_FULL), dh * 64, w.blk * kBwdBlk, w.hk, w.b);
+                            }
+                        }
+                        ok = ok && load_rows(C::kG, &tmG, C::G_FULL, C::G_EMPTY, NG, i, h0, 35);
+                    }
+                    i = in;
+                }
+                w = wn;
             }
         }
         __syncwarp();
@@ -638,157 +744,246 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         const bool is_dp = __shfl_sync(0xffffffffu, warp, 0) == 2;
         constexpr uint32_t idesc_s = idesc_bf16(128, 64, 0, 0);    // both operands K-major
         // A = Q (S) or dO (dP) of the stage; B = the key block's K or V.
-        const uint32_t b_lo = ((smem_base + (is_dp ? SM::kV : SM::kK)) >> 4) | (1u << 16);
-        bool ok = __all_sync(0xffffffffu, wait_bar(bar(KV_KV_FULL), 0, 1));
-        for (int e = 0; e < n && ok; ++e) {
-            const uint32_t bf = e & 1;
-            ok = __all_sync(0xffffffffu, wait_bar(bar(KV_QG_FULL + bf), (e >> 1) & 1, 3));
-            if (ok && e >= 2) ok = __all_sync(0xffffffffu, wait_bar(bar(KV_S_TAKEN + bf), ((e >> 1) - 1) & 1, 4));
-            if (!ok) break;
-            ptx::tc_fence_after_sync();
-            if (leader) {
-                const uint32_t a_lo = ((smem_base + SM::kQG + bf * SM::kStage + (is_dp ? 2 * kRowTile : 0u)) >> 4) | (1u << 16);
-                const uint32_t t_d = tmem_base + 128 * bf + (is_dp ? 64u : 0u);
-#pragma unroll
-                for (int kk = 0; kk < D / 16; ++kk)
-                    ptx::umma_ss_lohi(t_d, a_lo + (((kk / 4) * kRowTile + (kk % 4) * 32) >> 4), kDescHi,
-                                      b_lo + (((kk / 4) * kKeyTile + (kk % 4) * 32) >> 4), kDescHi, idesc_s, kk > 0 ? 1u : 0u);
-                ptx::umma_commit(bar(KV_SD_FULL + bf));
-            }
-            __syncwarp();
-        }
-    } else if (warp == 3) {
-        // -------------------------------------------------------------- tcgen05 issuer of dV^T and dK^T
-        // (its own warp: a Q / dO stage is free for the next load only when these have read it, and a
-        // single in-order issuer put them behind the next step's S and dP)
-        const bool leader = ptx::elect_one();
-        constexpr uint32_t idesc_t = idesc_bf16(128, 64, 1, 1);    // A feature-contiguous, B key-contiguous
+        const uint32_t b_lo = ((smem_base + (is_dp ? C::kV : C::kK)) >> 4) | (1u << 16);
+        const uint32_t rows_full = is_dp ? C::G_FULL : C::Q_FULL, stages = is_dp ? NG : NQ;
+        const uint32_t out_full = is_dp ? C::DP_FULL : C::S_FULL, out_taken = is_dp ? C::DP_TAKEN : C::S_TAKEN;
+        const uint32_t t_base = __shfl_sync(0xffffffffu, tmem_base + (is_dp ? 64u : 0u), 0);
+        uint32_t c = 0, st = 0, round = 0;  // step, its stage, how often the ring has come round
         bool ok = true;
-        for (int e1 = 0; e1 < n && ok; ++e1) {
-            {
-                const uint32_t bf = e1 & 1;
-                ok = __all_sync(0xffffffffu, wait_bar(bar(KV_PD_FULL + bf), (e1 >> 1) & 1, 5));
+        for (uint32_t k = 0; ok; ++k) {
+            BwdItem w;
+            ok = read_item(k, w);
+            const int n = __shfl_sync(0xffffffffu, w.n, 0) * a.npairs;
+            if (!ok || n < 0) break;
+            ok = wait_warp(bar(C::KV_FULL), k & 1, 36);
+            for (int e = 0; e < n && ok; ++e, ++c) {
+                const uint32_t bf = c & 1;
+                ok = wait_warp(bar(rows_full + st), round & 1, 37);
+                if (ok && c >= 2) ok = wait_warp(bar(out_taken + bf), ((c >> 1) - 1) & 1, 38);
                 if (!ok) break;
                 ptx::tc_fence_after_sync();
                 if (leader) {
-                    // A = the dO (Q) tile read feature-contiguous (its two 64-feature halves are kRowTile
-                    // apart), B = P (dS) read key-contiguous; 16 tile rows per MMA, 2048 bytes further each.
-                    const uint32_t qa = ((smem_base + SM::kQG + bf * SM::kStage) >> 4) | ((kRowTile >> 4) << 16);
-                    const uint32_t ga = qa + ((2 * kRowTile) >> 4);
-                    const uint32_t pb = ((smem_base + SM::kPD + bf * SM::kBuf) >> 4) | ((kRowTile >> 4) << 16);
-                    const uint32_t db = pb + (kRowTile >> 4);
+                    const uint32_t a_lo = ((smem_base + (is_dp ? C::kG : C::kQ) + st * C::kPitch) >> 4) | (1u << 16);
+                    const uint32_t t_d = t_base + 128 * bf;
+#pragma unroll
+                    for (int kk = 0; kk < D / 16; ++kk)
+                        ptx::umma_ss_lohi(t_d, a_lo + (((kk / 4) * kRowTile + (kk % 4) * 32) >> 4), kDescHi,
+                                          b_lo + (((kk / 4) * kKeyTile + (kk % 4) * 32) >> 4), kDescHi, idesc_s, kk > 0 ? 1u : 0u);
+                    ptx::umma_commit(bar(out_full + bf));
+                    if (is_dp) ptx::umma_commit(bar(C::G_EMPTY + st));
+                    if (e == n - 1) ptx::umma_commit(bar(C::KV_EMPTY));
+                }
+                __syncwarp();
+                if (++st == stages) {
+                    st = 0;
+                    ++round;
+                }
+            }
+        }
+    } else if (warp == 3) {
+        // -------------------------------------------------------------- tcgen05 issuer of dV^T and dK^T
+        // A = the dO (Q) tile read feature-contiguous (64-feature halves kRowTile apart), B = P (dS) read
+        // key-contiguous; 16 tile rows per MMA, 2048 bytes further each.
+        const bool leader = ptx::elect_one();
+        constexpr uint32_t idesc_t = idesc_bf16(128, D == 128 ? 64 : 128, 1, 1);
+        const uint32_t t_base = __shfl_sync(0xffffffffu, tmem_base + C::kColAcc, 0);
+        uint32_t c = 0;
+        bool ok = true;
+        for (uint32_t k = 0; ok; ++k) {
+            BwdItem w;
+            ok = read_item(k, w);
+            const int n = __shfl_sync(0xffffffffu, w.n, 0) * a.npairs;
+            if (!ok || n < 0) break;
+            // The previous item's accumulators must have been read.
+            if (k > 0) ok = wait_warp(bar(C::ACC_FREE), (k - 1) & 1, 39);
+            for (int e = 0; e < n && ok; ++e, ++c) {
+                const uint32_t sq = c % NQ, sg = c % NG, pb = c % NP, pphase = (c / NP) & 1;
+                const uint32_t qa = ((smem_base + C::kQ + sq * C::kPitch) >> 4) | ((kRowTile >> 4) << 16);
+                const uint32_t ga = ((smem_base + C::kG + sg * C::kPitch) >> 4) | ((kRowTile >> 4) << 16);
+                const uint32_t pp = ((smem_base + C::kPD + pb * 2 * kRowTile) >> 4) | ((kRowTile >> 4) << 16);
+                if (D == 128) {
+                    // (P needs S only, so dO may not have landed yet when it is there)
+                    ok = wait_warp(bar(C::G_FULL + sg), (c / NG) & 1, 47);
+                    ok = ok && wait_warp(bar(C::P_FULL + pb), pphase, 40);
+                    if (!ok) break;
+                    ptx::tc_fence_after_sync();
+                    if (leader) {
+#pragma unroll
+                        for (int kk = 0; kk < 8; ++kk)
+                            ptx::umma_ss_lohi(t_base + 64, ga + ((kk * 2048) >> 4), kDescHi, pp + ((kk * 2048) >> 4), kDescHi,
+                                              idesc_t, (e > 0 || kk > 0) ? 1u : 0u);
+                        ptx::umma_commit(bar(C::G_EMPTY + sg));
+                        ptx::umma_commit(bar(C::P_FREE + (c & 1)));
+                    }
+                    __syncwarp();
+                } else {
+                    ok = wait_warp(bar(C::P_FULL + pb), pphase, 40);
+                }
+                ok = ok && wait_warp(bar(C::DS_FULL + pb), pphase, 41);
+                if (!ok) break;
+                ptx::tc_fence_after_sync();
+                if (leader) {
+                    const uint32_t bb = D == 128 ? pp + (kRowTile >> 4) : pp;
 #pragma unroll
                     for (int kk = 0; kk < 8; ++kk)
-                        ptx::umma_ss_lohi(tmem_base + kColDv, ga + ((kk * 2048) >> 4), kDescHi, pb + ((kk * 2048) >> 4), kDescHi,
-                                          idesc_t, (e1 > 0 || kk > 0) ? 1u : 0u);
-#pragma unroll
-                    for (int kk = 0; kk < 8; ++kk)
-                        ptx::umma_ss_lohi(tmem_base + kColDk, qa + ((kk * 2048) >> 4), kDescHi, db + ((kk * 2048) >> 4), kDescHi,
-                                          idesc_t, (e1 > 0 || kk > 0) ? 1u : 0u);
-                    ptx::umma_commit(bar(KV_QG_EMPTY + bf));  // (frees the P / dS buffer as well)
-                    if (e1 == n - 1) ptx::umma_commit(bar(KV_DONE));
+                        ptx::umma_ss_lohi(t_base, qa + ((kk * 2048) >> 4), kDescHi, bb + ((kk * 2048) >> 4), kDescHi, idesc_t,
+                                          (e > 0 || kk > 0) ? 1u : 0u);
+                    ptx::umma_commit(bar(C::Q_EMPTY + sq));
+                    ptx::umma_commit(bar(C::DS_FREE + (c & 1)));
+                    if (D == 64) {
+                        ptx::umma_commit(bar(C::G_EMPTY + sg));
+                        ptx::umma_commit(bar(C::P_FREE + (c & 1)));
+                    }
+                    if (e == n - 1) ptx::umma_commit(bar(C::ACC_FULL));
                 }
                 __syncwarp();
             }
         }
-    } else if (warp >= 4) {
-        // -------------------------------------------------------------- compute groups
-        ptx::setmaxnreg_inc<PA_BWD_REG_COMP>();
-        const int wg = (warp - 4) >> 2, quad = warp & 3;
+    } else {
+        // -------------------------------------------------------------- compute warps
+        // Warpgroup wg: steps of parity wg & 1, keys 32 (wg >> 1) .. + 31.
+        ptx::setmaxnreg_inc<PA_DKV_REG_COMP>();
+        const int wg = (warp - 4) >> 2, quad = warp & 3, par = wg & 1, half = wg >> 1;
         const int row = quad * 32 + lane, qrow = row & 63;
         const uint32_t t_lane = tmem_base + ((uint32_t)(quad * 32) << 16);
-        // Row statistics of a step for this thread's row: LSE and delta; +inf / 0 for a row without
-        // weights (beyond the sequence, padding head, empty row): P = 0.  Nothing here uses a loaded
-        // value (the thread would wait for it on the spot): the query block index is loaded two of
-        // this group's steps ahead, LSE and delta one step ahead, and they are looked at when the step
-        // they belong to begins.
-        auto step_block = [&](int e) { return e < n ? __ldg(a.row_idx + e0 + e / a.npairs) : -1; };
-        auto request_stats = [&](int e, int32_t i, float &lse, float &delta, bool &diag) {
-            lse = INFINITY;
-            delta = 0.f;
-            diag = false;
-            if (e >= n) return;
-            const int head_local = 2 * (e % a.npairs) + (row >> 6);
-            const int64_t q = (int64_t)i * kBwdBlk + qrow;
-            diag = i == j;
-            if (head_local < a.G && q < a.N) {
-                const int64_t at = ((int64_t)b * a.Hq + hk * a.G + head_local) * a.N + q;
-                lse = __ldg(a.lse + at);
-                delta = __ldg(a.delta + at);
+        const uint64_t scale2 = ptx::pack_f32x2(a.scale_log2, a.scale_log2);
+        // Row statistics of this thread's next step, LSE and delta, are requested one of its steps ahead and its
+        // query block's index one more, across items as well; nothing uses a loaded value on the spot.
+        struct Place {
+            int x, hp;  // place in the chunk's list, head pair
+        };
+        auto advance = [&](Place &p, int steps) {
+            p.hp += steps;
+            while (p.hp >= a.npairs) {
+                p.hp -= a.npairs;
+                ++p.x;
             }
         };
-        float lse_raw, delta, lse_raw_n, delta_n;
-        bool diag, diag_n;
-        int32_t i_next = step_block(wg + 2);
-        request_stats(wg, step_block(wg), lse_raw, delta, diag);
-        const uint32_t p_row = smem_base + SM::kPD + wg * SM::kBuf + (uint32_t)row * 128u;
-        bool ok = true;
-        for (int e = wg; e < n; e += 2) {
-            const int32_t i_next2 = step_block(e + 4);
-            request_stats(e + 2, i_next, lse_raw_n, delta_n, diag_n);  // (in flight during this step)
-            ok = __all_sync(0xffffffffu, wait_bar(bar(KV_SD_FULL + wg), (e >> 1) & 1, 6));
+        auto block_at = [&](const BwdItem &w, const Place &p) { return p.x < w.n ? __ldg(a.row_idx + w.e0 + p.x) : -1; };
+        float lse_n = INFINITY, delta_n = 0.f;
+        auto request = [&](const BwdItem &w, int32_t i, const Place &p) {
+            lse_n = INFINITY;
+            delta_n = 0.f;
+            const int head_local = 2 * p.hp + (row >> 6);
+            const int64_t q = (int64_t)i * kBwdBlk + qrow;
+            if (i >= 0 && head_local < a.G && q < a.N) {
+                const int64_t at = ((int64_t)w.b * a.Hq + w.hk * a.G + head_local) * a.N + q;
+                lse_n = __ldg(a.lse + at);
+                delta_n = __ldg(a.delta + at);
+            }
+        };
+        uint32_t c = 0;      // step number at the item's start
+        BwdItem w, wn;
+        bool ok = read_item(0, w);
+        Place next = {0, 0};  // of the step after the current one
+        int32_t i_next = -1;
+        if (ok && w.n >= 0) {
+            advance(next, par);
+            i_next = block_at(w, next);
+            request(w, i_next, next);
+        }
+        for (uint32_t k = 0; ok && w.n >= 0; ++k) {
+            const int n = w.n * a.npairs;
+            // (next, i_next, lse_n and delta_n are those of this warp's first step in the item)
+            for (uint32_t e = (c ^ (uint32_t)par) & 1; e < (uint32_t)n; e += 2) {
+                const uint32_t cc = c + e, pb = cc % NP;
+                const bool diag = i_next == w.blk;
+                const float neg_lse2 = bwd_neg_lse2(lse_n);
+                const uint64_t neg_lse2_2 = ptx::pack_f32x2(neg_lse2, neg_lse2), neg_delta2 = ptx::pack_f32x2(-delta_n, -delta_n);
+                advance(next, 2);
+                i_next = block_at(w, next);
+                uint32_t x32[32];
+                uint64_t p[16];
+                ok = wait_warp(bar(C::S_FULL + par), (cc >> 1) & 1, 42);
+                if (!ok) break;
+                ptx::tc_fence_after_sync();
+                ptx::tmem_ld32(t_lane + 128 * par + 32 * half, x32);
+                ptx::tmem_wait_ld();
+                ptx::tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(bar(C::S_TAKEN + par));
+                request(w, i_next, next);  // (in flight during this step)
+                // Algorithm 1's causal term acts inside the diagonal pair only.
+                bwd_p(x32, diag, qrow - 32 * half, scale2, neg_lse2_2, p);
+                // The P / dS buffer was read by the products of step cc - NP.  (Their barriers alternate by step
+                // parity: with one buffer a warpgroup would otherwise wait for every other phase of a barrier only,
+                // whose parity cannot tell two phases ahead from none.)
+                if (cc >= NP) {
+                    ok = wait_warp(bar(C::P_FREE + ((cc - NP) & 1)), ((cc - NP) >> 1) & 1, 43);
+                    if (!ok) break;
+                }
+                // 16-byte chunk q of tile row r sits at chunk position q ^ (r & 7) (128-byte swizzle).
+                const uint32_t p_row = smem_base + C::kPD + pb * 2 * kRowTile + (uint32_t)row * 128u;
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    ptx::st_shared_v4(p_row + (uint32_t)(((4 * half + q) ^ (row & 7)) << 4), bwd_cvt(p[4 * q]), bwd_cvt(p[4 * q + 1]),
+                                      bwd_cvt(p[4 * q + 2]), bwd_cvt(p[4 * q + 3]));
+                ptx::fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(bar(C::P_FULL + pb));
+                ok = wait_warp(bar(C::DP_FULL + par), (cc >> 1) & 1, 44);
+                if (!ok) break;
+                ptx::tc_fence_after_sync();
+                ptx::tmem_ld32(t_lane + 128 * par + 64 + 32 * half, x32);
+                ptx::tmem_wait_ld();
+                ptx::tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(bar(C::DP_TAKEN + par));
+                if (cc >= NP) {
+                    ok = wait_warp(bar(C::DS_FREE + ((cc - NP) & 1)), ((cc - NP) >> 1) & 1, 45);
+                    if (!ok) break;
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    uint32_t v[4];
+#pragma unroll
+                    for (int y = 0; y < 4; ++y)
+                        v[y] = bwd_cvt(bwd_ds(p[4 * q + y], x32[8 * q + 2 * y], x32[8 * q + 2 * y + 1], neg_delta2));
+                    ptx::st_shared_v4(p_row + kRowTile + (uint32_t)(((4 * half + q) ^ (row & 7)) << 4), v[0], v[1], v[2], v[3]);
+                }
+                ptx::fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(bar(C::DS_FULL + pb));
+            }
+            if (!ok) break;
+            // The next item's first step, requested ahead of this item's output.
+            c += (uint32_t)n;
+            ok = read_item(k + 1, wn);
+            if (!ok) break;
+            next = {0, 0};
+            advance(next, (int)((c ^ (uint32_t)par) & 1));
+            i_next = block_at(wn, next);
+            // ---- output: thread = feature, one key per register, 128 contiguous bytes per warp instruction.  A
+            // key block of one chunk is written, the parts of others are added up in memory.
+            ok = wait_warp(bar(C::ACC_FULL), k & 1, 46);
             if (!ok) break;
             ptx::tc_fence_after_sync();
-            uint32_t s[64], dp[64];
-            ptx::tmem_ld32(t_lane + 128 * wg, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
-            ptx::tmem_ld32(t_lane + 128 * wg + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
-            ptx::tmem_ld32(t_lane + 128 * wg + 64, *reinterpret_cast<uint32_t(*)[32]>(&dp[0]));
-            ptx::tmem_ld32(t_lane + 128 * wg + 96, *reinterpret_cast<uint32_t(*)[32]>(&dp[32]));
+            constexpr int kKeys = D == 128 ? 32 : 16;  // keys per warp
+            const bool is_dk = D == 128 ? par == 0 : quad < 2;
+            const int key0 = D == 128 ? 32 * half : 16 * wg, feature = D == 128 ? row : row & 63;
+            const uint32_t col = C::kColAcc + (D == 128 ? (is_dk ? 0u : 64u) : (is_dk ? 64u : 0u)) + key0;
+            uint32_t acc[kKeys];
+            if (D == 128) ptx::tmem_ld32(t_lane + col, *reinterpret_cast<uint32_t(*)[32]>(acc));
+            else ptx::tmem_ld16(t_lane + col, *reinterpret_cast<uint32_t(*)[16]>(acc));
             ptx::tmem_wait_ld();
             ptx::tc_fence_before_sync();
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(bar(KV_S_TAKEN + wg));
-            // (The P / dS buffer is free: the second products of step e - 2 that read it had completed
-            // before this step's Q and dO could be loaded into the stage they also read, and so before
-            // the S and dP waited for above were issued.)
-            // Algorithm 1's causal term acts inside the diagonal pair only.
-            const int lim = diag ? qrow : 63;
-            const float lse2 = (lse_raw == -INFINITY || lse_raw == INFINITY) ? INFINITY : lse_raw * 1.4426950408889634f;
+            if (lane == 0) ptx::mbar_arrive(bar(C::ACC_FREE));
+            request(wn, i_next, next);
+            const int64_t tok0 = (int64_t)w.blk * kBwdBlk + key0;
+            float *dst = (is_dk ? a.dk : a.dv) + (((int64_t)w.b * a.N + tok0) * a.Hkv + w.hk) * D + feature;
+            const float f = is_dk ? a.scale : 1.0f;
+            const int64_t pitch = (int64_t)a.Hkv * D;
+            if (w.parts == 1) {
 #pragma unroll
-            for (int ch = 0; ch < 8; ++ch) {
-                uint32_t pp[4], pd[4];
+                for (int x = 0; x < kKeys; ++x)
+                    if (tok0 + x < a.N) dst[x * pitch] = __uint_as_float(acc[x]) * f;
+            } else {
 #pragma unroll
-                for (int x = 0; x < 4; ++x) {
-                    float p[2], ds[2];
-#pragma unroll
-                    for (int y = 0; y < 2; ++y) {
-                        const int col = 8 * ch + 2 * x + y;
-                        p[y] = (col <= lim) ? ptx::ex2(fmaf(__uint_as_float(s[col]), a.scale_log2, -lse2)) : 0.f;
-                        ds[y] = p[y] * (__uint_as_float(dp[col]) - delta);
-                    }
-                    pp[x] = ptx::cvt_bf16x2(p[0], p[1]);
-                    pd[x] = ptx::cvt_bf16x2(ds[0], ds[1]);
-                }
-                // 16-byte chunk ch of tile row r sits at chunk position ch ^ (r & 7) (128-byte swizzle).
-                const uint32_t off = (uint32_t)((ch ^ (row & 7)) << 4);
-                ptx::st_shared_v4(p_row + off, pp[0], pp[1], pp[2], pp[3]);
-                ptx::st_shared_v4(p_row + kRowTile + off, pd[0], pd[1], pd[2], pd[3]);
+                for (int x = 0; x < kKeys; ++x)
+                    if (tok0 + x < a.N) atomicAdd(dst + x * pitch, __uint_as_float(acc[x]) * f);
             }
-            ptx::fence_proxy_async_smem();
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(bar(KV_PD_FULL + wg));
-            lse_raw = lse_raw_n;
-            delta = delta_n;
-            diag = diag_n;
-            i_next = i_next2;
-        }
-        // Group 0 adds dK^T (x scale), group 1 dV^T: thread = feature, one key per register.
-        if (ok) ok = __all_sync(0xffffffffu, wait_bar(bar(KV_DONE), 0, 8));
-        if (ok) {
-            ptx::tc_fence_after_sync();
-            float *dst = (wg == 0 ? a.dk : a.dv) + (((int64_t)b * a.N + (int64_t)j * kBwdBlk) * a.Hkv + hk) * D + row;
-            const float f = wg == 0 ? a.scale : 1.0f;
-#pragma unroll
-            for (int ch = 0; ch < 2; ++ch) {
-                uint32_t acc[32];
-                ptx::tmem_ld32(t_lane + (wg == 0 ? kColDk : kColDv) + 32 * ch, acc);
-                ptx::tmem_wait_ld();
-#pragma unroll
-                for (int x = 0; x < 32; ++x) {
-                    const int key = 32 * ch + x;
-                    if ((int64_t)j * kBwdBlk + key < a.N) atomicAdd(dst + (int64_t)key * a.Hkv * D, __uint_as_float(acc[x]) * f);
-                }
-            }
+            w = wn;
         }
     }
 
@@ -807,25 +1002,10 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
 
 // ---------------------------------------------------------------------------------- host side
 template <int D>
-static pa_status launch_dq(const BackwardArgs &a, const pa_prefill_params *p, const CUtensorMap &tmQ, const CUtensorMap &tmG,
-                           const CUtensorMap &tmK, const CUtensorMap &tmV, int device, int sms, cudaStream_t st)
-{
-    CUtensorMap tmDq;
-    const TensorMapKey out = {a.dq, p->seq_len, (int64_t)a.Hq * D, D, (int64_t)a.N * a.Hq * D, device, D, a.Hq, p->batch, 1, 32, 1};
-    if (pa_status s = get_tensor_map(out, "dq", &tmDq)) return s;
-    const int64_t n_items = (int64_t)a.nqb * a.Hkv * a.npairs * a.batch;
-    if (n_items > (int64_t)0x3fffffff) return fail(PA_ERR_SHAPE, "too many work items (%lld)", (long long)n_items);
-    dq_kernel<D><<<(unsigned)(n_items < sms ? n_items : sms), kDqThreads, DqCfg<D>::kAlloc, st>>>(tmQ, tmG, tmK, tmV, tmDq, a,
-                                                                                                  (uint32_t)n_items);
-    PA_CUDA_OK(cudaGetLastError());
-    return PA_OK;
-}
-
-template <int D>
 static pa_status launch_tc(const BackwardArgs &a, const pa_prefill_params *p, int64_t nnz, int device, int sms, cudaStream_t st)
 {
     // Tensor maps (cached per buffer and shape): a Q or dO box holds the two heads of a tile, a K or V box one head.
-    CUtensorMap tmQ, tmG, tmK, tmV;
+    CUtensorMap tmQ, tmG, tmK, tmV, tmDq;
     auto map_of = [&](const void *base, int heads, const pa_strides &s, int box_heads, const char *what, CUtensorMap *m) {
         const TensorMapKey key = {base, p->seq_len, s.seq, s.head, s.batch, device, D, heads, p->batch, box_heads, kBwdBlk, 0};
         return get_tensor_map(key, what, m);
@@ -834,21 +1014,25 @@ static pa_status launch_tc(const BackwardArgs &a, const pa_prefill_params *p, in
     if (pa_status s = map_of(a.d_o, a.Hq, p->o, 2, "d_o", &tmG)) return s;
     if (pa_status s = map_of(a.k, a.Hkv, p->k, 1, "k", &tmK)) return s;
     if (pa_status s = map_of(a.v, a.Hkv, p->v, 1, "v", &tmV)) return s;
+    const TensorMapKey out = {a.dq, p->seq_len, (int64_t)a.Hq * D, D, (int64_t)a.N * a.Hq * D, device, D, a.Hq, p->batch, 1, 32, 1};
+    if (pa_status s = get_tensor_map(out, "dq", &tmDq)) return s;
     if (device_once_begin(device, D == 128 ? ONCE_BACKWARD_TC_ATTR : ONCE_BACKWARD_TC_ATTR_64)) {
         const cudaError_t e1 = cudaFuncSetAttribute(dq_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DqCfg<D>::kAlloc);
-        const cudaError_t e2 = cudaFuncSetAttribute(dkv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DkvSmem::kAlloc);
+        const cudaError_t e2 = cudaFuncSetAttribute(dkv_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DkvCfg<D>::kAlloc);
         if (e1 != cudaSuccess || e2 != cudaSuccess) {
             device_once_reset(device, D == 128 ? ONCE_BACKWARD_TC_ATTR : ONCE_BACKWARD_TC_ATTR_64);
             return fail(PA_ERR_CUDA, "cudaFuncSetAttribute failed: %s", cudaGetErrorString(e1 != cudaSuccess ? e1 : e2));
         }
     }
-    if (pa_status s = launch_dq<D>(a, p, tmQ, tmG, tmK, tmV, device, sms, st)) return s;
-    if (D == 128) {
-        // (an upper bound on the number of chunks; CTAs beyond the real count return at once)
-        const int64_t max_chunks = nnz / a.chunk + a.nqb;
-        dkv_kernel<<<dim3((unsigned)max_chunks, (unsigned)a.Hkv, (unsigned)a.batch), kTcThreads, DkvSmem::kAlloc, st>>>(tmQ, tmG, tmK, tmV, a);
-        PA_CUDA_OK(cudaGetLastError());
-    }
+    const int64_t dq_items = (int64_t)a.nqb * a.Hkv * a.npairs * a.batch;
+    const int64_t dkv_items = (nnz / a.chunk + a.nqb) * a.Hkv * a.batch;  // (chunk slots, some of them empty)
+    if (dq_items > (int64_t)0x3fffffff || dkv_items > (int64_t)0x3fffffff)
+        return fail(PA_ERR_SHAPE, "too many work items (%lld, %lld)", (long long)dq_items, (long long)dkv_items);
+    dq_kernel<D><<<(unsigned)(dq_items < sms ? dq_items : sms), kDqThreads, DqCfg<D>::kAlloc, st>>>(tmQ, tmG, tmK, tmV, tmDq, a,
+                                                                                                    (uint32_t)dq_items);
+    dkv_kernel<D><<<(unsigned)(dkv_items < sms ? dkv_items : sms), kDkvThreads, DkvCfg<D>::kAlloc, st>>>(tmQ, tmG, tmK, tmV, a,
+                                                                                                         (uint32_t)dkv_items);
+    PA_CUDA_OK(cudaGetLastError());
     return PA_OK;
 }
 

@@ -40,7 +40,7 @@ struct EnvSwitches {
     int decode_stages;   // PA_DECODE_STAGES=1..8, 0 = chosen from the problem size
     int decode_ctas_per_sm;  // PA_DECODE_CTAS_PER_SM=n: size of the persistent grid (default 2 per SM)
     int validate;        // PA_VALIDATE=1
-    int backward_mma;    // PA_BACKWARD_PATH=mma: the warp-level MMA kernels for head_dim 128 too
+    int backward_mma;    // PA_BACKWARD_PATH=mma: the warp-level MMA kernels
 };
 EnvSwitches env_switches();
 
