@@ -1,8 +1,10 @@
-"""ctypes binding of libpowerattn.so: argument marshalling only.
+"""Binding of libpowerattn.so: argument marshalling only.
 
 Every function has the name and meaning of its C entry point in include/powerattn.h.  Torch
 tensors are used as device buffers (data_ptr) and for the current CUDA stream; all computation
-happens inside the library's kernels.  Importing this module without a built library fails.
+happens inside the library's kernels.  The attention and cache calls forward to the CPython module
+_calls (csrc/calls.cpp), the others go through ctypes.  Importing this module without a built library
+fails.
 """
 from __future__ import annotations
 
@@ -134,6 +136,11 @@ def _load() -> ctypes.CDLL:
 lib = _load()
 
 
+from . import _calls  # noqa: E402  (linked against the library loaded above)
+
+_calls.set_error(PaError)
+
+
 def _check(status: int) -> None:
     if status != PA_OK:
         raise PaError(status, lib.pa_last_error_message().decode())
@@ -260,64 +267,22 @@ def pa_prefill(q, k, v, row_ptr, col_idx, o=None, lse=None, workspace=None, bloc
                softmax_scale: float = 0.0, o_dtype=torch.bfloat16, nnz: Optional[int] = None):
     """q [batch, N, Hq, D], k, v [batch, N, Hkv, D] bf16 device tensors; CSR int32 device tensors.
     Returns (o, lse, workspace); outputs and scratch are allocated here when not passed in."""
-    batch, seq, hq, d = q.shape
-    if o is None:
-        o = torch.empty((batch, seq, hq, d), dtype=o_dtype, device=q.device)
-    if lse is None:
-        lse = torch.empty((batch, hq, seq), dtype=torch.float32, device=q.device)
-    params = prefill_params(q, k, v, o, block, softmax_scale)
-    if workspace is None:
-        workspace = torch.empty(max(pa_prefill_workspace_bytes(params), 16), dtype=torch.uint8, device=q.device)
-    _check(lib.pa_prefill(ctypes.byref(params), _ptr(q), _ptr(k), _ptr(v), _ptr(row_ptr), _ptr(col_idx),
-                          col_idx.numel() if nnz is None else nnz, _ptr(o), _ptr(lse), _ptr(workspace),
-                          workspace.numel(), _stream()))
-    return o, lse, workspace
+    return _calls.prefill(q, k, v, row_ptr, col_idx, o, lse, workspace, block, softmax_scale, o_dtype, nnz)
 
 
 def pa_prefill_varlen(q, k, v, cu_seqlens, max_seq_len: int, row_ptr, col_idx, o=None, lse=None, workspace=None,
                       block: int = 64, softmax_scale: float = 0.0, o_dtype=torch.bfloat16):
     """Packed sequences: q [total, Hq, D], k, v [total, Hkv, D] bf16, cu_seqlens int32 [batch + 1] on the
     device.  Returns (o [total, Hq, D], lse [Hq, total], workspace)."""
-    total, hq, d = q.shape
-    assert q.stride(2) == 1 and k.stride(2) == 1 and v.stride(2) == 1 and cu_seqlens.dtype == torch.int32
-    if o is None:
-        o = torch.empty((total, hq, d), dtype=o_dtype, device=q.device)
-    if lse is None:
-        lse = torch.empty((hq, total), dtype=torch.float32, device=q.device)
-    st = lambda t: pa_strides(0, t.stride(0), t.stride(1))
-    params = pa_prefill_params(cu_seqlens.numel() - 1, hq, k.shape[1], d, max_seq_len, block, float(softmax_scale),
-                               st(q), st(k), st(v), st(o), PA_F32 if o.dtype == torch.float32 else PA_BF16)
-    if workspace is None:
-        workspace = torch.empty(max(pa_prefill_workspace_bytes(params), 16), dtype=torch.uint8, device=q.device)
-    _check(lib.pa_prefill_varlen(ctypes.byref(params), _ptr(q), _ptr(k), _ptr(v), _ptr(cu_seqlens), total,
-                                 _ptr(row_ptr), _ptr(col_idx), col_idx.numel(), _ptr(o), _ptr(lse), _ptr(workspace),
-                                 workspace.numel(), _stream()))
-    return o, lse, workspace
+    return _calls.prefill_varlen(q, k, v, cu_seqlens, max_seq_len, row_ptr, col_idx, o, lse, workspace, block,
+                                 softmax_scale, o_dtype)
 
 
 def pa_prefill_backward(q, k, v, o, lse, d_o, row_ptr, col_idx, dq=None, dk=None, dv=None, workspace=None,
                         block: int = 64, softmax_scale: float = 0.0):
     """Gradients of pa_prefill: q, k, v, o (bf16) and lse as in the forward call, d_o bf16 with o's
     strides.  Returns (dq, dk, dv, workspace), fp32 contiguous, allocated here when not passed in."""
-    batch, seq, hq, d = q.shape
-    hkv = k.shape[2]
-    assert d_o.stride() == o.stride() and o.dtype == torch.bfloat16 and d_o.dtype == torch.bfloat16
-    if dq is None:
-        dq = torch.empty((batch, seq, hq, d), dtype=torch.float32, device=q.device)
-    if dk is None:
-        dk = torch.empty((batch, seq, hkv, d), dtype=torch.float32, device=q.device)
-    if dv is None:
-        dv = torch.empty((batch, seq, hkv, d), dtype=torch.float32, device=q.device)
-    params = prefill_params(q, k, v, o, block, softmax_scale)
-    nnz = col_idx.numel()
-    if workspace is None:
-        workspace = torch.empty(int(lib.pa_prefill_backward_workspace_bytes(ctypes.byref(params), nnz)) + 256,
-                                dtype=torch.uint8, device=q.device)
-    ws_ptr = (workspace.data_ptr() + 255) & ~255
-    _check(lib.pa_prefill_backward(ctypes.byref(params), _ptr(q), _ptr(k), _ptr(v), _ptr(o), _ptr(lse), _ptr(d_o),
-                                   _ptr(row_ptr), _ptr(col_idx), nnz, _ptr(dq), _ptr(dk), _ptr(dv),
-                                   ctypes.c_void_p(ws_ptr), workspace.numel() - (ws_ptr - workspace.data_ptr()), _stream()))
-    return dq, dk, dv, workspace
+    return _calls.prefill_backward(q, k, v, o, lse, d_o, row_ptr, col_idx, dq, dk, dv, workspace, block, softmax_scale)
 
 
 def pa_prefill_status(workspace: torch.Tensor) -> int:
@@ -343,18 +308,8 @@ def pa_decode(q, k_cache, v_cache, cache_lens, window_blocks: int, sink_blocks: 
               workspace=None, block: int = 64, softmax_scale: float = 0.0, o_dtype=torch.bfloat16):
     """q [batch, Hq, D] bf16, caches [batch, max_len, Hkv, D] bf16, cache_lens int32 [batch], all on
     the device.  Returns (o, lse, workspace)."""
-    batch, hq, d = q.shape
-    if o is None:
-        o = torch.empty((batch, hq, d), dtype=o_dtype, device=q.device)
-    if lse is None:
-        lse = torch.empty((batch, hq), dtype=torch.float32, device=q.device)
-    params = decode_params(q, k_cache, v_cache, window_blocks, sink_blocks, block, softmax_scale, o.dtype)
-    if workspace is None:
-        workspace = torch.empty(max(pa_decode_workspace_bytes(params), 16), dtype=torch.uint8, device=q.device)
-    assert cache_lens.dtype == torch.int32 and q.is_contiguous() and o.is_contiguous()
-    _check(lib.pa_decode(ctypes.byref(params), _ptr(q), _ptr(k_cache), _ptr(v_cache), _ptr(cache_lens),
-                         _ptr(o), _ptr(lse), _ptr(workspace), workspace.numel(), _stream()))
-    return o, lse, workspace
+    return _calls.decode(q, k_cache, v_cache, cache_lens, window_blocks, sink_blocks, o, lse, workspace, block,
+                         softmax_scale, o_dtype)
 
 
 def pa_decode_block_list(cache_len: int, block: int, window_blocks: int, sink_blocks: int,
@@ -402,28 +357,13 @@ def pa_decode_paged_workspace_bytes(params: pa_paged_params) -> int:
 def pa_decode_paged(q, k_pool, v_pool, block_table, cache_lens, window_blocks: int, sink_blocks: int, o=None,
                     lse=None, workspace=None, block: int = 64, softmax_scale: float = 0.0, o_dtype=torch.bfloat16):
     """pa_decode against a pool of 64-token pages.  Returns (o, lse, workspace)."""
-    batch, hq, d = q.shape
-    if o is None:
-        o = torch.empty((batch, hq, d), dtype=o_dtype, device=q.device)
-    if lse is None:
-        lse = torch.empty((batch, hq), dtype=torch.float32, device=q.device)
-    params = paged_params(q, k_pool, v_pool, block_table, window_blocks, sink_blocks, block, softmax_scale, o.dtype)
-    if workspace is None:
-        workspace = torch.empty(max(pa_decode_paged_workspace_bytes(params), 16), dtype=torch.uint8, device=q.device)
-    assert cache_lens.dtype == torch.int32 and q.is_contiguous() and o.is_contiguous()
-    _check(lib.pa_decode_paged(ctypes.byref(params), _ptr(q), _ptr(k_pool), _ptr(v_pool), _ptr(block_table),
-                               _ptr(cache_lens), _ptr(o), _ptr(lse), _ptr(workspace), workspace.numel(), _stream()))
-    return o, lse, workspace
+    return _calls.decode_paged(q, k_pool, v_pool, block_table, cache_lens, window_blocks, sink_blocks, o, lse, workspace,
+                               block, softmax_scale, o_dtype)
 
 
 def pa_kv_append(k_new, v_new, k_pool, v_pool, block_table, cache_lens, block: int = 64) -> None:
     """k_new, v_new [batch, Hkv, D] go to position cache_lens[b] of each sequence; cache_lens grows by one."""
-    batch, hkv, d = k_new.shape
-    assert k_new.is_contiguous() and v_new.is_contiguous() and cache_lens.dtype == torch.int32
-    params = pa_paged_params(batch, hkv, hkv, d, block, 0, 0, k_pool.shape[0], block_table.shape[1], 0.0,
-                             _strides4(k_pool), _strides4(v_pool), PA_BF16)
-    _check(lib.pa_kv_append(ctypes.byref(params), _ptr(k_new), _ptr(v_new), _ptr(k_pool), _ptr(v_pool),
-                            _ptr(block_table), _ptr(cache_lens), _stream()))
+    _calls.kv_append(k_new, v_new, k_pool, v_pool, block_table, cache_lens, block)
 
 
 PA_DECODE_STATIC_SCRATCH_BYTES = 4 << 20
@@ -438,8 +378,5 @@ def pa_decode_static(q, k_cache, v_cache, cache_lens, window_blocks: int, sink_b
     PA_DECODE_STATIC_SCRATCH_BYTES raise PaError(PA_ERR_WORKSPACE).  Calls that overlap on the GPU
     share (and would corrupt) the one built-in scratch array: keep them on one stream.
     """
-    assert cache_lens.dtype == torch.int32 and q.is_contiguous() and o.is_contiguous()
-    params = decode_params(q, k_cache, v_cache, window_blocks, sink_blocks, block, softmax_scale, o.dtype)
-    _check(lib.pa_decode_static(ctypes.byref(params), _ptr(q), _ptr(k_cache), _ptr(v_cache), _ptr(cache_lens),
-                                _ptr(o), _ptr(lse), _stream()))
+    _calls.decode_static(q, k_cache, v_cache, cache_lens, window_blocks, sink_blocks, o, lse, block, softmax_scale)
     return o, lse

@@ -557,7 +557,7 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
 // (N = 128): two quadrants of the product are dV^T and dK^T, the other two are not used, and the eight MMAs take
 // 512 clk where two products of 64 accumulator rows take 768.
 // Measured, 28 / 4 heads at 32K tokens: 848 us, where one CTA per chunk with two common Q + dO stages and two
-// warpgroups took 985; 64 features, 16 / 4 heads, 2 x 8K tokens: 177 us, where the warp-level MMA kernel took 306.
+// warpgroups took 985; 64 features, 16 / 4 heads, 2 x 8K tokens: 177 us, where the warp-level MMA kernel took about 300.
 template <int D>
 struct DkvCfg {
     static constexpr int kDH = D / 64;

@@ -1,0 +1,44 @@
+"""The CPython module behind the attention calls: broken preconditions raise before anything is launched, and
+leave the interpreter usable (no GPU is present in this run)."""
+import pytest
+import torch
+
+
+@pytest.fixture(scope="module")
+def pa():
+    import paper_2503_03588_b200 as pa_
+
+    return pa_
+
+
+def _bf16(*shape):
+    return torch.zeros(shape, dtype=torch.bfloat16)
+
+
+def test_broken_preconditions_raise(pa):
+    q, kc, lens = _bf16(1, 4, 128), _bf16(1, 64, 2, 128), torch.ones(1, dtype=torch.int32)
+    with pytest.raises(AssertionError):
+        pa.pa_decode(q, kc, kc, lens.long(), 5, 1)                     # lengths of another type
+    with pytest.raises(AssertionError):
+        pa.pa_decode(q.transpose(1, 2), kc, kc, lens, 5, 1)            # q not contiguous
+    with pytest.raises(AssertionError):
+        pa.pa_decode_paged(q, kc, kc, torch.zeros((1, 1), dtype=torch.int64), lens, 5, 1)
+    with pytest.raises(AssertionError):
+        pa.pa_prefill(_bf16(1, 64, 4, 256)[..., ::2], kc, kc, lens, lens)   # head_dim not contiguous
+    with pytest.raises(AssertionError):
+        pa.pa_prefill_backward(_bf16(1, 64, 4, 128), kc, kc, _bf16(1, 64, 4, 128).float(), lens, _bf16(1, 64, 4, 128), lens, lens)
+    with pytest.raises(TypeError):
+        pa.pa_decode(q, None, kc, lens, 5, 1)
+    with pytest.raises(TypeError):
+        pa.pa_decode(q, kc, kc, lens, "5", 1)
+    with pytest.raises(OverflowError):
+        pa.pa_decode(q, kc, kc, lens, 1 << 40, 1)
+
+
+def test_library_errors_carry_status_and_message(pa):
+    if torch.cuda.is_available():
+        stream_error = pa.PaError
+    else:
+        stream_error = (pa.PaError, RuntimeError)  # (without a driver torch itself may refuse to name a stream)
+    with pytest.raises(stream_error):
+        pa.pa_decode(_bf16(1, 4, 96), _bf16(1, 64, 2, 96), _bf16(1, 64, 2, 96), torch.ones(1, dtype=torch.int32), 5, 1)
