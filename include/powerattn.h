@@ -79,7 +79,7 @@ pa_status pa_layout_size(int64_t seq_len, int32_t block, int32_t window_blocks,
 
 /* Writes the CSR on the device.  row_ptr: device int32[n_qblocks + 1]; col_idx: device
  * int32[col_capacity], col_capacity >= nnz from pa_layout_size (else PA_ERR_LAYOUT, nothing
- * launched).  Three small kernels are enqueued on `stream`; no scratch memory is used. */
+ * launched).  One small kernel is enqueued on `stream`; no scratch memory is used. */
 pa_status pa_build_layout(int64_t seq_len, int32_t block, int32_t window_blocks,
                           int32_t sink_blocks, int32_t *row_ptr, int32_t *col_idx,
                           int64_t col_capacity, void *stream);
@@ -126,7 +126,7 @@ pa_status pa_tile_layout_size(int64_t seq_len, int32_t block, int32_t window_blo
 
 /* Writes the tile CSR on the device.  row_ptr: device int32[n_qtiles + 1]; col_idx: device
  * int32[col_capacity], col_capacity >= nnz from pa_tile_layout_size (else PA_ERR_LAYOUT, nothing
- * launched).  Three small kernels are enqueued on `stream`; no scratch memory is used. */
+ * launched).  One small kernel is enqueued on `stream`; no scratch memory is used. */
 pa_status pa_build_tile_layout(int64_t seq_len, int32_t block, int32_t window_blocks,
                                int32_t sink_blocks, int32_t tile, int32_t *row_ptr,
                                int32_t *col_idx, int64_t col_capacity, void *stream);

@@ -185,15 +185,7 @@ def pa_build_layout(seq_len: int, block: int, window_blocks: int, sink_blocks: i
                     row_ptr: Optional[torch.Tensor] = None, col_idx: Optional[torch.Tensor] = None,
                     device="cuda"):
     """Returns (row_ptr, col_idx) int32 device tensors (allocated here when not passed in)."""
-    nqb, nnz = pa_layout_size(seq_len, block, window_blocks, sink_blocks)
-    if row_ptr is None:
-        row_ptr = torch.empty(nqb + 1, dtype=torch.int32, device=device)
-    if col_idx is None:
-        col_idx = torch.empty(nnz, dtype=torch.int32, device=device)
-    assert row_ptr.dtype == torch.int32 and col_idx.dtype == torch.int32 and row_ptr.numel() >= nqb + 1
-    _check(lib.pa_build_layout(seq_len, block, window_blocks, sink_blocks, _ptr(row_ptr), _ptr(col_idx),
-                               col_idx.numel(), _stream()))
-    return row_ptr, col_idx
+    return _calls.build_layout(seq_len, block, window_blocks, sink_blocks, None, row_ptr, col_idx, device)
 
 
 def pa_window_layout_size(seq_len: int, block: int, window_blocks: int, sink_blocks: int) -> Tuple[int, int]:
@@ -206,14 +198,7 @@ def pa_build_window_layout(seq_len: int, block: int, window_blocks: int, sink_bl
                            row_ptr: Optional[torch.Tensor] = None, col_idx: Optional[torch.Tensor] = None,
                            device="cuda"):
     """Sliding-window layout (window + sink blocks, no power-of-two term) as int32 device tensors."""
-    nqb, nnz = pa_window_layout_size(seq_len, block, window_blocks, sink_blocks)
-    if row_ptr is None:
-        row_ptr = torch.empty(nqb + 1, dtype=torch.int32, device=device)
-    if col_idx is None:
-        col_idx = torch.empty(nnz, dtype=torch.int32, device=device)
-    _check(lib.pa_build_window_layout(seq_len, block, window_blocks, sink_blocks, _ptr(row_ptr), _ptr(col_idx),
-                                      col_idx.numel(), _stream()))
-    return row_ptr, col_idx
+    return _calls.build_layout(seq_len, block, window_blocks, sink_blocks, 0, row_ptr, col_idx, device)
 
 
 def pa_reach_counts(row_ptr, col_idx, start: int, max_steps: int):
@@ -241,15 +226,9 @@ def pa_build_tile_layout(seq_len: int, block: int, window_blocks: int, sink_bloc
                          device="cuda"):
     """Returns (row_ptr, col_idx) int32 device tensors of the mask with `block`-token blocks listed by
     `tile`-token tiles (allocated here when not passed in)."""
-    nqt, nnz = pa_tile_layout_size(seq_len, block, window_blocks, sink_blocks, tile)
-    if row_ptr is None:
-        row_ptr = torch.empty(nqt + 1, dtype=torch.int32, device=device)
-    if col_idx is None:
-        col_idx = torch.empty(nnz, dtype=torch.int32, device=device)
-    assert row_ptr.dtype == torch.int32 and col_idx.dtype == torch.int32 and row_ptr.numel() >= nqt + 1
-    _check(lib.pa_build_tile_layout(seq_len, block, window_blocks, sink_blocks, tile, _ptr(row_ptr),
-                                    _ptr(col_idx), col_idx.numel(), _stream()))
-    return row_ptr, col_idx
+    if tile < 1:
+        pa_tile_layout_size(seq_len, block, window_blocks, sink_blocks, tile)  # raises
+    return _calls.build_layout(seq_len, block, window_blocks, sink_blocks, tile, row_ptr, col_idx, device)
 
 
 def prefill_params(q, k, v, o, block: int = 64, softmax_scale: float = 0.0) -> pa_prefill_params:

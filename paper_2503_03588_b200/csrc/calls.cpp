@@ -9,6 +9,7 @@
 
 #include <ATen/ops/empty.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Device.h>
 #include <torch/csrc/Dtype.h>
 #include <torch/csrc/autograd/python_variable.h>
 
@@ -286,6 +287,45 @@ PyObject *kv_append(PyObject *const *x)
     Py_RETURN_NONE;
 }
 
+// seq_len, block, window_blocks, sink_blocks, tile, row_ptr, col_idx, device; tile None: pa_build_layout, 0:
+// pa_build_window_layout, else pa_build_tile_layout
+PyObject *build_layout(PyObject *const *x)
+{
+    const int64_t seq_len = integer(x[0]);
+    const int32_t block = integer32(x[1]), window = integer32(x[2]), sink = integer32(x[3]);
+    const int32_t tile = x[4] == Py_None ? -1 : integer32(x[4]);
+    int32_t rows = 0;
+    int64_t nnz = 0;
+    run([&] {
+        return tile < 0    ? pa_layout_size(seq_len, block, window, sink, &rows, &nnz)
+               : tile == 0 ? pa_window_layout_size(seq_len, block, window, sink, &rows, &nnz)
+                           : pa_tile_layout_size(seq_len, block, window, sink, tile, &rows, &nnz);
+    });
+    auto fresh = [&](int64_t n) {
+        c10::Device device(c10::kCUDA);
+        if (THPDevice_Check(x[7])) {
+            device = reinterpret_cast<THPDevice *>(x[7])->device;
+        } else {
+            const char *name = PyUnicode_AsUTF8(x[7]);
+            if (!name) throw Raised();
+            device = c10::Device(std::string(name));
+        }
+        return at::empty({n}, at::TensorOptions().dtype(at::kInt).device(device));
+    };
+    const Out row_ptr(x[5], [&] { return fresh((int64_t)rows + 1); });
+    const Out col_idx(x[6], [&] { return fresh(nnz); });
+    expect(is_int32(row_ptr.t) && is_int32(col_idx.t) && row_ptr.t.numel() >= (int64_t)rows + 1,
+           "row_ptr and col_idx are int32, row_ptr has a row more than the layout");
+    run([&] {
+        int32_t *rp = (int32_t *)row_ptr.ptr(), *ci = (int32_t *)col_idx.ptr();
+        const int64_t room = col_idx.t.numel();
+        return tile < 0    ? pa_build_layout(seq_len, block, window, sink, rp, ci, room, stream())
+               : tile == 0 ? pa_build_window_layout(seq_len, block, window, sink, rp, ci, room, stream())
+                           : pa_build_tile_layout(seq_len, block, window, sink, tile, rp, ci, room, stream());
+    });
+    return Py_BuildValue("(NN)", row_ptr.object(), col_idx.object());
+}
+
 // Wraps a function of N positional arguments.
 template <int N, PyObject *(*F)(PyObject *const *)>
 PyObject *call(PyObject *, PyObject *const *args, Py_ssize_t n)
@@ -313,7 +353,8 @@ PyObject *set_error(PyObject *, PyObject *type)
 PyMethodDef methods[] = {
     {"set_error", set_error, METH_O, nullptr}, PA_METHOD(prefill, 12),       PA_METHOD(prefill_varlen, 13),
     PA_METHOD(prefill_backward, 14),           PA_METHOD(decode, 12),        PA_METHOD(decode_static, 10),
-    PA_METHOD(decode_paged, 13),               PA_METHOD(kv_append, 7),      {nullptr, nullptr, 0, nullptr}};
+    PA_METHOD(decode_paged, 13),               PA_METHOD(kv_append, 7),
+    PA_METHOD(build_layout, 8),                {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_calls", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
 }  // namespace

@@ -126,14 +126,9 @@ __global__ void __launch_bounds__(kDecThreads) decode_block_kernel(const DecodeA
     const bool valid = len >= 1 && len <= a.max_len;
     const int64_t p = len - 1;
     const int32_t row = valid ? (int32_t)(p / kDecBlock) : 0;  // max_len / 64 fits in 31 bits (host check)
-    // Every thread walks the (short) list; the chunk-th entry is this CTA's key block.
-    int32_t jblk = -1;
-    int n = 0;
-    if (valid)
-        n = for_each_key_block_t<int32_t>(row, a.W, a.S, [&](int pos, int32_t j) {
-            if (pos == chunk) jblk = j;
-        });
-    if (chunk >= n) return;
+    const LayoutRow list = layout_row(row, a.W, a.S);
+    if (!valid || chunk >= list.n) return;
+    const int32_t jblk = (int32_t)layout_entry(list, chunk);  // this CTA's key block
 
     {
         const int n_keys = jblk == row ? (int)(p % kDecBlock) + 1 : kDecBlock;
@@ -268,7 +263,7 @@ __global__ void __launch_bounds__(D) decode_combine_kernel(const DecodeArgs a)
     const int64_t len = a.lens[b];
     const bool valid = len >= 1 && len <= a.max_len;
     int n = 0;
-    if (valid) n = a.fixed_chunks > 0 ? a.fixed_chunks : row_length((len - 1) / kDecBlock, a.W, a.S);
+    if (valid) n = a.fixed_chunks > 0 ? a.fixed_chunks : (int)layout_row((len - 1) / kDecBlock, a.W, a.S).n;
     // The partial kernel's writes are visible only after this wait.
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
     const float *src = a.partial + (((int64_t)b * a.Hq + h) * a.chunks) * (D + 2);
@@ -807,11 +802,9 @@ __global__ void __launch_bounds__(kRowThreads, 2) decode_row_kernel(const __grid
 __global__ void decode_block_list_kernel(int64_t len, int32_t W, int32_t S, int32_t *out,
                                          int32_t *count, int32_t capacity)
 {
-    const int64_t row = (len - 1) / kDecBlock;
-    const int n = for_each_key_block(row, W, S, [=](int pos, int64_t j) {
-        if (pos < capacity) out[pos] = (int32_t)j;
-    });
-    *count = n;
+    const LayoutRow row = layout_row((len - 1) / kDecBlock, W, S);
+    for (int32_t pos = 0; pos < row.n && pos < capacity; ++pos) out[pos] = (int32_t)layout_entry(row, pos);
+    *count = (int32_t)row.n;
 }
 
 // One warp: the row kernel's own enumeration, compacted in lane order.
