@@ -337,8 +337,8 @@ pa_status pa_decode_paged(const pa_paged_params *p, const void *q, const void *k
  * contiguous) are written at position cache_lens[b] (the page block_table[b, cache_lens[b] / 64],
  * slot cache_lens[b] mod 64) and cache_lens[b] (device int32, read and written) grows by one.
  * A sequence whose table has no page for that position (position beyond 64 * max_blocks_per_seq,
- * or an entry outside [0, n_pages)) is left unchanged: nothing written, length kept.  Two small
- * kernels are enqueued on `stream`. */
+ * or an entry outside [0, n_pages)) is left unchanged: nothing written, length kept.  One small
+ * kernel is enqueued on `stream`. */
 pa_status pa_kv_append(const pa_paged_params *p, const void *k_new, const void *v_new,
                        void *k_pool, void *v_pool, const int32_t *block_table,
                        int32_t *cache_lens, void *stream);

@@ -48,6 +48,36 @@ EnvSwitches env_switches();
 // (0: each kernel's default).
 long long wait_limit_cycles();
 
+// Launch attribute under which a kernel may start while the kernel before it in the stream still runs
+// (programmatic dependent launch).  Such a kernel touches no global memory before pdl_wait(), which returns when
+// everything ahead of it in the stream has completed; what it does before that (barriers, tensor memory, the
+// launch itself) is hidden behind the other kernel's last microseconds.
+inline cudaLaunchAttribute pdl_attribute()
+{
+    cudaLaunchAttribute a;
+    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a.val.programmaticStreamSerializationAllowed = 1;
+    return a;
+}
+template <typename... Params, typename... Args>
+inline cudaError_t launch_pdl(void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr = pdl_attribute();
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+// The next kernel of the stream may be scheduled as soon as every block of this one has said so or ended.
+__device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+#endif
+
 #define PA_CUDA_OK(expr)                                                                    \
     do {                                                                                    \
         cudaError_t e_ = (expr);                                                            \

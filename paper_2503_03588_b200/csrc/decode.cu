@@ -112,7 +112,7 @@ template <int D>
 __global__ void __launch_bounds__(kDecThreads) decode_block_kernel(const DecodeArgs a)
 {
     // Let the combine kernel's CTAs be scheduled as soon as SM resources free up.
-    asm volatile("griddepcontrol.launch_dependents;\n" ::);
+    pdl_launch_next();
     constexpr int NJ = D / 32;  // 16-byte pieces per thread and row for Q and K
     __shared__ float sS[kMaxGroup][kDecBlock + 8];  // base-2 logits of the block
 
@@ -260,12 +260,14 @@ __global__ void __launch_bounds__(D) decode_combine_kernel(const DecodeArgs a)
 {
     __shared__ float s_red[D / 32];
     const int h = blockIdx.x, b = blockIdx.y, d = threadIdx.x;
+    // The partial kernel's writes are visible only after this wait (and so are the lengths: the kernel before it
+    // in the stream may have written them, and nothing has waited for that one yet).
+    pdl_wait();
+    pdl_launch_next();
     const int64_t len = a.lens[b];
     const bool valid = len >= 1 && len <= a.max_len;
     int n = 0;
     if (valid) n = a.fixed_chunks > 0 ? a.fixed_chunks : (int)layout_row((len - 1) / kDecBlock, a.W, a.S).n;
-    // The partial kernel's writes are visible only after this wait.
-    asm volatile("griddepcontrol.wait;\n" ::: "memory");
     const float *src = a.partial + (((int64_t)b * a.Hq + h) * a.chunks) * (D + 2);
     // Global maximum: the chunks are spread over the threads (independent loads), then reduced.
     float m = -INFINITY;
@@ -404,9 +406,9 @@ __global__ void __launch_bounds__(kRowThreads, 2) decode_row_kernel(const __grid
     // (item and row counts fit 31 bits; checked on the host)
     const uint32_t n_items = (uint32_t)a.items;
     const uint32_t it0 = blockIdx.x, it_step = gridDim.x;
-    // The first item's cache length is on the critical path of a small call: its load starts before
-    // the barrier set-up.
-    const int32_t len_first = it0 < n_items ? a.lens[(it0 / (uint32_t)R) / (uint32_t)a.Hkv] : 0;
+    // The launch after this one may take the places this one leaves; this one itself has started before the
+    // kernel ahead of it was done: up to pdl_wait() nothing of global memory is read or written.
+    pdl_launch_next();
     if (tid == 0) {
         for (int s = 0; s < stages; ++s) {
             ptx::mbar_init(bar_kfull(s), 1);
@@ -416,11 +418,13 @@ __global__ void __launch_bounds__(kRowThreads, 2) decode_row_kernel(const __grid
         *abort_flag = 0;
         ptx::fence_barrier_init();
         ptx::fence_proxy_async_smem();
-        if (blockIdx.x == 0) a.status[0] = 0;  // a wait that gives up (much later) sets it
+        ptx::prefetch_tensormap(&tmK);
+        ptx::prefetch_tensormap(&tmV);
     }
     __syncthreads();
-    // The combine kernel (kModePartial) may be scheduled as this grid's CTAs retire.
-    asm volatile("griddepcontrol.launch_dependents;\n" ::);
+    pdl_wait();
+    const int32_t len_first = it0 < n_items ? a.lens[(it0 / (uint32_t)R) / (uint32_t)a.Hkv] : 0;
+    if (blockIdx.x == 0 && tid == 0) a.status[0] = 0;  // a wait that gives up (much later) sets it
 
     // Item it -> (row of the call, chunk); a row -> (sequence, KV head).
     struct Item {
@@ -463,10 +467,6 @@ __global__ void __launch_bounds__(kRowThreads, 2) decode_row_kernel(const __grid
 
     if (wid == kRowConsumers) {
         // ------------------------------------------------------------------ producer
-        if (lane == 0) {
-            ptx::prefetch_tensormap(&tmK);
-            ptx::prefetch_tensormap(&tmV);
-        }
         bool ok = true;
         uint32_t ci = 0;  // blocks issued so far by this CTA (ring position)
         int32_t len_next = len_first;
@@ -820,48 +820,35 @@ __global__ void decode_row_block_set_kernel(int64_t len, int32_t W, int32_t S, i
     if (lane == 0) *count = __popc(have);
 }
 
-// pa_kv_append, first kernel: the new token's K and V rows go into the page that holds position
-// cache_lens[b].  One CTA per (sequence, KV head); a thread copies 16 bytes.  A sequence whose
-// block table has no valid page for that position is left alone.
-__global__ void kv_append_kernel(const __nv_bfloat16 *k_new, const __nv_bfloat16 *v_new, __nv_bfloat16 *k_pool,
-                                 __nv_bfloat16 *v_pool, const int32_t *table, int32_t *lens, int32_t table_stride,
-                                 int32_t n_pages, int32_t Hkv, int32_t D, int64_t k_sp, int64_t k_ss, int64_t k_sh,
-                                 int64_t v_sp, int64_t v_ss, int64_t v_sh)
-{
-    const int hk = blockIdx.x, b = blockIdx.y;
-    const int32_t pos = lens[b];
-    const int32_t blk = pos / kDecBlock;
-    bool ok = pos >= 0 && blk < table_stride;
-    int32_t page = 0;
-    if (ok) {
-        page = table[(int64_t)b * table_stride + blk];
-        ok = page >= 0 && page < n_pages;
-    }
-    if (ok) {
-        const int slot = pos % kDecBlock;
-        const int c = threadIdx.x;  // 16-byte piece of the row
-        if (c < D / 8) {
-            const uint4 kv = *reinterpret_cast<const uint4 *>(k_new + ((int64_t)b * Hkv + hk) * D + 8 * c);
-            const uint4 vv = *reinterpret_cast<const uint4 *>(v_new + ((int64_t)b * Hkv + hk) * D + 8 * c);
-            *reinterpret_cast<uint4 *>(k_pool + page * k_sp + slot * k_ss + hk * k_sh + 8 * c) = kv;
-            *reinterpret_cast<uint4 *>(v_pool + page * v_sp + slot * v_ss + hk * v_sh + 8 * c) = vv;
-        }
-    }
-}
+// pa_kv_append: a CTA per sequence.  The new token's K and V rows go into the page that holds position
+// cache_lens[b], 16 bytes per thread and turn; once every thread has read the old length it grows by one.  A
+// sequence whose block table has no valid page for that position is left alone.  (One launch: copying and
+// advancing the lengths in two kernels, each waiting for the one before it, cost a decoding step a third launch.)
+constexpr int kAppendThreads = 128;
 
-// pa_kv_append, second kernel: every CTA of the first one has read the old lengths by now; the
-// sequences that had a valid page grow by one token.
-__global__ void kv_advance_kernel(const int32_t *table, int32_t *lens, int32_t batch, int32_t table_stride,
-                                  int32_t n_pages)
+__global__ void __launch_bounds__(kAppendThreads)
+kv_append_kernel(const __nv_bfloat16 *k_new, const __nv_bfloat16 *v_new, __nv_bfloat16 *k_pool, __nv_bfloat16 *v_pool,
+                 const int32_t *table, int32_t *lens, int32_t table_stride, int32_t n_pages, int32_t Hkv, int32_t D,
+                 int64_t k_sp, int64_t k_ss, int64_t k_sh, int64_t v_sp, int64_t v_ss, int64_t v_sh)
 {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= batch) return;
+    pdl_launch_next();
+    pdl_wait();
+    const int b = blockIdx.x;
     const int32_t pos = lens[b];
     const int32_t blk = pos / kDecBlock;
     if (pos < 0 || blk >= table_stride) return;
     const int32_t page = table[(int64_t)b * table_stride + blk];
     if (page < 0 || page >= n_pages) return;
-    lens[b] = pos + 1;
+    const int slot = pos % kDecBlock, per_row = D / 8, pieces = Hkv * per_row;  // 16-byte pieces of K, then of V
+    for (int x = threadIdx.x; x < 2 * pieces; x += kAppendThreads) {
+        const bool is_v = x >= pieces;
+        const int y = is_v ? x - pieces : x, hk = y / per_row, c = y % per_row;
+        const uint4 piece = *reinterpret_cast<const uint4 *>((is_v ? v_new : k_new) + ((int64_t)b * Hkv + hk) * D + 8 * c);
+        __nv_bfloat16 *dst = is_v ? v_pool + page * v_sp + slot * v_ss + hk * v_sh : k_pool + page * k_sp + slot * k_ss + hk * k_sh;
+        *reinterpret_cast<uint4 *>(dst + 8 * c) = piece;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) lens[b] = pos + 1;
 }
 
 // Window distances + power-of-two distances beyond the window + sink blocks that a row below
@@ -1081,13 +1068,14 @@ static pa_status launch_decode(const DecodeShape &p, const void *q, const void *
         cfg.gridDim = dim3((unsigned)grid, 1, 1);
         cfg.blockDim = dim3(kRowThreads, 1, 1);
         cfg.stream = st;
-        cudaLaunchAttribute attr[1];
+        cudaLaunchAttribute attr[2];
+        attr[1] = pdl_attribute();
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = a.mode == kModeCluster ? (unsigned)R : 1u;
         attr[0].val.clusterDim.y = 1;
         attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
-        cfg.numAttrs = 1;
+        cfg.numAttrs = 2;
         if (p.head_dim == 128) {
             cfg.dynamicSmemBytes = RowSmem<128>::bytes(a.stages, a.mode == kModeCluster);
             PA_CUDA_OK(cudaLaunchKernelEx(&cfg, decode_row_kernel<128>, tmK, tmV, a));
@@ -1105,20 +1093,11 @@ static pa_status launch_decode(const DecodeShape &p, const void *q, const void *
         PA_CUDA_OK(cudaGetLastError());
     }
 
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)a.Hq, (unsigned)a.batch, 1);
-    cfg.blockDim = dim3((unsigned)p.head_dim, 1, 1);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    const dim3 heads((unsigned)a.Hq, (unsigned)a.batch, 1);
     if (p.head_dim == 128)
-        PA_CUDA_OK(cudaLaunchKernelEx(&cfg, decode_combine_kernel<128>, a));
+        PA_CUDA_OK(launch_pdl(decode_combine_kernel<128>, heads, 128, 0, st, a));
     else
-        PA_CUDA_OK(cudaLaunchKernelEx(&cfg, decode_combine_kernel<64>, a));
+        PA_CUDA_OK(launch_pdl(decode_combine_kernel<64>, heads, 64, 0, st, a));
     return PA_OK;
 }
 
@@ -1183,14 +1162,11 @@ extern "C" pa_status pa_kv_append(const pa_paged_params *p, const void *k_new, c
     if (!aligned16(k_new) || !aligned16(v_new) || !aligned16(k_pool) || !aligned16(v_pool))
         return fail(PA_ERR_ALIGNMENT, "k_new, v_new and the pools must be 16-byte aligned");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    kv_append_kernel<<<dim3((unsigned)p->n_kv_heads, (unsigned)p->batch), 32, 0, st>>>(
-        static_cast<const __nv_bfloat16 *>(k_new), static_cast<const __nv_bfloat16 *>(v_new),
-        static_cast<__nv_bfloat16 *>(k_pool), static_cast<__nv_bfloat16 *>(v_pool), block_table, cache_lens,
-        p->max_blocks_per_seq, p->n_pages, p->n_kv_heads, p->head_dim, p->k.batch, p->k.seq, p->k.head, p->v.batch,
-        p->v.seq, p->v.head);
-    kv_advance_kernel<<<(unsigned)((p->batch + 127) / 128), 128, 0, st>>>(block_table, cache_lens, p->batch,
-                                                                          p->max_blocks_per_seq, p->n_pages);
-    PA_CUDA_OK(cudaGetLastError());
+    PA_CUDA_OK(launch_pdl(kv_append_kernel, dim3((unsigned)p->batch), kAppendThreads, 0, st,
+                          static_cast<const __nv_bfloat16 *>(k_new), static_cast<const __nv_bfloat16 *>(v_new),
+                          static_cast<__nv_bfloat16 *>(k_pool), static_cast<__nv_bfloat16 *>(v_pool), block_table, cache_lens,
+                          p->max_blocks_per_seq, p->n_pages, p->n_kv_heads, p->head_dim, p->k.batch, p->k.seq, p->k.head,
+                          p->v.batch, p->v.seq, p->v.head));
     return PA_OK;
 }
 

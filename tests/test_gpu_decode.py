@@ -296,3 +296,24 @@ def test_decode_many_rows_through_the_persistent_grid(pa, oracle, pa_env, env):
     o_ref, lse_ref, _ = oracle.decode(q[good], kc[good], vc[good], lens[good], 64, 5, 1)
     compare(o[good], lse[good], o_ref, lse_ref, "persistent grid with invalid lengths")
 
+
+
+@pytest.mark.parametrize("Hkv,D", [(1, 64), (4, 128), (33, 128)])   # 16, 128 and 1056 pieces for 128 threads
+def test_append_copies_whole_rows(pa, Hkv, D):
+    """Back-to-back appends (each starts while the one before it still runs) land in order, bit for bit."""
+    batch, blocks, steps = 5, 3, 70
+    n_pages = batch * blocks
+    k_pool = torch.zeros((n_pages, 64, Hkv, D), dtype=torch.bfloat16, device="cuda")
+    v_pool = torch.zeros_like(k_pool)
+    table = torch.randperm(n_pages).to(torch.int32).view(batch, blocks).contiguous().cuda()
+    start = torch.tensor([0, 63, 64, 100, 191 - steps], dtype=torch.int32)
+    lens = start.cuda()
+    new = [si.bf16_randn((batch, Hkv, D), 1700 + t).cuda() for t in range(2 * steps)]
+    for t in range(steps):
+        pa.pa_kv_append(new[2 * t], new[2 * t + 1], k_pool, v_pool, table, lens)
+    assert lens.cpu().tolist() == (start + steps).tolist()
+    for b in range(batch):
+        for t in range(0, steps, 23):
+            pos = int(start[b]) + t
+            page = int(table[b, pos // 64])
+            assert torch.equal(k_pool[page, pos % 64], new[2 * t][b]) and torch.equal(v_pool[page, pos % 64], new[2 * t + 1][b])
