@@ -280,7 +280,7 @@ def run_ours(args):
             ev_p1[i].record(stream)
         pa.pa_decode(qd, kc, vc, lens_d, wd.window_blocks, wd.sink_blocks, o=Od, lse=LSEd, workspace=wsd)
 
-    launches_per_step = 3 + 1 + 1  # layout (count, scan, fill) + prefill + decode (one cluster kernel)
+    launches_per_step = 1 + 1 + 1  # layout + prefill + decode (one cluster kernel)
 
     for _ in range(max(args.warmup, 3)):
         step()
@@ -430,7 +430,7 @@ def run_ours(args):
         assert int(lens_s[0].item()) == ctx + steps
         pa.pa_decode_status(ws_s)
         return dict(workload="batch 8, 16K-token context + 1024 steps, paged cache (64-token pages), append + decode per step",
-                    us_per_step=1e3 * s0.elapsed_time(s1) / steps, steps=steps, launches_per_step=3)
+                    us_per_step=1e3 * s0.elapsed_time(s1) / steps, steps=steps, launches_per_step=2)
 
     decode_many = decode_steps()
 

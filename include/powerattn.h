@@ -169,7 +169,7 @@ size_t pa_prefill_workspace_bytes(const pa_prefill_params *p);
  * int32 CSR, shared by every batch entry and head (the mask does not depend on them).
  * o: device, o_dtype, strides p->o.  lse: device fp32 [batch, n_q_heads, seq_len] contiguous.
  * workspace: device, >= pa_prefill_workspace_bytes(p); cleared by the call itself.
- * Enqueues one memset and one kernel.  Errors: PA_ERR_INVALID_ARG, PA_ERR_SHAPE,
+ * Enqueues one kernel.  Errors: PA_ERR_INVALID_ARG, PA_ERR_SHAPE,
  * PA_ERR_ALIGNMENT, PA_ERR_LAYOUT (nnz outside [0, 2^31)), PA_ERR_WORKSPACE, PA_ERR_UNSUPPORTED,
  * PA_ERR_CUDA.  Outputs are undefined after a failure.  The CSR is trusted: extents that point
  * outside col_idx would be read out of bounds.  With PA_VALIDATE=1 in the environment (see

@@ -152,6 +152,8 @@ __global__ void __launch_bounds__(kPrepThreads) backward_prep_kernel(const Backw
                                                                      const int32_t cols_per_block)
 {
     extern __shared__ uint32_t prep_bits[];
+    if (a.early) pdl_launch_next();
+    pdl_wait();
     if (blockIdx.x == 0 && threadIdx.x < kBwdStatusBytes / sizeof(int32_t)) a.status[threadIdx.x] = 0;
     if (blockIdx.x < (unsigned)n_csc) {
         transpose_layout(a, (int32_t)blockIdx.x, cols_per_block, prep_bits);
@@ -533,8 +535,7 @@ static pa_status launch_backward(const BackwardArgs &a, const pa_prefill_params 
     const int32_t bitmap_cols = cols < a.nqb ? cols : a.nqb;
     const size_t bitmap = (size_t)bitmap_cols * ((a.nqb + 31) / 32) * sizeof(uint32_t);
     if (groups + n_csc > 0x7fffffff || bitmap > (size_t)kPrepMaxBitmap) return fail(PA_ERR_SHAPE, "batch x seq_len too large");
-    backward_prep_kernel<D><<<(unsigned)(n_csc + groups), kPrepThreads, bitmap, st>>>(a, n_csc, cols);
-    PA_CUDA_OK(cudaGetLastError());
+    PA_CUDA_OK(launch_pdl(backward_prep_kernel<D>, dim3((unsigned)(n_csc + groups)), kPrepThreads, bitmap, st, a, n_csc, cols));
     // dQ, dK and dV on the tcgen05 tensor cores (PA_BACKWARD_PATH=mma: on the warp-level kernels).
     if (!mma) return launch_backward_sm100(a, p, nnz, device, sms, st);
     backward_dq_kernel<D><<<dim3((unsigned)a.nqb, (unsigned)a.Hq, (unsigned)a.batch), kBwdThreads, kSmemDq, st>>>(a);
@@ -609,6 +610,7 @@ extern "C" pa_status pa_prefill_backward(const pa_prefill_params *p, const void 
     // clear those.
     const bool mma = env_switches().backward_mma != 0;
     a.prezero = mma || a.chunk < kBwdMaxChunk;
+    a.early = nqb * a.Hkv * a.npairs * a.batch <= dev.sms;
 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     return p->head_dim == 128 ? launch_backward<128>(a, p, nnz, dev.device, dev.sms, mma, st)

@@ -30,6 +30,7 @@ struct BackwardArgs {
     int64_t N;
     int32_t nqb, batch, Hq, Hkv, G;
     int32_t npairs;            // head pairs per KV group: ceil(G / 2)
+    int32_t early;             // one wave of work: the next kernel may start beside this one's last blocks
     int32_t prezero;           // dK and dV are cleared by the preparation (else: where needed, by the dQ kernel)
     float scale, scale_log2;
     long long wait_cycles;     // limit of every barrier wait of the tensor-core kernels

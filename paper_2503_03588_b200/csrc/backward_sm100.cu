@@ -211,6 +211,8 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
         ptx::tmem_alloc(ptx::smem_u32(&tail->tmem), kTcTmemCols);
         ptx::tmem_relinquish();
     }
+    if (a.early) pdl_launch_next();
+    pdl_wait();  // up to here this kernel may have run beside the one before it
     ptx::tc_fence_before_sync();
     __syncthreads();
     ptx::tc_fence_after_sync();
@@ -656,6 +658,8 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         ptx::tmem_alloc(ptx::smem_u32(&tail->tmem), kTcTmemCols);
         ptx::tmem_relinquish();
     }
+    if (a.early) pdl_launch_next();
+    pdl_wait();  // up to here this kernel may have run beside the one before it
     ptx::tc_fence_before_sync();
     __syncthreads();
     ptx::tc_fence_after_sync();
@@ -1028,11 +1032,10 @@ static pa_status launch_tc(const BackwardArgs &a, const pa_prefill_params *p, in
     const int64_t dkv_items = (nnz / a.chunk + a.nqb) * a.Hkv * a.batch;  // (chunk slots, some of them empty)
     if (dq_items > (int64_t)0x3fffffff || dkv_items > (int64_t)0x3fffffff)
         return fail(PA_ERR_SHAPE, "too many work items (%lld, %lld)", (long long)dq_items, (long long)dkv_items);
-    dq_kernel<D><<<(unsigned)(dq_items < sms ? dq_items : sms), kDqThreads, DqCfg<D>::kAlloc, st>>>(tmQ, tmG, tmK, tmV, tmDq, a,
-                                                                                                    (uint32_t)dq_items);
-    dkv_kernel<D><<<(unsigned)(dkv_items < sms ? dkv_items : sms), kDkvThreads, DkvCfg<D>::kAlloc, st>>>(tmQ, tmG, tmK, tmV, a,
-                                                                                                         (uint32_t)dkv_items);
-    PA_CUDA_OK(cudaGetLastError());
+    PA_CUDA_OK(launch_pdl(dq_kernel<D>, dim3((unsigned)(dq_items < sms ? dq_items : sms)), kDqThreads, DqCfg<D>::kAlloc, st, tmQ,
+                          tmG, tmK, tmV, tmDq, a, (uint32_t)dq_items));
+    PA_CUDA_OK(launch_pdl(dkv_kernel<D>, dim3((unsigned)(dkv_items < sms ? dkv_items : sms)), kDkvThreads, DkvCfg<D>::kAlloc, st,
+                          tmQ, tmG, tmK, tmV, a, (uint32_t)dkv_items));
     return PA_OK;
 }
 

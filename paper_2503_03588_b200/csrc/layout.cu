@@ -16,8 +16,10 @@ __global__ void __launch_bounds__(kLayoutThreads) layout_kernel(int32_t n_rows, 
 {
     const int64_t t = (int64_t)blockIdx.x * (kLayoutThreads / 32) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
-    if (t > n_rows) return;
+    pdl_launch_next();
     const int64_t start = tile_rows_before(t, r, W, S, power);
+    pdl_wait();
+    if (t > n_rows) return;
     if (lane == 0) row_ptr[t] = (int32_t)start;
     if (t == n_rows) return;
     const LayoutRow row = layout_row(t / r, W, S, power);
@@ -76,9 +78,8 @@ static pa_status build_layout(int64_t seq_len, int32_t tile, int32_t r, int32_t 
     if (col_capacity < nnz)
         return fail(PA_ERR_LAYOUT, "col_capacity %lld < nnz %lld", (long long)col_capacity, (long long)nnz);
     constexpr int kRowsPerBlock = kLayoutThreads / 32;
-    layout_kernel<<<(unsigned)(((int64_t)rows + kRowsPerBlock) / kRowsPerBlock), kLayoutThreads, 0,
-                    static_cast<cudaStream_t>(stream)>>>(rows, r, W, S, power, row_ptr, col_idx);
-    PA_CUDA_OK(cudaGetLastError());
+    PA_CUDA_OK(launch_pdl(layout_kernel, dim3((unsigned)(((int64_t)rows + kRowsPerBlock) / kRowsPerBlock)), kLayoutThreads, 0,
+                          static_cast<cudaStream_t>(stream), rows, r, W, S, power, row_ptr, col_idx));
     return PA_OK;
 }
 

@@ -53,6 +53,7 @@ constexpr uint32_t kTmemCols = 512;    // slot s: S at columns 128 s, P buffers 
 constexpr float kSumLimit = 1048576.0f;  // 2^20
 constexpr int kTurnAtColumn = 16;  // column of a pass at which the other slot gets its turn (a multiple of 4 below 64)
 constexpr float kRescaleThreshold = 8.0f;  // base-2 logits: rescale O only when the row max grows by more
+constexpr size_t kPrefillWorkspace = 256;  // bytes: the status block
 constexpr long long kWaitCycles = 4000000000ll;  // default limit of a barrier wait: ~2 s at 2 GHz
 
 struct PrefillArgs {
@@ -219,6 +220,14 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         ptx::tmem_alloc(ptx::smem_u32(tmem_slot), kTmemCols);
         ptx::tmem_relinquish();
     }
+    // Up to here the kernel may have run beside the one before it in the stream.  The next one may do so only if
+    // no CTA of this launch has more than one unit (2K tokens, 2 heads of 64 features: 11.4 us a launch in a graph
+    // with this and the status block cleared here, 15.5 without); in longer launches CTAs that wait on the SMs
+    // this launch is leaving cost more than they save (32K tokens, 28 / 4 heads: 383 us against 379).
+    if (a.n_units <= gridDim.x) pdl_launch_next();
+    pdl_wait();
+    // A clear status block (a wait that gives up, much later, writes to it).
+    if (blockIdx.x == 0 && threadIdx.x < kPrefillWorkspace / sizeof(int32_t)) a.status[threadIdx.x] = 0;
     ptx::tc_fence_before_sync();
     __syncthreads();
     ptx::tc_fence_after_sync();
@@ -837,8 +846,6 @@ static pa_status check_prefill(const pa_prefill_params *p)
     return PA_OK;
 }
 
-constexpr size_t kPrefillWorkspace = 256;
-
 // Optional check of a caller's CSR (PA_VALIDATE=1): one thread per row.  The first violation
 // found is recorded as (kind, row) in check[0..1]: 1 row_ptr does not start at 0 / end at nnz,
 // 2 row extent negative or beyond nnz, 3 block index outside [0, row], 4 indices not ascending.
@@ -944,12 +951,12 @@ static pa_status launch_prefill(const pa_prefill_params *p, const void *q, const
     a.wait_cycles = wait_cycles > 0 ? wait_cycles : kWaitCycles;
     const unsigned grid = (unsigned)(a.n_units < dev.sms ? a.n_units : dev.sms);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    PA_CUDA_OK(cudaMemsetAsync(workspace, 0, kPrefillWorkspace, st));
     {
         // PA_VALIDATE=1: check the CSR on the device before the attention kernel is enqueued.  This
         // synchronises the stream (so not during stream capture) and is meant for bring-up: a CSR
         // whose extents point outside col_idx would otherwise be read out of bounds.
         if (env_switches().validate) {
+            PA_CUDA_OK(cudaMemsetAsync(workspace, 0, kPrefillWorkspace, st));
             int32_t *check = static_cast<int32_t *>(workspace) + 32;
             validate_csr_kernel<<<(unsigned)((nqb + 127) / 128), 128, 0, st>>>(row_ptr, col_idx, (int32_t)nqb, nnz, check);
             PA_CUDA_OK(cudaGetLastError());
@@ -973,10 +980,9 @@ static pa_status launch_prefill(const pa_prefill_params *p, const void *q, const
         }
     }
     if (D == 128)
-        prefill_kernel<128><<<grid, kThreads, SmemMap<128>::kAlloc, st>>>(tmQ, tmK, tmV, tmO, a);
+        PA_CUDA_OK(launch_pdl(prefill_kernel<128>, dim3(grid), kThreads, SmemMap<128>::kAlloc, st, tmQ, tmK, tmV, tmO, a));
     else
-        prefill_kernel<64><<<grid, kThreads, SmemMap<64>::kAlloc, st>>>(tmQ, tmK, tmV, tmO, a);
-    PA_CUDA_OK(cudaGetLastError());
+        PA_CUDA_OK(launch_pdl(prefill_kernel<64>, dim3(grid), kThreads, SmemMap<64>::kAlloc, st, tmQ, tmK, tmV, tmO, a));
     return PA_OK;
 }
 
