@@ -10,13 +10,12 @@
 //   warp 3       issuer of the second products
 //   warps 4-19   four compute warpgroups
 //   warps 20-23  (dQ kernel) epilogue: the finished dQ out of tensor memory and out to global memory
-// A step is one query block and one (dK / dV kernel) or two (dQ kernel) of its key blocks for a pair of query
-// heads stacked on the 64 tokens of the query block: a 128-row tile, as in the forward kernel.  Per step the
-// tensor cores produce S = Q K^T and dP = dO V^T (fp32, tensor memory); the compute warps (thread = tile row =
-// TMEM lane, 32 keys each) turn them into P = exp2(S scale log2e - LSE log2e) and dS = P (dP - delta), rounded
+// A step is one (query block, key block) pair for a pair of query heads stacked on the 64 tokens of the query
+// block: a 128-row tile, as in the forward kernel.  Per step the tensor cores produce S = Q K^T and dP = dO V^T
+// (fp32, tensor memory); the compute warps (thread = tile row = TMEM lane) turn them into P = exp2(S scale log2e - LSE log2e) and dS = P (dP - delta), rounded
 // to bf16; the second products accumulate in tensor memory.
 //
-//   dq_kernel   an item is a (query block, head pair): walks the row's key blocks two at a time; dS goes back
+//   dq_kernel   an item is a (query block, head pair): walks the row's key blocks; dS goes back
 //               into tensor memory as the A operand of dQ += dS K (128 x D accumulator)
 //   dkv_kernel  an item is a (chunk of a key block's listing query blocks, KV head): walks the chunk for every
 //               head pair of the group; P and dS go to shared memory as the B operands of dV^T += dO^T P and
@@ -76,7 +75,14 @@ struct BwdTail {
 };
 static_assert(kBarBytes + sizeof(BwdTail) <= kBarArea, "barrier area");
 
-// P = exp2(S scale - lse2) of 32 keys, as packed pairs; keys beyond `lim` (causal term of the diagonal pair) are 0.
+// P = exp2(S scale - lse2) of a pair of keys.
+__device__ __forceinline__ uint64_t bwd_p2(uint32_t s0, uint32_t s1, uint64_t scale2, uint64_t neg_lse2)
+{
+    float y0, y1;
+    ptx::unpack_f32x2(ptx::fma_f32x2(ptx::pack_f32x2(__uint_as_float(s0), __uint_as_float(s1)), scale2, neg_lse2), y0, y1);
+    return ptx::pack_f32x2(ptx::ex2(y0), ptx::ex2(y1));
+}
+// P of 32 keys, as packed pairs; keys beyond `lim` (causal term of the diagonal pair) are 0.
 __device__ __forceinline__ void bwd_p(uint32_t (&s)[32], bool diag, int lim, uint64_t scale2, uint64_t neg_lse2,
                                       uint64_t (&p)[16])
 {
@@ -86,13 +92,7 @@ __device__ __forceinline__ void bwd_p(uint32_t (&s)[32], bool diag, int lim, uin
             if (x > lim) s[x] = 0xff800000u;
     }
 #pragma unroll
-    for (int x = 0; x < 16; ++x) {
-        const uint64_t y2 = ptx::fma_f32x2(ptx::pack_f32x2(__uint_as_float(s[2 * x]), __uint_as_float(s[2 * x + 1])), scale2,
-                                           neg_lse2);
-        float y0, y1;
-        ptx::unpack_f32x2(y2, y0, y1);
-        p[x] = ptx::pack_f32x2(ptx::ex2(y0), ptx::ex2(y1));
-    }
+    for (int x = 0; x < 16; ++x) p[x] = bwd_p2(s[2 * x], s[2 * x + 1], scale2, neg_lse2);
 }
 __device__ __forceinline__ uint32_t bwd_cvt(uint64_t v)
 {
@@ -112,38 +112,39 @@ __device__ __forceinline__ float bwd_neg_lse2(float lse)
 }
 
 // ------------------------------------------------------------------------------------- dQ
-// Two key blocks a step: S and dP are 128 x 128 MMAs (N = 64 reads A again for half the work: 48 clk instead of
-// 32 for 64 keys), and the fixed cost of a step, barrier round trips and the warps' loads and stores, is paid
-// once for both.  A row of odd length ends on a step of one block, for which the second block's compute warps
-// only keep the barriers going.  S and dP have one buffer each: the warps take them into registers at once, 32
-// keys a thread, and the next step's products run beside the arithmetic.  Q and dO have one buffer each as well:
-// the next item's tiles arrive while the last step is computed and its dQ product runs.
-// Measured, 28 / 4 heads at 32K tokens: 586 us, where steps of one block with two S and dP buffers took 661; 64
-// features, 16 / 4 heads, 2 x 8K tokens: 106 us, where the warp-level MMA kernel took 218.
+// A step's way is long and serial: S, dP, a warpgroup's loads, exponentials and stores, dQ, some 4500 cycles of which
+// the tensor cores work 1024.  So four steps are under way at a time, a warpgroup each.  Tensor memory decides the
+// rest: S has four buffers (dS goes over the S it was made from), dP two, which a warpgroup therefore loads whole
+// (64 registers a thread) before it works through S 16 keys at a time.  K stays in its ring until dQ has read
+// it, V only until dP has.  Q and dO have one buffer each: the next item's tiles arrive while the last steps are
+// computed and their dQ products run.  Bound by the issue of S and dP (1300 clk a step) and by the 128 KB that an
+// item starts with.  Measured, 28 / 4 heads at 32K tokens: 524 us at full clocks, where all four warpgroups on one
+// step of two key blocks took 583; 64 features, 16 / 4 heads, 2 x 8K tokens: 87 us against 106.
 template <int D>
 struct DqCfg {
     static constexpr int kDH = D / 64;
-    static constexpr int kStages = D == 128 ? 2 : 4;         // K and V rings, each of two blocks
-    static constexpr uint32_t kTile = kDH * kRowTile;        // Q, dO, and a pair of K or V blocks
+    static constexpr int kKStages = D == 128 ? 6 : 8, kVStages = D == 128 ? 3 : 4;
+    static constexpr uint32_t kTile = kDH * kRowTile, kBlkTile = kDH * kKeyTile;
     static constexpr uint32_t kQ = 0, kG = kTile;
-    static constexpr uint32_t kK = 2 * kTile, kV = kK + kStages * kTile;
-    static constexpr uint32_t kOut = kV + kStages * kTile;   // per epilogue warp two patches of 32 rows x 32 fp32
-    static constexpr uint32_t kBars = kOut + 4 * 2 * 4096;
+    static constexpr uint32_t kK = 2 * kTile, kV = kK + kKStages * kBlkTile;
+    static constexpr uint32_t kOut = kV + kVStages * kBlkTile;  // per epilogue warp a patch of 32 rows x 32 fp32
+    static constexpr uint32_t kBars = kOut + 4 * 4096;
     static constexpr uint32_t kAlloc = kBars + kBarArea + 1024;
     static_assert(kAlloc <= 227 * 1024, "shared memory budget");
     enum : uint32_t {
         Q_FULL, Q_EMPTY, G_FULL, G_EMPTY,
-        K_FULL, K_EMPTY = K_FULL + kStages,
-        V_FULL = K_EMPTY + kStages, V_EMPTY = V_FULL + kStages,
-        S_FULL = V_EMPTY + kStages, S_TAKEN, DP_FULL, DP_TAKEN,
-        DS_FULL, DS_FREE = DS_FULL + 2,      // [step parity]
-        DQ_DONE = DS_FREE + 2,               // the item's last dQ += dS K has completed
+        K_FULL, K_EMPTY = K_FULL + kKStages,
+        V_FULL = K_EMPTY + kKStages, V_EMPTY = V_FULL + kVStages,
+        S_FULL = V_EMPTY + kVStages, DP_FULL = S_FULL + 4,   // [warpgroup]
+        DP_TAKEN = DP_FULL + 4,                              // [step parity]: dP is in registers
+        DS_FULL = DP_TAKEN + 2, DS_FREE = DS_FULL + 4,       // [warpgroup]: dS is in tensor memory / dQ += dS K has read it
+        DQ_DONE = DS_FREE + 4,               // the item's last dQ += dS K has completed
         DQ_FREE,                             // the epilogue warps have read dQ out of tensor memory
         ITEM_FULL, ITEM_EMPTY = ITEM_FULL + kItemRing, COUNT = ITEM_EMPTY + kItemRing
     };
     static_assert(COUNT * 8 <= kBarBytes, "barrier area");
-    // Tensor memory columns: S, dP, dS (bf16 pairs, two buffers), dQ.
-    static constexpr uint32_t kColDp = 128, kColDs = 256, kColDq = 384;
+    // Tensor memory columns: S at 64 g (dS, bf16 pairs, over its first half), dP at 256 + 64 (step parity), dQ.
+    static constexpr uint32_t kColDp = 256, kColDq = 384;
 };
 
 template <int D>
@@ -154,7 +155,7 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
 {
     using C = DqCfg<D>;
     constexpr int DH = C::kDH;
-    constexpr uint32_t kStages = C::kStages;
+    constexpr uint32_t NK = C::kKStages, NV = C::kVStages;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *smem = smem_raw + (smem_base - ptx::smem_u32(smem_raw));
@@ -183,20 +184,22 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
         ptx::mbar_init(bar(C::Q_EMPTY), 1);
         ptx::mbar_init(bar(C::G_FULL), 1);
         ptx::mbar_init(bar(C::G_EMPTY), 1);
-        for (uint32_t s = 0; s < kStages; ++s) {
+        for (uint32_t s = 0; s < NK; ++s) {
             ptx::mbar_init(bar(C::K_FULL + s), 1);
             ptx::mbar_init(bar(C::K_EMPTY + s), 1);
+        }
+        for (uint32_t s = 0; s < NV; ++s) {
             ptx::mbar_init(bar(C::V_FULL + s), 1);
             ptx::mbar_init(bar(C::V_EMPTY + s), 1);
         }
-        ptx::mbar_init(bar(C::S_FULL), 1);
-        ptx::mbar_init(bar(C::DP_FULL), 1);
-        ptx::mbar_init(bar(C::S_TAKEN), kCompWarps);
-        ptx::mbar_init(bar(C::DP_TAKEN), kCompWarps);
-        for (int s = 0; s < 2; ++s) {
-            ptx::mbar_init(bar(C::DS_FULL + s), kCompWarps);
-            ptx::mbar_init(bar(C::DS_FREE + s), 1);
+        for (int g = 0; g < 4; ++g) {
+            ptx::mbar_init(bar(C::S_FULL + g), 1);
+            ptx::mbar_init(bar(C::DP_FULL + g), 1);
+            ptx::mbar_init(bar(C::DS_FULL + g), 4);
+            ptx::mbar_init(bar(C::DS_FREE + g), 1);
         }
+        ptx::mbar_init(bar(C::DP_TAKEN), 4);
+        ptx::mbar_init(bar(C::DP_TAKEN + 1), 4);
         ptx::mbar_init(bar(C::DQ_DONE), 1);
         ptx::mbar_init(bar(C::DQ_FREE), 4);
         for (uint32_t r = 0; r < kItemRing; ++r) {
@@ -268,29 +271,24 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
                             ptx::tma_load_4d(smem_base + dst + dh * kRowTile, tm, bar(full), dh * 64, w.blk * kBwdBlk, h0, w.b);
                         return true;
                     };
-                    auto load_pair = [&](uint32_t base, const CUtensorMap *tm, uint32_t full, uint32_t empty, int32_t j0, int32_t j1,
-                                         int code) {
-                        const uint32_t st = c % kStages;
-                        if (c >= kStages && !wait_bar(bar(empty + st), (c / kStages - 1) & 1, code)) return false;
-                        const uint32_t dst = smem_base + base + st * C::kTile;
-                        ptx::mbar_expect_tx(bar(full + st), (j1 >= 0 ? 2u : 1u) * DH * kKeyTile);
-                        for (int dh = 0; dh < DH; ++dh) {
-                            ptx::tma_load_4d(dst + dh * kRowTile, tm, bar(full + st), dh * 64, j0 * kBwdBlk, w.hk, w.b);
-                            if (j1 >= 0)
-                                ptx::tma_load_4d(dst + dh * kRowTile + kKeyTile, tm, bar(full + st), dh * 64, j1 * kBwdBlk, w.hk, w.b);
-                        }
+                    auto load_block = [&](uint32_t base, const CUtensorMap *tm, uint32_t full, uint32_t empty, uint32_t stages, int32_t j,
+                                          int code) {
+                        const uint32_t st = c % stages;
+                        if (c >= stages && !wait_bar(bar(empty + st), (c / stages - 1) & 1, code)) return false;
+                        ptx::mbar_expect_tx(bar(full + st), C::kBlkTile);
+                        for (int dh = 0; dh < DH; ++dh)
+                            ptx::tma_load_4d(smem_base + base + st * C::kBlkTile + dh * kKeyTile, tm, bar(full + st), dh * 64, j * kBwdBlk,
+                                             w.hk, w.b);
                         return true;
                     };
-                    int32_t j0 = __ldg(a.col_idx + w.e0), j1 = w.n > 1 ? __ldg(a.col_idx + w.e0 + 1) : -1;
-                    for (int e = 0; e < w.n && ok; e += 2, ++c) {
-                        const int32_t j0n = e + 2 < w.n ? __ldg(a.col_idx + w.e0 + e + 2) : 0;
-                        const int32_t j1n = e + 3 < w.n ? __ldg(a.col_idx + w.e0 + e + 3) : -1;
+                    int32_t j = __ldg(a.col_idx + w.e0);
+                    for (int e = 0; e < w.n && ok; ++e, ++c) {
+                        const int32_t jn = e + 1 < w.n ? __ldg(a.col_idx + w.e0 + e + 1) : 0;
                         if (e == 0) ok = load_rows(C::kQ, &tmQ, C::Q_FULL, C::Q_EMPTY, 3);
-                        ok = ok && load_pair(C::kK, &tmK, C::K_FULL, C::K_EMPTY, j0, j1, 4);
+                        ok = ok && load_block(C::kK, &tmK, C::K_FULL, C::K_EMPTY, NK, j, 4);
                         if (e == 0) ok = ok && load_rows(C::kG, &tmG, C::G_FULL, C::G_EMPTY, 5);
-                        ok = ok && load_pair(C::kV, &tmV, C::V_FULL, C::V_EMPTY, j0, j1, 6);
-                        j0 = j0n;
-                        j1 = j1n;
+                        ok = ok && load_block(C::kV, &tmV, C::V_FULL, C::V_EMPTY, NV, j, 6);
+                        j = jn;
                     }
                     ++kq;
                 }
@@ -302,13 +300,14 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
         // -------------------------------------------------------------- tcgen05 issuers of S (warp 1) and dP (warp 2)
         const bool leader = ptx::elect_one();
         const bool is_dp = __shfl_sync(0xffffffffu, warp, 0) == 2;
-        // A = Q (S) or dO (dP); B = the K or V blocks of the stage; both K-major.
+        // A = Q (S) or dO (dP); B = the K or V block of the stage; both K-major.
+        constexpr uint32_t idesc_s = idesc_bf16(128, 64, 0, 0);
         const uint32_t a_lo = ((smem_base + (is_dp ? C::kG : C::kQ)) >> 4) | (1u << 16);
         const uint32_t rows_full = is_dp ? C::G_FULL : C::Q_FULL, rows_empty = is_dp ? C::G_EMPTY : C::Q_EMPTY;
-        const uint32_t blk_full = is_dp ? C::V_FULL : C::K_FULL;
-        const uint32_t out_full = is_dp ? C::DP_FULL : C::S_FULL, out_taken = is_dp ? C::DP_TAKEN : C::S_TAKEN;
-        const uint32_t t_d = __shfl_sync(0xffffffffu, tmem_base + (is_dp ? C::kColDp : 0u), 0);
-        uint32_t c = 0, kq = 0;
+        const uint32_t blk_full = is_dp ? C::V_FULL : C::K_FULL, stages = is_dp ? NV : NK;
+        const uint32_t out_full = is_dp ? C::DP_FULL : C::S_FULL;
+        const uint32_t t_base = __shfl_sync(0xffffffffu, tmem_base + (is_dp ? C::kColDp : 0u), 0);
+        uint32_t c = 0, kq = 0, st = 0, round = 0;  // step, items, the step's stage, how often the ring has come round
         bool ok = true;
         for (uint32_t k = 0; ok; ++k) {
             BwdItem w;
@@ -316,25 +315,34 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
             const int n = __shfl_sync(0xffffffffu, w.n, 0);
             if (!ok || n < 0) break;
             if (n == 0) continue;
-            for (int e = 0; e < n; e += 2, ++c) {
-                const uint32_t st = c % kStages;
-                if (e == 0) ok = wait_warp(bar(rows_full), kq & 1, 7);
-                ok = ok && wait_warp(bar(blk_full + st), (c / kStages) & 1, 8);
-                if (c >= 1) ok = ok && wait_warp(bar(out_taken), (c - 1) & 1, 9);
+            for (int e = 0; e < n; ++e, ++c) {
+                // Three things to wait for, by three groups of lanes at a time (each wait costs some 200 clk even when it is
+                // over): the block; the item's rows; the buffer (dP of two steps before is in registers; the S
+                // buffer's last dS has been read).
+                uint32_t b_ = blk_full + st, parity = round & 1;
+                const int which = lane & 3;
+                if (which == 1 && e == 0) b_ = rows_full, parity = kq & 1;
+                if (which == 2 && is_dp && c >= 2) b_ = C::DP_TAKEN + (c & 1), parity = ((c >> 1) - 1) & 1;
+                if (which == 2 && !is_dp && c >= 4) b_ = C::DS_FREE + (c & 3), parity = ((c >> 2) - 1) & 1;
+                ok = wait_warp(bar(b_), parity, 7 + which);
                 if (!ok) break;
                 ptx::tc_fence_after_sync();
                 if (leader) {
-                    const uint32_t b_lo = ((smem_base + (is_dp ? C::kV : C::kK) + st * C::kTile) >> 4) | (1u << 16);
-                    const uint32_t idesc = e + 1 < n ? idesc_bf16(128, 128, 0, 0) : idesc_bf16(128, 64, 0, 0);
+                    const uint32_t b_lo = ((smem_base + (is_dp ? C::kV : C::kK) + st * C::kBlkTile) >> 4) | (1u << 16);
+                    const uint32_t t_d = t_base + 64 * (is_dp ? c & 1 : c & 3);
 #pragma unroll
                     for (int kk = 0; kk < D / 16; ++kk)
                         ptx::umma_ss_lohi(t_d, a_lo + (((kk / 4) * kRowTile + (kk % 4) * 32) >> 4), kDescHi,
-                                          b_lo + (((kk / 4) * kRowTile + (kk % 4) * 32) >> 4), kDescHi, idesc, kk > 0 ? 1u : 0u);
-                    ptx::umma_commit(bar(out_full));
+                                          b_lo + (((kk / 4) * kKeyTile + (kk % 4) * 32) >> 4), kDescHi, idesc_s, kk > 0 ? 1u : 0u);
+                    ptx::umma_commit(bar(out_full + (c & 3)));
                     if (is_dp) ptx::umma_commit(bar(C::V_EMPTY + st));
-                    if (e + 2 >= n) ptx::umma_commit(bar(rows_empty));  // this warp has read the item's Q (dO) tile
+                    if (e == n - 1) ptx::umma_commit(bar(rows_empty));  // this warp has read the item's Q (dO) tile
                 }
                 __syncwarp();
+                if (++st == stages) {
+                    st = 0;
+                    ++round;
+                }
             }
             ++kq;
         }
@@ -351,25 +359,24 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
             const int n = __shfl_sync(0xffffffffu, w.n, 0);
             if (!ok || n < 0) break;
             if (n == 0) continue;
-            for (int e = 0; e < n; e += 2, ++c) {
-                const uint32_t bf = c & 1, st = c % kStages;
-                ok = wait_warp(bar(C::DS_FULL + bf), (c >> 1) & 1, 10);
-                // The previous item's dQ must have left tensor memory.
-                if (ok && e == 0 && kq > 0) ok = wait_warp(bar(C::DQ_FREE), (kq - 1) & 1, 11);
+            for (int e = 0; e < n; ++e, ++c) {
+                const uint32_t g = c & 3, st = c % NK;
+                // (odd lanes: the previous item's dQ must have left tensor memory)
+                const bool free = (lane & 1) && e == 0 && kq > 0;
+                ok = wait_warp(bar(free ? C::DQ_FREE : C::DS_FULL + g), (free ? kq - 1 : c >> 2) & 1, free ? 11 : 10);
                 if (!ok) break;
                 ptx::tc_fence_after_sync();
                 if (leader) {
-                    // B = the K blocks read feature-contiguous: 16 keys per MMA, 2048 bytes further each.
-                    const uint32_t kb = ((smem_base + C::kK + st * C::kTile) >> 4) | ((kRowTile >> 4) << 16);
-                    const uint32_t t_ds = t_base + C::kColDs + 64 * bf;
+                    // B = the K block read feature-contiguous: 16 keys per MMA, 2048 bytes further each.
+                    const uint32_t kb = ((smem_base + C::kK + st * C::kBlkTile) >> 4) | ((kKeyTile >> 4) << 16);
+                    const uint32_t t_ds = t_base + 64 * g;
 #pragma unroll
-                    for (int kk = 0; kk < 8; ++kk)
-                        if (kk < 4 || e + 1 < n)
-                            ptx::umma_ts_lohi(t_base + C::kColDq, t_ds + kk * 8, kb + ((kk * 2048) >> 4), kDescHi, idesc_dq,
-                                              (e > 0 || kk > 0) ? 1u : 0u);
+                    for (int kk = 0; kk < kBwdBlk / 16; ++kk)
+                        ptx::umma_ts_lohi(t_base + C::kColDq, t_ds + kk * 8, kb + ((kk * 2048) >> 4), kDescHi, idesc_dq,
+                                          (e > 0 || kk > 0) ? 1u : 0u);
                     ptx::umma_commit(bar(C::K_EMPTY + st));
-                    ptx::umma_commit(bar(C::DS_FREE + bf));
-                    if (e + 2 >= n) ptx::umma_commit(bar(C::DQ_DONE));
+                    ptx::umma_commit(bar(C::DS_FREE + g));
+                    if (e == n - 1) ptx::umma_commit(bar(C::DQ_DONE));
                 }
                 __syncwarp();
             }
@@ -377,11 +384,13 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
         }
     } else if (warp < 4 + kCompWarps) {
         // -------------------------------------------------------------- compute warps
-        // Warpgroup wg: keys 32 wg .. 32 wg + 31 of the step's 128.
+        // Warpgroup g: every fourth step.
         ptx::setmaxnreg_inc<PA_DQ_REG_COMP>();
-        const int wg = (warp - 4) >> 2, quad = warp & 3, blk = wg >> 1;
+        const uint32_t g = (uint32_t)(warp - 4) >> 2;
+        const int quad = warp & 3;
         const int row = quad * 32 + lane, qrow = row & 63;
         const uint32_t t_lane = tmem_base + ((uint32_t)(quad * 32) << 16);
+        const uint32_t t_s = t_lane + 64 * g, t_dp = t_lane + C::kColDp + 64 * (g & 1);
         const uint64_t scale2 = ptx::pack_f32x2(a.scale_log2, a.scale_log2);
         // An item's row data for this thread, requested one item ahead.
         float lse_n = INFINITY, delta_n = 0.f;
@@ -400,72 +409,70 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
             }
             lastcol_n = __ldg(a.col_idx + w.e0 + w.n - 1);
         };
-        uint32_t c = 0;
-        BwdItem w, wn;
+        uint32_t c = 0;  // step number at the item's start
+        BwdItem w;
         bool ok = read_item(0, w);
         if (ok) request(w);
-        for (uint32_t k = 0; ok && w.n >= 0; ++k) {
+        int n = w.n, blk = w.blk;
+        for (uint32_t k = 0; ok && n >= 0; ++k) {
             const float neg_lse2 = bwd_neg_lse2(lse_n);
             const uint64_t neg_lse2_2 = ptx::pack_f32x2(neg_lse2, neg_lse2), neg_delta2 = ptx::pack_f32x2(-delta_n, -delta_n);
-            const bool last_is_diag = lastcol_n == w.blk;
-            ok = read_item(k + 1, wn);
+            const bool last_is_diag = lastcol_n == blk;
+            ok = read_item(k + 1, w);
             if (!ok) break;
-            request(wn);
-            for (int e = 0; e < w.n; e += 2, ++c) {
-                const bool active = e + blk < w.n;
-                uint32_t x32[32];
-                uint64_t p[16];
-                ok = wait_warp(bar(C::S_FULL), c & 1, 12);
+            request(w);
+            for (uint32_t e = (g - c) & 3; e < (uint32_t)n; e += 4) {
+                const uint32_t phase = ((c + e) >> 2) & 1;
+                uint32_t dp[64];
+                ok = wait_warp(bar(C::DP_FULL + g), phase, 13);
                 if (!ok) break;
                 ptx::tc_fence_after_sync();
-                if (active) {
-                    ptx::tmem_ld32(t_lane + 32 * wg, x32);
-                    ptx::tmem_wait_ld();
-                }
+                ptx::tmem_ld32(t_dp, *reinterpret_cast<uint32_t(*)[32]>(&dp[0]));
+                ptx::tmem_ld32(t_dp + 32, *reinterpret_cast<uint32_t(*)[32]>(&dp[32]));
+                ptx::tmem_wait_ld();
                 ptx::tc_fence_before_sync();
                 __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(bar(C::S_TAKEN));
+                if (lane == 0) ptx::mbar_arrive(bar(C::DP_TAKEN + (g & 1)));
+                ok = wait_warp(bar(C::S_FULL + g), phase, 12);
+                if (!ok) break;
+                ptx::tc_fence_after_sync();
                 // Algorithm 1's causal term acts inside the diagonal pair only (the row's last block).
-                if (active)
-                    bwd_p(x32, last_is_diag && e + blk == w.n - 1, qrow - 32 * (wg & 1), scale2, neg_lse2_2, p);
-                ok = wait_warp(bar(C::DP_FULL), c & 1, 13);
-                if (!ok) break;
-                ptx::tc_fence_after_sync();
-                if (active) {
-                    ptx::tmem_ld32(t_lane + C::kColDp + 32 * wg, x32);
-                    ptx::tmem_wait_ld();
-                }
-                ptx::tc_fence_before_sync();
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(bar(C::DP_TAKEN));
-                if (c >= 2) {
-                    ok = wait_warp(bar(C::DS_FREE + (c & 1)), ((c >> 1) - 1) & 1, 14);
-                    if (!ok) break;
-                }
-                if (active) {
-                    uint32_t pk[16];
+                const bool diag = last_is_diag && (int)e == n - 1;
 #pragma unroll
-                    for (int x = 0; x < 16; ++x) pk[x] = bwd_cvt(bwd_ds(p[x], x32[2 * x], x32[2 * x + 1], neg_delta2));
-                    ptx::tmem_st16(t_lane + C::kColDs + 64 * (c & 1) + 16 * wg, pk);
-                    ptx::tmem_wait_st();
+                for (int ch = 0; ch < 4; ++ch) {
+                    uint32_t sv[16], pk[8];
+                    ptx::tmem_ld16(t_s + 16 * ch, sv);
+                    ptx::tmem_wait_ld();
+                    if (diag) {
+#pragma unroll
+                        for (int x = 0; x < 16; ++x)
+                            if (16 * ch + x > qrow) sv[x] = 0xff800000u;
+                    }
+#pragma unroll
+                    for (int x = 0; x < 8; ++x)
+                        pk[x] = bwd_cvt(bwd_ds(bwd_p2(sv[2 * x], sv[2 * x + 1], scale2, neg_lse2_2), dp[16 * ch + 2 * x],
+                                               dp[16 * ch + 2 * x + 1], neg_delta2));
+                    ptx::tmem_st8(t_s + 8 * ch, pk);  // (over S of keys that are done)
                 }
+                ptx::tmem_wait_st();
                 ptx::tc_fence_before_sync();
                 __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(bar(C::DS_FULL + (c & 1)));
+                if (lane == 0) ptx::mbar_arrive(bar(C::DS_FULL + g));
             }
-            w = wn;
+            c += (uint32_t)(n > 0 ? n : 0);
+            n = w.n;
+            blk = w.blk;
         }
     } else {
         // -------------------------------------------------------------- epilogue
         // dQ = scale x the accumulator.  A warp's 32 rows leave 32 features at a time: through a swizzled patch of
-        // shared memory and a bulk tensor store each (rows beyond the sequence are clipped by the tensor map), two
-        // patches in turn.  (Plain stores moved 10 B/clk out of the SM: 7000 clk an item, during which the
+        // shared memory and a bulk tensor store each (rows beyond the sequence are clipped by the tensor map).  (Plain stores moved 10 B/clk out of the SM: 7000 clk an item, during which the
         // accumulator, or 128 registers a thread, was held.)
         ptx::setmaxnreg_dec<PA_DQ_REG_EPI>();
         const int quad = warp & 3;
         const int row = quad * 32 + lane, qrow = row & 63;
         const uint32_t t_lane = tmem_base + ((uint32_t)(quad * 32) << 16);
-        const uint32_t patch = smem_base + C::kOut + (uint32_t)quad * 8192u + (uint32_t)lane * 128u;
+        const uint32_t patch = smem_base + C::kOut + (uint32_t)quad * 4096u + (uint32_t)lane * 128u;
         // Key blocks whose dK and dV are added up from several chunks, or that nobody lists, start from zero
         // (where the preparation has not cleared everything).
         if (!a.prezero)
@@ -482,7 +489,7 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
                     }
                 }
             }
-        uint32_t kq = 0, np = 0;
+        uint32_t kq = 0;
         bool ok = true;
         for (uint32_t k = 0; ok; ++k) {
             BwdItem w;
@@ -502,7 +509,7 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
             ptx::tc_fence_after_sync();
             const int32_t tok = w.blk * kBwdBlk + 32 * (quad & 1);
 #pragma unroll 1
-            for (int ch = 0; ch < D / 32; ++ch, ++np) {
+            for (int ch = 0; ch < D / 32; ++ch) {
                 uint32_t acc[32];
                 ptx::tmem_ld32(t_lane + C::kColDq + 32 * ch, acc);
                 ptx::tmem_wait_ld();
@@ -511,12 +518,11 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
                     __syncwarp();
                     if (lane == 0) ptx::mbar_arrive(bar(C::DQ_FREE));
                 }
-                if (lane == 0) ptx::bulk_wait_read<1>();  // the store before last has read this patch
+                if (lane == 0) ptx::bulk_wait_read_all();  // the store before has read the patch
                 __syncwarp();
-                const uint32_t buf = 4096u * (np & 1), dst = patch + buf;
 #pragma unroll
                 for (int x = 0; x < 8; ++x)
-                    ptx::st_shared_v4(dst + (uint32_t)((x ^ (lane & 7)) << 4), __float_as_uint(__uint_as_float(acc[4 * x]) * a.scale),
+                    ptx::st_shared_v4(patch + (uint32_t)((x ^ (lane & 7)) << 4), __float_as_uint(__uint_as_float(acc[4 * x]) * a.scale),
                                       __float_as_uint(__uint_as_float(acc[4 * x + 1]) * a.scale),
                                       __float_as_uint(__uint_as_float(acc[4 * x + 2]) * a.scale),
                                       __float_as_uint(__uint_as_float(acc[4 * x + 3]) * a.scale));
@@ -524,7 +530,7 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
                 __syncwarp();
                 if (lane == 0) {
                     if (head_ok && tok < a.N)
-                        ptx::tma_store_4d(&tmDq, dst, 32 * ch, tok, w.hk * a.G + head_local, w.b);
+                        ptx::tma_store_4d(&tmDq, patch, 32 * ch, tok, w.hk * a.G + head_local, w.b);
                     ptx::bulk_commit_group();
                 }
             }
