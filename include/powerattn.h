@@ -259,7 +259,7 @@ size_t pa_decode_workspace_bytes(const pa_decode_params *p);
  * (window_blocks + sink_blocks + log2 of the row count: any default-window row up to millions of
  * tokens) the row kernel runs: a row's key blocks are dealt to R chunks; in each CTA a producer
  * warp fetches the blocks of its chunk by TMA into a ring of shared-memory stages and four warps
- * run an online softmax over them.  Small calls (batch x n_kv_heads up to about 70) are one
+ * run an online softmax over them.  Small calls (batch x n_kv_heads up to the number of SMs) are one
  * launch in which the R CTAs of a row form a thread-block cluster and merge their results through
  * distributed shared memory with the log-sum-exp rule
  * m = max m_c, l = sum l_c e^(m_c - m), o = sum o_c e^(m_c - m) / l.  Larger calls run a
@@ -271,8 +271,8 @@ size_t pa_decode_workspace_bytes(const pa_decode_params *p);
  * Calls that share a workspace must not overlap on the GPU.  Environment switches (for tests and
  * measurements, see pa_reload_environment): PA_DECODE_PATH=splitk forces the two-kernel path,
  * =cluster / =persist the two forms of the row kernel; PA_DECODE_CLUSTER=n (1..8) sets R (default:
- * for small calls as many CTAs per row as run all at once, for large ones one chunk per row once
- * there are as many rows as SMs, else two); PA_DECODE_STAGES=n (1..6) the number of key blocks a CTA keeps
+ * for small calls as many CTAs per row as run all at once, for large ones one chunk per row);
+ * PA_DECODE_STAGES=n (1..6) the number of key blocks a CTA keeps
  * in flight; PA_DECODE_CTAS_PER_SM=n the size of the persistent grid (default 2 per SM). */
 pa_status pa_decode(const pa_decode_params *p, const void *q, const void *k_cache,
                     const void *v_cache, const int32_t *cache_lens, void *o, float *lse,

@@ -1001,9 +1001,12 @@ static pa_status launch_decode(const DecodeShape &p, const void *q, const void *
         const int64_t rows_in_call = (int64_t)a.batch * a.Hkv;
         const int max_R = a.chunks < kRowMaxCluster ? a.chunks : kRowMaxCluster;
         const int64_t persistent_ctas = (env.decode_ctas_per_sm ? env.decode_ctas_per_sm : 2) * (int64_t)dev.sms;
-        // Small calls (latency-bound): one launch, a cluster of R CTAs per row, all resident at once.  Larger calls (bandwidth-bound): a persistent grid of
-        // two CTAs per SM over (row, chunk) items.
-        bool cluster = rows_in_call * kRowMaxCluster <= 2 * persistent_ctas;
+        // Small calls (latency-bound): a cluster of R CTAs per row, all resident at once.  Larger calls
+        // (bandwidth-bound): a persistent grid of two CTAs per SM over the rows.  The line lies where a row
+        // still gets two of the resident CTAs: rows of 18 blocks (30000 tokens, G = 7, head_dim 128) take
+        // 9.2 us at 80 rows in clusters of three and 11.5 us in the persistent form, 12.4 and 13.3 at 120
+        // rows, 18.8 (clusters of one) and 15.7 at 160.
+        bool cluster = rows_in_call * 2 <= persistent_ctas;
         if (env.decode_path == 2) cluster = true;
         if (env.decode_path == 3) cluster = false;
         int R = env.decode_cluster;
@@ -1017,9 +1020,9 @@ static pa_status launch_decode(const DecodeShape &p, const void *q, const void *
             if (R > max_R) R = max_R;
             a.mode = kModeCluster;
         } else {
-            // One chunk per row once there are enough rows for every SM; measured: finer items
-            // balance the SMs better on paper but pay more per item than they gain.
-            if (R == 0) R = rows_in_call >= dev.sms ? 1 : 2;
+            // One chunk per row: finer items balance the SMs better on paper but pay more per item
+            // than they gain, and need the merge kernel.
+            if (R == 0) R = 1;
             if (R > max_R) R = max_R;
             a.mode = R == 1 ? kModeDirect : kModePartial;
         }

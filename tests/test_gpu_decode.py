@@ -298,6 +298,18 @@ def test_decode_many_rows_through_the_persistent_grid(pa, oracle, pa_env, env):
 
 
 
+@pytest.mark.parametrize("rows", [37, 38, 74, 75, 148, 149])
+def test_decode_where_the_number_of_ctas_per_row_changes(pa, oracle, rows):
+    """On 148 SMs a row gets eight CTAs up to 37 rows, then seven, four up to 74, then three, two up to
+    148, and from 149 on the rows are walked by a persistent grid."""
+    max_len, D = 2100, 64
+    q = si.bf16_randn((rows, 2, D), 95)
+    kc, vc = si.bf16_randn((rows, max_len, 1, D), 96), si.bf16_randn((rows, max_len, 1, D), 97)
+    lens = np.random.default_rng(98).integers(1, max_len + 1, size=rows)
+    lens[:3] = [max_len, 1, 64]
+    _run(pa, oracle, q, kc, vc, lens, 5, 1)
+
+
 @pytest.mark.parametrize("Hkv,D", [(1, 64), (4, 128), (33, 128)])   # 16, 128 and 1056 pieces for 128 threads
 def test_append_copies_whole_rows(pa, Hkv, D):
     """Back-to-back appends (each starts while the one before it still runs) land in order, bit for bit."""
