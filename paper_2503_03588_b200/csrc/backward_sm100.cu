@@ -2,14 +2,14 @@
 // key-block lists of Algorithm 1, Section 3.3) on the sm_100a tensor cores, head_dim 64 and 128.
 //
 // Two persistent kernels with the same skeleton:
-//   warp 0       TMA producer (bf16 tiles, 128-byte swizzle, into rings of shared-memory stages); it also draws
-//                the CTA's next work item from a counter in memory and hands it to the other warps through a
-//                small ring in shared memory
+//   warp 0       TMA producer (bf16 tiles, 128-byte swizzle, into rings of shared-memory stages)
 //   warp 1       tcgen05 issuer of S (one elected lane)
 //   warp 2       tensor-memory allocation, issuer of dP
 //   warp 3       issuer of the second products
 //   warps 4-19   four compute warpgroups
-//   warps 20-23  (dQ kernel) epilogue: the finished dQ out of tensor memory and out to global memory
+//   warps 20-23  epilogue: an item's finished accumulators out of tensor memory and out to global memory
+// Work items are drawn from a counter in memory, by the producer (dQ) or by warp 20 (dK / dV), and handed to the
+// other warps through a small ring in shared memory.
 // A step is one (query block, key block) pair for a pair of query heads stacked on the 64 tokens of the query
 // block: a 128-row tile, as in the forward kernel.  Per step the tensor cores produce S = Q K^T and dP = dO V^T
 // (fp32, tensor memory); the compute warps (thread = tile row = TMEM lane) turn them into P = exp2(S scale log2e - LSE log2e) and dS = P (dP - delta), rounded
@@ -32,20 +32,16 @@
 #include "sm100_ptx.cuh"
 #include "tensor_map.cuh"
 
-// Registers per thread by role.  A warpgroup asking for more than the pool holds would wait for ever: the dK / dV
-// kernel starts 640 threads x 96, the dQ kernel 768 x 80.
-#define PA_DKV_REG_CTRL 56
-#define PA_DKV_REG_COMP 104
-static_assert(4 * PA_DKV_REG_CTRL + 16 * PA_DKV_REG_COMP <= 20 * 96, "register split exceeds the CTA's registers");
-#define PA_DQ_REG_CTRL 48
-#define PA_DQ_REG_COMP 96
-#define PA_DQ_REG_EPI 48
-static_assert(4 * PA_DQ_REG_CTRL + 16 * PA_DQ_REG_COMP + 4 * PA_DQ_REG_EPI <= 24 * 80, "register split exceeds the CTA's registers");
+// Registers per thread by role.  A warpgroup asking for more than the pool holds would wait for ever: both kernels
+// start 768 threads x 80.
+#define PA_BWD_REG_CTRL 48
+#define PA_BWD_REG_COMP 96
+#define PA_BWD_REG_EPI 48
+static_assert(4 * PA_BWD_REG_CTRL + 16 * PA_BWD_REG_COMP + 4 * PA_BWD_REG_EPI <= 24 * 80, "register split exceeds the CTA's registers");
 
 namespace pa {
 
-constexpr int kDkvThreads = 640;
-constexpr int kDqThreads = 768;
+constexpr int kTcThreads = 768;
 constexpr int kCompWarps = 16;
 constexpr uint32_t kTcTmemCols = 512;
 constexpr long long kBwdWaitCycles = 4000000000ll;
@@ -64,9 +60,10 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, int a_mn, int b_
 }
 
 // A work item as the producer publishes it.  blk: the query block (dQ) or key block (dK / dV); n: how many blocks
-// its row or chunk lists, from e0 on (negative: there are no more items); parts: chunks of the key block.
+// its row or chunk lists, from e0 on (negative: there are no more items); parts: chunks of the key block;
+// first: the first block listed (dK / dV).
 struct __align__(16) BwdItem {
-    int32_t blk, n, e0, hk, b, hp, parts, pad;
+    int32_t blk, n, e0, hk, b, hp, parts, first;
 };
 struct BwdTail {
     BwdItem items[kItemRing];
@@ -104,6 +101,19 @@ __device__ __forceinline__ uint32_t bwd_cvt(uint64_t v)
 __device__ __forceinline__ uint64_t bwd_ds(uint64_t p, uint32_t dp0, uint32_t dp1, uint64_t neg_delta2)
 {
     return ptx::mul_f32x2(p, ptx::add_f32x2(ptx::pack_f32x2(__uint_as_float(dp0), __uint_as_float(dp1)), neg_delta2));
+}
+// Lane t of every four lanes holds M[t][0..3] and gets M[0..3][t].
+__device__ __forceinline__ void transpose_quad(uint32_t &r0, uint32_t &r1, uint32_t &r2, uint32_t &r3, int lane)
+{
+    auto exchange = [&](uint32_t &lo, uint32_t &hi, int d) {
+        const bool upper = lane & d;
+        const uint32_t got = __shfl_xor_sync(0xffffffffu, upper ? lo : hi, d);
+        (upper ? lo : hi) = got;
+    };
+    exchange(r0, r1, 1);
+    exchange(r2, r3, 1);
+    exchange(r0, r2, 2);
+    exchange(r1, r3, 2);
 }
 // -LSE in base 2; a row without weights (beyond the sequence, padding head, empty row) gets -inf: P = 0.
 __device__ __forceinline__ float bwd_neg_lse2(float lse)
@@ -148,7 +158,7 @@ struct DqCfg {
 };
 
 template <int D>
-__global__ void __launch_bounds__(kDqThreads, 1)
+__global__ void __launch_bounds__(kTcThreads, 1)
 dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmG,
           const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
           const __grid_constant__ CUtensorMap tmDq, const BackwardArgs a, const uint32_t n_items)
@@ -204,7 +214,7 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
         ptx::mbar_init(bar(C::DQ_FREE), 4);
         for (uint32_t r = 0; r < kItemRing; ++r) {
             ptx::mbar_init(bar(C::ITEM_FULL + r), 1);
-            ptx::mbar_init(bar(C::ITEM_EMPTY + r), kDqThreads / 32 - 1);
+            ptx::mbar_init(bar(C::ITEM_EMPTY + r), kTcThreads / 32 - 1);
         }
         tail->abort_flag = 0;
         ptx::fence_barrier_init();
@@ -221,7 +231,7 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = tail->tmem;
 
-    if (warp < 4) ptx::setmaxnreg_dec<PA_DQ_REG_CTRL>();
+    if (warp < 4) ptx::setmaxnreg_dec<PA_BWD_REG_CTRL>();
     if (warp == 0) {
         // -------------------------------------------------------------- TMA producer
         if (lane == 0) {
@@ -255,7 +265,7 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
             };
             uint32_t c = 0, kq = 0;  // steps and non-empty items so far
             BwdItem w, wn;
-            w.parts = w.pad = wn.parts = wn.pad = 0;
+            w.parts = w.first = wn.parts = wn.first = 0;
             next_item(w);
             bool ok = publish(0, w);
             for (uint32_t k = 0; w.n >= 0 && ok; ++k) {
@@ -385,7 +395,7 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
     } else if (warp < 4 + kCompWarps) {
         // -------------------------------------------------------------- compute warps
         // Warpgroup g: every fourth step.
-        ptx::setmaxnreg_inc<PA_DQ_REG_COMP>();
+        ptx::setmaxnreg_inc<PA_BWD_REG_COMP>();
         const uint32_t g = (uint32_t)(warp - 4) >> 2;
         const int quad = warp & 3;
         const int row = quad * 32 + lane, qrow = row & 63;
@@ -468,7 +478,7 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
         // dQ = scale x the accumulator.  A warp's 32 rows leave 32 features at a time: through a swizzled patch of
         // shared memory and a bulk tensor store each (rows beyond the sequence are clipped by the tensor map).  (Plain stores moved 10 B/clk out of the SM: 7000 clk an item, during which the
         // accumulator, or 128 registers a thread, was held.)
-        ptx::setmaxnreg_dec<PA_DQ_REG_EPI>();
+        ptx::setmaxnreg_dec<PA_BWD_REG_EPI>();
         const int quad = warp & 3;
         const int row = quad * 32 + lane, qrow = row & 63;
         const uint32_t t_lane = tmem_base + ((uint32_t)(quad * 32) << 16);
@@ -564,8 +574,13 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
 // stage's Q and dO tiles lie side by side and are read as ONE 128-row A operand [Q | dO]^T against B = [P | dS]
 // (N = 128): two quadrants of the product are dV^T and dK^T, the other two are not used, and the eight MMAs take
 // 512 clk where two products of 64 accumulator rows take 768.
-// Measured, 28 / 4 heads at 32K tokens: 848 us, where one CTA per chunk with two common Q + dO stages and two
-// warpgroups took 985; 64 features, 16 / 4 heads, 2 x 8K tokens: 177 us, where the warp-level MMA kernel took about 300.
+// An item's accumulators have two buffers and warps of their own that write them out, the compute warps walk the
+// steps across the ends of items, and the next item is looked up by the epilogue's first warp while the one before
+// it is computed: with the lookup (a halving search, ten dependent loads) in the producer's way and the output in
+// that of the compute warps, every item began with some 8000 clk in which the tensor cores stood still, against
+// 10000 to 30000 of work.
+// Measured, 28 / 4 heads: the whole backward pass at 4K tokens 154 us (160 with items one after the other), at 32K
+// 1430 us at full clocks (1488); 64 features, 16 / 4 heads, 2 x 8K tokens: 234 us (269).
 template <int D>
 struct DkvCfg {
     static constexpr int kDH = D / 64;
@@ -587,17 +602,17 @@ struct DkvCfg {
         DP_FULL = S_TAKEN + 2, DP_TAKEN = DP_FULL + 2,
         P_FULL = DP_TAKEN + 2, DS_FULL = P_FULL + kPBufs,      // [P / dS buffer]
         P_FREE = DS_FULL + kPBufs, DS_FREE = P_FREE + 2,       // [step parity]: that step's product has read it
-        ACC_FULL = DS_FREE + 2, ACC_FREE,                      // the item's dK^T and dV^T are complete / have been read
-        ITEM_FULL, ITEM_EMPTY = ITEM_FULL + kItemRing, COUNT = ITEM_EMPTY + kItemRing
+        ACC_FULL = DS_FREE + 2, ACC_FREE = ACC_FULL + 2,       // [item parity]: dK^T and dV^T are complete / have been read
+        ITEM_FULL = ACC_FREE + 2, ITEM_EMPTY = ITEM_FULL + kItemRing, COUNT = ITEM_EMPTY + kItemRing
     };
     static_assert(COUNT * 8 <= kBarBytes, "barrier area");
-    // Tensor memory columns: S at 128 b, dP at 128 b + 64 (b = step parity); accumulators at 256: dK^T, then dV^T
-    // (head_dim 128), or the product with [P | dS] (head_dim 64).
+    // Tensor memory columns: S at 128 b, dP at 128 b + 64 (b = step parity); accumulators at 256 + 128 (item parity):
+    // dK^T, then dV^T (head_dim 128), or the product with [P | dS] (head_dim 64).
     static constexpr uint32_t kColAcc = 256;
 };
 
 template <int D>
-__global__ void __launch_bounds__(kDkvThreads, 1)
+__global__ void __launch_bounds__(kTcThreads, 1)
 dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmG,
            const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const BackwardArgs a,
            const uint32_t n_items)
@@ -650,11 +665,13 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             ptx::mbar_init(bar(C::P_FULL + s), kCompWarps / 2);
             ptx::mbar_init(bar(C::DS_FULL + s), kCompWarps / 2);
         }
-        ptx::mbar_init(bar(C::ACC_FULL), 1);
-        ptx::mbar_init(bar(C::ACC_FREE), kCompWarps);
+        for (int s = 0; s < 2; ++s) {
+            ptx::mbar_init(bar(C::ACC_FULL + s), 1);
+            ptx::mbar_init(bar(C::ACC_FREE + s), 4);
+        }
         for (uint32_t r = 0; r < kItemRing; ++r) {
             ptx::mbar_init(bar(C::ITEM_FULL + r), 1);
-            ptx::mbar_init(bar(C::ITEM_EMPTY + r), kDkvThreads / 32 - 1);
+            ptx::mbar_init(bar(C::ITEM_EMPTY + r), kTcThreads / 32);
         }
         tail->abort_flag = 0;
         ptx::fence_barrier_init();
@@ -671,7 +688,7 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = tail->tmem;
 
-    if (warp < 4) ptx::setmaxnreg_dec<PA_DKV_REG_CTRL>();
+    if (warp < 4) ptx::setmaxnreg_dec<PA_BWD_REG_CTRL>();
     if (warp == 0) {
         // -------------------------------------------------------------- TMA producer
         if (lane == 0) {
@@ -679,42 +696,14 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             ptx::prefetch_tensormap(&tmG);
             ptx::prefetch_tensormap(&tmK);
             ptx::prefetch_tensormap(&tmV);
-            // Items: chunk slots in column order (the sink block's long column first), and within a slot the KV
-            // heads and batch entries; slots without work are passed over.
-            uint32_t it = blockIdx.x;
-            auto next_item = [&](BwdItem &w) {
-                w.n = -1;
-                const uint32_t per_slot = (uint32_t)(a.Hkv * a.batch);
-                while (it < n_items) {
-                    const uint32_t slot = it / per_slot, yz = it - slot * per_slot;
-                    const BackwardChunk ch = backward_chunk_at(a, (int32_t)slot);
-                    it = gridDim.x + (uint32_t)atomicAdd(a.status + kBwdDkvCounter, 1);
-                    if (ch.e0 >= ch.e1) continue;
-                    w.blk = ch.j;
-                    w.e0 = ch.e0;
-                    w.n = ch.e1 - ch.e0;
-                    w.parts = ch.parts;
-                    w.b = (int32_t)(yz / (uint32_t)a.Hkv);
-                    w.hk = (int32_t)(yz % (uint32_t)a.Hkv);
-                    return;
-                }
-            };
-            auto publish = [&](uint32_t k, const BwdItem &w) {
-                const uint32_t r = k % kItemRing;
-                if (k >= kItemRing && !wait_bar(bar(C::ITEM_EMPTY + r), (k / kItemRing - 1) & 1, 32)) return false;
-                tail->items[r] = w;
-                ptx::mbar_arrive(bar(C::ITEM_FULL + r));
-                return true;
-            };
             uint32_t c = 0;  // steps so far
-            BwdItem w, wn;
-            w.hp = w.pad = wn.hp = wn.pad = 0;
-            next_item(w);
-            bool ok = publish(0, w);
-            for (uint32_t k = 0; w.n >= 0 && ok; ++k) {
-                next_item(wn);
-                ok = publish(k + 1, wn);
-                if (!ok) break;
+            bool ok = true;
+            for (uint32_t k = 0; ok; ++k) {
+                const uint32_t r = k % kItemRing;
+                if (!wait_bar(bar(C::ITEM_FULL + r), (k / kItemRing) & 1, 32)) break;
+                const BwdItem w = tail->items[r];
+                ptx::mbar_arrive(bar(C::ITEM_EMPTY + r));
+                if (w.n < 0) break;
                 auto load_rows = [&](uint32_t dst, const CUtensorMap *tm, uint32_t full, uint32_t empty, uint32_t stages, int32_t i,
                                      int h0, int code) {
                     const uint32_t st = c % stages;
@@ -725,7 +714,7 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                                          i * kBwdBlk, h0, w.b);
                     return true;
                 };
-                int32_t i = __ldg(a.row_idx + w.e0);
+                int32_t i = w.first;
                 for (int x = 0; x < w.n && ok; ++x) {
                     const int32_t in = x + 1 < w.n ? __ldg(a.row_idx + w.e0 + x + 1) : 0;
                     for (int hp = 0; hp < a.npairs && ok; ++hp, ++c) {
@@ -744,7 +733,6 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                     }
                     i = in;
                 }
-                w = wn;
             }
         }
         __syncwarp();
@@ -796,7 +784,7 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         // key-contiguous; 16 tile rows per MMA, 2048 bytes further each.
         const bool leader = ptx::elect_one();
         constexpr uint32_t idesc_t = idesc_bf16(128, D == 128 ? 64 : 128, 1, 1);
-        const uint32_t t_base = __shfl_sync(0xffffffffu, tmem_base + C::kColAcc, 0);
+        const uint32_t t_acc = __shfl_sync(0xffffffffu, tmem_base + C::kColAcc, 0);
         uint32_t c = 0;
         bool ok = true;
         for (uint32_t k = 0; ok; ++k) {
@@ -804,8 +792,9 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             ok = read_item(k, w);
             const int n = __shfl_sync(0xffffffffu, w.n, 0) * a.npairs;
             if (!ok || n < 0) break;
-            // The previous item's accumulators must have been read.
-            if (k > 0) ok = wait_warp(bar(C::ACC_FREE), (k - 1) & 1, 39);
+            // The accumulators of the item before the previous one must have been read.
+            const uint32_t t_base = t_acc + 128 * (k & 1);
+            if (k >= 2) ok = wait_warp(bar(C::ACC_FREE + (k & 1)), ((k >> 1) - 1) & 1, 39);
             for (int e = 0; e < n && ok; ++e, ++c) {
                 const uint32_t sq = c % NQ, sg = c % NG, pb = c % NP, pphase = (c / NP) & 1;
                 const uint32_t qa = ((smem_base + C::kQ + sq * C::kPitch) >> 4) | ((kRowTile >> 4) << 16);
@@ -826,8 +815,6 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                         ptx::umma_commit(bar(C::P_FREE + (c & 1)));
                     }
                     __syncwarp();
-                } else {
-                    ok = wait_warp(bar(C::P_FULL + pb), pphase, 40);
                 }
                 ok = ok && wait_warp(bar(C::DS_FULL + pb), pphase, 41);
                 if (!ok) break;
@@ -840,160 +827,208 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                                           (e > 0 || kk > 0) ? 1u : 0u);
                     ptx::umma_commit(bar(C::Q_EMPTY + sq));
                     ptx::umma_commit(bar(C::DS_FREE + (c & 1)));
-                    if (D == 64) {
-                        ptx::umma_commit(bar(C::G_EMPTY + sg));
-                        ptx::umma_commit(bar(C::P_FREE + (c & 1)));
-                    }
-                    if (e == n - 1) ptx::umma_commit(bar(C::ACC_FULL));
+                    if (D == 64) ptx::umma_commit(bar(C::G_EMPTY + sg));
+                    if (e == n - 1) ptx::umma_commit(bar(C::ACC_FULL + (k & 1)));
                 }
                 __syncwarp();
             }
         }
-    } else {
+    } else if (warp < 4 + kCompWarps) {
         // -------------------------------------------------------------- compute warps
         // Warpgroup wg: steps of parity wg & 1, keys 32 (wg >> 1) .. + 31.
-        ptx::setmaxnreg_inc<PA_DKV_REG_COMP>();
+        ptx::setmaxnreg_inc<PA_BWD_REG_COMP>();
         const int wg = (warp - 4) >> 2, quad = warp & 3, par = wg & 1, half = wg >> 1;
         const int row = quad * 32 + lane, qrow = row & 63;
         const uint32_t t_lane = tmem_base + ((uint32_t)(quad * 32) << 16);
         const uint64_t scale2 = ptx::pack_f32x2(a.scale_log2, a.scale_log2);
-        // Row statistics of this thread's next step, LSE and delta, are requested one of its steps ahead and its
-        // query block's index one more, across items as well; nothing uses a loaded value on the spot.
-        struct Place {
-            int x, hp;  // place in the chunk's list, head pair
-        };
-        auto advance = [&](Place &p, int steps) {
-            p.hp += steps;
-            while (p.hp >= a.npairs) {
-                p.hp -= a.npairs;
-                ++p.x;
-            }
-        };
-        auto block_at = [&](const BwdItem &w, const Place &p) { return p.x < w.n ? __ldg(a.row_idx + w.e0 + p.x) : -1; };
+        // The warp walks its steps without regard to where items end.  The place (item, query block in the list, head
+        // pair) is that of its next step: the query block's index is requested at the start of a step for the next
+        // one and the row statistics, LSE and delta, in its middle; nothing uses a loaded value on the spot.
+        BwdItem w;
+        uint32_t k = 0;
+        int x = 0, hp = 0;
+        int32_t i_next = -1;
         float lse_n = INFINITY, delta_n = 0.f;
-        auto request = [&](const BwdItem &w, int32_t i, const Place &p) {
+        bool ok = read_item(0, w);
+        auto advance = [&](int steps) {
+            hp += steps;
+            while (hp >= a.npairs) {
+                hp -= a.npairs;
+                ++x;
+            }
+            while (ok && w.n >= 0 && x >= w.n) {
+                x -= w.n;
+                ok = read_item(++k, w);
+            }
+            i_next = ok && w.n >= 0 ? __ldg(a.row_idx + w.e0 + x) : -1;
+        };
+        auto request = [&]() {
             lse_n = INFINITY;
             delta_n = 0.f;
-            const int head_local = 2 * p.hp + (row >> 6);
-            const int64_t q = (int64_t)i * kBwdBlk + qrow;
-            if (i >= 0 && head_local < a.G && q < a.N) {
+            const int head_local = 2 * hp + (row >> 6);
+            const int64_t q = (int64_t)i_next * kBwdBlk + qrow;
+            if (i_next >= 0 && head_local < a.G && q < a.N) {
                 const int64_t at = ((int64_t)w.b * a.Hq + w.hk * a.G + head_local) * a.N + q;
                 lse_n = __ldg(a.lse + at);
                 delta_n = __ldg(a.delta + at);
             }
         };
-        uint32_t c = 0;      // step number at the item's start
-        BwdItem w, wn;
-        bool ok = read_item(0, w);
-        Place next = {0, 0};  // of the step after the current one
-        int32_t i_next = -1;
-        if (ok && w.n >= 0) {
-            advance(next, par);
-            i_next = block_at(w, next);
-            request(w, i_next, next);
-        }
-        for (uint32_t k = 0; ok && w.n >= 0; ++k) {
-            const int n = w.n * a.npairs;
-            // (next, i_next, lse_n and delta_n are those of this warp's first step in the item)
-            for (uint32_t e = (c ^ (uint32_t)par) & 1; e < (uint32_t)n; e += 2) {
-                const uint32_t cc = c + e, pb = cc % NP;
-                const bool diag = i_next == w.blk;
-                const float neg_lse2 = bwd_neg_lse2(lse_n);
-                const uint64_t neg_lse2_2 = ptx::pack_f32x2(neg_lse2, neg_lse2), neg_delta2 = ptx::pack_f32x2(-delta_n, -delta_n);
-                advance(next, 2);
-                i_next = block_at(w, next);
-                uint32_t x32[32];
-                uint64_t p[16];
-                ok = wait_warp(bar(C::S_FULL + par), (cc >> 1) & 1, 42);
-                if (!ok) break;
-                ptx::tc_fence_after_sync();
-                ptx::tmem_ld32(t_lane + 128 * par + 32 * half, x32);
-                ptx::tmem_wait_ld();
-                ptx::tc_fence_before_sync();
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(bar(C::S_TAKEN + par));
-                request(w, i_next, next);  // (in flight during this step)
-                // Algorithm 1's causal term acts inside the diagonal pair only.
-                bwd_p(x32, diag, qrow - 32 * half, scale2, neg_lse2_2, p);
-                // The P / dS buffer was read by the products of step cc - NP.  (Their barriers alternate by step
-                // parity: with one buffer a warpgroup would otherwise wait for every other phase of a barrier only,
-                // whose parity cannot tell two phases ahead from none.)
-                if (cc >= NP) {
-                    ok = wait_warp(bar(C::P_FREE + ((cc - NP) & 1)), ((cc - NP) >> 1) & 1, 43);
-                    if (!ok) break;
-                }
-                // 16-byte chunk q of tile row r sits at chunk position q ^ (r & 7) (128-byte swizzle).
-                const uint32_t p_row = smem_base + C::kPD + pb * 2 * kRowTile + (uint32_t)row * 128u;
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    ptx::st_shared_v4(p_row + (uint32_t)(((4 * half + q) ^ (row & 7)) << 4), bwd_cvt(p[4 * q]), bwd_cvt(p[4 * q + 1]),
-                                      bwd_cvt(p[4 * q + 2]), bwd_cvt(p[4 * q + 3]));
-                ptx::fence_proxy_async_smem();
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(bar(C::P_FULL + pb));
-                ok = wait_warp(bar(C::DP_FULL + par), (cc >> 1) & 1, 44);
-                if (!ok) break;
-                ptx::tc_fence_after_sync();
-                ptx::tmem_ld32(t_lane + 128 * par + 64 + 32 * half, x32);
-                ptx::tmem_wait_ld();
-                ptx::tc_fence_before_sync();
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(bar(C::DP_TAKEN + par));
-                if (cc >= NP) {
-                    ok = wait_warp(bar(C::DS_FREE + ((cc - NP) & 1)), ((cc - NP) >> 1) & 1, 45);
-                    if (!ok) break;
-                }
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    uint32_t v[4];
-#pragma unroll
-                    for (int y = 0; y < 4; ++y)
-                        v[y] = bwd_cvt(bwd_ds(p[4 * q + y], x32[8 * q + 2 * y], x32[8 * q + 2 * y + 1], neg_delta2));
-                    ptx::st_shared_v4(p_row + kRowTile + (uint32_t)(((4 * half + q) ^ (row & 7)) << 4), v[0], v[1], v[2], v[3]);
-                }
-                ptx::fence_proxy_async_smem();
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(bar(C::DS_FULL + pb));
-            }
+        if (ok && w.n >= 0) advance(par);
+        request();
+        for (uint32_t cc = (uint32_t)par; ok && w.n >= 0; cc += 2) {
+            const uint32_t pb = cc % NP;
+            const bool diag = i_next == w.blk;
+            const float neg_lse2 = bwd_neg_lse2(lse_n);
+            const uint64_t neg_lse2_2 = ptx::pack_f32x2(neg_lse2, neg_lse2), neg_delta2 = ptx::pack_f32x2(-delta_n, -delta_n);
+            advance(2);
             if (!ok) break;
-            // The next item's first step, requested ahead of this item's output.
-            c += (uint32_t)n;
-            ok = read_item(k + 1, wn);
-            if (!ok) break;
-            next = {0, 0};
-            advance(next, (int)((c ^ (uint32_t)par) & 1));
-            i_next = block_at(wn, next);
-            // ---- output: thread = feature, one key per register, 128 contiguous bytes per warp instruction.  A
-            // key block of one chunk is written, the parts of others are added up in memory.
-            ok = wait_warp(bar(C::ACC_FULL), k & 1, 46);
+            uint32_t x32[32];
+            uint64_t p[16];
+            ok = wait_warp(bar(C::S_FULL + par), (cc >> 1) & 1, 42);
             if (!ok) break;
             ptx::tc_fence_after_sync();
-            constexpr int kKeys = D == 128 ? 32 : 16;  // keys per warp
-            const bool is_dk = D == 128 ? par == 0 : quad < 2;
-            const int key0 = D == 128 ? 32 * half : 16 * wg, feature = D == 128 ? row : row & 63;
-            const uint32_t col = C::kColAcc + (D == 128 ? (is_dk ? 0u : 64u) : (is_dk ? 64u : 0u)) + key0;
-            uint32_t acc[kKeys];
-            if (D == 128) ptx::tmem_ld32(t_lane + col, *reinterpret_cast<uint32_t(*)[32]>(acc));
-            else ptx::tmem_ld16(t_lane + col, *reinterpret_cast<uint32_t(*)[16]>(acc));
+            ptx::tmem_ld32(t_lane + 128 * par + 32 * half, x32);
             ptx::tmem_wait_ld();
             ptx::tc_fence_before_sync();
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(bar(C::ACC_FREE));
-            request(wn, i_next, next);
-            const int64_t tok0 = (int64_t)w.blk * kBwdBlk + key0;
-            float *dst = (is_dk ? a.dk : a.dv) + (((int64_t)w.b * a.N + tok0) * a.Hkv + w.hk) * D + feature;
-            const float f = is_dk ? a.scale : 1.0f;
-            const int64_t pitch = (int64_t)a.Hkv * D;
-            if (w.parts == 1) {
-#pragma unroll
-                for (int x = 0; x < kKeys; ++x)
-                    if (tok0 + x < a.N) dst[x * pitch] = __uint_as_float(acc[x]) * f;
-            } else {
-#pragma unroll
-                for (int x = 0; x < kKeys; ++x)
-                    if (tok0 + x < a.N) atomicAdd(dst + x * pitch, __uint_as_float(acc[x]) * f);
+            if (lane == 0) ptx::mbar_arrive(bar(C::S_TAKEN + par));
+            request();  // (in flight during this step)
+            // Algorithm 1's causal term acts inside the diagonal pair only.
+            bwd_p(x32, diag, qrow - 32 * half, scale2, neg_lse2_2, p);
+            // The P / dS buffer was read by the products of step cc - NP.  (Their barriers alternate by step
+            // parity: with one buffer a warpgroup would otherwise wait for every other phase of a barrier only,
+            // whose parity cannot tell two phases ahead from none.  With head_dim 64 one product reads both.)
+            if (cc >= NP) {
+                ok = wait_warp(bar((D == 128 ? C::P_FREE : C::DS_FREE) + ((cc - NP) & 1)), ((cc - NP) >> 1) & 1, 43);
+                if (!ok) break;
             }
-            w = wn;
+            // 16-byte chunk q of tile row r sits at chunk position q ^ (r & 7) (128-byte swizzle).
+            const uint32_t p_row = smem_base + C::kPD + pb * 2 * kRowTile + (uint32_t)row * 128u;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                ptx::st_shared_v4(p_row + (uint32_t)(((4 * half + q) ^ (row & 7)) << 4), bwd_cvt(p[4 * q]), bwd_cvt(p[4 * q + 1]),
+                                  bwd_cvt(p[4 * q + 2]), bwd_cvt(p[4 * q + 3]));
+            if (D == 128) {
+                ptx::fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(bar(C::P_FULL + pb));
+            }
+            ok = wait_warp(bar(C::DP_FULL + par), (cc >> 1) & 1, 44);
+            if (!ok) break;
+            ptx::tc_fence_after_sync();
+            ptx::tmem_ld32(t_lane + 128 * par + 64 + 32 * half, x32);
+            ptx::tmem_wait_ld();
+            ptx::tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(bar(C::DP_TAKEN + par));
+            if (D == 128 && cc >= NP) {
+                ok = wait_warp(bar(C::DS_FREE + ((cc - NP) & 1)), ((cc - NP) >> 1) & 1, 45);
+                if (!ok) break;
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                uint32_t v[4];
+#pragma unroll
+                for (int y = 0; y < 4; ++y)
+                    v[y] = bwd_cvt(bwd_ds(p[4 * q + y], x32[8 * q + 2 * y], x32[8 * q + 2 * y + 1], neg_delta2));
+                ptx::st_shared_v4(p_row + kRowTile + (uint32_t)(((4 * half + q) ^ (row & 7)) << 4), v[0], v[1], v[2], v[3]);
+            }
+            ptx::fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(bar(C::DS_FULL + pb));
+        }
+    } else {
+        // -------------------------------------------------------------- epilogue warps; the first one finds the items
+        ptx::setmaxnreg_dec<PA_BWD_REG_EPI>();
+        const int quad = warp & 3;
+        const uint32_t t_lane = tmem_base + ((uint32_t)(quad * 32) << 16);
+        // Items: chunk slots in column order (the sink block's long column first), and within a slot the KV heads and
+        // batch entries; slots without work are passed over.
+        uint32_t it = blockIdx.x;
+        auto publish_next = [&](uint32_t k) {
+            const uint32_t r = k % kItemRing, per_slot = (uint32_t)(a.Hkv * a.batch);
+            BwdItem w = {0, -1, 0, 0, 0, 0, 0, 0};
+            while (it < n_items && w.n < 0) {
+                const uint32_t slot = it / per_slot, yz = it - slot * per_slot;
+                const BackwardChunk ch = backward_chunk_by_warp(a, (int32_t)slot, lane);
+                if (ch.e0 < ch.e1) {
+                    w.blk = ch.j;
+                    w.e0 = ch.e0;
+                    w.n = ch.e1 - ch.e0;
+                    w.parts = ch.parts;
+                    w.b = (int32_t)(yz / (uint32_t)a.Hkv);
+                    w.hk = (int32_t)(yz % (uint32_t)a.Hkv);
+                    w.first = __ldg(a.row_idx + w.e0);
+                }
+                int drawn = 0;
+                if (lane == 0) drawn = atomicAdd(a.status + kBwdDkvCounter, 1);
+                it = gridDim.x + (uint32_t)__shfl_sync(0xffffffffu, drawn, 0);
+            }
+            if (k >= kItemRing && !wait_warp(bar(C::ITEM_EMPTY + r), (k / kItemRing - 1) & 1, 34)) return -2;
+            if (lane == 0) {
+                tail->items[r] = w;
+                ptx::mbar_arrive(bar(C::ITEM_FULL + r));
+            }
+            return w.n;
+        };
+        const bool finder = warp == 4 + kCompWarps;
+        int n_next = -1;  // (finder) length of item k + 1
+        bool ok = true;
+        if (finder && publish_next(0) >= 0) {
+            n_next = publish_next(1);
+            ok = wait_warp(bar(C::KV_FULL), 0, 35);
+        }
+        for (uint32_t k = 0; ok; ++k) {
+            BwdItem w;
+            ok = read_item(k, w);
+            if (!ok || w.n < 0) break;
+            // Item k + 2 is looked for when the loads have got to item k + 1.
+            if (finder && n_next >= 0) {
+                ok = wait_warp(bar(C::KV_FULL), (k + 1) & 1, 35);
+                if (!ok) break;
+                n_next = publish_next(k + 2);
+            }
+            ok = wait_warp(bar(C::ACC_FULL + (k & 1)), (k >> 1) & 1, 46);
+            if (!ok) break;
+            ptx::tc_fence_after_sync();
+            // A lane holds a feature and a register a key.  Quads of lanes transpose 4 x 4 among themselves, so that
+            // a lane gets four features of a key: 16 bytes.  A key block of one chunk is written, the parts of others
+            // are added up in memory.  (The four warps take 12000 clk for an item's 64 KB, 26000 with 4 bytes a lane
+            // and 14000 with 32 keys at a time, for which the addresses find no registers.)
+            const int64_t pitch = (int64_t)a.Hkv * D;
+            constexpr int kChunks = D == 128 ? 8 : 4;  // of 16 accumulator columns that the warp takes
+#pragma unroll 1
+            for (int ch = 0; ch < kChunks; ++ch) {
+                const bool is_dk = D == 128 ? ch < 4 : quad < 2;
+                uint32_t acc[16];
+                ptx::tmem_ld16(t_lane + C::kColAcc + 128 * (k & 1) + (D == 64 && is_dk ? 64 : 0) + 16 * ch, acc);
+                ptx::tmem_wait_ld();
+                if (ch == kChunks - 1) {
+                    ptx::tc_fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) ptx::mbar_arrive(bar(C::ACC_FREE + (k & 1)));
+                }
+                const int64_t tok0 = (int64_t)w.blk * kBwdBlk + 16 * (ch & 3) + (lane & 3);
+                const int keys = a.N - tok0 < 16 ? (int)(a.N - tok0) : 16;
+                float *dst = (is_dk ? a.dk : a.dv) + (((int64_t)w.b * a.N + tok0) * a.Hkv + w.hk) * D +
+                             ((quad * 32 + lane) & (D - 4));
+                const float f = is_dk ? a.scale : 1.0f;
+                float *at[4];
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    transpose_quad(acc[4 * x], acc[4 * x + 1], acc[4 * x + 2], acc[4 * x + 3], lane);
+                    at[x] = dst + 4 * x * pitch;
+                }
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    const float4 v = make_float4(__uint_as_float(acc[4 * x]) * f, __uint_as_float(acc[4 * x + 1]) * f,
+                                                 __uint_as_float(acc[4 * x + 2]) * f, __uint_as_float(acc[4 * x + 3]) * f);
+                    if (4 * x < keys) {
+                        if (w.parts == 1) *reinterpret_cast<float4 *>(at[x]) = v;
+                        else ptx::red_add_v4(at[x], v);
+                    }
+                }
+            }
         }
     }
 
@@ -1038,9 +1073,9 @@ static pa_status launch_tc(const BackwardArgs &a, const pa_prefill_params *p, in
     const int64_t dkv_items = (nnz / a.chunk + a.nqb) * a.Hkv * a.batch;  // (chunk slots, some of them empty)
     if (dq_items > (int64_t)0x3fffffff || dkv_items > (int64_t)0x3fffffff)
         return fail(PA_ERR_SHAPE, "too many work items (%lld, %lld)", (long long)dq_items, (long long)dkv_items);
-    PA_CUDA_OK(launch_pdl(dq_kernel<D>, dim3((unsigned)(dq_items < sms ? dq_items : sms)), kDqThreads, DqCfg<D>::kAlloc, st, tmQ,
+    PA_CUDA_OK(launch_pdl(dq_kernel<D>, dim3((unsigned)(dq_items < sms ? dq_items : sms)), kTcThreads, DqCfg<D>::kAlloc, st, tmQ,
                           tmG, tmK, tmV, tmDq, a, (uint32_t)dq_items));
-    PA_CUDA_OK(launch_pdl(dkv_kernel<D>, dim3((unsigned)(dkv_items < sms ? dkv_items : sms)), kDkvThreads, DkvCfg<D>::kAlloc, st,
+    PA_CUDA_OK(launch_pdl(dkv_kernel<D>, dim3((unsigned)(dkv_items < sms ? dkv_items : sms)), kTcThreads, DkvCfg<D>::kAlloc, st,
                           tmQ, tmG, tmK, tmV, a, (uint32_t)dkv_items));
     return PA_OK;
 }

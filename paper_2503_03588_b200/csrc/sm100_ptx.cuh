@@ -305,6 +305,12 @@ __device__ __forceinline__ void setmaxnreg_dec()
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(N));
 }
 
+// Four consecutive floats (16-byte aligned) added to global memory.
+__device__ __forceinline__ void red_add_v4(float *p, const float4 &v)
+{
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};\n" ::"l"(p), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+
 __device__ __forceinline__ float ex2(float x)
 {
     float y;

@@ -237,3 +237,27 @@ def test_backward_on_arbitrary_causal_layouts(pa, oracle, N, Hq, Hkv, D):
     pa.pa_prefill_status(wsb)
     for g, r, n in zip((dq, dk, dv), oracle.backward(Q, K, V, dO, 64, 5, 1, dense=dense), ("dQ", "dK", "dV")):
         _compare(g, r, n + " random layout")
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_backward_of_many_short_lists(pa, oracle, D):
+    """Key blocks listed by one or two rows, one head pair per group: work items of one and two steps, several per
+    CTA, so that a warp's next step lies one, two or three items ahead."""
+    nqb, Hkv = 12, 40
+    N, Hq = 64 * nqb - 5, 2 * Hkv
+    rows = [[i - 1, i] if i % 3 == 2 else [i] for i in range(nqb)]
+    rp = np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.int32)
+    ci = np.asarray([j for r in rows for j in r], dtype=np.int32)
+    dense = np.zeros((N, N), dtype=bool)
+    for i, r in enumerate(rows):
+        for j in r:
+            dense[i * 64:(i + 1) * 64, j * 64:(j + 1) * 64] = True
+    dense &= np.tril(np.ones((N, N), dtype=bool))
+    Q, K, V = (si.bf16_randn((1, N, h, D), 1700 + D + x) for x, h in enumerate((Hq, Hkv, Hkv)))
+    dO = si.bf16_randn((1, N, Hq, D), 1704 + D)
+    Qd, Kd, Vd, dOd, rpd, cid = (t.cuda() for t in (Q, K, V, dO, torch.as_tensor(rp), torch.as_tensor(ci)))
+    o, lse, _ = pa.pa_prefill(Qd, Kd, Vd, rpd, cid)
+    dq, dk, dv, wsb = pa.pa_prefill_backward(Qd, Kd, Vd, o, lse, dOd, rpd, cid)
+    pa.pa_prefill_status(wsb)
+    for g, r, n in zip((dq, dk, dv), oracle.backward(Q, K, V, dO, 64, 5, 1, dense=dense), ("dQ", "dK", "dV")):
+        _compare(g, r, n + " short lists")
