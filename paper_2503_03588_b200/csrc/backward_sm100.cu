@@ -126,24 +126,25 @@ __device__ __forceinline__ float bwd_neg_lse2(float lse)
 // the tensor cores work 1024.  So four steps are under way at a time, a warpgroup each.  Tensor memory decides the
 // rest: S has four buffers (dS goes over the S it was made from), dP two, which a warpgroup therefore loads whole
 // (64 registers a thread) before it works through S 16 keys at a time.  K stays in its ring until dQ has read
-// it, V only until dP has.  Q and dO have one buffer each: the next item's tiles arrive while the last steps are
-// computed and their dQ products run.  Bound by the issue of S and dP (1300 clk a step) and by the 128 KB that an
+// it, V only until dP has.  Q and dO have one buffer each with head_dim 128: the next item's tiles arrive while the last steps are
+// computed and their dQ products run.  With head_dim 64, whose steps are shorter than that, two.  Bound by the issue of S and dP (1300 clk a step) and by the 128 KB that an
 // item starts with.  Measured, 28 / 4 heads at 32K tokens: 524 us at full clocks, where all four warpgroups on one
-// step of two key blocks took 583; 64 features, 16 / 4 heads, 2 x 8K tokens: 87 us against 106.
+// step of two key blocks took 583; 64 features, 16 / 4 heads, 2 x 8K tokens: 87 us against 106, 82 with the second
+// pair of Q and dO buffers.
 template <int D>
 struct DqCfg {
     static constexpr int kDH = D / 64;
-    static constexpr int kKStages = D == 128 ? 6 : 8, kVStages = D == 128 ? 3 : 4;
+    static constexpr int kKStages = D == 128 ? 6 : 8, kVStages = D == 128 ? 3 : 4, kRowBufs = D == 128 ? 1 : 2;
     static constexpr uint32_t kTile = kDH * kRowTile, kBlkTile = kDH * kKeyTile;
-    static constexpr uint32_t kQ = 0, kG = kTile;
-    static constexpr uint32_t kK = 2 * kTile, kV = kK + kKStages * kBlkTile;
+    static constexpr uint32_t kQ = 0, kG = kTile;  // (further buffers 2 kTile apart)
+    static constexpr uint32_t kK = kRowBufs * 2 * kTile, kV = kK + kKStages * kBlkTile;
     static constexpr uint32_t kOut = kV + kVStages * kBlkTile;  // per epilogue warp a patch of 32 rows x 32 fp32
     static constexpr uint32_t kBars = kOut + 4 * 4096;
     static constexpr uint32_t kAlloc = kBars + kBarArea + 1024;
     static_assert(kAlloc <= 227 * 1024, "shared memory budget");
     enum : uint32_t {
-        Q_FULL, Q_EMPTY, G_FULL, G_EMPTY,
-        K_FULL, K_EMPTY = K_FULL + kKStages,
+        Q_FULL, Q_EMPTY = Q_FULL + kRowBufs, G_FULL = Q_EMPTY + kRowBufs, G_EMPTY = G_FULL + kRowBufs,
+        K_FULL = G_EMPTY + kRowBufs, K_EMPTY = K_FULL + kKStages,
         V_FULL = K_EMPTY + kKStages, V_EMPTY = V_FULL + kVStages,
         S_FULL = V_EMPTY + kVStages, DP_FULL = S_FULL + 4,   // [warpgroup]
         DP_TAKEN = DP_FULL + 4,                              // [step parity]: dP is in registers
@@ -165,7 +166,7 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
 {
     using C = DqCfg<D>;
     constexpr int DH = C::kDH;
-    constexpr uint32_t NK = C::kKStages, NV = C::kVStages;
+    constexpr uint32_t NK = C::kKStages, NV = C::kVStages, NR = C::kRowBufs;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *smem = smem_raw + (smem_base - ptx::smem_u32(smem_raw));
@@ -190,10 +191,12 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
     };
 
     if (threadIdx.x == 0) {
-        ptx::mbar_init(bar(C::Q_FULL), 1);
-        ptx::mbar_init(bar(C::Q_EMPTY), 1);
-        ptx::mbar_init(bar(C::G_FULL), 1);
-        ptx::mbar_init(bar(C::G_EMPTY), 1);
+        for (uint32_t s = 0; s < NR; ++s) {
+            ptx::mbar_init(bar(C::Q_FULL + s), 1);
+            ptx::mbar_init(bar(C::Q_EMPTY + s), 1);
+            ptx::mbar_init(bar(C::G_FULL + s), 1);
+            ptx::mbar_init(bar(C::G_EMPTY + s), 1);
+        }
         for (uint32_t s = 0; s < NK; ++s) {
             ptx::mbar_init(bar(C::K_FULL + s), 1);
             ptx::mbar_init(bar(C::K_EMPTY + s), 1);
@@ -275,10 +278,12 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
                 if (w.n > 0) {
                     const int h0 = w.hk * a.G + 2 * w.hp;
                     auto load_rows = [&](uint32_t dst, const CUtensorMap *tm, uint32_t full, uint32_t empty, int code) {
-                        if (kq >= 1 && !wait_bar(bar(empty), (kq - 1) & 1, code)) return false;
-                        ptx::mbar_expect_tx(bar(full), C::kTile);
+                        const uint32_t rb = kq % NR;
+                        if (kq >= NR && !wait_bar(bar(empty + rb), (kq / NR - 1) & 1, code)) return false;
+                        ptx::mbar_expect_tx(bar(full + rb), C::kTile);
                         for (int dh = 0; dh < DH; ++dh)
-                            ptx::tma_load_4d(smem_base + dst + dh * kRowTile, tm, bar(full), dh * 64, w.blk * kBwdBlk, h0, w.b);
+                            ptx::tma_load_4d(smem_base + dst + rb * 2 * C::kTile + dh * kRowTile, tm, bar(full + rb), dh * 64,
+                                             w.blk * kBwdBlk, h0, w.b);
                         return true;
                     };
                     auto load_block = [&](uint32_t base, const CUtensorMap *tm, uint32_t full, uint32_t empty, uint32_t stages, int32_t j,
@@ -312,7 +317,6 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
         const bool is_dp = __shfl_sync(0xffffffffu, warp, 0) == 2;
         // A = Q (S) or dO (dP); B = the K or V block of the stage; both K-major.
         constexpr uint32_t idesc_s = idesc_bf16(128, 64, 0, 0);
-        const uint32_t a_lo = ((smem_base + (is_dp ? C::kG : C::kQ)) >> 4) | (1u << 16);
         const uint32_t rows_full = is_dp ? C::G_FULL : C::Q_FULL, rows_empty = is_dp ? C::G_EMPTY : C::Q_EMPTY;
         const uint32_t blk_full = is_dp ? C::V_FULL : C::K_FULL, stages = is_dp ? NV : NK;
         const uint32_t out_full = is_dp ? C::DP_FULL : C::S_FULL;
@@ -325,13 +329,15 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
             const int n = __shfl_sync(0xffffffffu, w.n, 0);
             if (!ok || n < 0) break;
             if (n == 0) continue;
+            const uint32_t rb = kq % NR;
+            const uint32_t a_lo = ((smem_base + rb * 2 * C::kTile + (is_dp ? C::kG : C::kQ)) >> 4) | (1u << 16);
             for (int e = 0; e < n; ++e, ++c) {
                 // Three things to wait for, by three groups of lanes at a time (each wait costs some 200 clk even when it is
                 // over): the block; the item's rows; the buffer (dP of two steps before is in registers; the S
                 // buffer's last dS has been read).
                 uint32_t b_ = blk_full + st, parity = round & 1;
                 const int which = lane & 3;
-                if (which == 1 && e == 0) b_ = rows_full, parity = kq & 1;
+                if (which == 1 && e == 0) b_ = rows_full + rb, parity = (kq / NR) & 1;
                 if (which == 2 && is_dp && c >= 2) b_ = C::DP_TAKEN + (c & 1), parity = ((c >> 1) - 1) & 1;
                 if (which == 2 && !is_dp && c >= 4) b_ = C::DS_FREE + (c & 3), parity = ((c >> 2) - 1) & 1;
                 ok = wait_warp(bar(b_), parity, 7 + which);
@@ -346,7 +352,7 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
                                           b_lo + (((kk / 4) * kKeyTile + (kk % 4) * 32) >> 4), kDescHi, idesc_s, kk > 0 ? 1u : 0u);
                     ptx::umma_commit(bar(out_full + (c & 3)));
                     if (is_dp) ptx::umma_commit(bar(C::V_EMPTY + st));
-                    if (e == n - 1) ptx::umma_commit(bar(rows_empty));  // this warp has read the item's Q (dO) tile
+                    if (e == n - 1) ptx::umma_commit(bar(rows_empty + rb));  // this warp has read the item's Q (dO) tile
                 }
                 __syncwarp();
                 if (++st == stages) {
