@@ -56,6 +56,20 @@ def test_small_shapes(pa, oracle, N, Hq, Hkv, D, W, S):
     _full_compare(pa, oracle, Q, K, V, W, S, what=f"N={N} Hq={Hq} Hkv={Hkv} D={D} W={W} S={S}")
 
 
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("G", [1, 2, 3])
+def test_groups_that_leave_the_second_slot_idle(pa, oracle, G, D):
+    """One and two query heads per group run with one slot, three with two; several units per CTA, a ragged
+    last block.  Peaky logits (new reference maxima) with fp32 output: there |O| reaches 4 and rounding O to
+    bf16 alone costs 2^-7 of it."""
+    N, Hkv = 64 * 12 - 5, 40
+    Q = si.bf16_randn((1, N, G * Hkv, D), 1100 + G)
+    K = si.bf16_randn((1, N, Hkv, D), 1200 + G)
+    V = si.bf16_randn((1, N, Hkv, D), 1300 + G)
+    _full_compare(pa, oracle, Q, K, V, 2, 1, what=f"G={G} D={D}")
+    _full_compare(pa, oracle, Q, (K.float() * 3).bfloat16(), V, 2, 1, o_dtype=torch.float32, what=f"G={G} D={D} peaky")
+
+
 def test_peaky_logits_fp32_output_and_custom_scale(pa, oracle):
     N, Hq, Hkv, D = 1500, 14, 2, 128
     Q, K, V = si.bf16_randn((1, N, Hq, D), 1), si.bf16_randn((1, N, Hkv, D), 2, 3.0), si.bf16_randn((1, N, Hkv, D), 3)
