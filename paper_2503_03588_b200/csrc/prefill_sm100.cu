@@ -32,11 +32,12 @@
 #include "tensor_map.cuh"
 
 // Registers per thread by role: 4 control warps, 8 softmax warps, 4 epilogue warps share the
-// CTA's 16 x 128.
+// CTA's 16 x 128.  (56 / 176 / 104 spills eight bytes of the control warps: fp32 output, 18K tokens, 14 / 2 heads,
+// 159.4 us against 155.8, bf16 output the same.)
 #ifndef PA_REG_CTRL
-#define PA_REG_CTRL 56
-#define PA_REG_SOFT 176
-#define PA_REG_EPI 104
+#define PA_REG_CTRL 64
+#define PA_REG_SOFT 168
+#define PA_REG_EPI 112
 #endif
 // A warpgroup asking for more than the pool holds would wait for ever.
 static_assert(4 * PA_REG_CTRL + 8 * PA_REG_SOFT + 4 * PA_REG_EPI <= 16 * 128, "register split exceeds the CTA's registers");
