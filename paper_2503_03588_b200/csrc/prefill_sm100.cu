@@ -31,18 +31,6 @@
 #include "sm100_ptx.cuh"
 #include "tensor_map.cuh"
 
-// Registers per thread by role: 4 control warps, 8 softmax warps, 4 epilogue warps share the
-// CTA's 16 x 128.  (56 / 176 / 104 spills eight bytes of the control warps: fp32 output, 18K tokens, 14 / 2 heads,
-// 159.4 us against 155.8, bf16 output the same.)
-#ifndef PA_REG_CTRL
-#define PA_REG_CTRL 64
-#define PA_REG_SOFT 168
-#define PA_REG_EPI 112
-#endif
-// A warpgroup asking for more than the pool holds would wait for ever.
-static_assert(4 * PA_REG_CTRL + 8 * PA_REG_SOFT + 4 * PA_REG_EPI <= 16 * 128, "register split exceeds the CTA's registers");
-static_assert(PA_REG_CTRL % 8 == 0 && PA_REG_SOFT % 8 == 0 && PA_REG_EPI % 8 == 0, "setmaxnreg takes multiples of 8");
-
 namespace pa {
 
 constexpr int kBlk = 64;               // tokens per query / key block
@@ -56,6 +44,17 @@ constexpr int kTurnAtColumn = 16;  // column of a pass at which the other slot g
 constexpr float kRescaleThreshold = 8.0f;  // base-2 logits: rescale O only when the row max grows by more
 constexpr size_t kPrefillWorkspace = 256;  // bytes: the status block
 constexpr long long kWaitCycles = 4000000000ll;  // default limit of a barrier wait: ~2 s at 2 GHz
+
+// Registers per thread by role: 4 control warps, 8 softmax warps, 4 epilogue warps share the CTA's 16 x 128.
+// These splits spill nothing.  (56 / 176 / 104 spills eight bytes of the control warps with head_dim 128, reloaded
+// in every step: fp32 output, 18K tokens, 14 / 2 heads, 159.4 us against 155.8.)
+template <int D>
+struct RegSplit {
+    static constexpr int kCtrl = 64, kSoft = D == 128 ? 168 : 176, kEpi = D == 128 ? 112 : 96;
+    // A warpgroup asking for more than the pool holds would wait for ever.
+    static_assert(4 * kCtrl + 8 * kSoft + 4 * kEpi <= 16 * 128, "register split exceeds the CTA's registers");
+    static_assert(kCtrl % 8 == 0 && kSoft % 8 == 0 && kEpi % 8 == 0, "setmaxnreg takes multiples of 8");
+};
 
 struct PrefillArgs {
     const int32_t *row_ptr, *col_idx;
@@ -163,8 +162,8 @@ __device__ __forceinline__ Unit decode_unit(const PrefillArgs &a, uint32_t u)
     return r;
 }
 
-// kSlots: slots that have work (launch_prefill chooses).
-template <int D, int kSlots>
+// kSlots: slots that have work (launch_prefill chooses); kF32: fp32 output.
+template <int D, int kSlots, bool kF32>
 __global__ void __launch_bounds__(kThreads, 1)
 prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO,
@@ -236,7 +235,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     const uint32_t tmem_base_any = *tmem_slot;
     const uint32_t tmem_base = tmem_base_any;
 
-    if (warp < 4) ptx::setmaxnreg_dec<PA_REG_CTRL>();
+    if (warp < 4) ptx::setmaxnreg_dec<RegSplit<D>::kCtrl>();
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
         if (lane == 0) {
@@ -454,7 +453,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         __syncwarp();
     } else if (warp >= 4 && warp < 12) {
         // ------------------------------------------------------------------ online softmax
-        ptx::setmaxnreg_inc<PA_REG_SOFT>();
+        ptx::setmaxnreg_inc<RegSplit<D>::kSoft>();
         const int s = (warp - 4) >> 2;          // slot
         const int quad = warp & 3;              // TMEM lane quadrant this warp may access
         const int row = quad * 32 + lane;       // tile row = TMEM lane
@@ -670,11 +669,10 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     } else if (warp >= 12) {
         // ------------------------------------------------------------------ epilogue
         // O / l for both slots, off the softmax warps' critical path.  O is read out of tensor
-        // memory (which frees it for the next unit); bf16 output is staged in shared memory in
+        // memory (which frees it for the next unit); the output is staged in shared memory in
         // the 128-byte-swizzled box layout and leaves as bulk tensor stores, one per head and
-        // 64-feature half (rows beyond the sequence end are clipped by the tensor map), fp32
-        // output is written from registers.
-        ptx::setmaxnreg_dec<PA_REG_EPI>();
+        // 128 bytes of features (rows beyond the sequence end are clipped by the tensor map).
+        ptx::setmaxnreg_dec<RegSplit<D>::kEpi>();
         const int quad = warp & 3;
         const int row = quad * 32 + lane;
         const int qrow = row & 63;
@@ -696,7 +694,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 if (w.n <= 0) {  // empty row: defined outputs, no barrier traffic
                     if (valid) {
                         for (int c = 0; c < D; ++c) {
-                            if (a.o_is_f32) reinterpret_cast<float *>(a.o)[obase + c] = 0.f;
+                            if (kF32) reinterpret_cast<float *>(a.o)[obase + c] = 0.f;
                             else reinterpret_cast<__nv_bfloat16 *>(a.o)[obase + c] = __float2bfloat16_rn(0.f);
                         }
                         a.lse[w.b * a.lse_sb + head * a.lse_sh + w.tok0 + tok] = -INFINITY;
@@ -712,32 +710,69 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 if (!ok) break;
                 ptx::tc_fence_after_sync();
                 const uint32_t t_o = tmem_base + ((uint32_t)(quad * 32) << 16) + 256 + s * D;
-                if (a.o_is_f32) {
+                // A packed sequence's last block may reach into the next sequence's rows, which a
+                // box store would overwrite: its rows are written one by one from the registers.
+                const bool ragged = a.cu_seqlens != nullptr && (int64_t)(w.i + 1) * kBlk > w.len;
+                // Head 2 s + (row >> 6) of the unit: boxes of 64 tokens x 128 bytes; 16-byte chunk j of
+                // token t sits at chunk position j ^ (t & 7).
+                const uint32_t rbase = stage + (uint32_t)(2 * s + (row >> 6)) * SM::kOHead + (uint32_t)qrow * 128u;
+                // All four warps wait (not only the storing one), so none can arrive for the next time before
+                // this phase has completed.
+                auto meet = [&]() {
+                    __syncwarp();
+                    if (lane == 0) ptx::mbar_arrive(bar(BAR_STAGE_FULL));
+                    ok = wait_bar(bar(BAR_STAGE_FULL), ns & 1, abort_flag, a.status, 17);
+                    ok = __all_sync(0xffffffffu, ok);
+                    ++ns;
+                };
+                if (kF32) {
+                    // The slot's part of the Q buffer holds half of its fp32 rows: two rounds.  (Rows written from the
+                    // registers, 16 bytes a lane: 18K tokens, 14 / 2 heads 153.5 us, now 126.3; bf16 output 114.)
 #pragma unroll
-                    for (int ch = 0; ch < D / 32; ++ch) {
-                        uint32_t orr[32];
-                        ptx::tmem_ld32(t_o + ch * 32, orr);
-                        ptx::tmem_wait_ld();
-                        if (ch == D / 32 - 1) {
-                            ptx::tc_fence_before_sync();
-                            __syncwarp();
-                            if (lane == 0) ptx::mbar_arrive(bar(BAR_O_FREE + s));
+                    for (int half = 0; half < 2; ++half) {
+#pragma unroll
+                        for (int k = 0; k < DH; ++k) {
+                            const int ch = half * DH + k;  // of 32 features
+                            uint32_t orr[32];
+                            ptx::tmem_ld32(t_o + ch * 32, orr);
+                            ptx::tmem_wait_ld();
+                            if (ch == D / 32 - 1) {
+                                ptx::tc_fence_before_sync();
+                                __syncwarp();
+                                if (lane == 0) ptx::mbar_arrive(bar(BAR_O_FREE + s));
+                            }
+#pragma unroll
+                            for (int c = 0; c < 8; ++c) {
+                                uint32_t v[4];
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) v[e] = __float_as_uint(__uint_as_float(orr[4 * c + e]) * inv);
+                                ptx::st_shared_v4(rbase + (uint32_t)k * 8192u + ((uint32_t)(c ^ (qrow & 7)) << 4), v[0], v[1], v[2], v[3]);
+                                if (ragged && valid)
+                                    *reinterpret_cast<uint4 *>(reinterpret_cast<float *>(a.o) + obase + ch * 32 + 4 * c) =
+                                        make_uint4(v[0], v[1], v[2], v[3]);
+                            }
                         }
-                        if (valid) {
-                            float4 *dst = reinterpret_cast<float4 *>(reinterpret_cast<float *>(a.o) + obase + ch * 32);
-#pragma unroll
-                            for (int c = 0; c < 8; ++c)
-                                dst[c] = make_float4(__uint_as_float(orr[4 * c]) * inv, __uint_as_float(orr[4 * c + 1]) * inv,
-                                                     __uint_as_float(orr[4 * c + 2]) * inv, __uint_as_float(orr[4 * c + 3]) * inv);
+                        ptx::fence_proxy_async_smem();
+                        meet();
+                        if (!ok) break;
+                        if (store_thread) {
+                            for (int hh = 0; hh < 2; ++hh) {
+                                const int hl = w.sub * 4 + 2 * s + hh;
+                                if (hl >= a.G || ragged) continue;
+                                for (int k = 0; k < DH; ++k)
+                                    ptx::tma_store_4d(&tmO, stage + (uint32_t)(2 * s + hh) * SM::kOHead + (uint32_t)k * 8192u,
+                                                      (half * DH + k) * 32, w.tok0 + w.i * kBlk, w.hk * a.G + hl, w.bt);
+                            }
+                            ptx::bulk_commit_group();
+                        }
+                        if (half == 0) {  // the second half goes where the first one is read from
+                            if (store_thread) ptx::bulk_wait_read_all();
+                            meet();
+                            if (!ok) break;
                         }
                     }
+                    if (!ok) break;
                 } else {
-                    // Head 2 s + (row >> 6) of the unit: two boxes of 64 tokens x 128 bytes (one per
-                    // 64-feature half); 16-byte chunk j of token t sits at chunk position j ^ (t & 7).
-                    const uint32_t rbase = stage + (uint32_t)(2 * s + (row >> 6)) * SM::kOHead + (uint32_t)qrow * 128u;
-                    // A packed sequence's last block may reach into the next sequence's rows, which a
-                    // box store would overwrite: its rows are written one by one from the registers.
-                    const bool ragged = a.cu_seqlens != nullptr && (int64_t)(w.i + 1) * kBlk > w.len;
 #pragma unroll
                     for (int ch = 0; ch < D / 32; ++ch) {
                         uint32_t orr[32];
@@ -765,14 +800,8 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                         }
                     }
                     ptx::fence_proxy_async_smem();
-                    __syncwarp();
-                    if (lane == 0) ptx::mbar_arrive(bar(BAR_STAGE_FULL));
-                    // All four warps wait (not only the storing one), so none can arrive for the
-                    // next slot before this phase has completed.
-                    ok = wait_bar(bar(BAR_STAGE_FULL), ns & 1, abort_flag, a.status, 17);
-                    ok = __all_sync(0xffffffffu, ok);
+                    meet();
                     if (!ok) break;
-                    ++ns;
                     if (store_thread) {
                         for (int hh = 0; hh < 2; ++hh) {
                             const int hl = w.sub * 4 + 2 * s + hh;
@@ -884,21 +913,20 @@ namespace pa {
 
 // The launch behind pa_prefill (cu_seqlens null) and pa_prefill_varlen (packed sequences:
 // p->seq_len is the longest one, tokens run over [0, total_tokens)).
-template <int D, int kSlots>
+template <int D, int kSlots, bool kF32>
 static pa_status launch_kernel(unsigned grid, cudaStream_t st, int device, const CUtensorMap &tmQ, const CUtensorMap &tmK,
                                const CUtensorMap &tmV, const CUtensorMap &tmO, const PrefillArgs &a)
 {
-    constexpr DeviceOnce once = D == 128 ? (kSlots == 2 ? ONCE_PREFILL_ATTR : ONCE_PREFILL_ATTR_1)
-                                         : (kSlots == 2 ? ONCE_PREFILL_ATTR_64 : ONCE_PREFILL_ATTR_64_1);
+    constexpr DeviceOnce once = (DeviceOnce)(ONCE_PREFILL_ATTR + 4 * (D == 64) + 2 * (kSlots == 1) + kF32);
     if (device_once_begin(device, once)) {
-        const cudaError_t e = cudaFuncSetAttribute(prefill_kernel<D, kSlots>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        const cudaError_t e = cudaFuncSetAttribute(prefill_kernel<D, kSlots, kF32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    (int)SmemMap<D>::kAlloc);
         if (e != cudaSuccess) {
             device_once_reset(device, once);
             return fail(PA_ERR_CUDA, "cudaFuncSetAttribute failed: %s", cudaGetErrorString(e));
         }
     }
-    PA_CUDA_OK(launch_pdl(prefill_kernel<D, kSlots>, dim3(grid), kThreads, SmemMap<D>::kAlloc, st, tmQ, tmK, tmV, tmO, a));
+    PA_CUDA_OK(launch_pdl(prefill_kernel<D, kSlots, kF32>, dim3(grid), kThreads, SmemMap<D>::kAlloc, st, tmQ, tmK, tmV, tmO, a));
     return PA_OK;
 }
 
@@ -928,20 +956,16 @@ static pa_status launch_prefill(const pa_prefill_params *p, const void *q, const
     // boxes one head.
     CUtensorMap tmQ, tmK, tmV, tmO;
     const int D = p->head_dim;
-    auto map_of = [&](const void *base, int heads, const pa_strides &st, int box_heads, const char *what, CUtensorMap *m) {
+    auto map_of = [&](const void *base, int heads, const pa_strides &st, int box_heads, const char *what, CUtensorMap *m, bool f32 = false) {
         // (packed sequences: one "batch" entry of total_tokens tokens)
         const TensorMapKey key = {base, varlen ? total_tokens : p->seq_len, st.seq, st.head, varlen ? 0 : st.batch, dev.device, D,
-                                  heads, varlen ? 1 : p->batch, box_heads, kBlk, 0};
+                                  heads, varlen ? 1 : p->batch, box_heads, kBlk, f32 ? 1 : 0};
         return get_tensor_map(key, what, m);
     };
     if (pa_status s = map_of(q, p->n_q_heads, p->q, 2, "q", &tmQ)) return s;
     if (pa_status s = map_of(k, p->n_kv_heads, p->k, 1, "k", &tmK)) return s;
     if (pa_status s = map_of(v, p->n_kv_heads, p->v, 1, "v", &tmV)) return s;
-    if (p->o_dtype == PA_BF16) {
-        if (pa_status s = map_of(o, p->n_q_heads, p->o, 1, "o", &tmO)) return s;
-    } else {
-        tmO = tmQ;  // fp32 output is written from registers; the map is not used
-    }
+    if (pa_status s = map_of(o, p->n_q_heads, p->o, 1, "o", &tmO, p->o_dtype == PA_F32)) return s;
 
     PrefillArgs a;
     a.row_ptr = row_ptr;
@@ -993,10 +1017,13 @@ static pa_status launch_prefill(const pa_prefill_params *p, const void *q, const
     // long as one slot's chain alone.  With one head per group 2K tokens, 2 heads of 64 features take 9.1 us instead of
     // 11.4, 32K tokens, 8 heads of 128 features 266 us instead of 355; with two heads per group 8K tokens, batch 2,
     // 8 KV heads 118 us instead of 156 (burst).  Three heads need the second slot.
-    if (a.G > 2) return D == 128 ? launch_kernel<128, 2>(grid, st, dev.device, tmQ, tmK, tmV, tmO, a)
-                                 : launch_kernel<64, 2>(grid, st, dev.device, tmQ, tmK, tmV, tmO, a);
-    return D == 128 ? launch_kernel<128, 1>(grid, st, dev.device, tmQ, tmK, tmV, tmO, a)
-                    : launch_kernel<64, 1>(grid, st, dev.device, tmQ, tmK, tmV, tmO, a);
+    auto launch = [&](auto kernel) { return kernel(grid, st, dev.device, tmQ, tmK, tmV, tmO, a); };
+    if (a.o_is_f32) {
+        if (a.G > 2) return launch(D == 128 ? launch_kernel<128, 2, true> : launch_kernel<64, 2, true>);
+        return launch(D == 128 ? launch_kernel<128, 1, true> : launch_kernel<64, 1, true>);
+    }
+    if (a.G > 2) return launch(D == 128 ? launch_kernel<128, 2, false> : launch_kernel<64, 2, false>);
+    return launch(D == 128 ? launch_kernel<128, 1, false> : launch_kernel<64, 1, false>);
 }
 
 }  // namespace pa
