@@ -32,12 +32,18 @@
 #include "sm100_ptx.cuh"
 #include "tensor_map.cuh"
 
-// Registers per thread by role.  A warpgroup asking for more than the pool holds would wait for ever: both kernels
-// start 768 threads x 80.
-#define PA_BWD_REG_CTRL 48
-#define PA_BWD_REG_COMP 96
-#define PA_BWD_REG_EPI 48
-static_assert(4 * PA_BWD_REG_CTRL + 16 * PA_BWD_REG_COMP + 4 * PA_BWD_REG_EPI <= 24 * 80, "register split exceeds the CTA's registers");
+// Registers per thread by role (control, compute, epilogue warps).  A warpgroup asking for more than the pool holds
+// would wait for ever: both kernels start 768 threads x 80.  (48 / 96 / 48 for
+// both spills more, dK / dV not at all now: backward pass at 4K tokens, 28 / 4 heads, 162.7 us against 161.4, 2 x 8K
+// tokens, 16 / 4 heads of 64 features, 245.5 against 242.5.)
+#define PA_DQ_REG_CTRL 40
+#define PA_DQ_REG_COMP 96
+#define PA_DQ_REG_EPI 56
+static_assert(4 * PA_DQ_REG_CTRL + 16 * PA_DQ_REG_COMP + 4 * PA_DQ_REG_EPI <= 24 * 80, "register split exceeds the CTA's registers");
+#define PA_DKV_REG_CTRL 64
+#define PA_DKV_REG_COMP 88
+#define PA_DKV_REG_EPI 64
+static_assert(4 * PA_DKV_REG_CTRL + 16 * PA_DKV_REG_COMP + 4 * PA_DKV_REG_EPI <= 24 * 80, "register split exceeds the CTA's registers");
 
 namespace pa {
 
@@ -234,7 +240,7 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = tail->tmem;
 
-    if (warp < 4) ptx::setmaxnreg_dec<PA_BWD_REG_CTRL>();
+    if (warp < 4) ptx::setmaxnreg_dec<PA_DQ_REG_CTRL>();
     if (warp == 0) {
         // -------------------------------------------------------------- TMA producer
         if (lane == 0) {
@@ -401,7 +407,7 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
     } else if (warp < 4 + kCompWarps) {
         // -------------------------------------------------------------- compute warps
         // Warpgroup g: every fourth step.
-        ptx::setmaxnreg_inc<PA_BWD_REG_COMP>();
+        ptx::setmaxnreg_inc<PA_DQ_REG_COMP>();
         const uint32_t g = (uint32_t)(warp - 4) >> 2;
         const int quad = warp & 3;
         const int row = quad * 32 + lane, qrow = row & 63;
@@ -484,7 +490,7 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
         // dQ = scale x the accumulator.  A warp's 32 rows leave 32 features at a time: through a swizzled patch of
         // shared memory and a bulk tensor store each (rows beyond the sequence are clipped by the tensor map).  (Plain stores moved 10 B/clk out of the SM: 7000 clk an item, during which the
         // accumulator, or 128 registers a thread, was held.)
-        ptx::setmaxnreg_dec<PA_BWD_REG_EPI>();
+        ptx::setmaxnreg_dec<PA_DQ_REG_EPI>();
         const int quad = warp & 3;
         const int row = quad * 32 + lane, qrow = row & 63;
         const uint32_t t_lane = tmem_base + ((uint32_t)(quad * 32) << 16);
@@ -694,7 +700,7 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = tail->tmem;
 
-    if (warp < 4) ptx::setmaxnreg_dec<PA_BWD_REG_CTRL>();
+    if (warp < 4) ptx::setmaxnreg_dec<PA_DKV_REG_CTRL>();
     if (warp == 0) {
         // -------------------------------------------------------------- TMA producer
         if (lane == 0) {
@@ -842,7 +848,7 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     } else if (warp < 4 + kCompWarps) {
         // -------------------------------------------------------------- compute warps
         // Warpgroup wg: steps of parity wg & 1, keys 32 (wg >> 1) .. + 31.
-        ptx::setmaxnreg_inc<PA_BWD_REG_COMP>();
+        ptx::setmaxnreg_inc<PA_DKV_REG_COMP>();
         const int wg = (warp - 4) >> 2, quad = warp & 3, par = wg & 1, half = wg >> 1;
         const int row = quad * 32 + lane, qrow = row & 63;
         const uint32_t t_lane = tmem_base + ((uint32_t)(quad * 32) << 16);
@@ -945,7 +951,7 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         }
     } else {
         // -------------------------------------------------------------- epilogue warps; the first one finds the items
-        ptx::setmaxnreg_dec<PA_BWD_REG_EPI>();
+        ptx::setmaxnreg_dec<PA_DKV_REG_EPI>();
         const int quad = warp & 3;
         const uint32_t t_lane = tmem_base + ((uint32_t)(quad * 32) << 16);
         // Items: chunk slots in column order (the sink block's long column first); slots without work are passed over.
