@@ -12,8 +12,8 @@
 // other warps through a small ring in shared memory.
 // A step is one (query block, key block) pair for a pair of query heads stacked on the 64 tokens of the query
 // block: a 128-row tile, as in the forward kernel.  Per step the tensor cores produce S = Q K^T and dP = dO V^T
-// (fp32, tensor memory); the compute warps (thread = tile row = TMEM lane) turn them into P = exp2(S scale log2e - LSE log2e) and dS = P (dP - delta), rounded
-// to bf16; the second products accumulate in tensor memory.
+// (fp32, tensor memory); the compute warps (thread = tile row = TMEM lane) turn them into P = exp2(S scale
+// log2e - LSE log2e) and dS = P (dP - delta), rounded to bf16; the second products accumulate in tensor memory.
 //
 //   dq_kernel   an item is a (query block, head pair): walks the row's key blocks; dS goes back
 //               into tensor memory as the A operand of dQ += dS K (128 x D accumulator)
@@ -32,10 +32,10 @@
 #include "sm100_ptx.cuh"
 #include "tensor_map.cuh"
 
-// Registers per thread by role (control, compute, epilogue warps).  A warpgroup asking for more than the pool holds
-// would wait for ever: both kernels start 768 threads x 80.  (48 / 96 / 48 for
-// both spills more, dK / dV not at all now: backward pass at 4K tokens, 28 / 4 heads, 162.7 us against 161.4, 2 x 8K
-// tokens, 16 / 4 heads of 64 features, 245.5 against 242.5.)
+// Registers per thread by role (control, compute, epilogue warps).  A warpgroup asking for more than the pool
+// holds would wait for ever: both kernels start 768 threads x 80.  (48 / 96 / 48 for both spills more, dK / dV
+// not at all now: backward pass at 4K tokens, 28 / 4 heads, 162.7 us against 161.4, 2 x 8K tokens, 16 / 4 heads
+// of 64 features, 245.5 against 242.5.)
 #define PA_DQ_REG_CTRL 40
 #define PA_DQ_REG_COMP 96
 #define PA_DQ_REG_EPI 56
@@ -128,15 +128,16 @@ __device__ __forceinline__ float bwd_neg_lse2(float lse)
 }
 
 // ------------------------------------------------------------------------------------- dQ
-// A step's way is long and serial: S, dP, a warpgroup's loads, exponentials and stores, dQ, some 4500 cycles of which
-// the tensor cores work 1024.  So four steps are under way at a time, a warpgroup each.  Tensor memory decides the
-// rest: S has four buffers (dS goes over the S it was made from), dP two, which a warpgroup therefore loads whole
-// (64 registers a thread) before it works through S 16 keys at a time.  K stays in its ring until dQ has read
-// it, V only until dP has.  Q and dO have one buffer each with head_dim 128: the next item's tiles arrive while the last steps are
-// computed and their dQ products run.  With head_dim 64, whose steps are shorter than that, two.  Bound by the issue of S and dP (1300 clk a step) and by the 128 KB that an
-// item starts with.  Measured, 28 / 4 heads at 32K tokens: 524 us at full clocks, where all four warpgroups on one
-// step of two key blocks took 583; 64 features, 16 / 4 heads, 2 x 8K tokens: 87 us against 106, 82 with the second
-// pair of Q and dO buffers.
+// A step's way is long and serial: S, dP, a warpgroup's loads, exponentials and stores, dQ, some 4500 cycles of
+// which the tensor cores work 1024.  So four steps are under way at a time, a warpgroup each.  Tensor memory
+// decides the rest: S has four buffers (dS goes over the S it was made from), dP two, which a warpgroup
+// therefore loads whole (64 registers a thread) before it works through S 16 keys at a time.  K stays in its
+// ring until dQ has read it, V only until dP has.  Q and dO have one buffer each with head_dim 128: the next
+// item's tiles arrive while the last steps are computed and their dQ products run.  With head_dim 64, whose
+// steps are shorter than that, two.  Bound by the issue of S and dP (1300 clk a step) and by the 128 KB that an
+// item starts with.  Measured, 28 / 4 heads at 32K tokens: 524 us at full clocks, where all four warpgroups on
+// one step of two key blocks took 583; 64 features, 16 / 4 heads, 2 x 8K tokens: 87 us against 106, 82 with the
+// second pair of Q and dO buffers.
 template <int D>
 struct DqCfg {
     static constexpr int kDH = D / 64;
@@ -487,9 +488,10 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
         }
     } else {
         // -------------------------------------------------------------- epilogue
-        // dQ = scale x the accumulator.  A warp's 32 rows leave 32 features at a time: through a swizzled patch of
-        // shared memory and a bulk tensor store each (rows beyond the sequence are clipped by the tensor map).  (Plain stores moved 10 B/clk out of the SM: 7000 clk an item, during which the
-        // accumulator, or 128 registers a thread, was held.)
+        // dQ = scale x the accumulator.  A warp's 32 rows leave 32 features at a time: through a swizzled patch
+        // of shared memory and a bulk tensor store each (rows beyond the sequence are clipped by the tensor
+        // map).  (Plain stores moved 10 B/clk out of the SM: 7000 clk an item, during which the accumulator, or
+        // 128 registers a thread, was held.)
         ptx::setmaxnreg_dec<PA_DQ_REG_EPI>();
         const int quad = warp & 3;
         const int row = quad * 32 + lane, qrow = row & 63;
