@@ -157,9 +157,10 @@ pa_status get_tensor_map(const TensorMapKey &key, const char *what, CUtensorMap 
     const cuuint64_t dims[4] = {(cuuint64_t)key.head_dim, (cuuint64_t)key.seq, (cuuint64_t)key.heads,
                                 (cuuint64_t)key.batch};
     const cuuint64_t size = key.f32 ? 4 : 2;
-    const cuuint64_t strides[3] = {
-        (cuuint64_t)key.stride_seq * size, (cuuint64_t)key.stride_head * size,
-        (cuuint64_t)(key.stride_batch > 0 ? key.stride_batch : key.stride_seq * key.seq) * size};
+    // (A batch stride of 0 is an expanded tensor, one sequence that every batch entry reads, and goes into the map as
+    // it is; with a single entry the stride is never used and only has to be a valid one.)
+    const cuuint64_t strides[3] = {(cuuint64_t)key.stride_seq * size, (cuuint64_t)key.stride_head * size,
+                                   (cuuint64_t)(key.batch > 1 ? key.stride_batch : key.stride_seq * key.seq) * size};
     const cuuint32_t box[4] = {(cuuint32_t)(128 / size), (cuuint32_t)key.box_tokens, (cuuint32_t)key.box_heads, 1};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     CUtensorMap m;

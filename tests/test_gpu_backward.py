@@ -261,3 +261,20 @@ def test_backward_of_many_short_lists(pa, oracle, D):
     pa.pa_prefill_status(wsb)
     for g, r, n in zip((dq, dk, dv), oracle.backward(Q, K, V, dO, 64, 5, 1, dense=dense), ("dQ", "dK", "dV")):
         _compare(g, r, n + " short lists")
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_backward_of_keys_and_values_shared_by_the_batch(pa, D):
+    """Q, K and V expanded over the batch (stride 0): the gradients of their copies, per batch entry (dQ bit for bit,
+    dK and dV up to the order of their fp32 additions)."""
+    batch, N, Hq, Hkv = 3, 1000, 6, 2
+    q, k, v = (si.bf16_randn((1, N, h, D), 1820 + x).cuda().expand(batch, -1, -1, -1) for x, h in enumerate((Hq, Hkv, Hkv)))
+    d_o = si.bf16_randn((batch, N, Hq, D), 1823).cuda()
+    copies = [x.contiguous() for x in (q, k, v)]
+    rp, ci = pa.pa_build_layout(N, 64, 5, 1)
+    o, lse, _ = pa.pa_prefill(*copies, rp, ci)
+    dq, dk, dv, ws = pa.pa_prefill_backward(q, k, v, o, lse, d_o, rp, ci)
+    pa.pa_prefill_status(ws)
+    rq, rk, rv, _ = pa.pa_prefill_backward(*copies, o, lse, d_o, rp, ci)
+    assert torch.equal(dq, rq)
+    assert torch.allclose(dk, rk, rtol=1e-4, atol=1e-5) and torch.allclose(dv, rv, rtol=1e-4, atol=1e-5)

@@ -329,3 +329,17 @@ def test_append_copies_whole_rows(pa, Hkv, D):
             pos = int(start[b]) + t
             page = int(table[b, pos // 64])
             assert torch.equal(k_pool[page, pos % 64], new[2 * t][b]) and torch.equal(v_pool[page, pos % 64], new[2 * t + 1][b])
+
+
+@pytest.mark.parametrize("env", [{}, {"PA_DECODE_PATH": "persist"}, {"PA_DECODE_PATH": "splitk"}])
+def test_cache_shared_by_the_batch(pa, pa_env, env):
+    """A cache expanded over the batch (stride 0) gives what its copies give, bit for bit."""
+    pa_env(**env)
+    batch, max_len, D = 3, 1000, 128
+    q = si.bf16_randn((batch, 14, D), 1810).cuda()
+    kc, vc = (si.bf16_randn((1, max_len, 2, D), 1811 + x).cuda().expand(batch, -1, -1, -1) for x in range(2))
+    lens = torch.tensor([max_len, 64, 517], dtype=torch.int32, device="cuda")
+    o, lse, ws = pa.pa_decode(q, kc, vc, lens, 5, 1)
+    pa.pa_decode_status(ws)
+    o_ref, lse_ref, _ = pa.pa_decode(q, kc.contiguous(), vc.contiguous(), lens, 5, 1)
+    assert torch.equal(o, o_ref) and torch.equal(lse, lse_ref)

@@ -479,3 +479,16 @@ def test_kv_head_shards_reproduce_the_whole_call(pa):
             pa.pa_prefill_status(ws_r)
             lse[:, heads] = lse_r
         assert torch.equal(o, o_full) and torch.equal(lse, lse_full), world
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_keys_and_values_shared_by_the_batch(pa, D):
+    """K and V expanded over the batch (stride 0) give what their copies give, bit for bit."""
+    batch, N, Hq, Hkv = 3, 1000, 6, 2
+    q = si.bf16_randn((batch, N, Hq, D), 1800).cuda()
+    k, v = (si.bf16_randn((1, N, Hkv, D), 1801 + x).cuda().expand(batch, -1, -1, -1) for x in range(2))
+    rp, ci = pa.pa_build_layout(N, 64, 5, 1)
+    o, lse, ws = pa.pa_prefill(q, k, v, rp, ci)
+    pa.pa_prefill_status(ws)
+    o_ref, lse_ref, _ = pa.pa_prefill(q, k.contiguous(), v.contiguous(), rp, ci)
+    assert torch.equal(o, o_ref) and torch.equal(lse, lse_ref)
