@@ -422,6 +422,10 @@ __global__ void __launch_bounds__(kRowThreads, 2) decode_row_kernel(const __grid
         ptx::prefetch_tensormap(&tmV);
     }
     __syncthreads();
+    // A peer's shared memory may be written only once the peer has started.  Each CTA says so here and asks for the
+    // others just before it pushes its parts, which hides the answer's way behind the wait below and the loads.
+    const bool peers = a.mode == kModeCluster && R > 1;
+    if (peers) ptx::cluster_arrive_relaxed();
     pdl_wait();
     const int32_t len_first = it0 < n_items ? a.lens[(it0 / (uint32_t)R) / (uint32_t)a.Hkv] : 0;
     if (blockIdx.x == 0 && tid == 0) a.status[0] = 0;  // a wait that gives up (much later) sets it
@@ -499,6 +503,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) decode_row_kernel(const __grid
                 __syncwarp();
             }
         }
+        if (peers) ptx::cluster_wait();
     } else {
         // ------------------------------------------------------------------ consumers
         // ldmatrix row addresses inside a tile.  K (matrices: keys 0-7 / 8-15 of the warp x two
@@ -695,6 +700,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) decode_row_kernel(const __grid
                 const int64_t head = ((int64_t)w.b * a.Hq + (int64_t)w.hk * G + g);
                 const int f0 = wid * (D / 4) + 2 * t;
                 if (a.mode == kModeCluster) {
+                    if (peers) ptx::cluster_wait();  // (one item per CTA: every thread comes here once)
                     // Head g is merged by CTA g % R of the cluster: this CTA's part goes straight into
                     // that CTA's receive area (a store through distributed shared memory; the area is
                     // not used for anything else, so the owner may still be busy with its blocks).

@@ -311,6 +311,11 @@ __device__ __forceinline__ void red_add_v4(float *p, const float4 &v)
     asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};\n" ::"l"(p), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
 }
 
+// Barrier of the thread-block cluster in two halves, without an order of memory: every thread of every CTA arrives
+// once and waits once.  Behind the wait all CTAs of the cluster have started.
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed;\n" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait;\n" ::: "memory"); }
+
 __device__ __forceinline__ float ex2(float x)
 {
     float y;
