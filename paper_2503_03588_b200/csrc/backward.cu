@@ -86,18 +86,18 @@ __device__ void transpose_layout(const BackwardArgs &a, int32_t block, int32_t c
 #pragma unroll
         for (int x = 0; x < kAhead; ++x) {  // (the loads of four rows in flight together)
             const bool on = ib + x < a.nqb;
-            lo[x] = on ? __ldg(a.row_ptr + ib + x) : 0;
-            hi[x] = on ? __ldg(a.row_ptr + ib + x + 1) : 0;
+            lo[x] = on ? a.row_ptr[ib + x] : 0;
+            hi[x] = on ? a.row_ptr[ib + x + 1] : 0;
         }
 #pragma unroll
-        for (int x = 0; x < kAhead; ++x) col[x] = lo[x] + lane < hi[x] ? __ldg(a.col_idx + lo[x] + lane) : -1;
+        for (int x = 0; x < kAhead; ++x) col[x] = lo[x] + lane < hi[x] ? a.col_idx[lo[x] + lane] : -1;
 #pragma unroll
         for (int x = 0; x < kAhead; ++x) {
             const int32_t i = ib + x;
             for (int32_t e = lo[x], c = col[x]; e < hi[x]; e += 32) {
                 if (c >= j0 && c < j1) atomicOr(bits + (c - j0) * words + (i / 32 - w0), 1u << (i & 31));
                 before += (c >= 0 && c < j0) ? 1 : 0;
-                c = e + 32 + lane < hi[x] ? __ldg(a.col_idx + e + 32 + lane) : -1;
+                c = e + 32 + lane < hi[x] ? a.col_idx[e + 32 + lane] : -1;
             }
         }
     }
@@ -112,7 +112,7 @@ __device__ void transpose_layout(const BackwardArgs &a, int32_t block, int32_t c
     }
     __syncthreads();
     if (warp == 0) {  // exclusive prefix over the block's columns, from the entries before them
-        int32_t carry = s_before + __ldg(a.row_ptr + j0) - __ldg(a.row_ptr);
+        int32_t carry = s_before + a.row_ptr[j0] - a.row_ptr[0];
         for (int32_t x = 0; x < j1 - j0; x += 32) {
             const int32_t n = x + lane < j1 - j0 ? s_count[x + lane] : 0;
             int32_t incl = n;
@@ -186,8 +186,8 @@ __global__ void __launch_bounds__(kPrepThreads) backward_prep_kernel(const Backw
                 const int h = h0 + u * kHeadsPerStep + hsub;
                 const bool on = in && h < heads;
                 const int64_t off = base + (int64_t)(hb + h) * a.o_sh;
-                x[u] = on ? __ldg(reinterpret_cast<const uint4 *>(a.o + off)) : make_uint4(0, 0, 0, 0);
-                y[u] = on ? __ldg(reinterpret_cast<const uint4 *>(a.d_o + off)) : make_uint4(0, 0, 0, 0);
+                x[u] = on ? *reinterpret_cast<const uint4 *>(a.o + off) : make_uint4(0, 0, 0, 0);
+                y[u] = on ? *reinterpret_cast<const uint4 *>(a.d_o + off) : make_uint4(0, 0, 0, 0);
             }
 #pragma unroll
             for (int u = 0; u < kUnroll; ++u) {

@@ -50,10 +50,10 @@ __device__ __forceinline__ BackwardChunk backward_chunk_at(const BackwardArgs &a
     int32_t lo = 0, hi = a.nqb;  // last column whose slots start at or before c
     while (hi - lo > 1) {
         const int32_t mid = (lo + hi) >> 1;
-        if (__ldg(a.col_ptr + mid) / a.chunk + mid <= c) lo = mid;
+        if (a.col_ptr[mid] / a.chunk + mid <= c) lo = mid;
         else hi = mid;
     }
-    const int32_t p0 = __ldg(a.col_ptr + lo), cnt = __ldg(a.col_ptr + lo + 1) - p0;
+    const int32_t p0 = a.col_ptr[lo], cnt = a.col_ptr[lo + 1] - p0;
     const int32_t parts = (cnt + a.chunk - 1) / a.chunk, part = c - (p0 / a.chunk + lo);
     r.j = lo;
     r.parts = parts;
@@ -72,8 +72,8 @@ __device__ __forceinline__ BackwardChunk backward_chunk_by_warp(const BackwardAr
     do {
         step = (hi - lo + 31) / 32;
         const int32_t x = lo + lane * step;
-        p = x < hi ? __ldg(a.col_ptr + x) : 0;
-        p_next = x < hi ? __ldg(a.col_ptr + x + 1) : 0;
+        p = x < hi ? a.col_ptr[x] : 0;
+        p_next = x < hi ? a.col_ptr[x + 1] : 0;
         // (column lo starts at or before c, so the lanes that do are the first ones)
         at = __popc(__ballot_sync(0xffffffffu, x < hi && p / a.chunk + x <= c)) - 1;
         lo += at * step;

@@ -262,8 +262,8 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
                 w.b = (int32_t)bb;
                 w.hk = (int32_t)(hkp / (uint32_t)a.npairs);
                 w.hp = (int32_t)(hkp % (uint32_t)a.npairs);
-                w.e0 = __ldg(a.row_ptr + w.blk);
-                w.n = __ldg(a.row_ptr + w.blk + 1) - w.e0;
+                w.e0 = a.row_ptr[w.blk];
+                w.n = a.row_ptr[w.blk + 1] - w.e0;
                 it = gridDim.x + (uint32_t)atomicAdd(a.status + kBwdDqCounter, 1);
             };
             auto publish = [&](uint32_t k, const BwdItem &w) {
@@ -303,9 +303,9 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
                                              w.hk, w.b);
                         return true;
                     };
-                    int32_t j = __ldg(a.col_idx + w.e0);
+                    int32_t j = a.col_idx[w.e0];
                     for (int e = 0; e < w.n && ok; ++e, ++c) {
-                        const int32_t jn = e + 1 < w.n ? __ldg(a.col_idx + w.e0 + e + 1) : 0;
+                        const int32_t jn = e + 1 < w.n ? a.col_idx[w.e0 + e + 1] : 0;
                         if (e == 0) ok = load_rows(C::kQ, &tmQ, C::Q_FULL, C::Q_EMPTY, 3);
                         ok = ok && load_block(C::kK, &tmK, C::K_FULL, C::K_EMPTY, NK, j, 4);
                         if (e == 0) ok = ok && load_rows(C::kG, &tmG, C::G_FULL, C::G_EMPTY, 5);
@@ -427,10 +427,10 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
             const int64_t q = (int64_t)w.blk * kBwdBlk + qrow;
             if (head_local < a.G && q < a.N) {
                 const int64_t at = ((int64_t)w.b * a.Hq + w.hk * a.G + head_local) * a.N + q;
-                lse_n = __ldg(a.lse + at);
-                delta_n = __ldg(a.delta + at);
+                lse_n = a.lse[at];
+                delta_n = a.delta[at];
             }
-            lastcol_n = __ldg(a.col_idx + w.e0 + w.n - 1);
+            lastcol_n = a.col_idx[w.e0 + w.n - 1];
         };
         uint32_t c = 0;  // step number at the item's start
         BwdItem w;
@@ -501,7 +501,7 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
         // (where the preparation has not cleared everything).
         if (!a.prezero)
             for (int32_t j = blockIdx.x; j < a.nqb; j += gridDim.x) {
-                const int32_t cnt = __ldg(a.col_ptr + j + 1) - __ldg(a.col_ptr + j);
+                const int32_t cnt = a.col_ptr[j + 1] - a.col_ptr[j];
                 if (cnt > 0 && cnt <= a.chunk) continue;
                 const int64_t tok0 = (int64_t)j * kBwdBlk, toks = a.N - tok0 < kBwdBlk ? a.N - tok0 : kBwdBlk;
                 const int64_t words = toks * a.Hkv * (D / 4);
@@ -730,7 +730,7 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 };
                 int32_t i = w.first;
                 for (int x = 0; x < w.n && ok; ++x) {
-                    const int32_t in = x + 1 < w.n ? __ldg(a.row_idx + w.e0 + x + 1) : 0;
+                    const int32_t in = x + 1 < w.n ? a.row_idx[w.e0 + x + 1] : 0;
                     for (int hp = 0; hp < a.npairs && ok; ++hp, ++c) {
                         const int h0 = w.hk * a.G + 2 * hp;
                         ok = load_rows(C::kQ, &tmQ, C::Q_FULL, C::Q_EMPTY, NQ, i, h0, 33);
@@ -874,7 +874,7 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 x -= w.n;
                 ok = read_item(++k, w);
             }
-            i_next = ok && w.n >= 0 ? __ldg(a.row_idx + w.e0 + x) : -1;
+            i_next = ok && w.n >= 0 ? a.row_idx[w.e0 + x] : -1;
         };
         auto request = [&]() {
             lse_n = INFINITY;
@@ -883,8 +883,8 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             const int64_t q = (int64_t)i_next * kBwdBlk + qrow;
             if (i_next >= 0 && head_local < a.G && q < a.N) {
                 const int64_t at = ((int64_t)w.b * a.Hq + w.hk * a.G + head_local) * a.N + q;
-                lse_n = __ldg(a.lse + at);
-                delta_n = __ldg(a.delta + at);
+                lse_n = a.lse[at];
+                delta_n = a.delta[at];
             }
         };
         if (ok && w.n >= 0) advance(par);
@@ -979,7 +979,7 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                     w.parts = ch.parts;
                     w.b = (int32_t)(yz / (uint32_t)a.Hkv);
                     w.hk = (int32_t)(yz % (uint32_t)a.Hkv);
-                    w.first = __ldg(a.row_idx + w.e0);
+                    w.first = a.row_idx[w.e0];
                 }
                 int drawn = 0;
                 if (lane == 0) drawn = atomicAdd(a.status + kBwdDkvCounter, 1);

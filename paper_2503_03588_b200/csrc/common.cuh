@@ -53,6 +53,8 @@ long long wait_limit_cycles();
 // (programmatic dependent launch).  Such a kernel touches no global memory before pdl_wait(), which returns when
 // everything ahead of it in the stream has completed; what it does before that (barriers, tensor memory, the
 // launch itself) is hidden behind the other kernel's last microseconds.
+// Behind it, plain loads only: __ldg and ld.global.nc are for data that nobody writes while the kernel runs, which here
+// includes the time before the wait, and the compiler may move them across it.
 inline cudaLaunchAttribute pdl_attribute()
 {
     cudaLaunchAttribute a;

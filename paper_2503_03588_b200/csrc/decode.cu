@@ -70,19 +70,21 @@ __device__ __forceinline__ void block_origin(const DecodeArgs &a, int b, int32_t
     }
 }
 
-// 16-byte read-only global load.
-__device__ __forceinline__ uint4 ldg16(const void *p)
+// Loads that stay where they are written, ahead of the work that hides them.  (Not the read-only kind: decode_row_kernel
+// may start while the kernel that writes what it reads still runs.)
+__device__ __forceinline__ uint4 ld16(const void *p)
 {
     uint4 r;
-    asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];\n"
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];\n"
                  : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
-                 : "l"(p));
+                 : "l"(p)
+                 : "memory");
     return r;
 }
-__device__ __forceinline__ uint32_t ldg4(const void *p)
+__device__ __forceinline__ uint32_t ld4(const void *p)
 {
     uint32_t r;
-    asm volatile("ld.global.nc.u32 %0, [%1];\n" : "=r"(r) : "l"(p));
+    asm volatile("ld.global.u32 %0, [%1];\n" : "=r"(r) : "l"(p) : "memory");
     return r;
 }
 
@@ -148,17 +150,17 @@ __global__ void __launch_bounds__(kDecThreads) decode_block_kernel(const DecodeA
             const int key = base + nt * 8 + g;
 #pragma unroll
             for (int j = 0; j < NJ; ++j)
-                kr[nt][j] = key < n_keys ? ldg16(kb + key * a.k_ss + 8 * (4 * j + t)) : zero4;
+                kr[nt][j] = key < n_keys ? ld16(kb + key * a.k_ss + 8 * (4 * j + t)) : zero4;
         }
         const __nv_bfloat16 *qb = a.q + ((int64_t)b * a.Hq + (int64_t)hk * G + g) * D;
 #pragma unroll
-        for (int j = 0; j < NJ; ++j) qr[j] = g < G ? ldg16(qb + 8 * (4 * j + t)) : zero4;
+        for (int j = 0; j < NJ; ++j) qr[j] = g < G ? ld16(qb + 8 * (4 * j + t)) : zero4;
 #pragma unroll
         for (int ks = 0; ks < 4; ++ks)
 #pragma unroll
             for (int kx = 0; kx < 4; ++kx) {
                 const int key = 16 * ks + 2 * t + (kx & 1) + (kx >> 1) * 8;
-                vr[ks][kx] = (pv_warp && key < n_keys) ? ldg16(vb + key * a.v_ss + 8 * vchunk) : zero4;
+                vr[ks][kx] = (pv_warp && key < n_keys) ? ld16(vb + key * a.v_ss + 8 * vchunk) : zero4;
             }
 
         // ---- S = Q K^T: rows = heads, columns = the warp's 16 keys (two 8-key tiles)
@@ -521,8 +523,8 @@ __global__ void __launch_bounds__(kRowThreads, 2) decode_row_kernel(const __grid
             const __nv_bfloat16 *qb = a.q + ((int64_t)rowid * G + g) * D;
 #pragma unroll
             for (int ks = 0; ks < D / 16; ++ks) {
-                qn[ks][0] = in ? ldg4(qb + 16 * ks + 2 * t) : 0u;
-                qn[ks][1] = in ? ldg4(qb + 16 * ks + 8 + 2 * t) : 0u;
+                qn[ks][0] = in ? ld4(qb + 16 * ks + 2 * t) : 0u;
+                qn[ks][1] = in ? ld4(qb + 16 * ks + 8 + 2 * t) : 0u;
             }
         };
         load_q(it0);

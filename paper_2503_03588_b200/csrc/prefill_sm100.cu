@@ -147,12 +147,12 @@ __device__ __forceinline__ Unit decode_unit(const PrefillArgs &a, uint32_t u)
     r.i = a.nqb - 1 - (int32_t)rem;  // long rows first
     r.b = (int32_t)divmod(u, (uint32_t)a.Hkv, a.inv_Hkv, rem);
     r.hk = (int32_t)rem;
-    r.rs = __ldg(a.row_ptr + r.i);
-    r.n = __ldg(a.row_ptr + r.i + 1) - r.rs;
+    r.rs = a.row_ptr[r.i];
+    r.n = a.row_ptr[r.i + 1] - r.rs;
     if (a.cu_seqlens) {
         r.bt = 0;
-        r.tok0 = __ldg(a.cu_seqlens + r.b);
-        r.len = __ldg(a.cu_seqlens + r.b + 1) - r.tok0;
+        r.tok0 = a.cu_seqlens[r.b];
+        r.len = a.cu_seqlens[r.b + 1] - r.tok0;
         if ((int64_t)r.i * kBlk >= r.len) r.n = 0;  // the sequence ends before this query block: nothing to do
     } else {
         r.bt = r.b;
@@ -250,7 +250,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 for (; u < (uint32_t)a.n_units; u += gridDim.x) {
                     w = decode_unit(a, u);
                     if (w.n > 0) {
-                        j0 = __ldg(a.col_idx + w.rs);
+                        j0 = a.col_idx[w.rs];
                         break;
                     }
                 }
@@ -283,7 +283,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 const uint32_t un = next_unit(u + gridDim.x, wn, jnext);
                 bool q_pending = un < (uint32_t)a.n_units;  // the next unit's Q tiles are still to be requested
                 for (int t = 0; t < w.n; ++t, ++kc) {
-                    const int32_t jn = t + 1 < w.n ? __ldg(a.col_idx + w.rs + t + 1) : 0;
+                    const int32_t jn = t + 1 < w.n ? a.col_idx[w.rs + t + 1] : 0;
                     const uint32_t ks = kc % kKStages, vs = kc % kVStages;
                     if (kc >= (uint32_t)kKStages) {
                         ok = wait_bar(bar(BAR_K_EMPTY + ks), (kc / kKStages - 1) & 1, abort_flag, a.status, 2);
@@ -471,7 +471,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             if (u < (uint32_t)a.n_units) r = decode_unit(a, u);
             return r;
         };
-        auto fetch_lastcol = [&](const Unit &r) { return r.n > 0 ? __ldg(a.col_idx + r.rs + r.n - 1) : -1; };
+        auto fetch_lastcol = [&](const Unit &r) { return r.n > 0 ? a.col_idx[r.rs + r.n - 1] : -1; };
         Unit w_next = fetch_unit(blockIdx.x);
         Unit w_next2 = fetch_unit(blockIdx.x + gridDim.x);
         int32_t lastcol_next = fetch_lastcol(w_next);
