@@ -986,6 +986,10 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 it = gridDim.x + (uint32_t)__shfl_sync(0xffffffffu, drawn, 0);
             }
             if (k >= kItemRing && !wait_warp(bar(C::ITEM_EMPTY + r), (k / kItemRing - 1) & 1, 34)) return -2;
+            // The loop below follows KV_FULL phase by phase.  So that two of its phases are never over before this warp
+            // has asked for the first (their parity would then pass for that of a phase to come), item 1 is handed out
+            // once the loads of item 0 have landed, which its lookup mostly outlasts.
+            if (k == 1 && !wait_warp(bar(C::KV_FULL), 0, 35)) return -2;
             if (lane == 0) {
                 tail->items[r] = w;
                 ptx::mbar_arrive(bar(C::ITEM_FULL + r));
@@ -995,10 +999,7 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         const bool finder = warp == 4 + kCompWarps;
         int n_next = -1;  // (finder) length of item k + 1
         bool ok = true;
-        if (finder && publish_next(0) >= 0) {
-            n_next = publish_next(1);
-            ok = wait_warp(bar(C::KV_FULL), 0, 35);
-        }
+        if (finder && publish_next(0) >= 0) n_next = publish_next(1);
         for (uint32_t k = 0; ok; ++k) {
             BwdItem w;
             ok = read_item(k, w);
