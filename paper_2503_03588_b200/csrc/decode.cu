@@ -40,6 +40,7 @@ struct DecodeArgs {
     const int32_t *table;  // paged cache: [batch, table_stride] page numbers; null: contiguous cache
     float *partial;        // [batch, Hq, chunks, D + 2]
     int32_t *status;       // [0] error code, [1] detail
+    int32_t clear_status;  // the kernel clears the error code itself
     void *o;
     float *lse;
     // Element strides.  Contiguous cache: batch, token, head.  Paged: page, token in page, head.
@@ -430,7 +431,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) decode_row_kernel(const __grid
     if (peers) ptx::cluster_arrive_relaxed();
     pdl_wait();
     const int32_t len_first = it0 < n_items ? a.lens[(it0 / (uint32_t)R) / (uint32_t)a.Hkv] : 0;
-    if (blockIdx.x == 0 && tid == 0) a.status[0] = 0;  // a wait that gives up (much later) sets it
+    if (a.clear_status && blockIdx.x == 0 && tid == 0) a.status[0] = 0;  // a wait that gives up (much later) sets it
 
     // Item it -> (row of the call, chunk); a row -> (sequence, KV head).
     struct Item {
@@ -996,9 +997,14 @@ static pa_status launch_decode(const DecodeShape &p, const void *q, const void *
     a.stages = 0;
     const float scale = p.softmax_scale != 0.f ? p.softmax_scale : 1.0f / sqrtf((float)p.head_dim);
     a.scale_log2 = scale * 1.4426950408889634f;
-    a.wait_cycles = wait_limit_cycles() > 0 ? wait_limit_cycles() : kRowWaitCycles;
+    // Block 0 clears the error code as it starts, a second before any wait can run out; under a caller's limit, which
+    // may be shorter than the time from one CTA's start to another's, it is cleared ahead of the kernel.
+    const long long wait_cycles = wait_limit_cycles();
+    a.wait_cycles = wait_cycles > 0 ? wait_cycles : kRowWaitCycles;
+    a.clear_status = wait_cycles <= 0;
 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (!a.clear_status) PA_CUDA_OK(cudaMemsetAsync(a.status, 0, sizeof(int32_t), st));
     const EnvSwitches env = env_switches();
     a.fixed_chunks = 0;
     a.R = 1;

@@ -62,6 +62,7 @@ struct PrefillArgs {
     void *o;
     float *lse;
     int32_t *status;  // [0] error code, [1] detail
+    int32_t clear_status;  // the kernel clears the status block itself
     int64_t o_sb, o_ss, o_sh;
     int64_t lse_sb, lse_sh;  // LSE strides (batch, head); the token stride is 1
     int64_t N, n_units;     // N: sequence length (variable-length batch: the longest one, which sizes the unit grid)
@@ -227,8 +228,8 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     // this launch is leaving cost more than they save (32K tokens, 28 / 4 heads: 383 us against 379).
     if (a.n_units <= gridDim.x) pdl_launch_next();
     pdl_wait();
-    // A clear status block (a wait that gives up, much later, writes to it).
-    if (blockIdx.x == 0 && threadIdx.x < kPrefillWorkspace / sizeof(int32_t)) a.status[threadIdx.x] = 0;
+    // A clear status block (a wait that gives up, much later, writes to it: see launch_prefill).
+    if (a.clear_status && blockIdx.x == 0 && threadIdx.x < kPrefillWorkspace / sizeof(int32_t)) a.status[threadIdx.x] = 0;
     ptx::tc_fence_before_sync();
     __syncthreads();
     ptx::tc_fence_after_sync();
@@ -991,10 +992,14 @@ static pa_status launch_prefill(const pa_prefill_params *p, const void *q, const
     const float scale = p->softmax_scale != 0.f ? p->softmax_scale : 1.0f / sqrtf((float)D);
     a.scale_log2 = scale * 1.4426950408889634f;
 
+    // Block 0 clears the status block as it starts, two seconds before any wait can run out.  A caller's limit may be
+    // shorter than the time from one CTA's start to another's: then it is cleared ahead of the kernel.
     const long long wait_cycles = wait_limit_cycles();
     a.wait_cycles = wait_cycles > 0 ? wait_cycles : kWaitCycles;
+    a.clear_status = wait_cycles <= 0;
     const unsigned grid = (unsigned)(a.n_units < dev.sms ? a.n_units : dev.sms);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (!a.clear_status) PA_CUDA_OK(cudaMemsetAsync(workspace, 0, kPrefillWorkspace, st));
     {
         // PA_VALIDATE=1: check the CSR on the device before the attention kernel is enqueued.  This
         // synchronises the stream (so not during stream capture) and is meant for bring-up: a CSR

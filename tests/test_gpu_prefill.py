@@ -492,3 +492,24 @@ def test_keys_and_values_shared_by_the_batch(pa, D):
     pa.pa_prefill_status(ws)
     o_ref, lse_ref, _ = pa.pa_prefill(q, k.contiguous(), v.contiguous(), rp, ci)
     assert torch.equal(o, o_ref) and torch.equal(lse, lse_ref)
+
+
+def test_a_timeout_is_reported_whichever_cta_it_happens_in(pa):
+    """The first CTA has an empty row and waits for nothing; the others' waits run out at once.  What they report
+    outlives the first one's start."""
+    nqb, Hq, D = 40, 2, 64
+    rp = torch.arange(nqb + 1, dtype=torch.int32)
+    rp[nqb] = nqb - 1   # row i lists block i, the last row (the first CTA's) nothing
+    ci = torch.arange(nqb - 1, dtype=torch.int32)
+    q, k, v = (si.bf16_randn((1, 64 * nqb, Hq if x == 0 else 1, D), 1830 + x).cuda() for x in range(3))
+    rp, ci = rp.cuda(), ci.cuda()
+    try:
+        pa.pa_set_wait_limit_cycles(1)
+        for _ in range(50):
+            _, _, ws = pa.pa_prefill(q, k, v, rp, ci)
+            with pytest.raises(pa.PaError, match="PA_ERR_TIMEOUT"):
+                pa.pa_prefill_status(ws)
+    finally:
+        pa.pa_set_wait_limit_cycles(0)
+    _, _, ws = pa.pa_prefill(q, k, v, rp, ci)
+    assert pa.pa_prefill_status(ws) == 0
