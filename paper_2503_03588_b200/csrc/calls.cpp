@@ -11,6 +11,7 @@
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Device.h>
 #include <torch/csrc/Dtype.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include "powerattn.h"
@@ -337,8 +338,8 @@ PyObject *call(PyObject *, PyObject *const *args, Py_ssize_t n)
     try {
         return F(args);
     } catch (const Raised &) {
-    } catch (const std::exception &e) {
-        PyErr_SetString(PyExc_RuntimeError, e.what());
+    } catch (const std::exception &) {  // (as torch's own functions raise it: OutOfMemoryError and so on)
+        torch::translate_exception_to_python(std::current_exception());
     }
     return nullptr;
 }

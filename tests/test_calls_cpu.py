@@ -42,3 +42,12 @@ def test_library_errors_carry_status_and_message(pa):
         stream_error = (pa.PaError, RuntimeError)  # (without a driver torch itself may refuse to name a stream)
     with pytest.raises(stream_error):
         pa.pa_decode(_bf16(1, 4, 96), _bf16(1, 64, 2, 96), _bf16(1, 64, 2, 96), torch.ones(1, dtype=torch.int32), 5, 1)
+
+
+def test_errors_of_torch_keep_their_class(pa):
+    """A C++ exception of torch comes out as the Python exception torch itself would raise."""
+    with pytest.raises(RuntimeError) as expected:
+        torch.empty(1, device="vulkan")
+    with pytest.raises(type(expected.value)) as got:
+        pa.pa_build_layout(1000, 64, 5, 1, device="vulkan")
+    assert type(got.value) is type(expected.value) is NotImplementedError

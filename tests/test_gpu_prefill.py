@@ -513,3 +513,11 @@ def test_a_timeout_is_reported_whichever_cta_it_happens_in(pa):
         pa.pa_set_wait_limit_cycles(0)
     _, _, ws = pa.pa_prefill(q, k, v, rp, ci)
     assert pa.pa_prefill_status(ws) == 0
+
+
+def test_an_output_too_large_for_the_gpu_raises_out_of_memory(pa):
+    """(Nothing is launched: the output of 256 GiB is asked for first.)"""
+    q = torch.zeros((1, 64, 2, 64), dtype=torch.bfloat16, device="cuda").expand(1 << 24, -1, -1, -1)
+    rp, ci = pa.pa_build_layout(64, 64, 5, 1)
+    with pytest.raises(torch.OutOfMemoryError):
+        pa.pa_prefill(q, q, q, rp, ci)
