@@ -181,11 +181,15 @@ def pa_layout_size(seq_len: int, block: int, window_blocks: int, sink_blocks: in
     return int(nqb.value), int(nnz.value)
 
 
+def _device(device):
+    return torch.get_default_device() if device is None else torch.device(device)
+
+
 def pa_build_layout(seq_len: int, block: int, window_blocks: int, sink_blocks: int,
                     row_ptr: Optional[torch.Tensor] = None, col_idx: Optional[torch.Tensor] = None,
                     device="cuda"):
     """Returns (row_ptr, col_idx) int32 device tensors (allocated here when not passed in)."""
-    return _calls.build_layout(seq_len, block, window_blocks, sink_blocks, None, row_ptr, col_idx, device)
+    return _calls.build_layout(seq_len, block, window_blocks, sink_blocks, None, row_ptr, col_idx, _device(device))
 
 
 def pa_window_layout_size(seq_len: int, block: int, window_blocks: int, sink_blocks: int) -> Tuple[int, int]:
@@ -198,7 +202,7 @@ def pa_build_window_layout(seq_len: int, block: int, window_blocks: int, sink_bl
                            row_ptr: Optional[torch.Tensor] = None, col_idx: Optional[torch.Tensor] = None,
                            device="cuda"):
     """Sliding-window layout (window + sink blocks, no power-of-two term) as int32 device tensors."""
-    return _calls.build_layout(seq_len, block, window_blocks, sink_blocks, 0, row_ptr, col_idx, device)
+    return _calls.build_layout(seq_len, block, window_blocks, sink_blocks, 0, row_ptr, col_idx, _device(device))
 
 
 def pa_reach_counts(row_ptr, col_idx, start: int, max_steps: int):
@@ -228,7 +232,7 @@ def pa_build_tile_layout(seq_len: int, block: int, window_blocks: int, sink_bloc
     `tile`-token tiles (allocated here when not passed in)."""
     if tile < 1:
         pa_tile_layout_size(seq_len, block, window_blocks, sink_blocks, tile)  # raises
-    return _calls.build_layout(seq_len, block, window_blocks, sink_blocks, tile, row_ptr, col_idx, device)
+    return _calls.build_layout(seq_len, block, window_blocks, sink_blocks, tile, row_ptr, col_idx, _device(device))
 
 
 def prefill_params(q, k, v, o, block: int = 64, softmax_scale: float = 0.0) -> pa_prefill_params:

@@ -303,14 +303,8 @@ PyObject *build_layout(PyObject *const *x)
                            : pa_tile_layout_size(seq_len, block, window, sink, tile, &rows, &nnz);
     });
     auto fresh = [&](int64_t n) {
-        c10::Device device(c10::kCUDA);
-        if (THPDevice_Check(x[7])) {
-            device = reinterpret_cast<THPDevice *>(x[7])->device;
-        } else {
-            const char *name = PyUnicode_AsUTF8(x[7]);
-            if (!name) throw Raised();
-            device = c10::Device(std::string(name));
-        }
+        if (!THPDevice_Check(x[7])) raise(PyExc_TypeError, "expected a torch.device");
+        const c10::Device device = reinterpret_cast<THPDevice *>(x[7])->device;
         return at::empty({n}, at::TensorOptions().dtype(at::kInt).device(device));
     };
     const Out row_ptr(x[5], [&] { return fresh((int64_t)rows + 1); });

@@ -51,3 +51,20 @@ def test_errors_of_torch_keep_their_class(pa):
     with pytest.raises(type(expected.value)) as got:
         pa.pa_build_layout(1000, 64, 5, 1, device="vulkan")
     assert type(got.value) is type(expected.value) is NotImplementedError
+
+
+@pytest.mark.parametrize("device", [0, None, "cuda", torch.device("cuda", 0), "nowhere", 1.5])
+def test_devices_are_named_as_in_torch(pa, device):
+    """Layouts take what torch.empty takes for a device (None: the default one), and raise what it raises."""
+    def error_of(call):
+        try:
+            with torch.device("cuda"):
+                call()
+        except Exception as e:
+            return type(e)
+
+    expected = error_of(lambda: torch.empty(1, device=device))
+    for build in (lambda d: pa.pa_build_layout(1000, 64, 5, 1, device=d),
+                  lambda d: pa.pa_build_window_layout(1000, 64, 5, 1, device=d),
+                  lambda d: pa.pa_build_tile_layout(1000, 128, 5, 1, 64, device=d)):
+        assert error_of(lambda: build(device)) is expected
