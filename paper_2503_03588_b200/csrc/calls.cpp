@@ -8,6 +8,7 @@
 #include <Python.h>
 
 #include <ATen/ops/empty.h>
+#include <c10/core/DefaultDtype.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Device.h>
 #include <torch/csrc/Dtype.h>
@@ -57,6 +58,7 @@ float number(PyObject *o)
 }
 at::ScalarType dtype(PyObject *o)
 {
+    if (o == Py_None) return c10::get_default_dtype_as_scalartype();  // (as in torch.empty)
     if (!THPDtype_Check(o)) raise(PyExc_TypeError, "expected a torch.dtype");
     return reinterpret_cast<THPDtype *>(o)->scalar_type;
 }

@@ -68,3 +68,10 @@ def test_devices_are_named_as_in_torch(pa, device):
                   lambda d: pa.pa_build_window_layout(1000, 64, 5, 1, device=d),
                   lambda d: pa.pa_build_tile_layout(1000, 128, 5, 1, 64, device=d)):
         assert error_of(lambda: build(device)) is expected
+
+
+def test_no_output_type_is_no_type_error(pa):
+    """o_dtype None stands for torch's default type, as in torch.empty."""
+    q, kc, lens = _bf16(1, 4, 128), _bf16(1, 64, 2, 128), torch.ones(1, dtype=torch.int64)
+    with pytest.raises(AssertionError):   # the lengths' type, which is looked at after the output has been made
+        pa.pa_decode(q, kc, kc, lens, 5, 1, o_dtype=None)

@@ -521,3 +521,11 @@ def test_an_output_too_large_for_the_gpu_raises_out_of_memory(pa):
     rp, ci = pa.pa_build_layout(64, 64, 5, 1)
     with pytest.raises(torch.OutOfMemoryError):
         pa.pa_prefill(q, q, q, rp, ci)
+
+
+def test_output_type_none_is_the_default_type(pa):
+    q, k, v = (si.bf16_randn((1, 200, 2, 64), 1840 + x).cuda() for x in range(3))
+    rp, ci = pa.pa_build_layout(200, 64, 5, 1)
+    o, _, _ = pa.pa_prefill(q, k, v, rp, ci, o_dtype=None)
+    assert o.dtype is torch.get_default_dtype() is torch.float32
+    assert torch.equal(o, pa.pa_prefill(q, k, v, rp, ci, o_dtype=torch.float32)[0])
