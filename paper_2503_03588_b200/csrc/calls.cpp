@@ -71,6 +71,18 @@ pa_strides strides4(const at::Tensor &t)
     return {t.stride(0), t.stride(1), t.stride(2)};
 }
 
+struct WithoutGil {
+    PyThreadState *state = PyEval_SaveThread();
+    ~WithoutGil() { PyEval_RestoreThread(state); }
+};
+
+// (An allocation may wait for the device or another thread: without the interpreter lock, like torch's own.)
+at::Tensor empty(at::IntArrayRef size, const at::TensorOptions &options)
+{
+    const WithoutGil released;
+    return at::empty(size, options);
+}
+
 // An output or scratch tensor: the caller's, or one allocated here.
 struct Out {
     at::Tensor t;
@@ -90,7 +102,7 @@ struct Out {
 };
 at::Tensor make(const at::Tensor &like, at::IntArrayRef size, at::ScalarType type)
 {
-    return at::empty(size, like.options().dtype(type));
+    return empty(size, like.options().dtype(type));
 }
 at::Tensor make_bytes(const at::Tensor &like, size_t n)
 {
@@ -98,11 +110,6 @@ at::Tensor make_bytes(const at::Tensor &like, size_t n)
 }
 
 void *stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
-
-struct WithoutGil {
-    PyThreadState *state = PyEval_SaveThread();
-    ~WithoutGil() { PyEval_RestoreThread(state); }
-};
 
 // Runs a library call without the interpreter lock; raises on a status other than PA_OK.
 template <typename Call>
@@ -307,7 +314,7 @@ PyObject *build_layout(PyObject *const *x)
     auto fresh = [&](int64_t n) {
         if (!THPDevice_Check(x[7])) raise(PyExc_TypeError, "expected a torch.device");
         const c10::Device device = reinterpret_cast<THPDevice *>(x[7])->device;
-        return at::empty({n}, at::TensorOptions().dtype(at::kInt).device(device));
+        return empty({n}, at::TensorOptions().dtype(at::kInt).device(device));
     };
     const Out row_ptr(x[5], [&] { return fresh((int64_t)rows + 1); });
     const Out col_idx(x[6], [&] { return fresh(nnz); });

@@ -1,5 +1,8 @@
 """The CPython module behind the attention calls: broken preconditions raise before anything is launched, and
 leave the interpreter usable (no GPU is present in this run)."""
+import threading
+import time
+
 import pytest
 import torch
 
@@ -75,3 +78,31 @@ def test_no_output_type_is_no_type_error(pa):
     q, kc, lens = _bf16(1, 4, 128), _bf16(1, 64, 2, 128), torch.ones(1, dtype=torch.int64)
     with pytest.raises(AssertionError):   # the lengths' type, which is looked at after the output has been made
         pa.pa_decode(q, kc, kc, lens, 5, 1, o_dtype=None)
+
+
+def test_other_threads_run_while_an_output_is_allocated(pa, monkeypatch):
+    """An allocation that takes long (here: 160 MB filled with a pattern) does not hold the interpreter lock."""
+    if torch.cuda.is_available():
+        pytest.skip("the call is made to end before its launch, which takes a machine without a GPU")
+    monkeypatch.setattr(torch.utils.deterministic, "fill_uninitialized_memory", True)
+    torch.use_deterministic_algorithms(True)
+    ticks, stop = [], threading.Event()
+
+    def tick():
+        while not stop.is_set():
+            ticks.append(time.perf_counter())
+            time.sleep(0.001)
+
+    thread = threading.Thread(target=tick)
+    thread.start()
+    try:
+        t0 = time.perf_counter()
+        with pytest.raises(RuntimeError):
+            pa.pa_build_window_layout(40_000_000, 1, 1, 0, col_idx=torch.empty(1, dtype=torch.int32), device="cpu")
+        t1 = time.perf_counter()
+    finally:
+        stop.set()
+        thread.join()
+        torch.use_deterministic_algorithms(False)
+    inside = [t0] + [t for t in ticks if t0 < t < t1] + [t1]
+    assert max(b - a for a, b in zip(inside, inside[1:])) < 0.5 * (t1 - t0), (t1 - t0, len(inside))
