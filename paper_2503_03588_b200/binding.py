@@ -138,6 +138,9 @@ lib = _load()
 
 from . import _calls  # noqa: E402  (linked against the library loaded above)
 
+if _calls.torch_version != str(torch.__version__):  # (its tensors and types may be laid out differently)
+    raise ImportError("_calls.so was built against torch %s, this is %s: run %s" %
+                      (_calls.torch_version, torch.__version__, os.path.join(os.path.dirname(__file__), "build.py")))
 _calls.set_error(PaError)
 
 

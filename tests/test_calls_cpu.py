@@ -106,3 +106,22 @@ def test_other_threads_run_while_an_output_is_allocated(pa, monkeypatch):
         torch.use_deterministic_algorithms(False)
     inside = [t0] + [t for t in ticks if t0 < t < t1] + [t1]
     assert max(b - a for a, b in zip(inside, inside[1:])) < 0.5 * (t1 - t0), (t1 - t0, len(inside))
+
+
+def test_the_module_is_rebuilt_for_another_torch_or_python(pa, monkeypatch):
+    """Its file is as new as before, but it fits the versions it was built against only."""
+    import importlib.util
+    import os
+
+    path = os.path.join(os.path.dirname(pa.__file__), "build.py")
+    spec = importlib.util.spec_from_file_location("_powerattn_build_under_test", path)
+    build = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(build)
+    assert not build._calls_stale([])
+    version = build._torch_version()
+    for name, value in (("CALLS_STAMP", build.CALLS_STAMP + ".missing"), ("_torch_version", lambda: "2.99.0"),
+                        ("_torch_dir", lambda: "/elsewhere/torch")):
+        with monkeypatch.context() as m:
+            m.setattr(build, "_torch_version", lambda: version)   # (else read from where torch is)
+            m.setattr(build, name, value)
+            assert build._calls_stale([]), name
