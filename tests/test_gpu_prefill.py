@@ -497,10 +497,10 @@ def test_keys_and_values_shared_by_the_batch(pa, D):
 def test_a_timeout_is_reported_whichever_cta_it_happens_in(pa):
     """The first CTA has an empty row and waits for nothing; the others' waits run out at once.  What they report
     outlives the first one's start."""
-    nqb, Hq, D = 40, 2, 64
-    rp = torch.arange(nqb + 1, dtype=torch.int32)
-    rp[nqb] = nqb - 1   # row i lists block i, the last row (the first CTA's) nothing
-    ci = torch.arange(nqb - 1, dtype=torch.int32)
+    nqb, Hq, D = 120, 2, 64
+    rows = [i + 1 for i in range(nqb - 1)] + [0]   # dense rows, some 100 steps long; the last one (the first CTA's) empty
+    rp = torch.tensor([0] + rows).cumsum(0).to(torch.int32)
+    ci = torch.cat([torch.arange(n, dtype=torch.int32) for n in rows])
     q, k, v = (si.bf16_randn((1, 64 * nqb, Hq if x == 0 else 1, D), 1830 + x).cuda() for x in range(3))
     rp, ci = rp.cuda(), ci.cuda()
     try:
