@@ -833,9 +833,10 @@ __global__ void decode_row_block_set_kernel(int64_t len, int32_t W, int32_t S, i
 // cache_lens[b], 16 bytes per thread and turn; once every thread has read the old length it grows by one.  A
 // sequence whose block table has no valid page for that position is left alone.  (One launch: copying and
 // advancing the lengths in two kernels, each waiting for the one before it, cost a decoding step a third launch.)
-constexpr int kAppendThreads = 128;
-
-__global__ void __launch_bounds__(kAppendThreads)
+// kThreads: 128 or, beyond 256 pieces, 1024, since a thread's turns follow one another (64 heads of 128 features, 8
+// sequences: 4.6 us with 128 threads, 2.8 with 1024; 8 heads 1.9 and 1.8; one head of 64 features 1.7 and 1.7).
+template <int kThreads>
+__global__ void __launch_bounds__(kThreads)
 kv_append_kernel(const __nv_bfloat16 *k_new, const __nv_bfloat16 *v_new, __nv_bfloat16 *k_pool, __nv_bfloat16 *v_pool,
                  const int32_t *table, int32_t *lens, int32_t table_stride, int32_t n_pages, int32_t Hkv, int32_t D,
                  int64_t k_sp, int64_t k_ss, int64_t k_sh, int64_t v_sp, int64_t v_ss, int64_t v_sh)
@@ -849,7 +850,7 @@ kv_append_kernel(const __nv_bfloat16 *k_new, const __nv_bfloat16 *v_new, __nv_bf
     const int32_t page = table[(int64_t)b * table_stride + blk];
     if (page < 0 || page >= n_pages) return;
     const int slot = pos % kDecBlock, per_row = D / 8, pieces = Hkv * per_row;  // 16-byte pieces of K, then of V
-    for (int x = threadIdx.x; x < 2 * pieces; x += kAppendThreads) {
+    for (int x = threadIdx.x; x < 2 * pieces; x += kThreads) {
         const bool is_v = x >= pieces;
         const int y = is_v ? x - pieces : x, hk = y / per_row, c = y % per_row;
         const uint4 piece = *reinterpret_cast<const uint4 *>((is_v ? v_new : k_new) + ((int64_t)b * Hkv + hk) * D + 8 * c);
@@ -1179,11 +1180,15 @@ extern "C" pa_status pa_kv_append(const pa_paged_params *p, const void *k_new, c
     if (!aligned16(k_new) || !aligned16(v_new) || !aligned16(k_pool) || !aligned16(v_pool))
         return fail(PA_ERR_ALIGNMENT, "k_new, v_new and the pools must be 16-byte aligned");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    PA_CUDA_OK(launch_pdl(kv_append_kernel, dim3((unsigned)p->batch), kAppendThreads, 0, st,
-                          static_cast<const __nv_bfloat16 *>(k_new), static_cast<const __nv_bfloat16 *>(v_new),
-                          static_cast<__nv_bfloat16 *>(k_pool), static_cast<__nv_bfloat16 *>(v_pool), block_table, cache_lens,
-                          p->max_blocks_per_seq, p->n_pages, p->n_kv_heads, p->head_dim, p->k.batch, p->k.seq, p->k.head,
-                          p->v.batch, p->v.seq, p->v.head));
+    auto launch = [&](auto kernel, unsigned threads) {
+        return launch_pdl(kernel, dim3((unsigned)p->batch), threads, 0, st, static_cast<const __nv_bfloat16 *>(k_new),
+                          static_cast<const __nv_bfloat16 *>(v_new), static_cast<__nv_bfloat16 *>(k_pool),
+                          static_cast<__nv_bfloat16 *>(v_pool), block_table, cache_lens, p->max_blocks_per_seq, p->n_pages,
+                          p->n_kv_heads, p->head_dim, p->k.batch, p->k.seq, p->k.head, p->v.batch, p->v.seq, p->v.head);
+    };
+    const int pieces = 2 * p->n_kv_heads * (p->head_dim / 8);
+    if (pieces <= 256) PA_CUDA_OK(launch(kv_append_kernel<128>, 128));
+    else PA_CUDA_OK(launch(kv_append_kernel<1024>, 1024));
     return PA_OK;
 }
 
