@@ -259,9 +259,9 @@ size_t pa_decode_workspace_bytes(const pa_decode_params *p);
  * (window_blocks + sink_blocks + log2 of the row count: any default-window row up to millions of
  * tokens) the row kernel runs: a row's key blocks are dealt to R chunks; in each CTA a producer
  * warp fetches the blocks of its chunk by TMA into a ring of shared-memory stages and four warps
- * run an online softmax over them.  Small calls (batch x n_kv_heads up to the number of SMs) are one
- * launch in which the R CTAs of a row form a thread-block cluster and merge their results through
- * distributed shared memory with the log-sum-exp rule
+ * run an online softmax over them.  Small calls (batch x n_kv_heads up to the number of SMs, rows of
+ * more than one block) are one launch in which the R CTAs of a row form a thread-block cluster and
+ * merge their results through distributed shared memory with the log-sum-exp rule
  * m = max m_c, l = sum l_c e^(m_c - m), o = sum o_c e^(m_c - m) / l.  Larger calls run a
  * persistent grid (two CTAs per SM) over the (row, chunk) items and, unless R is 1, a second small
  * kernel that merges each row's R partial results from the workspace.  Rows with more candidates

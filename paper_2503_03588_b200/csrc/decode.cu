@@ -955,6 +955,49 @@ static size_t decode_workspace_bytes(const DecodeShape &s)
     return kDecStatusBytes + (size_t)s.batch * s.n_q_heads * chunks * (s.head_dim + 2) * sizeof(float);
 }
 
+static size_t row_smem_bytes(int head_dim, int stages, bool cluster)
+{
+    return head_dim == 128 ? RowSmem<128>::bytes(stages, cluster) : RowSmem<64>::bytes(stages, cluster);
+}
+
+// (The last attribute is the one that lets the kernel start early.)
+static cudaLaunchConfig_t row_launch_config(unsigned grid, int R, size_t smem, cudaLaunchAttribute (&attr)[2])
+{
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)R;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1] = pdl_attribute();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid, 1, 1);
+    cfg.blockDim = dim3(kRowThreads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cfg;
+}
+
+// How many clusters of R CTAs of the row kernel the device holds at once.  Asked once per device and kind of launch.
+static pa_status resident_clusters(int device, int head_dim, int stages, int R, int *out)
+{
+    static std::mutex mu;
+    static int known[kMaxDevices][2][kRowMaxStages + 1][kRowMaxCluster + 1];  // the number plus one; 0: not asked yet
+    std::lock_guard<std::mutex> lock(mu);
+    int &n = known[device][head_dim == 128][stages][R];
+    if (n == 0) {
+        cudaLaunchAttribute attr[2];
+        const cudaLaunchConfig_t cfg = row_launch_config((unsigned)R, R, row_smem_bytes(head_dim, stages, true), attr);
+        int found = 0;
+        if (head_dim == 128)
+            PA_CUDA_OK(cudaOccupancyMaxActiveClusters(&found, decode_row_kernel<128>, &cfg));
+        else
+            PA_CUDA_OK(cudaOccupancyMaxActiveClusters(&found, decode_row_kernel<64>, &cfg));
+        n = found + 1;
+    }
+    *out = n - 1;
+    return PA_OK;
+}
+
 // The launch shared by every decode entry point.  table == null: contiguous cache.
 static pa_status launch_decode(const DecodeShape &p, const void *q, const void *k_cache, const void *v_cache,
                                const int32_t *table, int32_t table_stride, int32_t n_pages,
@@ -1016,57 +1059,17 @@ static pa_status launch_decode(const DecodeShape &p, const void *q, const void *
         const int64_t rows_in_call = (int64_t)a.batch * a.Hkv;
         const int max_R = a.chunks < kRowMaxCluster ? a.chunks : kRowMaxCluster;
         const int64_t persistent_ctas = (env.decode_ctas_per_sm ? env.decode_ctas_per_sm : 2) * (int64_t)dev.sms;
-        // Small calls (latency-bound): a cluster of R CTAs per row, all resident at once.  Larger calls
-        // (bandwidth-bound): a persistent grid of two CTAs per SM over the rows.  The line lies where a row
-        // still gets two of the resident CTAs: rows of 18 blocks (30000 tokens, G = 7, head_dim 128) take
-        // 9.2 us at 80 rows in clusters of three and 11.5 us in the persistent form, 12.4 and 13.3 at 120
-        // rows, 18.8 (clusters of one) and 15.7 at 160.
-        bool cluster = rows_in_call * 2 <= persistent_ctas;
-        if (env.decode_path == 2) cluster = true;
-        if (env.decode_path == 3) cluster = false;
-        int R = env.decode_cluster;
-        if (cluster) {
-            if (R == 0) {
-                // as many CTAs per row as still run all at once (two CTAs fit an SM): a second wave
-                // of clusters doubles the call's latency (batch 16: 17.4 us with R = 8, 12.5 with R = 4)
-                R = (int)(persistent_ctas / rows_in_call);
-                if (R < 1) R = 1;
-            }
-            if (R > max_R) R = max_R;
-            a.mode = kModeCluster;
-        } else {
-            // One chunk per row: finer items balance the SMs better on paper but pay more per item
-            // than they gain, and need the merge kernel.
-            if (R == 0) R = 1;
-            if (R > max_R) R = max_R;
-            a.mode = R == 1 ? kModeDirect : kModePartial;
-        }
-        a.R = R;
-        a.items = rows_in_call * R;
-        const int64_t grid = a.mode == kModeCluster ? a.items : (a.items < persistent_ctas ? a.items : persistent_ctas);
-        if (a.items > 0x3fffffff) return fail(PA_ERR_SHAPE, "too many work items (%lld)", (long long)a.items);
         // Stages: 64 KB of blocks in flight per CTA, and no more than a CTA has blocks.
-        const int64_t blocks_per_cta = ((int64_t)a.chunks * rows_in_call + grid - 1) / grid;
         // (two stages measured 1-3 % faster than three at batch 64 and 256, head_dim 128)
-        const int fit = p.head_dim == 128 ? 2 : 4;
-        a.stages = env.decode_stages != 0 ? env.decode_stages : fit;
-        if (a.stages > kRowMaxStages) a.stages = kRowMaxStages;
-        if (a.stages > blocks_per_cta) a.stages = (int)blocks_per_cta;
-        if (a.stages < 1) a.stages = 1;
-        while (a.stages > 1 && (p.head_dim == 128 ? RowSmem<128>::bytes(a.stages, a.mode == kModeCluster)
-                                                  : RowSmem<64>::bytes(a.stages, a.mode == kModeCluster)) > (size_t)kRowMaxSmem)
-            --a.stages;
-
-        // Tensor maps over the cache: (feature, token, head, batch or page), one 64 x 64 box per copy.
-        CUtensorMap tmK, tmV;
-        const bool paged = table != nullptr;
-        TensorMapKey kk = {k_cache, paged ? (int64_t)kDecBlock : p.max_len, p.k.seq, p.k.head, p.k.batch, dev.device,
-                           p.head_dim, p.n_kv_heads, paged ? n_pages : p.batch, 1, kDecBlock, 0};
-        TensorMapKey kv = {v_cache, paged ? (int64_t)kDecBlock : p.max_len, p.v.seq, p.v.head, p.v.batch, dev.device,
-                           p.head_dim, p.n_kv_heads, paged ? n_pages : p.batch, 1, kDecBlock, 0};
-        if (pa_status s = get_tensor_map(kk, "k_cache", &tmK)) return s;
-        if (pa_status s = get_tensor_map(kv, "v_cache", &tmV)) return s;
-
+        auto stages_of = [&](int64_t ctas, bool cluster_form) {
+            const int64_t blocks_per_cta = ((int64_t)a.chunks * rows_in_call + ctas - 1) / ctas;
+            int n = env.decode_stages != 0 ? env.decode_stages : p.head_dim == 128 ? 2 : 4;
+            if (n > kRowMaxStages) n = kRowMaxStages;
+            if (n > blocks_per_cta) n = (int)blocks_per_cta;
+            if (n < 1) n = 1;
+            while (n > 1 && row_smem_bytes(p.head_dim, n, cluster_form) > (size_t)kRowMaxSmem) --n;
+            return n;
+        };
         if (device_once_begin(dev.device, ONCE_DECODE_ATTR)) {
             const cudaError_t e1 = cudaFuncSetAttribute(decode_row_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                         kRowMaxSmem);
@@ -1078,29 +1081,76 @@ static pa_status launch_decode(const DecodeShape &p, const void *q, const void *
                             cudaGetErrorString(e1 != cudaSuccess ? e1 : e2));
             }
         }
+        // Small calls (latency-bound): a cluster of R CTAs per row, all resident at once.  Larger calls
+        // (bandwidth-bound): a persistent grid of two CTAs per SM over the rows.  The line lies where a row
+        // still gets two of the resident CTAs: rows of 18 blocks (30000 tokens, G = 7, head_dim 128) take
+        // 9.2 us at 80 rows in clusters of three and 11.5 us in the persistent form, 12.4 and 13.3 at 120
+        // rows, 18.8 (clusters of one) and 15.7 at 160.
+        bool cluster = rows_in_call * 2 <= persistent_ctas;
+        if (env.decode_path == 2) cluster = true;
+        if (env.decode_path == 3) cluster = false;
+        int R = env.decode_cluster, fit = 0;  // fit: clusters of R CTAs that the device holds at once
+        if (cluster && R == 0) {
+            // As many CTAs per row as run all at once: a second wave of clusters nearly doubles the call's latency
+            // (4000 tokens, G = 7, head_dim 128: 74 rows in clusters of four 13.0 us, of three 8.2; 98 rows in clusters of
+            // three 14.4 us, of two 10.0).  How many clusters fit is asked of the device: all CTAs of a cluster lie
+            // within one GPU processing cluster, which may leave places that no further cluster fits in.
+            R = (int)(persistent_ctas / rows_in_call);
+            if (R > max_R) R = max_R;
+            for (; R > 1; --R) {
+                const int stages = stages_of(rows_in_call * R, true);
+                if (pa_status s = resident_clusters(dev.device, p.head_dim, stages, R, &fit)) return s;
+                if (rows_in_call <= fit) break;
+            }
+        }
+        // (Large calls: one chunk per row.  Finer items balance the SMs better on paper but pay more per item
+        // than they gain, and need the merge kernel.)
+        if (R < 1) R = 1;
+        if (R > max_R) R = max_R;
+        // A row in one piece has nothing to merge with: the cluster form's last step is spared (rows of one block, G = 7,
+        // head_dim 128: 6.4 to 7.6 us in the cluster form, 3.8 to 4.6 without).
+        if (R == 1 && env.decode_path != 2) cluster = false;
+        a.mode = cluster ? kModeCluster : R == 1 ? kModeDirect : kModePartial;
+        a.R = R;
+        a.items = rows_in_call * R;
+        const int64_t grid = cluster ? a.items : (a.items < persistent_ctas ? a.items : persistent_ctas);
+        if (a.items > 0x3fffffff) return fail(PA_ERR_SHAPE, "too many work items (%lld)", (long long)a.items);
+        a.stages = stages_of(grid, cluster);
+        // Started early, clusters take places as the CTAs of the kernel before leave them, one by one, and what is left
+        // in between may be of no use to a cluster until more have ended.  A call that needs nearly all places starts
+        // on the empty device instead, about 0.7 us later.  Where that begins to pay was measured for each size, early
+        // and late in us (4000 tokens, G = 7, head_dim 128; 148 SMs): clusters of three 8.1 and 8.9 at 80 rows, 10.7 and
+        // 8.9 at 84, 12.9 and 8.9 at 93; of five 7.1 and 7.7 at 52, 8.2 and 7.6 at 54; of six 7.7 and 7.7 at 43, 8.8 and
+        // 7.5 at 45; of seven 6.5 and 7.1 at 34, 8.3 and 7.1 at 37; of four and eight, which find the places of their
+        // like, 8.1 and 8.3 at 70, 9.6 and 8.3 at 71, 6.8 and 6.9 at 32, 8.3 and 7.0 at 33.  Pairs fit in any order.
+        const bool full = R == 3             ? rows_in_call * 10 > fit * 9
+                          : (R & (R - 1)) == 0 ? rows_in_call == fit
+                                               : rows_in_call * 25 > fit * 24;
+        const bool early = !(cluster && R > 2 && fit > 0 && full);
+
+        // Tensor maps over the cache: (feature, token, head, batch or page), one 64 x 64 box per copy.
+        CUtensorMap tmK, tmV;
+        const bool paged = table != nullptr;
+        TensorMapKey kk = {k_cache, paged ? (int64_t)kDecBlock : p.max_len, p.k.seq, p.k.head, p.k.batch, dev.device,
+                           p.head_dim, p.n_kv_heads, paged ? n_pages : p.batch, 1, kDecBlock, 0};
+        TensorMapKey kv = {v_cache, paged ? (int64_t)kDecBlock : p.max_len, p.v.seq, p.v.head, p.v.batch, dev.device,
+                           p.head_dim, p.n_kv_heads, paged ? n_pages : p.batch, 1, kDecBlock, 0};
+        if (pa_status s = get_tensor_map(kk, "k_cache", &tmK)) return s;
+        if (pa_status s = get_tensor_map(kv, "v_cache", &tmV)) return s;
+
         if (a.mode == kModePartial) {
             a.chunks = R;  // the partials of a row are its R chunks
             a.fixed_chunks = R;
         }
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)grid, 1, 1);
-        cfg.blockDim = dim3(kRowThreads, 1, 1);
-        cfg.stream = st;
         cudaLaunchAttribute attr[2];
-        attr[1] = pdl_attribute();
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = a.mode == kModeCluster ? (unsigned)R : 1u;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 2;
-        if (p.head_dim == 128) {
-            cfg.dynamicSmemBytes = RowSmem<128>::bytes(a.stages, a.mode == kModeCluster);
+        cudaLaunchConfig_t cfg =
+            row_launch_config((unsigned)grid, cluster ? R : 1, row_smem_bytes(p.head_dim, a.stages, cluster), attr);
+        cfg.stream = st;
+        if (!early) cfg.numAttrs = 1;
+        if (p.head_dim == 128)
             PA_CUDA_OK(cudaLaunchKernelEx(&cfg, decode_row_kernel<128>, tmK, tmV, a));
-        } else {
-            cfg.dynamicSmemBytes = RowSmem<64>::bytes(a.stages, a.mode == kModeCluster);
+        else
             PA_CUDA_OK(cudaLaunchKernelEx(&cfg, decode_row_kernel<64>, tmK, tmV, a));
-        }
         if (a.mode != kModePartial) return PA_OK;
     } else {
         const dim3 grid1((unsigned)a.chunks, (unsigned)a.Hkv, (unsigned)a.batch);

@@ -300,8 +300,8 @@ def test_decode_many_rows_through_the_persistent_grid(pa, oracle, pa_env, env):
 
 @pytest.mark.parametrize("rows", [37, 38, 74, 75, 148, 149])
 def test_decode_where_the_number_of_ctas_per_row_changes(pa, oracle, rows):
-    """On 148 SMs a row gets eight CTAs up to 37 rows, then seven, four up to 74, then three, two up to
-    148, and from 149 on the rows are walked by a persistent grid."""
+    """A row gets as many CTAs, up to eight, as the clusters of all rows fit on the device at once (on 148 SMs seven
+    at 37 rows, six at 38, three at 74 and 75, two at 148); from 149 rows on they are walked by a persistent grid."""
     max_len, D = 2100, 64
     q = si.bf16_randn((rows, 2, D), 95)
     kc, vc = si.bf16_randn((rows, max_len, 1, D), 96), si.bf16_randn((rows, max_len, 1, D), 97)
@@ -343,3 +343,27 @@ def test_cache_shared_by_the_batch(pa, pa_env, env):
     pa.pa_decode_status(ws)
     o_ref, lse_ref, _ = pa.pa_decode(q, kc.contiguous(), vc.contiguous(), lens, 5, 1)
     assert torch.equal(o, o_ref) and torch.equal(lse, lse_ref)
+
+
+@pytest.mark.parametrize("rows", [33, 36, 45, 56, 71, 84, 93])
+def test_decode_calls_that_fill_the_device_back_to_back(pa, oracle, rows):
+    """Clusters that need nearly all places of the device (on 148 SMs), call after call on one stream."""
+    max_len, D = 2100, 64
+    q = si.bf16_randn((rows, 2, D), 1850)
+    kc, vc = si.bf16_randn((rows, max_len, 1, D), 1851), si.bf16_randn((rows, max_len, 1, D), 1852)
+    lens = np.random.default_rng(1853).integers(1, max_len + 1, size=rows)
+    qd, kd, vd, ld = q.cuda(), kc.cuda(), vc.cuda(), torch.as_tensor(lens, dtype=torch.int32).cuda()
+    calls = [pa.pa_decode(qd, kd, vd, ld, 5, 1) for _ in range(20)]
+    o_ref, lse_ref, _ = oracle.decode(q, kc, vc, lens, 64, 5, 1)
+    compare(calls[0][0], calls[0][1], o_ref, lse_ref, f"{rows} rows")
+    for o, lse, ws in calls:
+        pa.pa_decode_status(ws)
+        assert torch.equal(o, calls[0][0]) and torch.equal(lse, calls[0][1])
+
+
+@pytest.mark.parametrize("rows", [1, 100])
+def test_decode_of_caches_of_one_block(pa, oracle, rows):
+    """A row of one block has nothing to merge: no cluster."""
+    q = si.bf16_randn((rows, 7, 128), 1860)
+    kc, vc = si.bf16_randn((rows, 64, 1, 128), 1861), si.bf16_randn((rows, 64, 1, 128), 1862)
+    _run(pa, oracle, q, kc, vc, np.random.default_rng(1863).integers(1, 65, size=rows), 5, 1)
