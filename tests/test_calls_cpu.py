@@ -125,3 +125,14 @@ def test_the_module_is_rebuilt_for_another_torch_or_python(pa, monkeypatch):
             m.setattr(build, "_torch_version", lambda: version)   # (else read from where torch is)
             m.setattr(build, name, value)
             assert build._calls_stale([]), name
+
+
+def test_status_and_message_of_the_library(pa):
+    """Sizes are checked on the host, before anything that needs a GPU."""
+    for call, status, message in (
+            (lambda: pa.pa_build_layout(0, 64, 5, 1), 1, "seq_len must be >= 1 (got 0)"),
+            (lambda: pa.pa_build_window_layout(100, 64, 0, 1), 1, "a sliding-window layout needs window_blocks >= 1"),
+            (lambda: pa.pa_build_tile_layout(100, 100, 5, 1, 64), 2, "block 100 is not a multiple of tile 64")):
+        with pytest.raises(pa.PaError) as e:
+            call()
+        assert e.value.status == status and message in str(e.value)

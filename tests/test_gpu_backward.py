@@ -81,11 +81,21 @@ def test_backward_sliding_window_layout(pa, oracle):
     (4200, 8, 2, 5, 1),      # the sink column in three chunks
 ])
 def test_backward_head_dim_128_on_the_warp_level_kernels(pa, pa_env, oracle, N, Hq, Hkv, W, S):
-    """head_dim 128 takes the tcgen05 kernels by default; PA_BACKWARD_PATH=mma sends it through the
-    warp-level MMA kernels that head_dim 64 uses.  Both meet the oracle."""
+    """The tcgen05 kernels run by default; PA_BACKWARD_PATH=mma asks for the warp-level MMA kernels.  Both meet
+    the oracle."""
     _run(pa, oracle, N, Hq, Hkv, 128, W, S, seed=N)
     pa_env(PA_BACKWARD_PATH="mma")
     _run(pa, oracle, N, Hq, Hkv, 128, W, S, seed=N)
+
+
+@pytest.mark.parametrize("N,Hq,Hkv,W,S", [
+    (1000, 5, 1, 5, 1),      # an odd group
+    (777, 8, 2, 0, 0),       # pure power-of-two pattern, ragged
+    (4200, 4, 2, 5, 1),      # the sink column in several chunks
+])
+def test_backward_head_dim_64_on_the_warp_level_kernels(pa, pa_env, oracle, N, Hq, Hkv, W, S):
+    pa_env(PA_BACKWARD_PATH="mma")
+    _run(pa, oracle, N, Hq, Hkv, 64, W, S, batch=2, seed=N + 1)
 
 
 def test_backward_many_items_per_cta(pa, oracle):
@@ -278,3 +288,47 @@ def test_backward_of_keys_and_values_shared_by_the_batch(pa, D):
     rq, rk, rv, _ = pa.pa_prefill_backward(*copies, o, lse, d_o, rp, ci)
     assert torch.equal(dq, rq)
     assert torch.allclose(dk, rk, rtol=1e-4, atol=1e-5) and torch.allclose(dv, rv, rtol=1e-4, atol=1e-5)
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_backward_with_chunks_of_full_size(pa, oracle, D):
+    """Enough work that chunks have their full 32 query blocks: only the columns of several chunks, and those that
+    nobody lists, are cleared beforehand, and the KV heads are walked one after the other (Q and dO exceed 64 MB).
+    Columns nobody lists, of one chunk and of two; ragged length, batch 3.  The same gradients come out of calls on
+    eight KV heads of one batch entry each, which clear everything and deal a slot's heads together; two heads are
+    compared with the oracle."""
+    nqb, batch, H = 41, 3, 64
+    N = 64 * nqb - 20
+    rng = np.random.default_rng(1900)
+    rows = [[j for j in range(i + 1) if j < 2 or j == i or (j % 4 and rng.random() < 0.25)] for i in range(nqb)]
+    rows[12] = [j for j in rows[12] if j != 12]
+    rows = [r if i < 12 else [j for j in r if j != 12] for i, r in enumerate(rows)]   # nobody lists block 12
+    rp = np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.int32)
+    ci = np.asarray([j for r in rows for j in r], dtype=np.int32)
+    listers = np.bincount(ci, minlength=nqb)
+    assert listers[12] == 0 and listers[0] > 32 and 0 < listers[nqb - 1] <= 32
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert len(ci) * H * batch >= 32 * 8 * sms and batch * N * H * D * 4 > 64 << 20
+    Q, K, V, dO = (si.bf16_randn((batch, N, H, D), 1901 + x).cuda() for x in range(4))
+    rpd, cid = torch.as_tensor(rp).cuda(), torch.as_tensor(ci).cuda()
+    o, lse, ws = pa.pa_prefill(Q, K, V, rpd, cid)
+    pa.pa_prefill_status(ws)
+    dq, dk, dv, ws = pa.pa_prefill_backward(Q, K, V, o, lse, dO, rpd, cid, *(torch.full((batch, N, H, D), 7.0, device="cuda")
+                                                                             for _ in range(3)))
+    pa.pa_prefill_status(ws)
+    assert not dk[:, 64 * 12:64 * 13].any() and not dv[:, 64 * 12:64 * 13].any()
+    for b in range(batch):
+        for h in range(0, H, 8):
+            part = [x[b:b + 1, :, h:h + 8] for x in (Q, K, V, o, dO)]
+            pq, pk, pv, _ = pa.pa_prefill_backward(*part[:4], lse[b:b + 1, h:h + 8].contiguous(), part[4], rpd, cid)
+            assert torch.equal(dq[b:b + 1, :, h:h + 8], pq), (b, h)
+            for got, ref in ((dk, pk), (dv, pv)):
+                assert torch.allclose(got[b:b + 1, :, h:h + 8], ref, rtol=1e-4, atol=1e-5), (b, h)
+    dense = np.zeros((N, N), dtype=bool)
+    for i, r in enumerate(rows):
+        for j in r:
+            dense[i * 64:(i + 1) * 64, j * 64:(j + 1) * 64] = True
+    dense &= np.tril(np.ones((N, N), dtype=bool))
+    two = [x[1:2, :, 30:32].cpu().contiguous() for x in (Q, K, V, dO)]
+    for g, r, n in zip((dq, dk, dv), oracle.backward(*two, 64, 5, 1, dense=dense), ("dQ", "dK", "dV")):
+        _compare(g[1:2, :, 30:32], r, n + " full chunks")
