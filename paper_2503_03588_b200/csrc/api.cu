@@ -135,7 +135,8 @@ static bool same_key(const TensorMapKey &a, const TensorMapKey &b)
 {
     return a.base == b.base && a.seq == b.seq && a.stride_seq == b.stride_seq && a.stride_head == b.stride_head &&
            a.stride_batch == b.stride_batch && a.device == b.device && a.head_dim == b.head_dim &&
-           a.heads == b.heads && a.batch == b.batch && a.box_heads == b.box_heads && a.box_tokens == b.box_tokens && a.f32 == b.f32;
+           a.heads == b.heads && a.batch == b.batch && a.box_heads == b.box_heads && a.box_tokens == b.box_tokens &&
+           a.f32 == b.f32;
 }
 
 pa_status get_tensor_map(const TensorMapKey &key, const char *what, CUtensorMap *out)
@@ -164,8 +165,9 @@ pa_status get_tensor_map(const TensorMapKey &key, const char *what, CUtensorMap 
     const cuuint32_t box[4] = {(cuuint32_t)(128 / size), (cuuint32_t)key.box_tokens, (cuuint32_t)key.box_heads, 1};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     CUtensorMap m;
-    const CUresult r = g_encode(&m, key.f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(key.base), dims, strides,
-                                box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+    const CUtensorMapDataType type = key.f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
+    const CUresult r = g_encode(&m, type, 4, const_cast<void *>(key.base), dims, strides, box, estr,
+                                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS)
         return fail(PA_ERR_CUDA, "cuTensorMapEncodeTiled failed for %s (CUresult %d)", what, (int)r);

@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(kPrepThreads) backward_prep_kernel(const Backw
 {
     extern __shared__ uint32_t prep_bits[];
     if (a.early) pdl_launch_next();
-    pdl_wait();
+    pdl_wait();  // (nothing of global memory is touched before this)
     if (blockIdx.x == 0 && threadIdx.x < kBwdStatusBytes / sizeof(int32_t)) a.status[threadIdx.x] = 0;
     if (blockIdx.x < (unsigned)n_csc) {
         transpose_layout(a, (int32_t)blockIdx.x, cols_per_block, prep_bits);
@@ -520,10 +520,11 @@ static pa_status launch_backward(const BackwardArgs &a, const pa_prefill_params 
 {
     constexpr int kSmemDq = 4 * BwdTile<D>::kBytes, kSmemDkv = 4 * BwdTile<D>::kBytes + 2 * kBwdBlk * 4;
     if (device_once_begin(device, D == 128 ? ONCE_BACKWARD_ATTR : ONCE_BACKWARD_ATTR_64)) {
-        const cudaError_t e1 = cudaFuncSetAttribute(backward_dq_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemDq);
-        const cudaError_t e2 = cudaFuncSetAttribute(backward_dkv_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemDkv);
+        constexpr cudaFuncAttribute kSmem = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        const cudaError_t e1 = cudaFuncSetAttribute(backward_dq_kernel<D>, kSmem, kSmemDq);
+        const cudaError_t e2 = cudaFuncSetAttribute(backward_dkv_kernel<D>, kSmem, kSmemDkv);
         // (a bitmap row of more than the 32 KB aimed at is needed from 16 million tokens on)
-        const cudaError_t e3 = cudaFuncSetAttribute(backward_prep_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPrepMaxBitmap);
+        const cudaError_t e3 = cudaFuncSetAttribute(backward_prep_kernel<D>, kSmem, kPrepMaxBitmap);
         if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess) {
             device_once_reset(device, D == 128 ? ONCE_BACKWARD_ATTR : ONCE_BACKWARD_ATTR_64);
             return fail(PA_ERR_CUDA, "cudaFuncSetAttribute failed: %s",

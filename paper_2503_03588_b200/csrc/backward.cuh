@@ -1,5 +1,5 @@
 // Shared between the backward pass's two translation units: the argument block of its kernels and
-// the entry of the tensor-core (tcgen05) kernels for head_dim 128.
+// the entry of the tensor-core (tcgen05) kernels.
 #pragma once
 
 #include <cuda.h>

@@ -34,16 +34,19 @@
 
 // Registers per thread by role (control, compute, epilogue warps).  A warpgroup asking for more than the pool
 // holds would wait for ever: both kernels start 768 threads x 80.  (48 / 96 / 48 for both spills more, dK / dV
-// not at all now: backward pass at 4K tokens, 28 / 4 heads, 162.7 us against 161.4, 2 x 8K tokens, 16 / 4 heads
-// of 64 features, 245.5 against 242.5.)
+// not at all now.  Backward pass, two runs each: 4001 tokens, 28 / 4 heads, 154.0 and 154.6 us against 151.8 and
+// 151.9; 4 x 4096 tokens, 8 / 8 heads, 342 and 344 against 332 and 333; 2 x 8K tokens, 16 / 4 heads of 64 features,
+// 270 and 265 against 260 and 254.)
 #define PA_DQ_REG_CTRL 40
 #define PA_DQ_REG_COMP 96
 #define PA_DQ_REG_EPI 56
-static_assert(4 * PA_DQ_REG_CTRL + 16 * PA_DQ_REG_COMP + 4 * PA_DQ_REG_EPI <= 24 * 80, "register split exceeds the CTA's registers");
+static_assert(4 * PA_DQ_REG_CTRL + 16 * PA_DQ_REG_COMP + 4 * PA_DQ_REG_EPI <= 24 * 80,
+              "register split exceeds the CTA's registers");
 #define PA_DKV_REG_CTRL 64
 #define PA_DKV_REG_COMP 88
 #define PA_DKV_REG_EPI 64
-static_assert(4 * PA_DKV_REG_CTRL + 16 * PA_DKV_REG_COMP + 4 * PA_DKV_REG_EPI <= 24 * 80, "register split exceeds the CTA's registers");
+static_assert(4 * PA_DKV_REG_CTRL + 16 * PA_DKV_REG_COMP + 4 * PA_DKV_REG_EPI <= 24 * 80,
+              "register split exceeds the CTA's registers");
 
 namespace pa {
 
@@ -293,14 +296,14 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
                                              w.blk * kBwdBlk, h0, w.b);
                         return true;
                     };
-                    auto load_block = [&](uint32_t base, const CUtensorMap *tm, uint32_t full, uint32_t empty, uint32_t stages, int32_t j,
-                                          int code) {
+                    auto load_block = [&](uint32_t base, const CUtensorMap *tm, uint32_t full, uint32_t empty, uint32_t stages,
+                                          int32_t j, int code) {
                         const uint32_t st = c % stages;
                         if (c >= stages && !wait_bar(bar(empty + st), (c / stages - 1) & 1, code)) return false;
                         ptx::mbar_expect_tx(bar(full + st), C::kBlkTile);
                         for (int dh = 0; dh < DH; ++dh)
-                            ptx::tma_load_4d(smem_base + base + st * C::kBlkTile + dh * kKeyTile, tm, bar(full + st), dh * 64, j * kBwdBlk,
-                                             w.hk, w.b);
+                            ptx::tma_load_4d(smem_base + base + st * C::kBlkTile + dh * kKeyTile, tm, bar(full + st), dh * 64,
+                                             j * kBwdBlk, w.hk, w.b);
                         return true;
                     };
                     int32_t j = a.col_idx[w.e0];
@@ -356,7 +359,8 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
 #pragma unroll
                     for (int kk = 0; kk < D / 16; ++kk)
                         ptx::umma_ss_lohi(t_d, a_lo + (((kk / 4) * kRowTile + (kk % 4) * 32) >> 4), kDescHi,
-                                          b_lo + (((kk / 4) * kKeyTile + (kk % 4) * 32) >> 4), kDescHi, idesc_s, kk > 0 ? 1u : 0u);
+                                          b_lo + (((kk / 4) * kKeyTile + (kk % 4) * 32) >> 4), kDescHi, idesc_s,
+                                          kk > 0 ? 1u : 0u);
                     ptx::umma_commit(bar(out_full + (c & 3)));
                     if (is_dp) ptx::umma_commit(bar(C::V_EMPTY + st));
                     if (e == n - 1) ptx::umma_commit(bar(rows_empty + rb));  // this warp has read the item's Q (dO) tile
@@ -546,7 +550,8 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
                 __syncwarp();
 #pragma unroll
                 for (int x = 0; x < 8; ++x)
-                    ptx::st_shared_v4(patch + (uint32_t)((x ^ (lane & 7)) << 4), __float_as_uint(__uint_as_float(acc[4 * x]) * a.scale),
+                    ptx::st_shared_v4(patch + (uint32_t)((x ^ (lane & 7)) << 4),
+                                      __float_as_uint(__uint_as_float(acc[4 * x]) * a.scale),
                                       __float_as_uint(__uint_as_float(acc[4 * x + 1]) * a.scale),
                                       __float_as_uint(__uint_as_float(acc[4 * x + 2]) * a.scale),
                                       __float_as_uint(__uint_as_float(acc[4 * x + 3]) * a.scale));
@@ -718,8 +723,8 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 const BwdItem w = tail->items[r];
                 ptx::mbar_arrive(bar(C::ITEM_EMPTY + r));
                 if (w.n < 0) break;
-                auto load_rows = [&](uint32_t dst, const CUtensorMap *tm, uint32_t full, uint32_t empty, uint32_t stages, int32_t i,
-                                     int h0, int code) {
+                auto load_rows = [&](uint32_t dst, const CUtensorMap *tm, uint32_t full, uint32_t empty, uint32_t stages,
+                                     int32_t i, int h0, int code) {
                     const uint32_t st = c % stages;
                     if (c >= stages && !wait_bar(bar(empty + st), (c / stages - 1) & 1, code)) return false;
                     ptx::mbar_expect_tx(bar(full + st), C::kTile);
@@ -739,8 +744,10 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                             if (!ok) break;
                             ptx::mbar_expect_tx(bar(C::KV_FULL), 2 * C::kBlkTile);
                             for (int dh = 0; dh < DH; ++dh) {
-                                ptx::tma_load_4d(smem_base + C::kK + dh * kKeyTile, &tmK, bar(C::KV_FULL), dh * 64, w.blk * kBwdBlk, w.hk, w.b);
-                                ptx::tma_load_4d(smem_base + C::kV + dh * kKeyTile, &tmV, bar(C::KV_FULL), dh * 64, w.blk * kBwdBlk, w.hk, w.b);
+                                ptx::tma_load_4d(smem_base + C::kK + dh * kKeyTile, &tmK, bar(C::KV_FULL), dh * 64, w.blk * kBwdBlk,
+                                                 w.hk, w.b);
+                                ptx::tma_load_4d(smem_base + C::kV + dh * kKeyTile, &tmV, bar(C::KV_FULL), dh * 64, w.blk * kBwdBlk,
+                                                 w.hk, w.b);
                             }
                         }
                         ok = ok && load_rows(C::kG, &tmG, C::G_FULL, C::G_EMPTY, NG, i, h0, 35);
@@ -780,7 +787,8 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
 #pragma unroll
                     for (int kk = 0; kk < D / 16; ++kk)
                         ptx::umma_ss_lohi(t_d, a_lo + (((kk / 4) * kRowTile + (kk % 4) * 32) >> 4), kDescHi,
-                                          b_lo + (((kk / 4) * kKeyTile + (kk % 4) * 32) >> 4), kDescHi, idesc_s, kk > 0 ? 1u : 0u);
+                                          b_lo + (((kk / 4) * kKeyTile + (kk % 4) * 32) >> 4), kDescHi, idesc_s,
+                                          kk > 0 ? 1u : 0u);
                     ptx::umma_commit(bar(out_full + bf));
                     if (is_dp) ptx::umma_commit(bar(C::G_EMPTY + st));
                     if (e == n - 1) ptx::umma_commit(bar(C::KV_EMPTY));
@@ -959,9 +967,11 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         // Items: chunk slots in column order (the sink block's long column first); slots without work are passed over.
         // A column's listers are read by some ten columns.  Where Q and dO of all heads do not fit half of L2, one KV
         // head of one batch entry comes after the other, so that what is read again is still there; else a slot's heads
-        // come together, which leaves more of the last, short columns for the end.  Whole backward pass, heads together
-        // and one after the other: 57 MB of Q and dO (4K tokens, 28 heads) 163.9 and 164.9 us, 67 MB (2 x 8K, 16 heads of
-        // 64 features) 245 and 245, 470 MB (32K) 1665 and 1640 (this kernel's DRAM reads 2.4 and 1.7 GB).
+        // come together, which leaves more of the last, short columns for the end.  (L2 of an sm_100 GPU: 126 MB.)  Whole
+        // backward pass in us, heads together and one after the other, by MB of Q and dO: 54 to 67 MB equal but for
+        // what two runs differ by (4K tokens, 28 heads: 163.9 and 164.9; 2 x 8K, 16 heads of 64 features: 255 and 253),
+        // 117 (8K) 370 and 357, 235 (16K) 778 to 838 and 685 to 788, 268 (2 x 32K of 64 features) 1120 and 1096, 470
+        // (32K) 1665 and 1640 (this kernel's DRAM reads 2.4 and 1.7 GB).
         const bool by_head = (int64_t)a.batch * a.N * a.Hq * D * 4 > (int64_t)64 << 20;
         const uint32_t heads = (uint32_t)(a.Hkv * a.batch), slots = n_items / heads;
         uint32_t it = blockIdx.x;
@@ -1081,11 +1091,13 @@ static pa_status launch_tc(const BackwardArgs &a, const pa_prefill_params *p, in
     if (pa_status s = map_of(a.d_o, a.Hq, p->o, 2, "d_o", &tmG)) return s;
     if (pa_status s = map_of(a.k, a.Hkv, p->k, 1, "k", &tmK)) return s;
     if (pa_status s = map_of(a.v, a.Hkv, p->v, 1, "v", &tmV)) return s;
-    const TensorMapKey out = {a.dq, p->seq_len, (int64_t)a.Hq * D, D, (int64_t)a.N * a.Hq * D, device, D, a.Hq, p->batch, 1, 32, 1};
+    const int64_t dq_seq = (int64_t)a.Hq * D;
+    const TensorMapKey out = {a.dq, p->seq_len, dq_seq, D, a.N * dq_seq, device, D, a.Hq, p->batch, 1, 32, 1};
     if (pa_status s = get_tensor_map(out, "dq", &tmDq)) return s;
     if (device_once_begin(device, D == 128 ? ONCE_BACKWARD_TC_ATTR : ONCE_BACKWARD_TC_ATTR_64)) {
-        const cudaError_t e1 = cudaFuncSetAttribute(dq_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DqCfg<D>::kAlloc);
-        const cudaError_t e2 = cudaFuncSetAttribute(dkv_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DkvCfg<D>::kAlloc);
+        constexpr cudaFuncAttribute kSmem = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        const cudaError_t e1 = cudaFuncSetAttribute(dq_kernel<D>, kSmem, (int)DqCfg<D>::kAlloc);
+        const cudaError_t e2 = cudaFuncSetAttribute(dkv_kernel<D>, kSmem, (int)DkvCfg<D>::kAlloc);
         if (e1 != cudaSuccess || e2 != cudaSuccess) {
             device_once_reset(device, D == 128 ? ONCE_BACKWARD_TC_ATTR : ONCE_BACKWARD_TC_ATTR_64);
             return fail(PA_ERR_CUDA, "cudaFuncSetAttribute failed: %s", cudaGetErrorString(e1 != cudaSuccess ? e1 : e2));

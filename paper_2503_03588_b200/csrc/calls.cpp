@@ -164,7 +164,8 @@ PyObject *prefill_varlen(PyObject *const *x)
 {
     const at::Tensor &q = tensor(x[0]), &k = tensor(x[1]), &v = tensor(x[2]), &cu = tensor(x[3]), &row_ptr = tensor(x[5]),
                      &col_idx = tensor(x[6]);
-    expect(q.dim() == 3 && k.dim() == 3 && v.dim() == 3 && q.stride(2) == 1 && k.stride(2) == 1 && v.stride(2) == 1 && is_int32(cu),
+    expect(q.dim() == 3 && k.dim() == 3 && v.dim() == 3 && q.stride(2) == 1 && k.stride(2) == 1 && v.stride(2) == 1 &&
+               is_int32(cu),
            "expected [total, head, head_dim] tensors with contiguous head_dim and int32 cu_seqlens");
     const Out o(x[7], [&] { return make(q, q.sizes(), dtype(x[12])); });
     const Out lse(x[8], [&] { return make(q, {q.size(1), q.size(0)}, at::kFloat); });
@@ -256,8 +257,8 @@ pa_paged_params paged_params(int64_t batch, int64_t hq, int64_t hkv, int64_t d, 
 {
     const pa_strides sk = strides4(k), sv = strides4(v);
     expect(table.dim() == 2, "expected a block table [batch, max_blocks]");
-    return {(int32_t)batch, (int32_t)hq, (int32_t)hkv, (int32_t)d, block, window, sink, (int32_t)k.size(0), (int32_t)table.size(1),
-            scale, sk, sv, o_type};
+    return {(int32_t)batch, (int32_t)hq, (int32_t)hkv, (int32_t)d, block, window, sink, (int32_t)k.size(0),
+            (int32_t)table.size(1), scale, sk, sv, o_type};
 }
 
 // q, k_pool, v_pool, block_table, cache_lens, window_blocks, sink_blocks, o, lse, workspace, block, softmax_scale, o_dtype
@@ -268,7 +269,8 @@ PyObject *decode_paged(PyObject *const *x)
     const Out o(x[7], [&] { return make(q, q.sizes(), dtype(x[12])); });
     const Out lse(x[8], [&] { return make(q, {q.size(0), q.size(1)}, at::kFloat); });
     const int32_t block = integer32(x[10]);
-    expect(k.size(1) == block && is_int32(table) && table.is_contiguous(), "pages hold `block` tokens, the table is contiguous int32");
+    expect(k.size(1) == block && is_int32(table) && table.is_contiguous(),
+           "pages hold `block` tokens, the table is contiguous int32");
     const pa_paged_params p = paged_params(q.size(0), q.size(1), k.size(2), q.size(2), k, v, table, block, integer32(x[5]),
                                            integer32(x[6]), number(x[11]), out_dtype(o.t.scalar_type()));
     const Out ws(x[9], [&] { return make_bytes(q, pa_decode_paged_workspace_bytes(&p)); });
@@ -288,8 +290,8 @@ PyObject *kv_append(PyObject *const *x)
                      &lens = tensor(x[5]);
     expect(kn.dim() == 3 && kn.is_contiguous() && vn.is_contiguous() && is_int32(lens),
            "k_new and v_new [batch, head, head_dim] are contiguous, cache_lens is int32");
-    const pa_paged_params p = paged_params(kn.size(0), kn.size(1), kn.size(1), kn.size(2), k, v, table, integer32(x[6]), 0, 0, 0.f,
-                                           PA_BF16);
+    const pa_paged_params p = paged_params(kn.size(0), kn.size(1), kn.size(1), kn.size(2), k, v, table, integer32(x[6]), 0, 0,
+                                           0.f, PA_BF16);
     run([&] {
         return pa_kv_append(&p, kn.data_ptr(), vn.data_ptr(), k.data_ptr(), v.data_ptr(), (const int32_t *)table.data_ptr(),
                             (int32_t *)lens.data_ptr(), stream());

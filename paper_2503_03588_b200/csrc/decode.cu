@@ -334,7 +334,7 @@ constexpr int kRowMaxStages = 6;                     // shared-memory stages (ke
 constexpr int kRowMaxCluster = 8;                    // portable cluster size limit
 constexpr int kRowMaxSmem = 227 * 1024;              // dynamic shared memory a CTA may ask for
 constexpr long long kRowWaitCycles = 2000000000ll;   // default limit of a barrier wait: ~1 s
-enum : int32_t { kModeCluster = 0, kModePartial = 1, kModeDirect = 2 };
+enum : int32_t { kModeCluster = 0, kModePartial = 1 /* only under PA_DECODE_CLUSTER */, kModeDirect = 2 };
 
 template <int D>
 struct RowSmem {
@@ -614,7 +614,8 @@ __global__ void __launch_bounds__(kRowThreads, 2) decode_row_kernel(const __grid
                         keep0 = (key0 < n_keys ? 0x0000ffffu : 0u) | (key0 + 1 < n_keys ? 0xffff0000u : 0u);
                         keep1 = (key0 + 8 < n_keys ? 0x0000ffffu : 0u) | (key0 + 9 < n_keys ? 0xffff0000u : 0u);
                     }
-                    ok = ptx::mbar_wait_bounded(bar_vfull(s), parity, abort_flag, a.status, 3, a.wait_cycles, (int)PA_ERR_TIMEOUT);
+                    ok = ptx::mbar_wait_bounded(bar_vfull(s), parity, abort_flag, a.status, 3, a.wait_cycles,
+                                                (int)PA_ERR_TIMEOUT);
                     ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
                     // ---- O = alpha O + P V: rows = heads, 16 keys, all D features (8 per MMA)
@@ -854,7 +855,8 @@ kv_append_kernel(const __nv_bfloat16 *k_new, const __nv_bfloat16 *v_new, __nv_bf
         const bool is_v = x >= pieces;
         const int y = is_v ? x - pieces : x, hk = y / per_row, c = y % per_row;
         const uint4 piece = *reinterpret_cast<const uint4 *>((is_v ? v_new : k_new) + ((int64_t)b * Hkv + hk) * D + 8 * c);
-        __nv_bfloat16 *dst = is_v ? v_pool + page * v_sp + slot * v_ss + hk * v_sh : k_pool + page * k_sp + slot * k_ss + hk * k_sh;
+        __nv_bfloat16 *dst = is_v ? v_pool + page * v_sp + slot * v_ss + hk * v_sh
+                                  : k_pool + page * k_sp + slot * k_ss + hk * k_sh;
         *reinterpret_cast<uint4 *>(dst + 8 * c) = piece;
     }
     __syncthreads();

@@ -18,7 +18,7 @@ __global__ void __launch_bounds__(kLayoutThreads) layout_kernel(int32_t n_rows, 
     const int lane = threadIdx.x & 31;
     pdl_launch_next();
     const int64_t start = tile_rows_before(t, r, W, S, power);
-    pdl_wait();
+    pdl_wait();  // (nothing of global memory is touched before this)
     if (t > n_rows) return;
     if (lane == 0) row_ptr[t] = (int32_t)start;
     if (t == n_rows) return;

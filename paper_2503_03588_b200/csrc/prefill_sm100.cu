@@ -4,7 +4,8 @@
 // One persistent CTA per SM walks work units (batch, KV head, query block, head quad).  A unit
 // holds two 128-row tiles ("slots"); a tile stacks two query heads of the KV group on the 64
 // tokens of the query block (the mask does not depend on the head, so they share the key list
-// and the K/V tiles).  (Groups of one or two query heads have one slot.)  The key list is walked one 64-key block per step.  Warp roles:
+// and the K/V tiles).  (Groups of one or two query heads have one slot.)  The key list is walked one
+// 64-key block per step.  Warp roles:
 //   warp 0      TMA producer: the listed K and V blocks, gathered by block index, into two rings
 //               of shared-memory tiles (128-byte swizzle); the next unit's Q tiles early in
 //               the current unit, into the second of two Q buffers
@@ -66,7 +67,7 @@ struct PrefillArgs {
     int64_t o_sb, o_ss, o_sh;
     int64_t lse_sb, lse_sh;  // LSE strides (batch, head); the token stride is 1
     int64_t N, n_units;     // N: sequence length (variable-length batch: the longest one, which sizes the unit grid)
-    int32_t nqb, batch, Hq, Hkv, G, nsub, o_is_f32;
+    int32_t nqb, batch, Hq, Hkv, G, nsub;
     uint32_t inv_nsub, inv_Hkv, inv_nqb;  // floor(2^32 / d) of the three divisors of a unit index
     float scale_log2;
     long long wait_cycles;  // limit of every barrier wait, in clock cycles
@@ -267,7 +268,8 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             auto load_q = [&](const Unit &w, uint32_t ul_q) {
                 const uint32_t qb = ul_q & 1;
                 if (ul_q >= 2 && !wait_bar(bar(BAR_Q_EMPTY + qb), ((ul_q >> 1) - 1) & 1, abort_flag, a.status, 1)) return false;
-                if (ul_q >= 2 && !wait_bar(bar(BAR_STAGE_FREE + qb), ((ul_q >> 1) - 1) & 1, abort_flag, a.status, 16)) return false;
+                if (ul_q >= 2 && !wait_bar(bar(BAR_STAGE_FREE + qb), ((ul_q >> 1) - 1) & 1, abort_flag, a.status, 16))
+                    return false;
                 ptx::mbar_expect_tx(bar(BAR_Q_FULL + qb), kSlots * SM::kQSlot);
                 for (int s = 0; s < kSlots; ++s)
                     for (int dh = 0; dh < DH; ++dh)
@@ -387,7 +389,8 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             bool ok = true;
             // S(c1) of this slot; `first` / `final`: c1 is the first / last step of unit number ul1.
             auto qk_step = [&](uint32_t c1, uint32_t ul1, bool first, bool final, bool wait_taken) {
-                if (first) ok = __all_sync(0xffffffffu, wait_bar(bar(BAR_Q_FULL + (ul1 & 1)), (ul1 >> 1) & 1, abort_flag, a.status, 4));
+                if (first)
+                    ok = __all_sync(0xffffffffu, wait_bar(bar(BAR_Q_FULL + (ul1 & 1)), (ul1 >> 1) & 1, abort_flag, a.status, 4));
                 if (ok)
                     ok = __all_sync(0xffffffffu, wait_bar(bar(BAR_K_FULL + c1 % kKStages), (c1 / kKStages) & 1,
                                                           abort_flag, a.status, 5));
@@ -408,7 +411,8 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 ok = __all_sync(0xffffffffu, wait_bar(bar(BAR_V_FULL + c % kVStages), (c / kVStages) & 1,
                                                       abort_flag, a.status, 6));
                 if (ok)
-                    ok = __all_sync(0xffffffffu, wait_bar(bar(BAR_P_FULL + 2 * s + (c & 1)), (c >> 1) & 1, abort_flag, a.status, 7));
+                    ok = wait_bar(bar(BAR_P_FULL + 2 * s + (c & 1)), (c >> 1) & 1, abort_flag, a.status, 7);
+                    ok = __all_sync(0xffffffffu, ok);
                 // The previous unit's O must have left tensor memory.
                 if (ok && t == 0 && ul > 0)
                     ok = __all_sync(0xffffffffu, wait_bar(bar(BAR_O_FREE + s), (ul - 1) & 1, abort_flag, a.status, 14));
@@ -439,7 +443,9 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                         // Unit boundary: the next unit's first S goes first if its Q tile has
                         // arrived (normally long ago), else behind this unit's last P V, for which
                         // the epilogue waits.
-                        const bool q_here = has_next && __all_sync(0xffffffffu, ptx::mbar_test_wait(bar(BAR_Q_FULL + ((ul + 1) & 1)), ((ul + 1) >> 1) & 1));
+                        const uint32_t q_next = ul + 1;
+                        const bool q_here = has_next && __all_sync(0xffffffffu, ptx::mbar_test_wait(
+                                                            bar(BAR_Q_FULL + (q_next & 1)), (q_next >> 1) & 1));
                         if (q_here) qk_step(c + 1, ul + 1, true, nn == 1, true);
                         if (ok) pv_step(c, ul, t, n);
                         if (ok && has_next && !q_here) qk_step(c + 1, ul + 1, true, nn == 1, true);
@@ -483,7 +489,8 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             lastcol_next = fetch_lastcol(w_next);
             w_next2 = fetch_unit(u + 2 * gridDim.x);
         };
-        for (uint32_t u = kSlots == 2 || s == 0 ? blockIdx.x : (uint32_t)a.n_units; u < (uint32_t)a.n_units && ok; u += gridDim.x) {
+        const uint32_t n_units = (uint32_t)a.n_units;
+        for (uint32_t u = kSlots == 2 || s == 0 ? blockIdx.x : n_units; u < n_units && ok; u += gridDim.x) {
             const Unit w = w_next;
             const int32_t lastcol = lastcol_next;
             const int head_local = w.sub * 4 + 2 * s + (row >> 6);
@@ -747,7 +754,8 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                                 uint32_t v[4];
 #pragma unroll
                                 for (int e = 0; e < 4; ++e) v[e] = __float_as_uint(__uint_as_float(orr[4 * c + e]) * inv);
-                                ptx::st_shared_v4(rbase + (uint32_t)k * 8192u + ((uint32_t)(c ^ (qrow & 7)) << 4), v[0], v[1], v[2], v[3]);
+                                ptx::st_shared_v4(rbase + (uint32_t)k * 8192u + ((uint32_t)(c ^ (qrow & 7)) << 4), v[0], v[1], v[2],
+                                                  v[3]);
                                 if (ragged && valid)
                                     *reinterpret_cast<uint4 *>(reinterpret_cast<float *>(a.o) + obase + ch * 32 + 4 * c) =
                                         make_uint4(v[0], v[1], v[2], v[3]);
@@ -957,7 +965,8 @@ static pa_status launch_prefill(const pa_prefill_params *p, const void *q, const
     // boxes one head.
     CUtensorMap tmQ, tmK, tmV, tmO;
     const int D = p->head_dim;
-    auto map_of = [&](const void *base, int heads, const pa_strides &st, int box_heads, const char *what, CUtensorMap *m, bool f32 = false) {
+    auto map_of = [&](const void *base, int heads, const pa_strides &st, int box_heads, const char *what, CUtensorMap *m,
+                      bool f32 = false) {
         // (packed sequences: one "batch" entry of total_tokens tokens)
         const TensorMapKey key = {base, varlen ? total_tokens : p->seq_len, st.seq, st.head, varlen ? 0 : st.batch, dev.device, D,
                                   heads, varlen ? 1 : p->batch, box_heads, kBlk, f32 ? 1 : 0};
@@ -988,7 +997,6 @@ static pa_status launch_prefill(const pa_prefill_params *p, const void *q, const
     auto inv32 = [](int32_t d) { return d == 1 ? 0xffffffffu : (uint32_t)((1ull << 32) / (uint64_t)d); };
     a.inv_nsub = inv32(a.nsub); a.inv_Hkv = inv32(a.Hkv); a.inv_nqb = inv32(a.nqb);
     if (a.n_units > (int64_t)0x3fffffff) return fail(PA_ERR_SHAPE, "too many work units (%lld)", (long long)a.n_units);
-    a.o_is_f32 = p->o_dtype == PA_F32;
     const float scale = p->softmax_scale != 0.f ? p->softmax_scale : 1.0f / sqrtf((float)D);
     a.scale_log2 = scale * 1.4426950408889634f;
 
@@ -1023,7 +1031,7 @@ static pa_status launch_prefill(const pa_prefill_params *p, const void *q, const
     // 11.4, 32K tokens, 8 heads of 128 features 266 us instead of 355; with two heads per group 8K tokens, batch 2,
     // 8 KV heads 118 us instead of 156 (burst).  Three heads need the second slot.
     auto launch = [&](auto kernel) { return kernel(grid, st, dev.device, tmQ, tmK, tmV, tmO, a); };
-    if (a.o_is_f32) {
+    if (p->o_dtype == PA_F32) {
         if (a.G > 2) return launch(D == 128 ? launch_kernel<128, 2, true> : launch_kernel<64, 2, true>);
         return launch(D == 128 ? launch_kernel<128, 1, true> : launch_kernel<64, 1, true>);
     }
