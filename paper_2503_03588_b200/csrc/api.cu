@@ -166,9 +166,15 @@ pa_status get_tensor_map(const TensorMapKey &key, const char *what, CUtensorMap 
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     CUtensorMap m;
     const CUtensorMapDataType type = key.f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
-    const CUresult r = g_encode(&m, type, 4, const_cast<void *>(key.base), dims, strides, box, estr,
-                                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    auto encode = [&] {
+        return g_encode(&m, type, 4, const_cast<void *>(key.base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                        CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    };
+    CUresult r = encode();
+    if (r == CUDA_ERROR_INVALID_CONTEXT) {  // a thread's first CUDA call: the driver has no context for it yet
+        PA_CUDA_OK(cudaSetDevice(key.device));
+        r = encode();
+    }
     if (r != CUDA_SUCCESS)
         return fail(PA_ERR_CUDA, "cuTensorMapEncodeTiled failed for %s (CUresult %d)", what, (int)r);
     MapEntry &e = g_maps[g_map_next];

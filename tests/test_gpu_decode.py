@@ -367,3 +367,36 @@ def test_decode_of_caches_of_one_block(pa, oracle, rows):
     q = si.bf16_randn((rows, 7, 128), 1860)
     kc, vc = si.bf16_randn((rows, 64, 1, 128), 1861), si.bf16_randn((rows, 64, 1, 128), 1862)
     _run(pa, oracle, q, kc, vc, np.random.default_rng(1863).integers(1, 65, size=rows), 5, 1)
+
+
+def test_first_calls_from_several_threads(pa):
+    """The one-time set-up of a kernel is done before another thread's call launches it (a process of its own, so that
+    the calls are its first ones)."""
+    import os
+    import subprocess
+    import sys
+
+    program = """
+import threading
+import torch
+import paper_2503_03588_b200 as pa
+q, kc = torch.ones((2, 8, 128), device="cuda").bfloat16(), torch.ones((2, 2048, 2, 128), device="cuda").bfloat16()
+p, lens = kc[:, :, :1].repeat(1, 1, 4, 1), torch.full((2,), 2048, dtype=torch.int32, device="cuda")
+rp, ci = pa.pa_build_layout(2048, 64, 5, 1)
+torch.cuda.synchronize()
+start, errors = threading.Barrier(16), []
+def work(i):
+    try:
+        start.wait()
+        o, lse, ws = pa.pa_decode(q, kc, kc, lens, 5, 1) if i % 2 else pa.pa_prefill(p, p, p, rp, ci)
+        torch.cuda.synchronize()
+        assert (o == 1).all() and pa.pa_decode_status(ws) == 0
+    except Exception as e:
+        errors.append(e)
+threads = [threading.Thread(target=work, args=(i,)) for i in range(16)]
+[t.start() for t in threads]
+[t.join() for t in threads]
+assert not errors, errors
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    subprocess.run([sys.executable, "-c", program], check=True, cwd=root, timeout=300)
