@@ -26,7 +26,7 @@ pa_status fail(pa_status s, const char *fmt, ...)
 
 void clear_error() { g_err[0] = '\0'; }
 
-static std::mutex g_mu;  // guards every cache below
+static std::mutex g_mu;  // guards the caches below (g_once: device_once_mutex)
 
 // ---------------------------------------------------------------- devices
 static DeviceInfo g_dev[kMaxDevices];
@@ -65,19 +65,13 @@ pa_status current_sm100_device(DeviceInfo *out)
     return PA_OK;
 }
 
-bool device_once_begin(int device, DeviceOnce slot)
+std::mutex &device_once_mutex()
 {
-    std::lock_guard<std::mutex> lock(g_mu);
-    if (g_once[device][slot]) return false;
-    g_once[device][slot] = true;
-    return true;
+    static std::mutex mu;
+    return mu;
 }
 
-void device_once_reset(int device, DeviceOnce slot)
-{
-    std::lock_guard<std::mutex> lock(g_mu);
-    g_once[device][slot] = false;
-}
+bool &device_once_done(int device, DeviceOnce slot) { return g_once[device][slot]; }
 
 // ---------------------------------------------------------------- environment
 static EnvSwitches g_env;

@@ -519,18 +519,14 @@ static pa_status launch_backward(const BackwardArgs &a, const pa_prefill_params 
                                  bool mma, cudaStream_t st)
 {
     constexpr int kSmemDq = 4 * BwdTile<D>::kBytes, kSmemDkv = 4 * BwdTile<D>::kBytes + 2 * kBwdBlk * 4;
-    if (device_once_begin(device, D == 128 ? ONCE_BACKWARD_ATTR : ONCE_BACKWARD_ATTR_64)) {
-        constexpr cudaFuncAttribute kSmem = cudaFuncAttributeMaxDynamicSharedMemorySize;
-        const cudaError_t e1 = cudaFuncSetAttribute(backward_dq_kernel<D>, kSmem, kSmemDq);
-        const cudaError_t e2 = cudaFuncSetAttribute(backward_dkv_kernel<D>, kSmem, kSmemDkv);
-        // (a bitmap row of more than the 32 KB aimed at is needed from 16 million tokens on)
-        const cudaError_t e3 = cudaFuncSetAttribute(backward_prep_kernel<D>, kSmem, kPrepMaxBitmap);
-        if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess) {
-            device_once_reset(device, D == 128 ? ONCE_BACKWARD_ATTR : ONCE_BACKWARD_ATTR_64);
-            return fail(PA_ERR_CUDA, "cudaFuncSetAttribute failed: %s",
-                        cudaGetErrorString(e1 != cudaSuccess ? e1 : e2 != cudaSuccess ? e2 : e3));
-        }
-    }
+    if (pa_status s = device_once(device, D == 128 ? ONCE_BACKWARD_ATTR : ONCE_BACKWARD_ATTR_64, [] {
+            constexpr cudaFuncAttribute kSmem = cudaFuncAttributeMaxDynamicSharedMemorySize;
+            // (a bitmap row of more than the 32 KB aimed at is needed from 16 million tokens on)
+            const cudaError_t e = cudaFuncSetAttribute(backward_prep_kernel<D>, kSmem, kPrepMaxBitmap);
+            return first_error(e, first_error(cudaFuncSetAttribute(backward_dq_kernel<D>, kSmem, kSmemDq),
+                                              cudaFuncSetAttribute(backward_dkv_kernel<D>, kSmem, kSmemDkv)));
+        }))
+        return s;
     const int32_t cols = prep_cols_per_block(a.nqb), n_csc = (a.nqb + cols - 1) / cols;
     const int64_t groups = (int64_t)a.batch * ((a.N + kPrepTokens - 1) / kPrepTokens);
     const int32_t bitmap_cols = cols < a.nqb ? cols : a.nqb;

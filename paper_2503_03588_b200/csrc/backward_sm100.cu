@@ -1094,15 +1094,12 @@ static pa_status launch_tc(const BackwardArgs &a, const pa_prefill_params *p, in
     const int64_t dq_seq = (int64_t)a.Hq * D;
     const TensorMapKey out = {a.dq, p->seq_len, dq_seq, D, a.N * dq_seq, device, D, a.Hq, p->batch, 1, 32, 1};
     if (pa_status s = get_tensor_map(out, "dq", &tmDq)) return s;
-    if (device_once_begin(device, D == 128 ? ONCE_BACKWARD_TC_ATTR : ONCE_BACKWARD_TC_ATTR_64)) {
-        constexpr cudaFuncAttribute kSmem = cudaFuncAttributeMaxDynamicSharedMemorySize;
-        const cudaError_t e1 = cudaFuncSetAttribute(dq_kernel<D>, kSmem, (int)DqCfg<D>::kAlloc);
-        const cudaError_t e2 = cudaFuncSetAttribute(dkv_kernel<D>, kSmem, (int)DkvCfg<D>::kAlloc);
-        if (e1 != cudaSuccess || e2 != cudaSuccess) {
-            device_once_reset(device, D == 128 ? ONCE_BACKWARD_TC_ATTR : ONCE_BACKWARD_TC_ATTR_64);
-            return fail(PA_ERR_CUDA, "cudaFuncSetAttribute failed: %s", cudaGetErrorString(e1 != cudaSuccess ? e1 : e2));
-        }
-    }
+    if (pa_status s = device_once(device, D == 128 ? ONCE_BACKWARD_TC_ATTR : ONCE_BACKWARD_TC_ATTR_64, [] {
+            constexpr cudaFuncAttribute kSmem = cudaFuncAttributeMaxDynamicSharedMemorySize;
+            return first_error(cudaFuncSetAttribute(dq_kernel<D>, kSmem, (int)DqCfg<D>::kAlloc),
+                               cudaFuncSetAttribute(dkv_kernel<D>, kSmem, (int)DkvCfg<D>::kAlloc));
+        }))
+        return s;
     const int64_t dq_items = (int64_t)a.nqb * a.Hkv * a.npairs * a.batch;
     const int64_t dkv_items = (nnz / a.chunk + a.nqb) * a.Hkv * a.batch;  // (chunk slots, some of them empty)
     if (dq_items > (int64_t)0x3fffffff || dkv_items > (int64_t)0x3fffffff)

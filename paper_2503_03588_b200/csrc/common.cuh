@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
+
 #include "powerattn.h"
 
 namespace pa {
@@ -32,10 +34,22 @@ enum DeviceOnce : int {
     ONCE_BACKWARD_ATTR, ONCE_BACKWARD_ATTR_64, ONCE_BACKWARD_TC_ATTR, ONCE_BACKWARD_TC_ATTR_64,
     ONCE_COUNT
 };
-// True exactly once per (device, slot); the caller then performs the step and, if it fails, calls
-// device_once_reset so that a later call tries again.
-bool device_once_begin(int device, DeviceOnce slot);
-void device_once_reset(int device, DeviceOnce slot);
+std::mutex &device_once_mutex();
+bool &device_once_done(int device, DeviceOnce slot);
+// Performs the step, a cudaError_t(), once per (device, slot); a step that fails is tried again by the next call.
+// Another thread's call goes on only when the step is done.
+template <typename Step>
+pa_status device_once(int device, DeviceOnce slot, Step step)
+{
+    std::lock_guard<std::mutex> lock(device_once_mutex());
+    bool &done = device_once_done(device, slot);
+    if (done) return PA_OK;
+    const cudaError_t e = step();
+    if (e != cudaSuccess) return fail(PA_ERR_CUDA, "cudaFuncSetAttribute failed: %s", cudaGetErrorString(e));
+    done = true;
+    return PA_OK;
+}
+inline cudaError_t first_error(cudaError_t a, cudaError_t b) { return a != cudaSuccess ? a : b; }
 
 // Environment switches (for tests and measurements).  They are read when the library first needs
 // them and again on pa_reload_environment().

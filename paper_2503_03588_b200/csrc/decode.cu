@@ -1072,17 +1072,12 @@ static pa_status launch_decode(const DecodeShape &p, const void *q, const void *
             while (n > 1 && row_smem_bytes(p.head_dim, n, cluster_form) > (size_t)kRowMaxSmem) --n;
             return n;
         };
-        if (device_once_begin(dev.device, ONCE_DECODE_ATTR)) {
-            const cudaError_t e1 = cudaFuncSetAttribute(decode_row_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                        kRowMaxSmem);
-            const cudaError_t e2 = cudaFuncSetAttribute(decode_row_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                        kRowMaxSmem);
-            if (e1 != cudaSuccess || e2 != cudaSuccess) {
-                device_once_reset(dev.device, ONCE_DECODE_ATTR);
-                return fail(PA_ERR_CUDA, "cudaFuncSetAttribute failed: %s",
-                            cudaGetErrorString(e1 != cudaSuccess ? e1 : e2));
-            }
-        }
+        if (pa_status s = device_once(dev.device, ONCE_DECODE_ATTR, [] {
+                constexpr cudaFuncAttribute kSmem = cudaFuncAttributeMaxDynamicSharedMemorySize;
+                return first_error(cudaFuncSetAttribute(decode_row_kernel<128>, kSmem, kRowMaxSmem),
+                                   cudaFuncSetAttribute(decode_row_kernel<64>, kSmem, kRowMaxSmem));
+            }))
+            return s;
         // Small calls (latency-bound): a cluster of R CTAs per row, all resident at once.  Larger calls
         // (bandwidth-bound): a persistent grid of two CTAs per SM over the rows.  The line lies where a row
         // still gets two of the resident CTAs: rows of 18 blocks (30000 tokens, G = 7, head_dim 128) take

@@ -927,14 +927,11 @@ static pa_status launch_kernel(unsigned grid, cudaStream_t st, int device, const
                                const CUtensorMap &tmV, const CUtensorMap &tmO, const PrefillArgs &a)
 {
     constexpr DeviceOnce once = (DeviceOnce)(ONCE_PREFILL_ATTR + 4 * (D == 64) + 2 * (kSlots == 1) + kF32);
-    if (device_once_begin(device, once)) {
-        const cudaError_t e = cudaFuncSetAttribute(prefill_kernel<D, kSlots, kF32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)SmemMap<D>::kAlloc);
-        if (e != cudaSuccess) {
-            device_once_reset(device, once);
-            return fail(PA_ERR_CUDA, "cudaFuncSetAttribute failed: %s", cudaGetErrorString(e));
-        }
-    }
+    if (pa_status s = device_once(device, once, [] {
+            return cudaFuncSetAttribute(prefill_kernel<D, kSlots, kF32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)SmemMap<D>::kAlloc);
+        }))
+        return s;
     PA_CUDA_OK(launch_pdl(prefill_kernel<D, kSlots, kF32>, dim3(grid), kThreads, SmemMap<D>::kAlloc, st, tmQ, tmK, tmV, tmO, a));
     return PA_OK;
 }
