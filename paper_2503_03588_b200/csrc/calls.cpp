@@ -14,6 +14,7 @@
 #include <torch/csrc/Dtype.h>
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
+#include <torch/csrc/utils/device_lazy_init.h>
 
 #include "powerattn.h"
 
@@ -76,9 +77,11 @@ struct WithoutGil {
     ~WithoutGil() { PyEval_RestoreThread(state); }
 };
 
-// (An allocation may wait for the device or another thread: without the interpreter lock, like torch's own.)
+// As torch.empty: the device's Python side is set up first, and the allocation, which may wait for the device or another
+// thread, goes without the interpreter lock.
 at::Tensor empty(at::IntArrayRef size, const at::TensorOptions &options)
 {
+    torch::utils::maybe_initialize_device(options);
     const WithoutGil released;
     return at::empty(size, options);
 }

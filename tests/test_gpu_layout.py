@@ -96,3 +96,21 @@ def test_window_layout_bit_exact(pa, oracle):
     rp, ci = pa.pa_build_window_layout(128 * 256, 256, 9, 1)
     assert (ci[int(rp[-2]):].cpu().numpy() + 1).tolist() == [1, 120, 121, 122, 123, 124, 125, 126, 127, 128]
     assert pa.pa_reach_counts(rp.cpu().numpy(), ci.cpu().numpy(), 127, 1) == [10]
+
+
+def test_a_process_whose_first_cuda_call_is_a_layout(pa):
+    """torch's CUDA state is set up on the way, as by torch's own functions (what was asked of it before, such as a
+    seed, then holds, and forked children are told)."""
+    import os
+    import subprocess
+    import sys
+
+    program = """
+import torch
+import paper_2503_03588_b200 as pa
+torch.cuda.manual_seed(5)
+row_ptr, _ = pa.pa_build_layout(1000, 64, 5, 1)
+assert torch.cuda.is_initialized() and torch.cuda.initial_seed() == 5 and int(row_ptr[-1]) == 88
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    subprocess.run([sys.executable, "-c", program], check=True, cwd=root, timeout=300)
