@@ -130,7 +130,7 @@ static bool same_key(const TensorMapKey &a, const TensorMapKey &b)
     return a.base == b.base && a.seq == b.seq && a.stride_seq == b.stride_seq && a.stride_head == b.stride_head &&
            a.stride_batch == b.stride_batch && a.device == b.device && a.head_dim == b.head_dim &&
            a.heads == b.heads && a.batch == b.batch && a.box_heads == b.box_heads && a.box_tokens == b.box_tokens &&
-           a.f32 == b.f32;
+           a.f32 == b.f32 && a.group == b.group;
 }
 
 pa_status get_tensor_map(const TensorMapKey &key, const char *what, CUtensorMap *out)
@@ -149,19 +149,24 @@ pa_status get_tensor_map(const TensorMapKey &key, const char *what, CUtensorMap 
             return fail(PA_ERR_CUDA, "cuTensorMapEncodeTiled is not available from this driver");
         g_encode = reinterpret_cast<EncodeTiledFn>(fn);
     }
-    const cuuint64_t dims[4] = {(cuuint64_t)key.head_dim, (cuuint64_t)key.seq, (cuuint64_t)key.heads,
-                                (cuuint64_t)key.batch};
+    // Feature, token, head (or head in the group, group), batch.
+    const int rank = key.group > 0 ? 5 : 4;
+    const cuuint64_t group = (cuuint64_t)(key.group > 0 ? key.group : key.heads);
+    const cuuint64_t batch = (cuuint64_t)key.batch;
+    const cuuint64_t dims[5] = {(cuuint64_t)key.head_dim, (cuuint64_t)key.seq, group,
+                                rank == 5 ? (cuuint64_t)key.heads / group : batch, batch};
     const cuuint64_t size = key.f32 ? 4 : 2;
     // (A batch stride of 0 is an expanded tensor, one sequence that every batch entry reads, and goes into the map as
     // it is; with a single entry the stride is never used and only has to be a valid one.)
-    const cuuint64_t strides[3] = {(cuuint64_t)key.stride_seq * size, (cuuint64_t)key.stride_head * size,
-                                   (cuuint64_t)(key.batch > 1 ? key.stride_batch : key.stride_seq * key.seq) * size};
-    const cuuint32_t box[4] = {(cuuint32_t)(128 / size), (cuuint32_t)key.box_tokens, (cuuint32_t)key.box_heads, 1};
-    const cuuint32_t estr[4] = {1, 1, 1, 1};
+    const cuuint64_t stride_batch = (cuuint64_t)(key.batch > 1 ? key.stride_batch : key.stride_seq * key.seq) * size;
+    const cuuint64_t strides[4] = {(cuuint64_t)key.stride_seq * size, (cuuint64_t)key.stride_head * size,
+                                   rank == 5 ? (cuuint64_t)key.stride_head * group * size : stride_batch, stride_batch};
+    const cuuint32_t box[5] = {(cuuint32_t)(128 / size), (cuuint32_t)key.box_tokens, (cuuint32_t)key.box_heads, 1, 1};
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
     CUtensorMap m;
     const CUtensorMapDataType type = key.f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
     auto encode = [&] {
-        return g_encode(&m, type, 4, const_cast<void *>(key.base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+        return g_encode(&m, type, (cuuint32_t)rank, const_cast<void *>(key.base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                         CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     };
     CUresult r = encode();

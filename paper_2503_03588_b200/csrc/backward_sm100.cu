@@ -286,14 +286,13 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
                 ok = publish(k + 1, wn);
                 if (!ok) break;
                 if (w.n > 0) {
-                    const int h0 = w.hk * a.G + 2 * w.hp;
                     auto load_rows = [&](uint32_t dst, const CUtensorMap *tm, uint32_t full, uint32_t empty, int code) {
                         const uint32_t rb = kq % NR;
                         if (kq >= NR && !wait_bar(bar(empty + rb), (kq / NR - 1) & 1, code)) return false;
                         ptx::mbar_expect_tx(bar(full + rb), C::kTile);
                         for (int dh = 0; dh < DH; ++dh)
-                            ptx::tma_load_4d(smem_base + dst + rb * 2 * C::kTile + dh * kRowTile, tm, bar(full + rb), dh * 64,
-                                             w.blk * kBwdBlk, h0, w.b);
+                            ptx::tma_load_5d(smem_base + dst + rb * 2 * C::kTile + dh * kRowTile, tm, bar(full + rb), dh * 64,
+                                             w.blk * kBwdBlk, 2 * w.hp, w.hk, w.b);
                         return true;
                     };
                     auto load_block = [&](uint32_t base, const CUtensorMap *tm, uint32_t full, uint32_t empty, uint32_t stages,
@@ -724,21 +723,20 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 ptx::mbar_arrive(bar(C::ITEM_EMPTY + r));
                 if (w.n < 0) break;
                 auto load_rows = [&](uint32_t dst, const CUtensorMap *tm, uint32_t full, uint32_t empty, uint32_t stages,
-                                     int32_t i, int h0, int code) {
+                                     int32_t i, int hp, int code) {
                     const uint32_t st = c % stages;
                     if (c >= stages && !wait_bar(bar(empty + st), (c / stages - 1) & 1, code)) return false;
                     ptx::mbar_expect_tx(bar(full + st), C::kTile);
                     for (int dh = 0; dh < DH; ++dh)
-                        ptx::tma_load_4d(smem_base + dst + st * C::kPitch + dh * kRowTile, tm, bar(full + st), dh * 64,
-                                         i * kBwdBlk, h0, w.b);
+                        ptx::tma_load_5d(smem_base + dst + st * C::kPitch + dh * kRowTile, tm, bar(full + st), dh * 64,
+                                         i * kBwdBlk, 2 * hp, w.hk, w.b);
                     return true;
                 };
                 int32_t i = w.first;
                 for (int x = 0; x < w.n && ok; ++x) {
                     const int32_t in = x + 1 < w.n ? a.row_idx[w.e0 + x + 1] : 0;
                     for (int hp = 0; hp < a.npairs && ok; ++hp, ++c) {
-                        const int h0 = w.hk * a.G + 2 * hp;
-                        ok = load_rows(C::kQ, &tmQ, C::Q_FULL, C::Q_EMPTY, NQ, i, h0, 33);
+                        ok = load_rows(C::kQ, &tmQ, C::Q_FULL, C::Q_EMPTY, NQ, i, hp, 33);
                         if (ok && x == 0 && hp == 0) {
                             ok = k == 0 || wait_bar(bar(C::KV_EMPTY), (k - 1) & 1, 34);
                             if (!ok) break;
@@ -750,7 +748,7 @@ dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                                                  w.hk, w.b);
                             }
                         }
-                        ok = ok && load_rows(C::kG, &tmG, C::G_FULL, C::G_EMPTY, NG, i, h0, 35);
+                        ok = ok && load_rows(C::kG, &tmG, C::G_FULL, C::G_EMPTY, NG, i, hp, 35);
                     }
                     i = in;
                 }
@@ -1082,15 +1080,19 @@ template <int D>
 static pa_status launch_tc(const BackwardArgs &a, const pa_prefill_params *p, int64_t nnz, int device, int sms, cudaStream_t st)
 {
     // Tensor maps (cached per buffer and shape): a Q or dO box holds the two heads of a tile, a K or V box one head.
+    // The last tile of a group with an odd number of heads gets zeros for the second: both products of a tile sum over its
+    // rows, so that whatever another group's head holds there (infinities, NaN) would reach this group's dK and dV.
     CUtensorMap tmQ, tmG, tmK, tmV, tmDq;
-    auto map_of = [&](const void *base, int heads, const pa_strides &s, int box_heads, const char *what, CUtensorMap *m) {
-        const TensorMapKey key = {base, p->seq_len, s.seq, s.head, s.batch, device, D, heads, p->batch, box_heads, kBwdBlk, 0};
+    auto map_of = [&](const void *base, int heads, const pa_strides &s, int box_heads, int group, const char *what,
+                      CUtensorMap *m) {
+        const TensorMapKey key = {base,  p->seq_len, s.seq,     s.head,  s.batch, device, D,
+                                  heads, p->batch,   box_heads, kBwdBlk, 0,       group};
         return get_tensor_map(key, what, m);
     };
-    if (pa_status s = map_of(a.q, a.Hq, p->q, 2, "q", &tmQ)) return s;
-    if (pa_status s = map_of(a.d_o, a.Hq, p->o, 2, "d_o", &tmG)) return s;
-    if (pa_status s = map_of(a.k, a.Hkv, p->k, 1, "k", &tmK)) return s;
-    if (pa_status s = map_of(a.v, a.Hkv, p->v, 1, "v", &tmV)) return s;
+    if (pa_status s = map_of(a.q, a.Hq, p->q, 2, a.G, "q", &tmQ)) return s;
+    if (pa_status s = map_of(a.d_o, a.Hq, p->o, 2, a.G, "d_o", &tmG)) return s;
+    if (pa_status s = map_of(a.k, a.Hkv, p->k, 1, 0, "k", &tmK)) return s;
+    if (pa_status s = map_of(a.v, a.Hkv, p->v, 1, 0, "v", &tmV)) return s;
     const int64_t dq_seq = (int64_t)a.Hq * D;
     const TensorMapKey out = {a.dq, p->seq_len, dq_seq, D, a.N * dq_seq, device, D, a.Hq, p->batch, 1, 32, 1};
     if (pa_status s = get_tensor_map(out, "dq", &tmDq)) return s;

@@ -19,6 +19,9 @@ struct TensorMapKey {
     int64_t seq, stride_seq, stride_head, stride_batch;
     int32_t device, head_dim, heads, batch, box_heads, box_tokens;
     int32_t f32;  // fp32 elements, 32 (not 64) of them per box row
+    // Heads per group, or 0.  With groups the head dimension is two, head in the group and group: a box that reaches
+    // beyond its group's heads is filled with zeros there instead of with the next group's.
+    int32_t group;
 };
 
 // Encoded map for `key` (from the cache, or encoded now and cached).  Thread-safe.

@@ -332,3 +332,21 @@ def test_backward_with_chunks_of_full_size(pa, oracle, D):
     two = [x[1:2, :, 30:32].cpu().contiguous() for x in (Q, K, V, dO)]
     for g, r, n in zip((dq, dk, dv), oracle.backward(*two, 64, 5, 1, dense=dense), ("dQ", "dK", "dV")):
         _compare(g[1:2, :, 30:32], r, n + " full chunks")
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_backward_of_a_group_beside_one_that_is_not_finite(pa, D, bad):
+    """Groups of three heads: the second tile of a group has room for a head that is not there, next to which the
+    next group's first head lies in memory.  What that one holds changes nothing in this group's gradients."""
+    N, Hq, Hkv = 500, 6, 2
+    Q, K, V, dO = (si.bf16_randn((1, N, h, D), 1950 + x).cuda() for x, h in enumerate((Hq, Hkv, Hkv, Hq)))
+    rp, ci = pa.pa_build_layout(N, 64, 5, 1)
+    o, lse, _ = pa.pa_prefill(Q, K, V, rp, ci)
+    clean = pa.pa_prefill_backward(Q, K, V, o, lse, dO, rp, ci)[:3]
+    Q[:, :, 3:], dO[:, :, 3:] = bad, bad
+    dq, dk, dv, ws = pa.pa_prefill_backward(Q, K, V, o, lse, dO, rp, ci)
+    pa.pa_prefill_status(ws)
+    assert torch.equal(dq[:, :, :3], clean[0][:, :, :3])
+    for got, ref in ((dk, clean[1]), (dv, clean[2])):
+        assert torch.allclose(got[:, :, 0], ref[:, :, 0], rtol=1e-4, atol=1e-5)
