@@ -77,12 +77,10 @@ __device__ void transpose_layout(const BackwardArgs &a, int32_t block, int32_t c
     constexpr int kWarps = kPrepThreads / 32, kAhead = 4;
     const int32_t j0 = block * cols, j1 = j0 + cols < a.nqb ? j0 + cols : a.nqb;
     const int32_t w0 = j0 / 32, words = (a.nqb + 31) / 32 - w0;  // (rows below j0 list nothing here)
-    for (int32_t x = tid; x < (j1 - j0) * words; x += kPrepThreads) bits[x] = 0;
-    if (tid == 0) s_before = 0;
-    __syncthreads();
-    int32_t before = 0;
-    for (int32_t ib = j0 + warp * kAhead; ib < a.nqb; ib += kWarps * kAhead) {
-        int32_t lo[kAhead], hi[kAhead], col[kAhead];
+    // Loads go ahead of the work that they need not wait for: nothing but their order here lets them overlap it.
+    const int32_t listed_above = a.row_ptr[j0] - a.row_ptr[0];
+    int32_t lo[kAhead], hi[kAhead], col[kAhead];
+    auto fetch = [&](int32_t ib) {
 #pragma unroll
         for (int x = 0; x < kAhead; ++x) {  // (the loads of four rows in flight together)
             const bool on = ib + x < a.nqb;
@@ -91,6 +89,14 @@ __device__ void transpose_layout(const BackwardArgs &a, int32_t block, int32_t c
         }
 #pragma unroll
         for (int x = 0; x < kAhead; ++x) col[x] = lo[x] + lane < hi[x] ? a.col_idx[lo[x] + lane] : -1;
+    };
+    int32_t ib = j0 + warp * kAhead;
+    fetch(ib);
+    for (int32_t x = tid; x < (j1 - j0) * words; x += kPrepThreads) bits[x] = 0;
+    if (tid == 0) s_before = 0;
+    __syncthreads();
+    int32_t before = 0;
+    while (ib < a.nqb) {
 #pragma unroll
         for (int x = 0; x < kAhead; ++x) {
             const int32_t i = ib + x;
@@ -100,6 +106,8 @@ __device__ void transpose_layout(const BackwardArgs &a, int32_t block, int32_t c
                 c = e + 32 + lane < hi[x] ? a.col_idx[e + 32 + lane] : -1;
             }
         }
+        ib += kWarps * kAhead;
+        fetch(ib);
     }
     before = __reduce_add_sync(0xffffffffu, before);
     if (lane == 0 && before) atomicAdd(&s_before, before);
@@ -112,7 +120,7 @@ __device__ void transpose_layout(const BackwardArgs &a, int32_t block, int32_t c
     }
     __syncthreads();
     if (warp == 0) {  // exclusive prefix over the block's columns, from the entries before them
-        int32_t carry = s_before + a.row_ptr[j0] - a.row_ptr[0];
+        int32_t carry = s_before + listed_above;
         for (int32_t x = 0; x < j1 - j0; x += 32) {
             const int32_t n = x + lane < j1 - j0 ? s_count[x + lane] : 0;
             int32_t incl = n;
@@ -167,15 +175,6 @@ __global__ void __launch_bounds__(kPrepThreads) backward_prep_kernel(const Backw
     const int64_t groups = (a.N + kPrepTokens - 1) / kPrepTokens, grp = (int64_t)blockIdx.x - n_csc;
     const int64_t b = grp / groups, t0 = (grp - b * groups) * kPrepTokens, t = t0 + warp;
     const bool in = t < a.N;
-    if (a.prezero) {  // dK and dV of these tokens: contiguous
-        const int64_t per_token = (int64_t)a.Hkv * D / 4, tokens = a.N - t0 < kPrepTokens ? a.N - t0 : kPrepTokens;
-        float4 *zk = reinterpret_cast<float4 *>(a.dk) + (b * a.N + t0) * per_token;
-        float4 *zv = reinterpret_cast<float4 *>(a.dv) + (b * a.N + t0) * per_token;
-        for (int64_t x = tid; x < tokens * per_token; x += kPrepThreads) {
-            zk[x] = make_float4(0.f, 0.f, 0.f, 0.f);
-            zv[x] = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-    }
     const int64_t base = b * a.o_sb + (in ? t : 0) * a.o_ss + 8 * sub;
     for (int hb = 0; hb < a.Hq; hb += kPrepHeads) {
         const int heads = a.Hq - hb < kPrepHeads ? a.Hq - hb : kPrepHeads;
@@ -212,6 +211,15 @@ __global__ void __launch_bounds__(kPrepThreads) backward_prep_kernel(const Backw
             if (t0 + w < a.N) a.delta[(b * a.Hq + hb + h) * a.N + t0 + w] = s_delta[h][w];
         }
         __syncthreads();
+    }
+    if (a.prezero) {  // dK and dV of these tokens: contiguous (behind the loads, which do not wait for it so)
+        const int64_t per_token = (int64_t)a.Hkv * D / 4, tokens = a.N - t0 < kPrepTokens ? a.N - t0 : kPrepTokens;
+        float4 *zk = reinterpret_cast<float4 *>(a.dk) + (b * a.N + t0) * per_token;
+        float4 *zv = reinterpret_cast<float4 *>(a.dv) + (b * a.N + t0) * per_token;
+        for (int64_t x = tid; x < tokens * per_token; x += kPrepThreads) {
+            zk[x] = make_float4(0.f, 0.f, 0.f, 0.f);
+            zv[x] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
     }
 }
 
