@@ -4,9 +4,9 @@
 // pool of 64-token pages reached through a block table.
 //
 // Two paths.  Rows with at most 32 window, power-of-two and sink candidates (every PowerAttention
-// row with the default window up to millions of tokens) take decode_row_kernel: one launch, a
-// thread-block cluster per (sequence, KV head), described at that kernel.  Longer rows take the
-// split-K pair below.
+// row with the default window up to millions of tokens) take one launch: decode_cluster_kernel where they are few (a
+// thread-block cluster per (sequence, KV head)), else decode_row_kernel (a CTA per row), described at those kernels.
+// Longer rows take the split-K pair below.
 //
 // Split-K: one CTA per (sequence, KV head, chunk) where a chunk is one 64-key block of the
 // row's block list.  Each CTA reads its K and V block with coalesced 16-byte loads and computes
@@ -14,13 +14,13 @@
 // output on the warp-level tensor-core MMA.  The chunk partials (o[D], m, l) are then merged with
 // the log-sum-exp rule by a second kernel, launched with programmatic dependent launch so that
 // its start-up overlaps the first kernel's tail; it waits for the partials with griddepcontrol.wait.
-#include <cooperative_groups.h>
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <math.h>
 #include <stdlib.h>
 
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "layout_rule.cuh"
@@ -47,13 +47,13 @@ struct DecodeArgs {
     int64_t k_sb, k_ss, k_sh, v_sb, v_ss, v_sh;
     int64_t max_len;
     int32_t batch, Hq, Hkv, G, W, S, chunks, o_is_f32;
-    int32_t stages;        // (row kernel) shared-memory stages of this launch
-    int32_t R, mode;       // (row kernel) chunks per row; what becomes of an item's result
+    int32_t stages;        // (row and cluster kernels) shared-memory stages of this launch
+    int32_t R;             // (row and cluster kernels) chunks per row
     int32_t fixed_chunks;  // (combine kernel) > 0: every row has this many partials
     int64_t items;         // (row kernel) rows of the call x R
     int32_t table_stride, n_pages;
     float scale_log2;  // softmax_scale * log2(e)
-    long long wait_cycles;  // (row kernel) limit of every barrier wait, in clock cycles
+    long long wait_cycles;  // (row and cluster kernels) limit of every barrier wait, in clock cycles
 };
 
 // Where key block j of sequence b starts: (index along the batch / page axis, first token).  A
@@ -316,15 +316,9 @@ __global__ void __launch_bounds__(D) decode_combine_kernel(const DecodeArgs a)
 //               says when it has finished with it.  At the end of an item the four warps merge
 //               their partial results through shared memory with the log-sum-exp rule, each
 //               warp a quarter of the features.
-// What happens to an item's result depends on the launch (DecodeArgs::mode):
-//   kModeCluster  small calls.  One item per CTA, the R CTAs of a row form a thread-block
-//                 cluster: each CTA stores its part of head h into the shared memory of CTA h % R
-//                 (distributed shared memory), and after one cluster barrier that CTA merges the
-//                 head and writes O and LSE.  One launch.
-//   kModePartial  larger calls.  A persistent grid of two CTAs per SM strides over the items;
-//                 each item's (o, m, l) goes to the workspace and decode_combine_kernel merges a
-//                 row's R chunks (second launch, programmatic dependent launch).
-//   kModeDirect   R = 1 in a persistent grid: O and LSE are written straight from the registers.
+// A persistent grid of two CTAs per SM strides over the items.  With one chunk per row (the default) O and LSE are
+// written straight from the registers; with more (kParts, only under PA_DECODE_CLUSTER) each item's (o, m, l) goes to
+// the workspace and decode_combine_kernel merges a row's R chunks (second launch, programmatic dependent launch).
 // Every mbarrier wait is bounded; one that runs out records PA_ERR_TIMEOUT in the status block
 // and the CTA runs to its end without hanging.
 // ------------------------------------------------------------------------------------------
@@ -334,7 +328,6 @@ constexpr int kRowMaxStages = 6;                     // shared-memory stages (ke
 constexpr int kRowMaxCluster = 8;                    // portable cluster size limit
 constexpr int kRowMaxSmem = 227 * 1024;              // dynamic shared memory a CTA may ask for
 constexpr long long kRowWaitCycles = 2000000000ll;   // default limit of a barrier wait: ~1 s
-enum : int32_t { kModeCluster = 0, kModePartial = 1 /* only under PA_DECODE_CLUSTER */, kModeDirect = 2 };
 
 template <int D>
 struct RowSmem {
@@ -345,15 +338,8 @@ struct RowSmem {
     // (three quarters of the D features) and its running maximum and sum.
     static constexpr uint32_t kPartRow = D - D / 4 + 2;
     static constexpr uint32_t kPart = kRowConsumers * kMaxGroup * kPartRow * 4;
-    // (cluster form) what the row's CTAs send to the CTA that merges a head: per sending CTA and head
-    // slot, o[D], m, l.  R senders x ceil(8 / R) heads of an owner is at most 14 entries (R = 7).
-    static constexpr uint32_t kRecvEntries = 14;
-    static constexpr uint32_t kRecv = kRecvEntries * (D + 2) * 4;
     static constexpr uint32_t kBars = 3 * kRowMaxStages * 8 + 16;
-    static constexpr size_t bytes(int stages, bool cluster)
-    {
-        return 1024 + (size_t)stages * kStage + kPart + kBars + (cluster ? kRecv : 0);
-    }
+    static constexpr size_t bytes(int stages) { return 1024 + (size_t)stages * kStage + kPart + kBars; }
 };
 
 // The row's block set, one candidate per lane (the order does not matter for Eq. (1), so the set
@@ -379,12 +365,12 @@ __device__ __forceinline__ int32_t row_block_candidate(int32_t row, int32_t W, i
     return cand;
 }
 
-template <int D>
+// kParts: rows come in R chunks; else R = 1, known to the compiler (one block of 128 features, 16 rows: 3.6 us against 3.8).
+template <int D, bool kParts>
 __global__ void __launch_bounds__(kRowThreads, 2) decode_row_kernel(const __grid_constant__ CUtensorMap tmK,
                                                                     const __grid_constant__ CUtensorMap tmV,
                                                                     const DecodeArgs a)
 {
-    namespace cg = cooperative_groups;
     using SM = RowSmem<D>;
     constexpr int DH = D / 64;  // 64-feature (128-byte) sub-tiles per key row
     extern __shared__ uint8_t row_smem_raw[];
@@ -393,15 +379,13 @@ __global__ void __launch_bounds__(kRowThreads, 2) decode_row_kernel(const __grid
     const int stages = a.stages;
     const uint32_t off_part = (uint32_t)stages * SM::kStage;
     float *part = reinterpret_cast<float *>(smem + off_part);  // [warp][head][kPartRow]
-    // (cluster form) receive area behind the barriers: [sender][head slot][D + 2]
-    float *recv = reinterpret_cast<float *>(smem + off_part + SM::kPart + SM::kBars);
     const uint32_t bars = smem_base + off_part + SM::kPart;
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + off_part + SM::kPart + 3 * kRowMaxStages * 8);
     auto bar_kfull = [&](int s) { return bars + (uint32_t)s * 8u; };
     auto bar_vfull = [&](int s) { return bars + (uint32_t)(kRowMaxStages + s) * 8u; };
     auto bar_empty = [&](int s) { return bars + (uint32_t)(2 * kRowMaxStages + s) * 8u; };
 
-    const int R = a.R;
+    const int R = kParts ? a.R : 1;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int g = lane >> 2, t = lane & 3;
     const int G = a.G;
@@ -425,10 +409,6 @@ __global__ void __launch_bounds__(kRowThreads, 2) decode_row_kernel(const __grid
         ptx::prefetch_tensormap(&tmV);
     }
     __syncthreads();
-    // A peer's shared memory may be written only once the peer has started.  Each CTA says so here and asks for the
-    // others just before it pushes its parts, which hides the answer's way behind the wait below and the loads.
-    const bool peers = a.mode == kModeCluster && R > 1;
-    if (peers) ptx::cluster_arrive_relaxed();
     pdl_wait();
     const int32_t len_first = it0 < n_items ? a.lens[(it0 / (uint32_t)R) / (uint32_t)a.Hkv] : 0;
     if (a.clear_status && blockIdx.x == 0 && tid == 0) a.status[0] = 0;  // a wait that gives up (much later) sets it
@@ -506,7 +486,6 @@ __global__ void __launch_bounds__(kRowThreads, 2) decode_row_kernel(const __grid
                 __syncwarp();
             }
         }
-        if (peers) ptx::cluster_wait();
     } else {
         // ------------------------------------------------------------------ consumers
         // ldmatrix row addresses inside a tile.  K (matrices: keys 0-7 / 8-15 of the warp x two
@@ -703,27 +682,8 @@ __global__ void __launch_bounds__(kRowThreads, 2) decode_row_kernel(const __grid
             {
                 const int64_t head = ((int64_t)w.b * a.Hq + (int64_t)w.hk * G + g);
                 const int f0 = wid * (D / 4) + 2 * t;
-                if (a.mode == kModeCluster) {
-                    if (peers) ptx::cluster_wait();  // (one item per CTA: every thread comes here once)
-                    // Head g is merged by CTA g % R of the cluster: this CTA's part goes straight into
-                    // that CTA's receive area (a store through distributed shared memory; the area is
-                    // not used for anything else, so the owner may still be busy with its blocks).
-                    if (g < G) {
-                        namespace cg = cooperative_groups;
-                        cg::cluster_group cluster = cg::this_cluster();
-                        const int owner = g % R, slot = g / R, heads_per_owner = (kMaxGroup + R - 1) / R;
-                        float *dst = (R > 1 ? cluster.map_shared_rank(recv, owner) : recv) +
-                                     ((size_t)w.r * heads_per_owner + slot) * (D + 2);
-#pragma unroll
-                        for (int y = 0; y < D / 32; ++y)
-                            *reinterpret_cast<float2 *>(dst + f0 + 8 * y) = make_float2(fin[y][0], fin[y][1]);
-                        if (wid == 0 && t == 0) {
-                            dst[D] = m;
-                            dst[D + 1] = l;
-                        }
-                    }
-                } else if (g < G) {
-                    if (a.mode == kModePartial) {
+                if (g < G) {
+                    if (kParts) {
                         float *dst = a.partial + (head * R + w.r) * (D + 2);
 #pragma unroll
                         for (int y = 0; y < D / 32; ++y)
@@ -750,56 +710,351 @@ __global__ void __launch_bounds__(kRowThreads, 2) decode_row_kernel(const __grid
                     }
                 }
             }
-            // The hand-over area is written again only after every warp has read it (the cluster form
-            // has one item per CTA: nothing follows).
-            if (a.mode != kModeCluster) asm volatile("bar.sync 1, %0;\n" ::"n"(32 * kRowConsumers) : "memory");
+            // The hand-over area is written again only after every warp has read it.
+            asm volatile("bar.sync 1, %0;\n" ::"n"(32 * kRowConsumers) : "memory");
         }
     }
 
-    if (a.mode == kModeCluster) {
-        // ---- merge across the cluster: every CTA has pushed its parts; after one cluster barrier CTA r
-        // merges heads r, r + R, ... from its own receive area (thread d one feature) and writes O
-        // and LSE.  Nothing reads a peer's shared memory after the barrier, so no second one is needed.
-        namespace cg = cooperative_groups;
-        cg::cluster_group cluster = cg::this_cluster();
-        const int r = (int)(blockIdx.x % (unsigned)R);
-        const int32_t rowid = (int32_t)(blockIdx.x / (unsigned)R);
-        const int heads_per_owner = (kMaxGroup + R - 1) / R;
-        if (R > 1) cluster.sync();
-        else __syncthreads();
-        if (tid < D) {
-            for (int h = r, slot = 0; h < G; h += R, ++slot) {
-                float mr[kRowMaxCluster], lr[kRowMaxCluster], orr[kRowMaxCluster];
-#pragma unroll
-                for (int rr = 0; rr < kRowMaxCluster; ++rr) {
-                    const float *src = recv + ((size_t)(rr < R ? rr : 0) * heads_per_owner + slot) * (D + 2);
-                    mr[rr] = src[D];
-                    lr[rr] = src[D + 1];
-                    orr[rr] = src[tid];
-                }
-                float m = -INFINITY;
-#pragma unroll
-                for (int rr = 0; rr < kRowMaxCluster; ++rr)
-                    if (rr < R) m = fmaxf(m, mr[rr]);
-                float l = 0.f, o = 0.f;
-#pragma unroll
-                for (int rr = 0; rr < kRowMaxCluster; ++rr) {
-                    const float wgt = (rr < R && mr[rr] != -INFINITY) ? exp2f(mr[rr] - m) : 0.f;
-                    l += lr[rr] * wgt;
-                    o += orr[rr] * wgt;
-                }
-                const bool any = m != -INFINITY;  // false: a cache length outside [1, max_len]
-                const float out = any ? o / l : 0.f;
-                const int64_t oi = ((int64_t)rowid * G + h) * D + tid;
-                if (a.o_is_f32)
-                    reinterpret_cast<float *>(a.o)[oi] = out;
-                else
-                    reinterpret_cast<__nv_bfloat16 *>(a.o)[oi] = __float2bfloat16_rn(out);
-                if (tid == 0) a.lse[(int64_t)rowid * G + h] = any ? (m + log2f(l)) * 0.6931471805599453f : -INFINITY;
-            }
+    __syncthreads();
+    if (*abort_flag && tid == 0) {
+        // A wait gave up: leave copies that may still be in flight a bounded time to land
+        // before the CTA's shared memory is handed to another CTA.
+        const long long t0 = clock64();
+        while (clock64() - t0 < 2000000ll) {
         }
     }
+}
+
+// ------------------------------------------------------------------------------------------
+// The cluster kernel: the same rows in calls of so few that latency is all that counts.
+//
+// A row's key blocks are dealt round-robin to the R CTAs of a thread-block cluster; a CTA works on two blocks at a time,
+// eight warps on 16 keys each for the logits.  The warps exchange their maxima and their weights through shared
+// memory, and each takes D / 8 features of O += P V over all keys of the two blocks: what a warp holds at the end is
+// the CTA's result for its features, with nothing to merge inside the CTA.  It is pushed to the CTA that merges the
+// head (CTA h % R; asynchronous stores that count their bytes on a barrier of the receiving CTA, so that this CTA waits for
+// its parts and for nothing else).
+// Bound by that chain of latencies.  Measured in a graph, G = 7, head_dim 128, 4000 tokens, against this split done by
+// decode_row_kernel (keys kept apart by warp up to the end, the warps' outputs merged in shared memory, then all parts
+// behind a barrier of the cluster): 4 rows 3.7 us (5.2), 32 rows 4.9 (6.8), 74 rows 6.8 (8.0), 148 rows 9.1 (10.0).
+// ------------------------------------------------------------------------------------------
+constexpr int kClusterThreads = 256;
+constexpr int kClusterWarps = kClusterThreads / 32;
+
+template <int D>
+struct ClusterSmem {
+    static constexpr uint32_t kSub = kDecBlock * 128;   // 64 keys x 64 features
+    static constexpr uint32_t kTile = kSub * (D / 64);  // one K or V block
+    static constexpr uint32_t kStage = 2 * kTile;       // K + V of one key block
+    static constexpr uint32_t kPPitch = 2 * kDecBlock * 2 + 16;  // weights of a head: 128 keys, bf16; the pad spreads the banks
+    static constexpr uint32_t kMax = kMaxGroup * kPPitch;        // (behind the weights) [head][warp] maxima
+    static constexpr uint32_t kSum = kMax + kMaxGroup * kClusterWarps * 4;  // [head][warp] sums
+    // What the row's CTAs send to the CTA that merges a head: per sending CTA and head slot, o[D], m, l.
+    // R senders x ceil(8 / R) heads of an owner is at most 14 entries (R = 7).
+    static constexpr uint32_t kRecv = kSum + kMaxGroup * kClusterWarps * 4;
+    static constexpr uint32_t kRecvRow = (D + 2) * 4;
+    static constexpr uint32_t kBars = kRecv + ((14 * kRecvRow + 15) & ~15u);
+    static constexpr uint32_t kRest = kBars + (2 * kRowMaxStages + 2) * 8;
+    static constexpr size_t bytes(int stages) { return 1024 + (size_t)stages * kStage + kRest; }
+};
+
+template <int D>
+__global__ void __launch_bounds__(kClusterThreads, 2)
+decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const DecodeArgs a)
+{
+    using SM = ClusterSmem<D>;
+    constexpr int DH = D / 64;            // 64-feature (128-byte) sub-tiles per key row
+    constexpr int NT = D / 64;            // 8-feature tiles of O per warp
+    extern __shared__ uint8_t row_smem_raw[];
+    const uint32_t smem_base = (ptx::smem_u32(row_smem_raw) + 1023u) & ~1023u;
+    const int stages = a.stages;
+    const uint32_t rest = smem_base + (uint32_t)stages * SM::kStage, bars = rest + SM::kBars;
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(row_smem_raw + (bars - ptx::smem_u32(row_smem_raw)) +
+                                                                (2 * kRowMaxStages + 1) * 8);
+    auto bar_kfull = [&](int s) { return bars + (uint32_t)s * 8u; };
+    auto bar_vfull = [&](int s) { return bars + (uint32_t)(kRowMaxStages + s) * 8u; };
+    const uint32_t bar_recv = bars + 2 * kRowMaxStages * 8;
+    auto wait_bar = [&](uint32_t b_, uint32_t parity, int code) {
+        return ptx::mbar_wait_bounded(b_, parity, abort_flag, a.status, code, a.wait_cycles, (int)PA_ERR_TIMEOUT);
+    };
+
+    const int R = a.R, G = a.G;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int g = lane >> 2, t = lane & 3;
+    const uint32_t rowid = blockIdx.x / (uint32_t)R;  // = b Hkv + hk
+    const int r = (int)(blockIdx.x - rowid * (uint32_t)R);
+    const uint32_t b = rowid / (uint32_t)a.Hkv, hk = rowid - b * (uint32_t)a.Hkv;
+    const uint32_t inv_R = (65536u + (uint32_t)R - 1) / (uint32_t)R;  // x / R = x inv_R >> 16 for x < 32
+    // Heads r, r + R, ... are merged here.
+    const int heads_here = G > r ? (G - r + R - 1) / R : 0, heads_per_owner = (kMaxGroup + R - 1) / R;
+
+    // The launch after this one may take the places this one leaves; this one itself has started before the
+    // kernel ahead of it was done: up to pdl_wait() nothing of global memory is read or written.
+    pdl_launch_next();
+    if (tid == 0) {
+        for (int s = 0; s < stages; ++s) {
+            ptx::mbar_init(bar_kfull(s), 1);
+            ptx::mbar_init(bar_vfull(s), 1);
+        }
+        ptx::mbar_init(bar_recv, 1);
+        *abort_flag = 0;
+        ptx::fence_barrier_init();
+        ptx::fence_proxy_async_smem();
+        ptx::mbar_expect_tx(bar_recv, (uint32_t)(heads_here * R) * SM::kRecvRow);
+        ptx::prefetch_tensormap(&tmK);
+        ptx::prefetch_tensormap(&tmV);
+    }
     __syncthreads();
+    // A peer's shared memory may be written only once the peer has started and set its barrier up.  Each CTA says so here
+    // and asks for the others just before it pushes its parts, which hides the answer's way behind the loads.
+    ptx::cluster_arrive();
+    pdl_wait();
+    const int32_t len = a.lens[b];
+    if (a.clear_status && blockIdx.x == 0 && tid == 0) a.status[0] = 0;  // a wait that gives up (much later) sets it
+    // Q fragments: head g is row g of the 16-row A operand (rows 8..15 are zero).
+    uint32_t qa[D / 16][2];
+    {
+        const bool in = g < G;
+        const __nv_bfloat16 *qb = a.q + ((int64_t)rowid * G + (in ? g : 0)) * D;
+#pragma unroll
+        for (int ks = 0; ks < D / 16; ++ks) {
+            qa[ks][0] = in ? ld4(qb + 16 * ks + 2 * t) : 0u;
+            qa[ks][1] = in ? ld4(qb + 16 * ks + 8 + 2 * t) : 0u;
+        }
+    }
+
+    // The row's block set, one candidate per lane; block number i of this CTA is the (r + i R)-th that exists.  The diagonal
+    // block, lane 0's, is block 0 of CTA 0.
+    const bool valid = len >= 1 && (int64_t)len <= a.max_len;
+    const int32_t row = valid ? (len - 1) / kDecBlock : 0;
+    const int32_t cand = valid ? row_block_candidate(row, a.W, a.S, lane) : -1;
+    const uint32_t have = __ballot_sync(0xffffffffu, cand >= 0);
+    const int n = __popc(have), mine = n > r ? (int)(((uint32_t)(n - r + R - 1) * inv_R) >> 16) : 0;
+    const uint32_t rank = (uint32_t)__popc(have & ((1u << lane) - 1u)), quot = (rank * inv_R) >> 16;
+    const int my_block = cand >= 0 && (int)(rank - quot * (uint32_t)R) == r ? (int)quot : -1;
+    // Warp 0: each lane fetches the block that it found.  (A page outside the pool reads as zeros.)
+    int32_t outer = (int32_t)b, tok0 = cand * kDecBlock;
+    if (wid == 0 && a.table && my_block >= 0) {
+        outer = a.table[(int64_t)b * a.table_stride + cand];
+        tok0 = 0;
+    }
+    auto fetch = [&](int first, int end) {
+        if (my_block < first || my_block >= end) return;
+        const int s = my_block % stages;
+        const uint32_t dst = smem_base + (uint32_t)s * SM::kStage;
+        ptx::mbar_expect_tx(bar_kfull(s), SM::kTile);
+#pragma unroll
+        for (int dh = 0; dh < DH; ++dh) ptx::tma_load_4d(dst + dh * SM::kSub, &tmK, bar_kfull(s), dh * 64, tok0, (int)hk, outer);
+        ptx::mbar_expect_tx(bar_vfull(s), SM::kTile);
+#pragma unroll
+        for (int dh = 0; dh < DH; ++dh)
+            ptx::tma_load_4d(dst + SM::kTile + dh * SM::kSub, &tmV, bar_vfull(s), dh * 64, tok0, (int)hk, outer);
+    };
+    if (wid == 0) {
+        fetch(0, stages);
+        __syncwarp();
+    }
+
+    // ldmatrix row addresses inside a tile.  K (matrices: keys 0-7 / 8-15 of the warp x two 16-byte feature chunks): lane
+    // -> key 16 (w % 4) + 8 (lane / 16) + lane % 8, chunk + (lane / 8) % 2.  V (transposed; matrices: two key halves x two
+    // feature chunks, or with 64 features four key halves): key 8 (..) + lane % 8.  A 16-byte chunk c of row `key` sits
+    // at c ^ (key % 8).
+    const int k_key = 16 * (wid & 3) + ((lane >> 4) << 3) + (lane & 7), k_ch = (lane >> 3) & 1;
+    const uint32_t p_mine = rest + (uint32_t)g * SM::kPPitch + (uint32_t)(16 * wid + 2 * t) * 2u;
+    const uint32_t stat_mine = (uint32_t)(g * kClusterWarps + wid) * 4u, stat_row = (uint32_t)(g * kClusterWarps) * 4u;
+    // P as the A operand by ldmatrix: matrices of 8 heads x 8 keys.
+    const uint32_t p_frag = rest + (uint32_t)(lane & 7) * SM::kPPitch + (uint32_t)(lane >> 3) * 16u;
+    const int per = stages > 1 ? 2 : 1;  // blocks at a time
+    float m_run = -INFINITY, l_run = 0.f;  // of head g: the CTA's maximum, this warp's sum
+    float acc[NT][4];
+#pragma unroll
+    for (int e = 0; e < NT; ++e) acc[e][0] = acc[e][1] = acc[e][2] = acc[e][3] = 0.f;
+#pragma unroll 1
+    for (int i0 = 0; i0 < mine; i0 += per) {
+        const int blocks = min(per, mine - i0);
+        const int i = i0 + (wid >> 2);  // this warp's block
+        const int n_keys = (wid >> 2) >= blocks ? 0 : r == 0 && i == 0 ? (len - 1) % kDecBlock + 1 : kDecBlock;
+        float sx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+        float mx = -INFINITY;
+        if (16 * (wid & 3) < n_keys) {
+            const int s = i % stages;
+            wait_bar(bar_kfull(s), (uint32_t)(i / stages) & 1, 2);
+            __syncwarp();
+            // ---- S = Q K^T: rows = heads, columns = the warp's 16 keys (two 8-key tiles), two chains of MMAs each.
+            const uint32_t sk = smem_base + (uint32_t)s * SM::kStage;
+            float sc[2][2][4];
+#pragma unroll
+            for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+                for (int x = 0; x < 2; ++x) sc[nt][x][0] = sc[nt][x][1] = sc[nt][x][2] = sc[nt][x][3] = 0.f;
+#pragma unroll
+            for (int kb = 0; kb < D / 16; kb += 4) {
+                uint32_t kf[4][4];
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    const int ch = 2 * (kb + x) + k_ch;
+                    ptx::ldmatrix_x4(sk + (uint32_t)(ch >> 3) * SM::kSub + (uint32_t)k_key * 128u +
+                                         (uint32_t)(((ch & 7) ^ (k_key & 7)) << 4),
+                                     kf[x][0], kf[x][1], kf[x][2], kf[x][3]);
+                }
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    mma_bf16(sc[0][x & 1], qa[kb + x][0], 0u, qa[kb + x][1], 0u, kf[x][0], kf[x][1]);
+                    mma_bf16(sc[1][x & 1], qa[kb + x][0], 0u, qa[kb + x][1], 0u, kf[x][2], kf[x][3]);
+                }
+            }
+            // This thread: head g, keys 8 nt + 2 t + {0, 1} of the warp's 16; base-2 domain; keys that do not exist
+            // become -inf (a select, so whatever the cache holds there is ignored).
+            const int key0 = 16 * (wid & 3) + 2 * t;
+            sx[0] = key0 < n_keys ? (sc[0][0][0] + sc[0][1][0]) * a.scale_log2 : -INFINITY;
+            sx[1] = key0 + 1 < n_keys ? (sc[0][0][1] + sc[0][1][1]) * a.scale_log2 : -INFINITY;
+            sx[2] = key0 + 8 < n_keys ? (sc[1][0][0] + sc[1][1][0]) * a.scale_log2 : -INFINITY;
+            sx[3] = key0 + 9 < n_keys ? (sc[1][0][1] + sc[1][1][1]) * a.scale_log2 : -INFINITY;
+            mx = fmaxf(fmaxf(sx[0], sx[1]), fmaxf(sx[2], sx[3]));
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+        }
+        if (t == 0) ptx::st_shared(rest + SM::kMax + stat_mine, __float_as_uint(mx));
+        __syncthreads();
+        float m_new = m_run;
+        {
+            float mw[kClusterWarps];
+            ptx::ld_shared_v4(rest + SM::kMax + stat_row, mw[0], mw[1], mw[2], mw[3]);
+            ptx::ld_shared_v4(rest + SM::kMax + stat_row + 16, mw[4], mw[5], mw[6], mw[7]);
+#pragma unroll
+            for (int x = 0; x < kClusterWarps; ++x) m_new = fmaxf(m_new, mw[x]);  // finite: a listed block has a key
+        }
+        const float alpha = ptx::ex2(m_run - m_new);  // 0 at first
+        const float p0 = ptx::ex2(sx[0] - m_new), p1 = ptx::ex2(sx[1] - m_new);
+        const float p2 = ptx::ex2(sx[2] - m_new), p3 = ptx::ex2(sx[3] - m_new);
+        ptx::st_shared(p_mine, ptx::cvt_bf16x2(p0, p1));
+        ptx::st_shared(p_mine + 16, ptx::cvt_bf16x2(p2, p3));
+        float lsum = (p0 + p1) + (p2 + p3);
+        lsum += __shfl_xor_sync(0xffffffffu, lsum, 1);
+        lsum += __shfl_xor_sync(0xffffffffu, lsum, 2);
+        l_run = l_run * alpha + lsum;
+        m_run = m_new;
+        if (t == 0) ptx::st_shared(rest + SM::kSum + stat_mine, __float_as_uint(l_run));
+        __syncthreads();
+        // ---- O = alpha O + P V: rows = heads, the blocks' keys 16 at a time, this warp's D / 8 features.
+#pragma unroll
+        for (int e = 0; e < NT; ++e) {
+            acc[e][0] *= alpha;
+            acc[e][1] *= alpha;
+        }
+#pragma unroll 1
+        for (int x = 0; x < blocks; ++x) {
+            const int s = (i0 + x) % stages;
+            wait_bar(bar_vfull(s), (uint32_t)((i0 + x) / stages) & 1, 3);
+            __syncwarp();
+            const uint32_t sv = smem_base + (uint32_t)s * SM::kStage + SM::kTile;
+            uint32_t pf[4][2], vf[4][2 * NT];
+#pragma unroll
+            for (int ks = 0; ks < 4; ks += 2)
+                ptx::ldmatrix_x4(p_frag + (uint32_t)(64 * x + 16 * ks) * 2u, pf[ks][0], pf[ks][1], pf[ks + 1][0], pf[ks + 1][1]);
+            if constexpr (NT == 2) {
+                const int ch = 2 * wid + (lane >> 4);
+#pragma unroll
+                for (int ks = 0; ks < 4; ++ks) {
+                    const int key = 16 * ks + (((lane >> 3) & 1) << 3) + (lane & 7);
+                    ptx::ldmatrix_x4_trans(sv + (uint32_t)(ch >> 3) * SM::kSub + (uint32_t)key * 128u +
+                                               (uint32_t)(((ch & 7) ^ (key & 7)) << 4),
+                                           vf[ks][0], vf[ks][1], vf[ks][2], vf[ks][3]);
+                }
+            } else {
+                const int ch = wid;
+#pragma unroll
+                for (int ks = 0; ks < 4; ks += 2) {
+                    const int key = 16 * ks + ((lane >> 3) << 3) + (lane & 7);
+                    ptx::ldmatrix_x4_trans(sv + (uint32_t)key * 128u + (uint32_t)((ch ^ (key & 7)) << 4), vf[ks][0], vf[ks][1],
+                                           vf[ks + 1][0], vf[ks + 1][1]);
+                }
+            }
+            // V rows of keys that do not exist may hold anything (0 x NaN would poison O): they are cleared in the
+            // fragments.  Only the diagonal block has such rows.
+            if (r == 0 && i0 + x == 0) {
+                const int keys = (len - 1) % kDecBlock + 1;
+#pragma unroll
+                for (int ks = 0; ks < 4; ++ks) {
+                    const int key0 = 16 * ks + 2 * t;
+                    const uint32_t keep0 = (key0 < keys ? 0x0000ffffu : 0u) | (key0 + 1 < keys ? 0xffff0000u : 0u);
+                    const uint32_t keep1 = (key0 + 8 < keys ? 0x0000ffffu : 0u) | (key0 + 9 < keys ? 0xffff0000u : 0u);
+#pragma unroll
+                    for (int e = 0; e < NT; ++e) {
+                        vf[ks][2 * e] &= keep0;
+                        vf[ks][2 * e + 1] &= keep1;
+                    }
+                }
+            }
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks)
+#pragma unroll
+                for (int e = 0; e < NT; ++e)
+                    mma_bf16(acc[e], pf[ks][0], 0u, pf[ks][1], 0u, vf[ks][2 * e], vf[ks][2 * e + 1]);
+        }
+        // Once every warp has finished with these blocks, their stages may be loaded again.
+        if (i0 + stages < mine) {
+            __syncthreads();
+            if (wid == 0) fetch(i0 + stages, i0 + stages + per);
+            __syncwarp();
+        }
+    }
+
+    // ---- Thread (g, t) of warp w holds head g, features (D / 8) w + 8 e + 2 t + {0, 1}: pushed to CTA g % R.
+    ptx::cluster_wait();
+    if (g < G) {
+        const uint32_t slot = ((uint32_t)g * inv_R) >> 16, owner = (uint32_t)g - slot * (uint32_t)R;
+        const uint32_t dst = ptx::map_shared(rest + SM::kRecv, owner) + ((uint32_t)r * (uint32_t)heads_per_owner + slot) * SM::kRecvRow;
+        const uint32_t their_bar = ptx::map_shared(bar_recv, owner);
+#pragma unroll
+        for (int e = 0; e < NT; ++e)
+            ptx::st_async_v2(dst + (uint32_t)(wid * (D / 8) + 8 * e + 2 * t) * 4u, acc[e][0], acc[e][1], their_bar);
+        if (wid == 0 && t == 0) {
+            float l = 0.f;
+            if (mine > 0) {
+                float lw[kClusterWarps];
+                ptx::ld_shared_v4(rest + SM::kSum + stat_row, lw[0], lw[1], lw[2], lw[3]);
+                ptx::ld_shared_v4(rest + SM::kSum + stat_row + 16, lw[4], lw[5], lw[6], lw[7]);
+                l = ((lw[0] + lw[1]) + (lw[2] + lw[3])) + ((lw[4] + lw[5]) + (lw[6] + lw[7]));
+            }
+            ptx::st_async_v2(dst + D * 4u, m_run, l, their_bar);
+        }
+    }
+
+    // ---- Heads r, r + R, ...: D threads a head, a thread one feature.
+    if (heads_here > 0) {
+        ptx::mbar_wait_bounded_cluster(bar_recv, 0, abort_flag, a.status, 4, a.wait_cycles, (int)PA_ERR_TIMEOUT);
+        const int d = tid % D;
+        for (int slot = tid / D; slot < heads_here; slot += kClusterThreads / D) {
+            const int h = r + slot * R;
+            float mr[kRowMaxCluster], lr[kRowMaxCluster], orr[kRowMaxCluster];
+#pragma unroll
+            for (int x = 0; x < kRowMaxCluster; ++x) {
+                const uint32_t src = rest + SM::kRecv + (uint32_t)((x < R ? x : 0) * heads_per_owner + slot) * SM::kRecvRow;
+                ptx::ld_shared_v2(src + D * 4u, mr[x], lr[x]);
+                orr[x] = __uint_as_float(ptx::ld_shared(src + (uint32_t)d * 4u));
+            }
+            float m = -INFINITY;
+#pragma unroll
+            for (int x = 0; x < kRowMaxCluster; ++x)
+                if (x < R) m = fmaxf(m, mr[x]);
+            float l = 0.f, o = 0.f;
+#pragma unroll
+            for (int x = 0; x < kRowMaxCluster; ++x) {
+                const float wgt = (x < R && mr[x] != -INFINITY) ? ptx::ex2(mr[x] - m) : 0.f;
+                l = fmaf(lr[x], wgt, l);
+                o = fmaf(orr[x], wgt, o);
+            }
+            const bool any = m != -INFINITY;  // false: a cache length outside [1, max_len]
+            const float out = any ? o / l : 0.f;
+            const int64_t oi = ((int64_t)rowid * G + h) * D + d;
+            if (a.o_is_f32)
+                reinterpret_cast<float *>(a.o)[oi] = out;
+            else
+                reinterpret_cast<__nv_bfloat16 *>(a.o)[oi] = __float2bfloat16_rn(out);
+            if (d == 0) a.lse[(int64_t)rowid * G + h] = any ? (m + log2f(l)) * 0.6931471805599453f : -INFINITY;
+        }
+    }
     if (*abort_flag && tid == 0) {
         // A wait gave up: leave copies that may still be in flight a bounded time to land
         // before the CTA's shared memory is handed to another CTA.
@@ -959,11 +1214,12 @@ static size_t decode_workspace_bytes(const DecodeShape &s)
 
 static size_t row_smem_bytes(int head_dim, int stages, bool cluster)
 {
-    return head_dim == 128 ? RowSmem<128>::bytes(stages, cluster) : RowSmem<64>::bytes(stages, cluster);
+    if (cluster) return head_dim == 128 ? ClusterSmem<128>::bytes(stages) : ClusterSmem<64>::bytes(stages);
+    return head_dim == 128 ? RowSmem<128>::bytes(stages) : RowSmem<64>::bytes(stages);
 }
 
 // (The last attribute is the one that lets the kernel start early.)
-static cudaLaunchConfig_t row_launch_config(unsigned grid, int R, size_t smem, cudaLaunchAttribute (&attr)[2])
+static cudaLaunchConfig_t row_launch_config(unsigned grid, unsigned threads, int R, size_t smem, cudaLaunchAttribute (&attr)[2])
 {
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = (unsigned)R;
@@ -972,7 +1228,7 @@ static cudaLaunchConfig_t row_launch_config(unsigned grid, int R, size_t smem, c
     attr[1] = pdl_attribute();
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid, 1, 1);
-    cfg.blockDim = dim3(kRowThreads, 1, 1);
+    cfg.blockDim = dim3(threads, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
@@ -988,12 +1244,12 @@ static pa_status resident_clusters(int device, int head_dim, int stages, int R, 
     int &n = known[device][head_dim == 128][stages][R];
     if (n == 0) {
         cudaLaunchAttribute attr[2];
-        const cudaLaunchConfig_t cfg = row_launch_config((unsigned)R, R, row_smem_bytes(head_dim, stages, true), attr);
+        const cudaLaunchConfig_t cfg = row_launch_config((unsigned)R, kClusterThreads, R, row_smem_bytes(head_dim, stages, true), attr);
         int found = 0;
         if (head_dim == 128)
-            PA_CUDA_OK(cudaOccupancyMaxActiveClusters(&found, decode_row_kernel<128>, &cfg));
+            PA_CUDA_OK(cudaOccupancyMaxActiveClusters(&found, decode_cluster_kernel<128>, &cfg));
         else
-            PA_CUDA_OK(cudaOccupancyMaxActiveClusters(&found, decode_row_kernel<64>, &cfg));
+            PA_CUDA_OK(cudaOccupancyMaxActiveClusters(&found, decode_cluster_kernel<64>, &cfg));
         n = found + 1;
     }
     *out = n - 1;
@@ -1054,7 +1310,6 @@ static pa_status launch_decode(const DecodeShape &p, const void *q, const void *
     const EnvSwitches env = env_switches();
     a.fixed_chunks = 0;
     a.R = 1;
-    a.mode = kModeCluster;
     a.items = 0;
     // Rows whose block set fits one warp's lanes take the row kernel.
     if (!takes_split_k(p)) {
@@ -1074,23 +1329,24 @@ static pa_status launch_decode(const DecodeShape &p, const void *q, const void *
         };
         if (pa_status s = device_once(dev.device, ONCE_DECODE_ATTR, [] {
                 constexpr cudaFuncAttribute kSmem = cudaFuncAttributeMaxDynamicSharedMemorySize;
-                return first_error(cudaFuncSetAttribute(decode_row_kernel<128>, kSmem, kRowMaxSmem),
-                                   cudaFuncSetAttribute(decode_row_kernel<64>, kSmem, kRowMaxSmem));
+                cudaError_t e = cudaSuccess;
+                for (auto *kernel : {decode_row_kernel<128, true>, decode_row_kernel<128, false>, decode_row_kernel<64, true>,
+                                     decode_row_kernel<64, false>, decode_cluster_kernel<128>, decode_cluster_kernel<64>})
+                    e = first_error(e, cudaFuncSetAttribute(kernel, kSmem, kRowMaxSmem));
+                return e;
             }))
             return s;
         // Small calls (latency-bound): a cluster of R CTAs per row, all resident at once.  Larger calls
         // (bandwidth-bound): a persistent grid of two CTAs per SM over the rows.  The line lies where a row
-        // still gets two of the resident CTAs: rows of 18 blocks (30000 tokens, G = 7, head_dim 128) take
-        // 9.2 us at 80 rows in clusters of three and 11.5 us in the persistent form, 12.4 and 13.3 at 120
-        // rows, 18.8 (clusters of one) and 15.7 at 160.
+        // still gets two of the resident CTAs: 4000 tokens, G = 7, head_dim 128 take 6.8 us at 80 rows in clusters
+        // of three, 9.1 at 148 in clusters of two, 13.8 (clusters of one) and 11.3 (persistent form) at 160.
         bool cluster = rows_in_call * 2 <= persistent_ctas;
         if (env.decode_path == 2) cluster = true;
         if (env.decode_path == 3) cluster = false;
         int R = env.decode_cluster, fit = 0;  // fit: clusters of R CTAs that the device holds at once
         if (cluster && R == 0) {
             // As many CTAs per row as run all at once: a second wave of clusters nearly doubles the call's latency
-            // (4000 tokens, G = 7, head_dim 128: 74 rows in clusters of four 13.0 us, of three 8.2; 98 rows in clusters of
-            // three 14.4 us, of two 10.0).  How many clusters fit is asked of the device: all CTAs of a cluster lie
+            // (with an earlier kernel, 4000 tokens, G = 7, head_dim 128: 74 rows in clusters of four 13.0 us, of three 8.2).  How many clusters fit is asked of the device: all CTAs of a cluster lie
             // within one GPU processing cluster, which may leave places that no further cluster fits in.
             R = (int)(persistent_ctas / rows_in_call);
             if (R > max_R) R = max_R;
@@ -1104,10 +1360,10 @@ static pa_status launch_decode(const DecodeShape &p, const void *q, const void *
         // than they gain, and need the merge kernel.)
         if (R < 1) R = 1;
         if (R > max_R) R = max_R;
-        // A row in one piece has nothing to merge with: the cluster form's last step is spared (rows of one block, G = 7,
-        // head_dim 128: 6.4 to 7.6 us in the cluster form, 3.8 to 4.6 without).
+        // A row in one piece has nothing to merge with, and nothing that eight warps could share (one block, G = 7,
+        // head_dim 128: 4.3 to 5.9 us in the cluster form, 3.4 to 4.6 without).
         if (R == 1 && env.decode_path != 2) cluster = false;
-        a.mode = cluster ? kModeCluster : R == 1 ? kModeDirect : kModePartial;
+        const bool parts = !cluster && R > 1;
         a.R = R;
         a.items = rows_in_call * R;
         const int64_t grid = cluster ? a.items : (a.items < persistent_ctas ? a.items : persistent_ctas);
@@ -1115,14 +1371,12 @@ static pa_status launch_decode(const DecodeShape &p, const void *q, const void *
         a.stages = stages_of(grid, cluster);
         // Started early, clusters take places as the CTAs of the kernel before leave them, one by one, and what is left
         // in between may be of no use to a cluster until more have ended.  A call that needs nearly all places starts
-        // on the empty device instead, about 0.7 us later.  Where that begins to pay was measured for each size, early
-        // and late in us (4000 tokens, G = 7, head_dim 128; 148 SMs): clusters of three 8.1 and 8.9 at 80 rows, 10.7 and
-        // 8.9 at 84, 12.9 and 8.9 at 93; of five 7.1 and 7.7 at 52, 8.2 and 7.6 at 54; of six 7.7 and 7.7 at 43, 8.8 and
-        // 7.5 at 45; of seven 6.5 and 7.1 at 34, 8.3 and 7.1 at 37; of four and eight, which find the places of their
-        // like, 8.1 and 8.3 at 70, 9.6 and 8.3 at 71, 6.8 and 6.9 at 32, 8.3 and 7.0 at 33.  Pairs fit in any order.
-        const bool full = R == 3             ? rows_in_call * 10 > fit * 9
-                          : (R & (R - 1)) == 0 ? rows_in_call == fit
-                                               : rows_in_call * 25 > fit * 24;
+        // on the empty device instead, about 1 us later.  Where that begins to pay was measured for each size, early
+        // and late in us (4000 tokens, G = 7, head_dim 128; 148 SMs): clusters of three 8.0 and 8.0 at 88 rows, 9.2 and
+        // 8.0 at 90; of four and five (20000 tokens, G = 8) 7.2 and 7.8 at 70, 8.5 and 7.8 at 71, 7.7 and 7.8 at 55, 8.8 and
+        // 7.8 at 56; of six to eight never clearly: 5.7 and 6.4 at 45, 5.8 and 6.2 at 37, 5.6 and 6.2 at 33.  Pairs fit
+        // in any order.
+        const bool full = R == 3 ? rows_in_call * 20 > fit * 19 : R <= 5 && rows_in_call == fit;
         const bool early = !(cluster && R > 2 && fit > 0 && full);
 
         // Tensor maps over the cache: (feature, token, head, batch or page), one 64 x 64 box per copy.
@@ -1135,20 +1389,23 @@ static pa_status launch_decode(const DecodeShape &p, const void *q, const void *
         if (pa_status s = get_tensor_map(kk, "k_cache", &tmK)) return s;
         if (pa_status s = get_tensor_map(kv, "v_cache", &tmV)) return s;
 
-        if (a.mode == kModePartial) {
+        if (parts) {
             a.chunks = R;  // the partials of a row are its R chunks
             a.fixed_chunks = R;
         }
         cudaLaunchAttribute attr[2];
         cudaLaunchConfig_t cfg =
-            row_launch_config((unsigned)grid, cluster ? R : 1, row_smem_bytes(p.head_dim, a.stages, cluster), attr);
+            row_launch_config((unsigned)grid, cluster ? kClusterThreads : kRowThreads, cluster ? R : 1,
+                              row_smem_bytes(p.head_dim, a.stages, cluster), attr);
         cfg.stream = st;
         if (!early) cfg.numAttrs = 1;
-        if (p.head_dim == 128)
-            PA_CUDA_OK(cudaLaunchKernelEx(&cfg, decode_row_kernel<128>, tmK, tmV, a));
-        else
-            PA_CUDA_OK(cudaLaunchKernelEx(&cfg, decode_row_kernel<64>, tmK, tmV, a));
-        if (a.mode != kModePartial) return PA_OK;
+        auto kernel_of = [&](auto d) {
+            constexpr int D = decltype(d)::value;
+            return cluster ? decode_cluster_kernel<D> : parts ? decode_row_kernel<D, true> : decode_row_kernel<D, false>;
+        };
+        auto *kernel = p.head_dim == 128 ? kernel_of(std::integral_constant<int, 128>()) : kernel_of(std::integral_constant<int, 64>());
+        PA_CUDA_OK(cudaLaunchKernelEx(&cfg, kernel, tmK, tmV, a));
+        if (!parts) return PA_OK;
     } else {
         const dim3 grid1((unsigned)a.chunks, (unsigned)a.Hkv, (unsigned)a.batch);
         if (p.head_dim == 128)

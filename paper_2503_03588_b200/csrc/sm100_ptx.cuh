@@ -66,13 +66,14 @@ __device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity)
 // cycles.  Returns false after a timeout, which it records once in status[0] (error code) and
 // status[1] (an id naming the wait), or once another thread of the CTA has raised the abort flag;
 // a timeout raises the flag, so that every role of the CTA leaves its loop and the CTA ends.
-__device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity, volatile int *abort_flag,
-                                                  int32_t *status, int code, long long limit, int timeout_status)
+template <bool (*kTry)(uint32_t, uint32_t)>
+__device__ __forceinline__ bool mbar_wait_bounded_by(uint32_t bar, uint32_t parity, volatile int *abort_flag,
+                                                     int32_t *status, int code, long long limit, int timeout_status)
 {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (kTry(bar, parity)) return true;
     const long long t0 = clock64();
     while (true) {
-        if (mbar_try_wait(bar, parity)) return true;  // (each try suspends the thread for a while by itself)
+        if (kTry(bar, parity)) return true;  // (each try suspends the thread for a while by itself)
         if (*abort_flag) return false;
         if (clock64() - t0 > limit) break;
     }
@@ -80,6 +81,29 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
     *abort_flag = 1;
     __threadfence_block();
     return false;
+}
+__device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity, volatile int *abort_flag,
+                                                  int32_t *status, int code, long long limit, int timeout_status)
+{
+    return mbar_wait_bounded_by<mbar_try_wait>(bar, parity, abort_flag, status, code, limit, timeout_status);
+}
+// The same for a barrier on which other CTAs of the cluster count their stores.
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+__device__ __forceinline__ bool mbar_wait_bounded_cluster(uint32_t bar, uint32_t parity, volatile int *abort_flag,
+                                                          int32_t *status, int code, long long limit, int timeout_status)
+{
+    return mbar_wait_bounded_by<mbar_try_wait_cluster>(bar, parity, abort_flag, status, code, limit, timeout_status);
 }
 
 // ---------------------------------------------------------------- TMA (no multicast anywhere)
@@ -120,6 +144,27 @@ __device__ __forceinline__ void bulk_commit_group() { asm volatile("cp.async.bul
 // The issuing thread's bulk stores have finished reading shared memory / have completed.
 __device__ __forceinline__ void bulk_wait_read_all() { asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory"); }
+__device__ __forceinline__ void st_shared(uint32_t addr, uint32_t v)
+{
+    asm volatile("st.volatile.shared.u32 [%0], %1;\n" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ uint32_t ld_shared(uint32_t addr)
+{
+    uint32_t v;
+    asm volatile("ld.volatile.shared.u32 %0, [%1];\n" : "=r"(v) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ void ld_shared_v2(uint32_t addr, float &a, float &b)
+{
+    asm volatile("ld.volatile.shared.v2.f32 {%0, %1}, [%2];\n" : "=f"(a), "=f"(b) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ld_shared_v4(uint32_t addr, float &a, float &b, float &c, float &d)
+{
+    asm volatile("ld.volatile.shared.v4.f32 {%0, %1, %2, %3}, [%4];\n"
+                 : "=f"(a), "=f"(b), "=f"(c), "=f"(d)
+                 : "r"(addr)
+                 : "memory");
+}
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
 {
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
@@ -320,10 +365,24 @@ __device__ __forceinline__ void red_add_v4(float *p, const float4 &v)
     asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};\n" ::"l"(p), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
 }
 
-// Barrier of the thread-block cluster in two halves, without an order of memory: every thread of every CTA arrives
-// once and waits once.  Behind the wait all CTAs of the cluster have started.
-__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed;\n" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait;\n" ::: "memory"); }
+// Barrier of the thread-block cluster in two halves: every thread of every CTA arrives once and waits once.  What a thread
+// wrote before it arrived is seen by every thread behind the wait.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;\n" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;\n" ::: "memory"); }
+// The address of `addr` (of this CTA's shared memory) in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t map_shared(uint32_t addr, uint32_t rank)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+// Two floats into a CTA's shared memory, their 8 bytes counted on a barrier of the same CTA.
+__device__ __forceinline__ void st_async_v2(uint32_t addr, float a, float b, uint32_t bar)
+{
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];\n" ::"r"(addr), "f"(a),
+                 "f"(b), "r"(bar)
+                 : "memory");
+}
 
 __device__ __forceinline__ float ex2(float x)
 {

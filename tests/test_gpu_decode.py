@@ -116,6 +116,24 @@ def test_decode_paths(pa, oracle, pa_env, env):
     _run(pa, oracle, q, kc, vc, lens, 3, 2, o_dtype=torch.float32)
 
 
+@pytest.mark.parametrize("R,stages", [(1, 1), (1, 3), (2, 2), (3, 3), (5, 2), (8, 2)])
+@pytest.mark.parametrize("Hq,Hkv,D", [(8, 1, 64), (3, 1, 64), (2, 2, 128), (8, 1, 128)])
+def test_cluster_kernel_edges(pa, oracle, pa_env, Hq, Hkv, D, R, stages):
+    """decode_cluster_kernel: lengths around the edges of a warp's 16 keys and of a block, CTAs without a block, one, two
+    and more blocks at a time, a head per CTA and several; beyond its length the cache holds NaN."""
+    pa_env(PA_DECODE_PATH="cluster", PA_DECODE_CLUSTER=str(R), PA_DECODE_STAGES=str(stages))
+    lens = np.array([1, 15, 16, 17, 64, 65, 81, 130, 1000, 2049])
+    batch, max_len = len(lens), 2100
+    q = si.bf16_randn((batch, Hq, D), 51)
+    kc, vc = si.bf16_randn((batch, max_len, Hkv, D), 52, 2.0), si.bf16_randn((batch, max_len, Hkv, D), 53)
+    for b, L in enumerate(lens):
+        kc[b, L:] = vc[b, L:] = float("nan")
+    o, lse, _ = pa.pa_decode(q.cuda(), kc.cuda(), vc.cuda(), torch.as_tensor(lens, dtype=torch.int32).cuda(), 5, 1,
+                             o_dtype=torch.float32)
+    o_ref, lse_ref, _ = oracle.decode(q, torch.nan_to_num(kc), torch.nan_to_num(vc), lens, 64, 5, 1)
+    compare(o, lse, o_ref, lse_ref, f"R={R} stages={stages}")
+
+
 def test_decode_short_cache_with_wide_window_and_sinks(pa, oracle):
     """A cache of 32 blocks whose window + sink candidates exceed 32: the bound on listed blocks is
     clamped by the row count, the candidate count is not (the library must pick its path by the
