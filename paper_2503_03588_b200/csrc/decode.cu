@@ -1100,16 +1100,25 @@ kv_append_kernel(const __nv_bfloat16 *k_new, const __nv_bfloat16 *v_new, __nv_bf
     pdl_launch_next();
     pdl_wait();
     const int b = blockIdx.x;
+    const int per_row = D / 8, pieces = Hkv * per_row;  // 16-byte pieces of K, then of V
+    auto piece_of = [&](int x) {
+        const bool is_v = x >= pieces;
+        return ld16((is_v ? v_new : k_new) + ((int64_t)b * pieces + (is_v ? x - pieces : x)) * 8);
+    };
+    // A thread's first piece is on its way while the length and then the page are looked up.
+    const int first = threadIdx.x;
+    uint4 piece = make_uint4(0, 0, 0, 0);
     const int32_t pos = lens[b];
+    if (first < 2 * pieces) piece = piece_of(first);
     const int32_t blk = pos / kDecBlock;
     if (pos < 0 || blk >= table_stride) return;
     const int32_t page = table[(int64_t)b * table_stride + blk];
     if (page < 0 || page >= n_pages) return;
-    const int slot = pos % kDecBlock, per_row = D / 8, pieces = Hkv * per_row;  // 16-byte pieces of K, then of V
-    for (int x = threadIdx.x; x < 2 * pieces; x += kThreads) {
+    const int slot = pos % kDecBlock;
+    for (int x = first; x < 2 * pieces; x += kThreads) {
         const bool is_v = x >= pieces;
         const int y = is_v ? x - pieces : x, hk = y / per_row, c = y % per_row;
-        const uint4 piece = *reinterpret_cast<const uint4 *>((is_v ? v_new : k_new) + ((int64_t)b * Hkv + hk) * D + 8 * c);
+        if (x != first) piece = piece_of(x);
         __nv_bfloat16 *dst = is_v ? v_pool + page * v_sp + slot * v_ss + hk * v_sh
                                   : k_pool + page * k_sp + slot * k_ss + hk * k_sh;
         *reinterpret_cast<uint4 *>(dst + 8 * c) = piece;
