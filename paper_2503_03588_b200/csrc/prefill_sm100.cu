@@ -4,7 +4,7 @@
 // One persistent CTA per SM walks work units (batch, KV head, query block, head quad).  A unit
 // holds two 128-row tiles ("slots"); a tile stacks two query heads of the KV group on the 64
 // tokens of the query block (the mask does not depend on the head, so they share the key list
-// and the K/V tiles).  (Groups of one or two query heads have one slot.)  The key list is walked one
+// and the K/V tiles).  (One slot where the group has one or two query heads, or units are few.)  The key list is walked one
 // 64-key block per step.  Warp roles:
 //   warp 0      TMA producer: the listed K and V blocks, gathered by block index, into two rings
 //               of shared-memory tiles (128-byte swizzle); the next unit's Q tiles early in
@@ -275,7 +275,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                     for (int dh = 0; dh < DH; ++dh)
                         ptx::tma_load_4d(smem_base + SM::kQ + qb * SM::kQBuf + s * SM::kQSlot + dh * SM::kQSub, &tmQ,
                                          bar(BAR_Q_FULL + qb), dh * 64, w.tok0 + w.i * kBlk,
-                                         w.hk * a.G + w.sub * 4 + 2 * s, w.bt);
+                                         w.hk * a.G + w.sub * 2 * kSlots + 2 * s, w.bt);
                 return true;
             };
             Unit w, wn;
@@ -493,7 +493,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         for (uint32_t u = kSlots == 2 || s == 0 ? blockIdx.x : n_units; u < n_units && ok; u += gridDim.x) {
             const Unit w = w_next;
             const int32_t lastcol = lastcol_next;
-            const int head_local = w.sub * 4 + 2 * s + (row >> 6);
+            const int head_local = w.sub * 2 * kSlots + 2 * s + (row >> 6);
             const int head = w.hk * a.G + head_local;
             const int64_t tok = (int64_t)w.i * kBlk + qrow;
             const bool valid = head_local < a.G && tok < w.len;
@@ -695,7 +695,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             const uint32_t stage = smem_base + SM::kQ + (ul & 1) * SM::kQBuf;
 #pragma unroll 1
             for (int s = 0; s < kSlots; ++s) {
-                const int head_local = w.sub * 4 + 2 * s + (row >> 6);
+                const int head_local = w.sub * 2 * kSlots + 2 * s + (row >> 6);
                 const int head = w.hk * a.G + head_local;
                 const bool valid = head_local < a.G && tok < w.len;
                 const int64_t obase = w.bt * a.o_sb + (w.tok0 + tok) * a.o_ss + (int64_t)head * a.o_sh;
@@ -766,7 +766,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                         if (!ok) break;
                         if (store_thread) {
                             for (int hh = 0; hh < 2; ++hh) {
-                                const int hl = w.sub * 4 + 2 * s + hh;
+                                const int hl = w.sub * 2 * kSlots + 2 * s + hh;
                                 if (hl >= a.G || ragged) continue;
                                 for (int k = 0; k < DH; ++k)
                                     ptx::tma_store_4d(&tmO, stage + (uint32_t)(2 * s + hh) * SM::kOHead + (uint32_t)k * 8192u,
@@ -813,7 +813,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                     if (!ok) break;
                     if (store_thread) {
                         for (int hh = 0; hh < 2; ++hh) {
-                            const int hl = w.sub * 4 + 2 * s + hh;
+                            const int hl = w.sub * 2 * kSlots + 2 * s + hh;
                             if (hl >= a.G || ragged) continue;  // the padding head of an odd group; rows already written
                             for (int dh = 0; dh < DH; ++dh)
                                 ptx::tma_store_4d(&tmO, stage + (uint32_t)(2 * s + hh) * SM::kOHead + (uint32_t)dh * 8192u,
@@ -989,8 +989,17 @@ static pa_status launch_prefill(const pa_prefill_params *p, const void *q, const
     a.nqb = (int32_t)nqb;
     a.batch = p->batch; a.Hq = p->n_q_heads; a.Hkv = p->n_kv_heads;
     a.G = p->n_q_heads / p->n_kv_heads;
-    a.nsub = (a.G + 3) / 4;
-    a.n_units = (int64_t)p->batch * nqb * a.Hkv * a.nsub;
+    // Slots.  Groups of one or two query heads have nothing for a second one: its roles stay idle then, and a step is as
+    // long as one slot's chain alone.  With one head per group 2K tokens, 2 heads of 64 features take 9.1 us instead of
+    // 11.4, 32K tokens, 8 heads of 128 features 266 us instead of 355; with two heads per group 8K tokens, batch 2,
+    // 8 KV heads 118 us instead of 156 (burst).  Larger groups are taken two heads a CTA, too, where every such unit
+    // finds an SM of its own: then nothing counts but the length of the chain (in a graph, 28 / 4 heads: 64 tokens 6.3 ->
+    // 5.3 us, 500 tokens 11.6 -> 9.9; 8 / 2 heads: 2048 tokens 13.7 -> 11.5).  One unit more and two rounds of one slot
+    // take longer than one of two.
+    const int64_t rows = (int64_t)p->batch * nqb * a.Hkv;
+    const int slots = a.G <= 2 || rows * ((a.G + 1) / 2) <= dev.sms ? 1 : 2;
+    a.nsub = (a.G + 2 * slots - 1) / (2 * slots);
+    a.n_units = rows * a.nsub;
     auto inv32 = [](int32_t d) { return d == 1 ? 0xffffffffu : (uint32_t)((1ull << 32) / (uint64_t)d); };
     a.inv_nsub = inv32(a.nsub); a.inv_Hkv = inv32(a.Hkv); a.inv_nqb = inv32(a.nqb);
     if (a.n_units > (int64_t)0x3fffffff) return fail(PA_ERR_SHAPE, "too many work units (%lld)", (long long)a.n_units);
@@ -1023,16 +1032,12 @@ static pa_status launch_prefill(const pa_prefill_params *p, const void *q, const
                 return fail(PA_ERR_LAYOUT, "CSR check: %s (row %d)", what[found[0]], (int)found[1]);
         }
     }
-    // Groups of one or two query heads have nothing for a second slot: its roles stay idle then, and a step is as
-    // long as one slot's chain alone.  With one head per group 2K tokens, 2 heads of 64 features take 9.1 us instead of
-    // 11.4, 32K tokens, 8 heads of 128 features 266 us instead of 355; with two heads per group 8K tokens, batch 2,
-    // 8 KV heads 118 us instead of 156 (burst).  Three heads need the second slot.
     auto launch = [&](auto kernel) { return kernel(grid, st, dev.device, tmQ, tmK, tmV, tmO, a); };
     if (p->o_dtype == PA_F32) {
-        if (a.G > 2) return launch(D == 128 ? launch_kernel<128, 2, true> : launch_kernel<64, 2, true>);
+        if (slots == 2) return launch(D == 128 ? launch_kernel<128, 2, true> : launch_kernel<64, 2, true>);
         return launch(D == 128 ? launch_kernel<128, 1, true> : launch_kernel<64, 1, true>);
     }
-    if (a.G > 2) return launch(D == 128 ? launch_kernel<128, 2, false> : launch_kernel<64, 2, false>);
+    if (slots == 2) return launch(D == 128 ? launch_kernel<128, 2, false> : launch_kernel<64, 2, false>);
     return launch(D == 128 ? launch_kernel<128, 1, false> : launch_kernel<64, 1, false>);
 }
 

@@ -70,6 +70,22 @@ def test_groups_that_leave_the_second_slot_idle(pa, oracle, G, D):
     _full_compare(pa, oracle, Q, (K.float() * 3).bfloat16(), V, 2, 1, o_dtype=torch.float32, what=f"G={G} D={D} peaky")
 
 
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("G", [3, 4, 5, 7, 8])
+def test_large_groups_with_few_units(pa, oracle, G, D):
+    """Calls whose units of two heads find an SM each run larger groups with one slot, longer ones with two: lengths on both
+    sides of the line for 148 SMs, two KV heads, a ragged last block, the padding head of odd groups."""
+    Hkv, pairs = 2, (G + 1) // 2
+    most = 148 // (Hkv * pairs)   # query blocks up to which there is one slot
+    for blocks in (1, 3, most, most + 1):
+        N = 64 * blocks - 5
+        Q = si.bf16_randn((1, N, G * Hkv, D), 1400 + G)
+        K = si.bf16_randn((1, N, Hkv, D), 1500 + G)
+        V = si.bf16_randn((1, N, Hkv, D), 1600 + G)
+        _full_compare(pa, oracle, Q, K, V, 2, 1, o_dtype=torch.float32, what=f"G={G} D={D} blocks={blocks}")
+        _full_compare(pa, oracle, Q, K, V, 2, 1, what=f"G={G} D={D} blocks={blocks}")
+
+
 def test_peaky_logits_fp32_output_and_custom_scale(pa, oracle):
     N, Hq, Hkv, D = 1500, 14, 2, 128
     Q, K, V = si.bf16_randn((1, N, Hq, D), 1), si.bf16_randn((1, N, Hkv, D), 2, 3.0), si.bf16_randn((1, N, Hkv, D), 3)
