@@ -476,13 +476,14 @@ __global__ void __launch_bounds__(kBwdThreads) backward_dkv_kernel(const Backwar
 namespace pa {
 
 // Query blocks per chunk of a key block's list.  A chunk is walked by one CTA of the dK / dV kernels for the
-// whole head group, so it is also the granularity at which the work is dealt to the SMs: about eight chunks per
-// SM, no more than 32 blocks, and no less than four, below which a chunk's own cost (K and V in, dK and dV added
-// to memory) outweighs the balance.  (4K tokens, 28 / 4 heads: 112 us with chunks of 4, 229 us with chunks of 32,
-// of which the sink block's two are then the whole call's tail.)
+// whole head group, so it is also the granularity at which the work is dealt to the SMs: about four chunks per
+// SM (the dQ kernel fills what their last round leaves), no more than 32 blocks, and no less than four, below which a
+// chunk's own cost (K and V in, dK and dV added to memory) outweighs the balance.  (Whole backward pass in a loop, eight
+// and four chunks per SM: 32K tokens, 28 / 4 heads 1567 and 1543 us, 2 x 8K, 16 / 4 heads of 64 features 239 and 234; no less
+// than four and eight blocks: 2K tokens 81 and 95.)
 static int32_t backward_chunk(int64_t nnz, int64_t kv_rows, int sms)
 {
-    const int64_t c = nnz * kv_rows / (8 * (int64_t)sms);
+    const int64_t c = nnz * kv_rows / (4 * (int64_t)sms);
     return c < 4 ? 4 : c > kBwdMaxChunk ? kBwdMaxChunk : (int32_t)c;
 }
 
@@ -610,9 +611,9 @@ extern "C" pa_status pa_prefill_backward(const pa_prefill_params *p, const void 
     a.npairs = (a.G + 1) / 2;
     a.wait_cycles = 0;
     a.chunk = backward_chunk(nnz, (int64_t)a.batch * a.Hkv, dev.sms);
-    // dK and dV are cleared by the preparation where most key blocks are added up from several chunks (small
-    // problems, small chunks); with chunks of full size the tcgen05 kernels write all but a few columns once and
-    // clear those.
+    // The preparation clears all of dK and dV where most key blocks are added up from several chunks (small problems,
+    // small chunks); with chunks of full size all but a few columns are written once, and those few get a kernel of their
+    // own, which longer calls do not notice.
     const bool mma = env_switches().backward_mma != 0;
     a.prezero = mma || a.chunk < kBwdMaxChunk;
     a.early = nqb * a.Hkv * a.npairs * a.batch <= dev.sms;

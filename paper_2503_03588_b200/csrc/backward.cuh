@@ -14,7 +14,8 @@ namespace pa {
 constexpr int kBwdBlk = 64;       // tokens per block
 constexpr int kBwdMaxChunk = 32;  // query blocks per chunk of the dK / dV kernels, at most
 constexpr size_t kBwdStatusBytes = 256;  // status block at the head of the workspace ([0] error code, [1] detail)
-constexpr int kBwdDqCounter = 16, kBwdDkvCounter = 24;  // words of the status block: items drawn by the tcgen05 kernels
+// Words of the status block: items drawn by the tcgen05 kernels; 1 once the preparation is over.
+constexpr int kBwdDqCounter = 16, kBwdDkvCounter = 24, kBwdPrepared = 32;
 
 struct BackwardArgs {
     const __nv_bfloat16 *q, *k, *v, *o, *d_o;
@@ -31,7 +32,7 @@ struct BackwardArgs {
     int32_t nqb, batch, Hq, Hkv, G;
     int32_t npairs;            // head pairs per KV group: ceil(G / 2)
     int32_t early;             // one wave of work: the next kernel may start beside this one's last blocks
-    int32_t prezero;           // dK and dV are cleared by the preparation (else: where needed, by the dQ kernel)
+    int32_t prezero;           // the preparation clears all of dK and dV (else a kernel of its own clears what needs it)
     float scale, scale_log2;
     long long wait_cycles;     // limit of every barrier wait of the tensor-core kernels
 };
