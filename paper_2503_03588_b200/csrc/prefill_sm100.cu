@@ -28,6 +28,8 @@
 #include <math.h>
 #include <stdlib.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "sm100_ptx.cuh"
 #include "tensor_map.cuh"
@@ -68,7 +70,7 @@ struct PrefillArgs {
     int64_t lse_sb, lse_sh;  // LSE strides (batch, head); the token stride is 1
     int64_t N, n_units;     // N: sequence length (variable-length batch: the longest one, which sizes the unit grid)
     int32_t nqb, batch, Hq, Hkv, G, nsub;
-    uint32_t inv_nsub, inv_Hkv, inv_nqb;  // floor(2^32 / d) of the three divisors of a unit index
+    uint32_t inv_nsub, inv_Hkv, inv_nqb, inv_batch;  // floor(2^32 / d) of the divisors of a unit index
     float scale_log2;
     long long wait_cycles;  // limit of every barrier wait, in clock cycles
 };
@@ -137,18 +139,30 @@ __device__ __forceinline__ uint32_t divmod(uint32_t u, uint32_t d, uint32_t inv,
 }
 
 // Unit index -> coordinates (the unit count fits in 30 bits; checked on the host).
+template <bool kRowsFirst>
 __device__ __forceinline__ Unit decode_unit(const PrefillArgs &a, uint32_t u)
 {
     Unit r;
     uint32_t rem;
-    // Order: head quad fastest, then query block (long rows first), then KV head, then batch entry:
-    // the CTAs work on one KV head at a time, whose K and V (67 MB at 128K tokens) stay in L2.
+    // Order: a group's heads fastest, then
+    //   kRowsFirst: KV head, batch entry, query block (long rows first): the units get shorter and shorter, so that the
+    //               CTAs, which take them in turn, end together;
+    //   else:       query block, KV head, batch entry: the CTAs work on one KV head at a time, whose K and V (67 MB at
+    //               128K tokens) stay in L2.
     u = divmod(u, (uint32_t)a.nsub, a.inv_nsub, rem);
     r.sub = (int32_t)rem;
-    u = divmod(u, (uint32_t)a.nqb, a.inv_nqb, rem);
-    r.i = a.nqb - 1 - (int32_t)rem;  // long rows first
-    r.b = (int32_t)divmod(u, (uint32_t)a.Hkv, a.inv_Hkv, rem);
-    r.hk = (int32_t)rem;
+    if (kRowsFirst) {
+        u = divmod(u, (uint32_t)a.Hkv, a.inv_Hkv, rem);
+        r.hk = (int32_t)rem;
+        u = divmod(u, (uint32_t)a.batch, a.inv_batch, rem);
+        r.b = (int32_t)rem;
+        r.i = a.nqb - 1 - (int32_t)u;
+    } else {
+        u = divmod(u, (uint32_t)a.nqb, a.inv_nqb, rem);
+        r.i = a.nqb - 1 - (int32_t)rem;
+        r.b = (int32_t)divmod(u, (uint32_t)a.Hkv, a.inv_Hkv, rem);
+        r.hk = (int32_t)rem;
+    }
     r.rs = a.row_ptr[r.i];
     r.n = a.row_ptr[r.i + 1] - r.rs;
     if (a.cu_seqlens) {
@@ -164,8 +178,22 @@ __device__ __forceinline__ Unit decode_unit(const PrefillArgs &a, uint32_t u)
     return r;
 }
 
-// kSlots: slots that have work (launch_prefill chooses); kF32: fp32 output.
-template <int D, int kSlots, bool kF32>
+// The units of a CTA: number k is the one at the CTA's place in round k of the grid; with kRowsFirst from the front in even
+// rounds and from the back in odd ones, since in every round the first places have the longer rows.
+template <bool kRowsFirst>
+struct UnitCursor {
+    uint32_t u = blockIdx.x;                               // the unit
+    uint32_t ahead = 2 * (gridDim.x - blockIdx.x) - 1;     // (kRowsFirst) how far the next one is from it
+    __device__ __forceinline__ uint32_t next() const { return u + (kRowsFirst ? ahead : gridDim.x); }
+    __device__ __forceinline__ void advance()
+    {
+        u = next();
+        if (kRowsFirst) ahead = 2 * gridDim.x - ahead;
+    }
+};
+
+// kSlots: slots that have work; kRowsFirst: order of the units (launch_prefill chooses both); kF32: fp32 output.
+template <int D, int kSlots, bool kF32, bool kRowsFirst>
 __global__ void __launch_bounds__(kThreads, 1)
 prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO,
@@ -248,15 +276,16 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             bool ok = true;
             // A unit's coordinates and its first block index are fetched while the previous unit's
             // loads are still waiting for ring space, the other block indices one block ahead.
-            auto next_unit = [&](uint32_t u, Unit &w, int32_t &j0) {
-                for (; u < (uint32_t)a.n_units; u += gridDim.x) {
-                    w = decode_unit(a, u);
+            UnitCursor<kRowsFirst> cur;
+            auto next_unit = [&](Unit &w, int32_t &j0) {
+                for (; cur.u < (uint32_t)a.n_units; cur.advance()) {
+                    w = decode_unit<kRowsFirst>(a, cur.u);
                     if (w.n > 0) {
                         j0 = a.col_idx[w.rs];
                         break;
                     }
                 }
-                return u;
+                return cur.u;
             };
             // Q tiles of unit number ul_q go to Q buffer ul_q & 1 once the unit two before has
             // issued its last S and its output, staged in that buffer, has left.  (Both barriers
@@ -280,10 +309,11 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             };
             Unit w, wn;
             int32_t j = 0, jnext = 0;
-            uint32_t u = next_unit(blockIdx.x, w, j);
+            uint32_t u = next_unit(w, j);
             if (u < (uint32_t)a.n_units) ok = load_q(w, 0);
             while (u < (uint32_t)a.n_units && ok) {
-                const uint32_t un = next_unit(u + gridDim.x, wn, jnext);
+                cur.advance();
+                const uint32_t un = next_unit(wn, jnext);
                 bool q_pending = un < (uint32_t)a.n_units;  // the next unit's Q tiles are still to be requested
                 for (int t = 0; t < w.n; ++t, ++kc) {
                     const int32_t jn = t + 1 < w.n ? a.col_idx[w.rs + t + 1] : 0;
@@ -374,15 +404,18 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                                       (acc || kk > 0) ? 1u : 0u);
             };
             auto unit_blocks = [&](uint32_t u) {
-                return __shfl_sync(0xffffffffu, u < (uint32_t)a.n_units ? decode_unit(a, u).n : 0, 0);
+                return __shfl_sync(0xffffffffu, u < (uint32_t)a.n_units ? decode_unit<kRowsFirst>(a, u).n : 0, 0);
             };
             // Next non-empty unit after u.  Its block count `n` is already loaded (`ahead`); the
             // count after that is requested now, so no unit boundary waits for a load.
-            auto next_unit = [&](uint32_t u, int &n, int &ahead) {
+            UnitCursor<kRowsFirst> cur;  // the unit that `ahead` is of
+            auto next_unit = [&](int &n, int &ahead) {
+                uint32_t u;
                 do {
-                    u += gridDim.x;
+                    u = cur.u;
+                    cur.advance();
                     n = ahead;
-                    ahead = unit_blocks(u + gridDim.x);
+                    ahead = unit_blocks(cur.u);
                 } while (u < (uint32_t)a.n_units && n <= 0);
                 return u;
             };
@@ -428,11 +461,11 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             };
             uint32_t kc = 0, ul = 0;
             int n = 0, nn = 0;  // key blocks of this unit and of the next
-            int ahead = unit_blocks(blockIdx.x);
-            uint32_t u = next_unit(blockIdx.x - gridDim.x, n, ahead);  // (the sum wraps back to blockIdx.x)
+            int ahead = unit_blocks(cur.u);
+            uint32_t u = next_unit(n, ahead);
             if (u < (uint32_t)a.n_units) qk_step(0, 0, true, n == 1, false);
             while (u < (uint32_t)a.n_units && ok) {
-                const uint32_t un = next_unit(u, nn, ahead);
+                const uint32_t un = next_unit(nn, ahead);
                 const bool has_next = un < (uint32_t)a.n_units;
                 for (int t = 0; t < n && ok; ++t) {
                     const uint32_t c = kc + t;
@@ -475,22 +508,23 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         // extent two units ahead, the row's last block index (needs the extent) one unit ahead.
         auto fetch_unit = [&](uint32_t u) {
             Unit r = {};
-            if (u < (uint32_t)a.n_units) r = decode_unit(a, u);
+            if (u < (uint32_t)a.n_units) r = decode_unit<kRowsFirst>(a, u);
             return r;
         };
         auto fetch_lastcol = [&](const Unit &r) { return r.n > 0 ? a.col_idx[r.rs + r.n - 1] : -1; };
-        Unit w_next = fetch_unit(blockIdx.x);
-        Unit w_next2 = fetch_unit(blockIdx.x + gridDim.x);
+        UnitCursor<kRowsFirst> cur;
+        Unit w_next = fetch_unit(cur.u);
+        Unit w_next2 = fetch_unit(cur.next());
         int32_t lastcol_next = fetch_lastcol(w_next);
         // Called once per unit, after the first step's hand-over (the issuer is busy with it then),
         // not between two units where the next logits are already waiting.
-        auto advance_metadata = [&](uint32_t u) {
+        auto advance_metadata = [&]() {
             w_next = w_next2;
             lastcol_next = fetch_lastcol(w_next);
-            w_next2 = fetch_unit(u + 2 * gridDim.x);
+            w_next2 = fetch_unit(cur.u + 2 * gridDim.x);  // (two rounds on, so the same place from the front or back)
         };
         const uint32_t n_units = (uint32_t)a.n_units;
-        for (uint32_t u = kSlots == 2 || s == 0 ? blockIdx.x : n_units; u < n_units && ok; u += gridDim.x) {
+        for (; (kSlots == 2 || s == 0) && cur.u < n_units && ok; cur.advance()) {
             const Unit w = w_next;
             const int32_t lastcol = lastcol_next;
             const int head_local = w.sub * 2 * kSlots + 2 * s + (row >> 6);
@@ -651,7 +685,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 ptx::tc_fence_before_sync();
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive(bar(BAR_P_FULL + 2 * s + (kc & 1)));
-                if (t == 0) advance_metadata(u);
+                if (t == 0) advance_metadata();
                 if (t + 1 == w.n) {
                     // Softmax denominators for the epilogue warps (they finish O / l).  The previous
                     // unit's must have been read: that also keeps this slot's statistics barrier at
@@ -672,7 +706,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 }
             }
             if (w.n > 0) ++ul;
-            else advance_metadata(u);
+            else advance_metadata();
         }
     } else if (warp >= 12) {
         // ------------------------------------------------------------------ epilogue
@@ -687,8 +721,8 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         const bool store_thread = threadIdx.x == 12 * 32;
         uint32_t ul = 0, ns = 0;  // units and staged slots so far
         bool ok = true;
-        for (uint32_t u = blockIdx.x; u < (uint32_t)a.n_units && ok; u += gridDim.x) {
-            const Unit w = decode_unit(a, u);
+        for (UnitCursor<kRowsFirst> cur; cur.u < (uint32_t)a.n_units && ok; cur.advance()) {
+            const Unit w = decode_unit<kRowsFirst>(a, cur.u);
             const int64_t tok = (int64_t)w.i * kBlk + qrow;
             // The unit's Q buffer is no longer read once its last P V has completed (every S of
             // the unit was issued before it); its output is staged there.
@@ -922,17 +956,17 @@ namespace pa {
 
 // The launch behind pa_prefill (cu_seqlens null) and pa_prefill_varlen (packed sequences:
 // p->seq_len is the longest one, tokens run over [0, total_tokens)).
-template <int D, int kSlots, bool kF32>
+template <int D, int kSlots, bool kF32, bool kRowsFirst>
 static pa_status launch_kernel(unsigned grid, cudaStream_t st, int device, const CUtensorMap &tmQ, const CUtensorMap &tmK,
                                const CUtensorMap &tmV, const CUtensorMap &tmO, const PrefillArgs &a)
 {
-    constexpr DeviceOnce once = (DeviceOnce)(ONCE_PREFILL_ATTR + 4 * (D == 64) + 2 * (kSlots == 1) + kF32);
+    constexpr DeviceOnce once = (DeviceOnce)(ONCE_PREFILL_ATTR + 8 * kRowsFirst + 4 * (D == 64) + 2 * (kSlots == 1) + kF32);
     if (pa_status s = device_once(device, once, [] {
-            return cudaFuncSetAttribute(prefill_kernel<D, kSlots, kF32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            return cudaFuncSetAttribute(prefill_kernel<D, kSlots, kF32, kRowsFirst>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)SmemMap<D>::kAlloc);
         }))
         return s;
-    PA_CUDA_OK(launch_pdl(prefill_kernel<D, kSlots, kF32>, dim3(grid), kThreads, SmemMap<D>::kAlloc, st, tmQ, tmK, tmV, tmO, a));
+    PA_CUDA_OK(launch_pdl(prefill_kernel<D, kSlots, kF32, kRowsFirst>, dim3(grid), kThreads, SmemMap<D>::kAlloc, st, tmQ, tmK, tmV, tmO, a));
     return PA_OK;
 }
 
@@ -1001,7 +1035,14 @@ static pa_status launch_prefill(const pa_prefill_params *p, const void *q, const
     a.nsub = (a.G + 2 * slots - 1) / (2 * slots);
     a.n_units = rows * a.nsub;
     auto inv32 = [](int32_t d) { return d == 1 ? 0xffffffffu : (uint32_t)((1ull << 32) / (uint64_t)d); };
-    a.inv_nsub = inv32(a.nsub); a.inv_Hkv = inv32(a.Hkv); a.inv_nqb = inv32(a.nqb);
+    a.inv_nsub = inv32(a.nsub); a.inv_Hkv = inv32(a.Hkv); a.inv_nqb = inv32(a.nqb); a.inv_batch = inv32(a.batch);
+    // The order that balances the CTAs is taken where they have more than one unit each and K and V of all heads may stay
+    // in L2 together, of whose 126 MB Q and O take their share: in a loop, 28 / 4 heads, the other order and this, 4001
+    // tokens (8 MB of K and V) 44.7 and 42.2 us, 8192 (17 MB) 93.6 and 90.9, 16100 (33 MB) 193.4 and 193.9, in 256-token
+    // blocks 523 and 505; 4 x 16384 tokens, 8 / 8 heads (268 MB) 500 and 520; packed prompts of 22 MB 125 and 119, of 95 MB
+    // 514 and 522.
+    const int64_t kv_bytes = (varlen ? total_tokens : p->batch * p->seq_len) * a.Hkv * D * 4;
+    const bool rows_first = a.n_units > dev.sms && kv_bytes <= (int64_t)48 << 20;
     if (a.n_units > (int64_t)0x3fffffff) return fail(PA_ERR_SHAPE, "too many work units (%lld)", (long long)a.n_units);
     const float scale = p->softmax_scale != 0.f ? p->softmax_scale : 1.0f / sqrtf((float)D);
     a.scale_log2 = scale * 1.4426950408889634f;
@@ -1032,13 +1073,18 @@ static pa_status launch_prefill(const pa_prefill_params *p, const void *q, const
                 return fail(PA_ERR_LAYOUT, "CSR check: %s (row %d)", what[found[0]], (int)found[1]);
         }
     }
-    auto launch = [&](auto kernel) { return kernel(grid, st, dev.device, tmQ, tmK, tmV, tmO, a); };
-    if (p->o_dtype == PA_F32) {
-        if (slots == 2) return launch(D == 128 ? launch_kernel<128, 2, true> : launch_kernel<64, 2, true>);
-        return launch(D == 128 ? launch_kernel<128, 1, true> : launch_kernel<64, 1, true>);
-    }
-    if (slots == 2) return launch(D == 128 ? launch_kernel<128, 2, false> : launch_kernel<64, 2, false>);
-    return launch(D == 128 ? launch_kernel<128, 1, false> : launch_kernel<64, 1, false>);
+    auto launch = [&](auto d, auto one_slot, auto f32, auto rows) {
+        return launch_kernel<d.value, one_slot.value ? 1 : 2, f32.value, rows.value>(grid, st, dev.device, tmQ, tmK, tmV, tmO, a);
+    };
+    auto choose = [](bool x, auto then) { return x ? then(std::true_type()) : then(std::false_type()); };
+    return choose(slots == 1, [&](auto one_slot) {
+        return choose(p->o_dtype == PA_F32, [&](auto f32) {
+            return choose(rows_first, [&](auto rows) {
+                return D == 128 ? launch(std::integral_constant<int, 128>(), one_slot, f32, rows)
+                                : launch(std::integral_constant<int, 64>(), one_slot, f32, rows);
+            });
+        });
+    });
 }
 
 }  // namespace pa

@@ -86,6 +86,24 @@ def test_large_groups_with_few_units(pa, oracle, G, D):
         _full_compare(pa, oracle, Q, K, V, 2, 1, what=f"G={G} D={D} blocks={blocks}")
 
 
+@pytest.mark.parametrize("N,batch,Hkv", [(64 * 37, 1, 4), (64 * 37 + 1, 1, 4), (64 * 75, 1, 4), (500, 3, 40), (64 * 20, 2, 60)])
+def test_orders_of_units_agree(pa, N, batch, Hkv):
+    """Whole rounds of the grid, one unit more and rounds that end early: the same rows in one call, whose units come row by
+    row, and beside so many other heads that they come head by head."""
+    G, D = 1, 64
+    Q, K, V = (si.bf16_randn((batch, N, h, D), 1700 + i).cuda() for i, h in enumerate((G * Hkv, Hkv, Hkv)))
+    many = (48 << 20) // (batch * N * D * 4) + 1 + Hkv   # KV heads at which the order changes
+    rp, ci = pa.pa_build_layout(N, 64, 2, 1)
+    o, lse, ws = pa.pa_prefill(Q, K, V, rp, ci)
+    pa.pa_prefill_status(ws)
+    rest = many - Hkv
+    more = [torch.cat([x, torch.zeros((batch, N, rest, D), dtype=x.dtype, device="cuda")], dim=2) for x in (Q, K, V)]
+    o2, lse2, ws = pa.pa_prefill(*more, rp, ci)
+    pa.pa_prefill_status(ws)
+    assert torch.equal(o, o2[:, :, :Hkv]) and torch.equal(lse, lse2[:, :Hkv])
+    assert (o2[:, :, Hkv:] == 0).all()
+
+
 def test_peaky_logits_fp32_output_and_custom_scale(pa, oracle):
     N, Hq, Hkv, D = 1500, 14, 2, 128
     Q, K, V = si.bf16_randn((1, N, Hq, D), 1), si.bf16_randn((1, N, Hkv, D), 2, 3.0), si.bf16_randn((1, N, Hkv, D), 3)
