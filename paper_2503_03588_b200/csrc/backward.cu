@@ -170,7 +170,10 @@ __global__ void __launch_bounds__(kPrepThreads) backward_prep_kernel(const Backw
     __shared__ float s_delta[kPrepHeads][kPrepTokens + 1];
     constexpr int kLanes = D / 8;             // lanes that share a head's row, 16 bytes each
     constexpr int kHeadsPerStep = 32 / kLanes;
-    constexpr int kUnroll = 7;                // (28 heads of 128 features: two rounds)
+    // Heads a thread takes at a time.  With more blocks per SM doing less each the loads overlap better than within a thread
+    // (whole backward pass with 1, 2, 3 and 7: 16 / 4 heads of 64 features, 2 x 32K tokens 1031, 1029, 1036 and 1042 us;
+    // 28 / 4 heads of 128, 4001 tokens 155, 152, 155 and 154).
+    constexpr int kUnroll = 2;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, sub = lane % kLanes, hsub = lane / kLanes;
     const int64_t groups = (a.N + kPrepTokens - 1) / kPrepTokens, grp = (int64_t)blockIdx.x - n_csc;
     const int64_t b = grp / groups, t0 = (grp - b * groups) * kPrepTokens, t = t0 + warp;

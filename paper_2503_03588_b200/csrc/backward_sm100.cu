@@ -1096,7 +1096,7 @@ __global__ void __launch_bounds__(kClearThreads) backward_clear_kernel(const Bac
         for (int32_t b = 0; b < a.batch; ++b) {
             float4 *zk = reinterpret_cast<float4 *>(a.dk) + (b * a.N + tok0) * per_token;
             float4 *zv = reinterpret_cast<float4 *>(a.dv) + (b * a.N + tok0) * per_token;
-            for (int64_t x = threadIdx.x; x < toks * per_token; x += kClearThreads)
+            for (int64_t x = blockIdx.y * kClearThreads + threadIdx.x; x < toks * per_token; x += gridDim.y * kClearThreads)
                 zk[x] = zv[x] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
     }
@@ -1134,7 +1134,7 @@ static pa_status launch_tc(const BackwardArgs &a, const pa_prefill_params *p, in
     if (dq_items > (int64_t)0x3fffffff || dkv_items > (int64_t)0x3fffffff)
         return fail(PA_ERR_SHAPE, "too many work items (%lld, %lld)", (long long)dq_items, (long long)dkv_items);
     if (!a.prezero)
-        PA_CUDA_OK(launch_pdl(backward_clear_kernel, dim3((unsigned)(a.nqb < 4 * sms ? a.nqb : 4 * sms)), kClearThreads, 0, st, a,
+        PA_CUDA_OK(launch_pdl(backward_clear_kernel, dim3((unsigned)(a.nqb < sms ? a.nqb : sms), 8), kClearThreads, 0, st, a,
                               (int32_t)D));
     PA_CUDA_OK(launch_pdl(dkv_kernel<D>, dim3((unsigned)(dkv_items < sms ? dkv_items : sms)), kTcThreads, DkvCfg<D>::kAlloc, st,
                           tmQ, tmG, tmK, tmV, a, (uint32_t)dkv_items));
