@@ -192,14 +192,20 @@ struct UnitCursor {
     }
 };
 
-// kSlots: slots that have work; kRowsFirst: order of the units (launch_prefill chooses both); kF32: fp32 output.
-template <int D, int kSlots, bool kF32, bool kRowsFirst>
+// What a call's length asks for: kOne, at most a unit per CTA; kMid, the units row by row; kLong, head by head, and the
+// heads that a group's last unit lacks are zeros.
+enum Length : int { kOne, kMid, kLong };
+
+// kSlots: slots that have work, kLength (launch_prefill chooses both); kF32: fp32 output.
+template <int D, int kSlots, bool kF32, Length kLength>
 __global__ void __launch_bounds__(kThreads, 1)
 prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO,
                const PrefillArgs a)
 {
     using SM = SmemMap<D>;
+    constexpr bool kRowsFirst = kLength == kMid;
+    constexpr bool kZeros = kLength == kLong;  // (the Q map has a group dimension)
     constexpr int DH = D / 64;  // 64-feature (128-byte) sub-tiles per row
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -302,9 +308,14 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 ptx::mbar_expect_tx(bar(BAR_Q_FULL + qb), kSlots * SM::kQSlot);
                 for (int s = 0; s < kSlots; ++s)
                     for (int dh = 0; dh < DH; ++dh)
-                        ptx::tma_load_4d(smem_base + SM::kQ + qb * SM::kQBuf + s * SM::kQSlot + dh * SM::kQSub, &tmQ,
-                                         bar(BAR_Q_FULL + qb), dh * 64, w.tok0 + w.i * kBlk,
-                                         w.hk * a.G + w.sub * 2 * kSlots + 2 * s, w.bt);
+                        if constexpr (kZeros)
+                            ptx::tma_load_5d(smem_base + SM::kQ + qb * SM::kQBuf + s * SM::kQSlot + dh * SM::kQSub, &tmQ,
+                                             bar(BAR_Q_FULL + qb), dh * 64, w.tok0 + w.i * kBlk, w.sub * 2 * kSlots + 2 * s,
+                                             w.hk, w.bt);
+                        else
+                            ptx::tma_load_4d(smem_base + SM::kQ + qb * SM::kQBuf + s * SM::kQSlot + dh * SM::kQSub, &tmQ,
+                                             bar(BAR_Q_FULL + qb), dh * 64, w.tok0 + w.i * kBlk,
+                                             w.hk * a.G + w.sub * 2 * kSlots + 2 * s, w.bt);
                 return true;
             };
             Unit w, wn;
@@ -581,6 +592,10 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                         for (int e = 0; e < 4; ++e) mx4[e] = fmaxf(mx4[e], __uint_as_float(sr[c + e]));
                     }
                     m = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * sl2;
+                    // A group's missing heads get P = 0: products with zeros take less power, of which long calls have no more than
+                    // enough (28 / 4 heads, whose padding is an eighth of the rows, 128K tokens in a loop: 1933 us, 1915 with
+                    // zeros in Q and P; the cycles stay the same, the clock rises from 1635 to 1660 MHz).
+                    if (kZeros && head_local >= a.G) m = INFINITY;
                 }
                 const uint64_t negm_2 = ptx::pack_f32x2(-m, -m);
                 uint64_t sum2[2] = {0ull, 0ull};
@@ -956,17 +971,17 @@ namespace pa {
 
 // The launch behind pa_prefill (cu_seqlens null) and pa_prefill_varlen (packed sequences:
 // p->seq_len is the longest one, tokens run over [0, total_tokens)).
-template <int D, int kSlots, bool kF32, bool kRowsFirst>
+template <int D, int kSlots, bool kF32, Length kLength>
 static pa_status launch_kernel(unsigned grid, cudaStream_t st, int device, const CUtensorMap &tmQ, const CUtensorMap &tmK,
                                const CUtensorMap &tmV, const CUtensorMap &tmO, const PrefillArgs &a)
 {
-    constexpr DeviceOnce once = (DeviceOnce)(ONCE_PREFILL_ATTR + 8 * kRowsFirst + 4 * (D == 64) + 2 * (kSlots == 1) + kF32);
+    constexpr DeviceOnce once = (DeviceOnce)(ONCE_PREFILL_ATTR + 8 * (int)kLength + 4 * (D == 64) + 2 * (kSlots == 1) + kF32);
     if (pa_status s = device_once(device, once, [] {
-            return cudaFuncSetAttribute(prefill_kernel<D, kSlots, kF32, kRowsFirst>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            return cudaFuncSetAttribute(prefill_kernel<D, kSlots, kF32, kLength>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)SmemMap<D>::kAlloc);
         }))
         return s;
-    PA_CUDA_OK(launch_pdl(prefill_kernel<D, kSlots, kF32, kRowsFirst>, dim3(grid), kThreads, SmemMap<D>::kAlloc, st, tmQ, tmK, tmV, tmO, a));
+    PA_CUDA_OK(launch_pdl(prefill_kernel<D, kSlots, kF32, kLength>, dim3(grid), kThreads, SmemMap<D>::kAlloc, st, tmQ, tmK, tmV, tmO, a));
     return PA_OK;
 }
 
@@ -992,18 +1007,37 @@ static pa_status launch_prefill(const pa_prefill_params *p, const void *q, const
     DeviceInfo dev;
     if (pa_status s = current_sm100_device(&dev)) return s;
 
+    const int G = p->n_q_heads / p->n_kv_heads;
+    // Slots.  Groups of one or two query heads have nothing for a second one: its roles stay idle then, and a step is as
+    // long as one slot's chain alone.  With one head per group 2K tokens, 2 heads of 64 features take 9.1 us instead of
+    // 11.4, 32K tokens, 8 heads of 128 features 266 us instead of 355; with two heads per group 8K tokens, batch 2,
+    // 8 KV heads 118 us instead of 156 (burst).  Larger groups are taken two heads a CTA, too, where every such unit
+    // finds an SM of its own: then nothing counts but the length of the chain (in a graph, 28 / 4 heads: 64 tokens 6.3 ->
+    // 5.3 us, 500 tokens 11.6 -> 9.9; 8 / 2 heads: 2048 tokens 13.7 -> 11.5).  One unit more and two rounds of one slot
+    // take longer than one of two.
+    const int64_t rows = (int64_t)p->batch * nqb * p->n_kv_heads;
+    const int slots = G <= 2 || rows * ((G + 1) / 2) <= dev.sms ? 1 : 2;
+    // The order that balances the CTAs is taken where K and V of all heads may stay in L2 together, of whose 126 MB Q and
+    // O take their share: in a loop, 28 / 4 heads, the other order and this, 4001 tokens (8 MB of K and V) 44.7 and 42.2 us,
+    // 8192 (17 MB) 93.6 and 90.9, 16100 (33 MB) 193.4 and 193.9, in 256-token blocks 523 and 505; 4 x 16384 tokens, 8 / 8
+    // heads (268 MB) 500 and 520; packed prompts of 22 MB 125 and 119, of 95 MB 514 and 522.  The calls beyond are
+    // those that last: what saves power goes with them (it costs calls of one unit per CTA 1.4 %).
+    const int64_t kv_bytes = (varlen ? total_tokens : p->batch * p->seq_len) * p->n_kv_heads * p->head_dim * 4;
+    const int64_t units = rows * ((G + 2 * slots - 1) / (2 * slots));
+    const Length length = units <= dev.sms ? kOne : kv_bytes <= (int64_t)48 << 20 ? kMid : slots == 2 ? kLong : kOne;
+
     // Tensor maps (cached per buffer and shape): a Q box holds the two heads of a tile, K, V and O
     // boxes one head.
     CUtensorMap tmQ, tmK, tmV, tmO;
     const int D = p->head_dim;
     auto map_of = [&](const void *base, int heads, const pa_strides &st, int box_heads, const char *what, CUtensorMap *m,
-                      bool f32 = false) {
+                      bool f32 = false, int group = 0) {
         // (packed sequences: one "batch" entry of total_tokens tokens)
         const TensorMapKey key = {base, varlen ? total_tokens : p->seq_len, st.seq, st.head, varlen ? 0 : st.batch, dev.device, D,
-                                  heads, varlen ? 1 : p->batch, box_heads, kBlk, f32 ? 1 : 0};
+                                  heads, varlen ? 1 : p->batch, box_heads, kBlk, f32 ? 1 : 0, group};
         return get_tensor_map(key, what, m);
     };
-    if (pa_status s = map_of(q, p->n_q_heads, p->q, 2, "q", &tmQ)) return s;
+    if (pa_status s = map_of(q, p->n_q_heads, p->q, 2, "q", &tmQ, false, length == kLong ? G : 0)) return s;
     if (pa_status s = map_of(k, p->n_kv_heads, p->k, 1, "k", &tmK)) return s;
     if (pa_status s = map_of(v, p->n_kv_heads, p->v, 1, "v", &tmV)) return s;
     if (pa_status s = map_of(o, p->n_q_heads, p->o, 1, "o", &tmO, p->o_dtype == PA_F32)) return s;
@@ -1022,27 +1056,11 @@ static pa_status launch_prefill(const pa_prefill_params *p, const void *q, const
     a.N = p->seq_len;
     a.nqb = (int32_t)nqb;
     a.batch = p->batch; a.Hq = p->n_q_heads; a.Hkv = p->n_kv_heads;
-    a.G = p->n_q_heads / p->n_kv_heads;
-    // Slots.  Groups of one or two query heads have nothing for a second one: its roles stay idle then, and a step is as
-    // long as one slot's chain alone.  With one head per group 2K tokens, 2 heads of 64 features take 9.1 us instead of
-    // 11.4, 32K tokens, 8 heads of 128 features 266 us instead of 355; with two heads per group 8K tokens, batch 2,
-    // 8 KV heads 118 us instead of 156 (burst).  Larger groups are taken two heads a CTA, too, where every such unit
-    // finds an SM of its own: then nothing counts but the length of the chain (in a graph, 28 / 4 heads: 64 tokens 6.3 ->
-    // 5.3 us, 500 tokens 11.6 -> 9.9; 8 / 2 heads: 2048 tokens 13.7 -> 11.5).  One unit more and two rounds of one slot
-    // take longer than one of two.
-    const int64_t rows = (int64_t)p->batch * nqb * a.Hkv;
-    const int slots = a.G <= 2 || rows * ((a.G + 1) / 2) <= dev.sms ? 1 : 2;
+    a.G = G;
     a.nsub = (a.G + 2 * slots - 1) / (2 * slots);
-    a.n_units = rows * a.nsub;
+    a.n_units = units;
     auto inv32 = [](int32_t d) { return d == 1 ? 0xffffffffu : (uint32_t)((1ull << 32) / (uint64_t)d); };
     a.inv_nsub = inv32(a.nsub); a.inv_Hkv = inv32(a.Hkv); a.inv_nqb = inv32(a.nqb); a.inv_batch = inv32(a.batch);
-    // The order that balances the CTAs is taken where they have more than one unit each and K and V of all heads may stay
-    // in L2 together, of whose 126 MB Q and O take their share: in a loop, 28 / 4 heads, the other order and this, 4001
-    // tokens (8 MB of K and V) 44.7 and 42.2 us, 8192 (17 MB) 93.6 and 90.9, 16100 (33 MB) 193.4 and 193.9, in 256-token
-    // blocks 523 and 505; 4 x 16384 tokens, 8 / 8 heads (268 MB) 500 and 520; packed prompts of 22 MB 125 and 119, of 95 MB
-    // 514 and 522.
-    const int64_t kv_bytes = (varlen ? total_tokens : p->batch * p->seq_len) * a.Hkv * D * 4;
-    const bool rows_first = a.n_units > dev.sms && kv_bytes <= (int64_t)48 << 20;
     if (a.n_units > (int64_t)0x3fffffff) return fail(PA_ERR_SHAPE, "too many work units (%lld)", (long long)a.n_units);
     const float scale = p->softmax_scale != 0.f ? p->softmax_scale : 1.0f / sqrtf((float)D);
     a.scale_log2 = scale * 1.4426950408889634f;
@@ -1073,18 +1091,17 @@ static pa_status launch_prefill(const pa_prefill_params *p, const void *q, const
                 return fail(PA_ERR_LAYOUT, "CSR check: %s (row %d)", what[found[0]], (int)found[1]);
         }
     }
-    auto launch = [&](auto d, auto one_slot, auto f32, auto rows) {
-        return launch_kernel<d.value, one_slot.value ? 1 : 2, f32.value, rows.value>(grid, st, dev.device, tmQ, tmK, tmV, tmO, a);
+    auto launch = [&](auto d, auto f32) {
+        constexpr int kD = decltype(d)::value;
+        constexpr bool kF32 = decltype(f32)::value;
+        auto go = [&](auto kernel) { return kernel(grid, st, dev.device, tmQ, tmK, tmV, tmO, a); };
+        if (slots == 1) return go(length == kMid ? launch_kernel<kD, 1, kF32, kMid> : launch_kernel<kD, 1, kF32, kOne>);
+        return go(length == kMid    ? launch_kernel<kD, 2, kF32, kMid>
+                  : length == kLong ? launch_kernel<kD, 2, kF32, kLong>
+                                    : launch_kernel<kD, 2, kF32, kOne>);
     };
-    auto choose = [](bool x, auto then) { return x ? then(std::true_type()) : then(std::false_type()); };
-    return choose(slots == 1, [&](auto one_slot) {
-        return choose(p->o_dtype == PA_F32, [&](auto f32) {
-            return choose(rows_first, [&](auto rows) {
-                return D == 128 ? launch(std::integral_constant<int, 128>(), one_slot, f32, rows)
-                                : launch(std::integral_constant<int, 64>(), one_slot, f32, rows);
-            });
-        });
-    });
+    auto launch_of = [&](auto d) { return p->o_dtype == PA_F32 ? launch(d, std::true_type()) : launch(d, std::false_type()); };
+    return D == 128 ? launch_of(std::integral_constant<int, 128>()) : launch_of(std::integral_constant<int, 64>());
 }
 
 }  // namespace pa

@@ -86,22 +86,23 @@ def test_large_groups_with_few_units(pa, oracle, G, D):
         _full_compare(pa, oracle, Q, K, V, 2, 1, what=f"G={G} D={D} blocks={blocks}")
 
 
-@pytest.mark.parametrize("N,batch,Hkv", [(64 * 37, 1, 4), (64 * 37 + 1, 1, 4), (64 * 75, 1, 4), (500, 3, 40), (64 * 20, 2, 60)])
-def test_orders_of_units_agree(pa, N, batch, Hkv):
+@pytest.mark.parametrize("N,batch,Hkv,G", [(64 * 37, 1, 4, 1), (64 * 37 + 1, 1, 4, 3), (64 * 75, 1, 4, 1), (500, 3, 40, 5),
+                                           (64 * 20, 2, 60, 1)])
+def test_orders_of_units_agree(pa, N, batch, Hkv, G):
     """Whole rounds of the grid, one unit more and rounds that end early: the same rows in one call, whose units come row by
-    row, and beside so many other heads that they come head by head."""
-    G, D = 1, 64
+    row, and beside so many other heads that they come head by head (with zeros for the heads that odd groups lack)."""
+    D = 64
     Q, K, V = (si.bf16_randn((batch, N, h, D), 1700 + i).cuda() for i, h in enumerate((G * Hkv, Hkv, Hkv)))
-    many = (48 << 20) // (batch * N * D * 4) + 1 + Hkv   # KV heads at which the order changes
+    rest = (48 << 20) // (batch * N * D * 4) + 1   # KV heads beyond which the order changes
     rp, ci = pa.pa_build_layout(N, 64, 2, 1)
     o, lse, ws = pa.pa_prefill(Q, K, V, rp, ci)
     pa.pa_prefill_status(ws)
-    rest = many - Hkv
-    more = [torch.cat([x, torch.zeros((batch, N, rest, D), dtype=x.dtype, device="cuda")], dim=2) for x in (Q, K, V)]
+    more = [torch.cat([x, torch.zeros((batch, N, g * rest, D), dtype=x.dtype, device="cuda")], dim=2)
+            for x, g in ((Q, G), (K, 1), (V, 1))]
     o2, lse2, ws = pa.pa_prefill(*more, rp, ci)
     pa.pa_prefill_status(ws)
-    assert torch.equal(o, o2[:, :, :Hkv]) and torch.equal(lse, lse2[:, :Hkv])
-    assert (o2[:, :, Hkv:] == 0).all()
+    assert torch.equal(o, o2[:, :, :G * Hkv]) and torch.equal(lse, lse2[:, :G * Hkv])
+    assert (o2[:, :, G * Hkv:] == 0).all()
 
 
 def test_peaky_logits_fp32_output_and_custom_scale(pa, oracle):
