@@ -257,12 +257,12 @@ size_t pa_decode_workspace_bytes(const pa_decode_params *p);
  * o: device [batch, n_q_heads, head_dim] contiguous, o_dtype.  lse: device fp32
  * [batch, n_q_heads].  When a row's window, power-of-two and sink candidates number at most 32
  * (window_blocks + sink_blocks + log2 of the row count: any default-window row up to millions of
- * tokens) the row kernel runs: a row's key blocks are dealt to R chunks; in each CTA a producer
- * warp fetches the blocks of its chunk by TMA into a ring of shared-memory stages and four warps
- * run an online softmax over them.  Small calls (batch x n_kv_heads up to the number of SMs, rows of
- * more than one block) are one launch in which the R CTAs of a row form a thread-block cluster and
+ * tokens) a row's key blocks are dealt to R chunks, which are fetched by TMA into a ring of
+ * shared-memory stages and run through an online softmax.  Small calls (batch x n_kv_heads up to the
+ * number of SMs, rows of more than one block) take the cluster kernel: one launch in which the R CTAs
+ * of a row form a thread-block cluster and
  * merge their results through distributed shared memory with the log-sum-exp rule
- * m = max m_c, l = sum l_c e^(m_c - m), o = sum o_c e^(m_c - m) / l.  Larger calls run a
+ * m = max m_c, l = sum l_c e^(m_c - m), o = sum o_c e^(m_c - m) / l.  Larger calls take the row kernel, a
  * persistent grid (two CTAs per SM) over the (row, chunk) items and, unless R is 1, a second small
  * kernel that merges each row's R partial results from the workspace.  Rows with more candidates
  * take two kernels: partial attention per (sequence, KV head, block) into the workspace, then
@@ -270,7 +270,7 @@ size_t pa_decode_workspace_bytes(const pa_decode_params *p);
  * be given; its first word is a status block (see pa_decode_status).
  * Calls that share a workspace must not overlap on the GPU.  Environment switches (for tests and
  * measurements, see pa_reload_environment): PA_DECODE_PATH=splitk forces the two-kernel path,
- * =cluster / =persist the two forms of the row kernel; PA_DECODE_CLUSTER=n (1..8) sets R (default:
+ * =cluster / =persist one of the other two kernels; PA_DECODE_CLUSTER=n (1..8) sets R (default:
  * for small calls as many CTAs per row as run all at once, for large ones one chunk per row);
  * PA_DECODE_STAGES=n (1..6) the number of key blocks a CTA keeps
  * in flight; PA_DECODE_CTAS_PER_SM=n the size of the persistent grid (default 2 per SM). */

@@ -1355,8 +1355,9 @@ static pa_status launch_decode(const DecodeShape &p, const void *q, const void *
         int R = env.decode_cluster, fit = 0;  // fit: clusters of R CTAs that the device holds at once
         if (cluster && R == 0) {
             // As many CTAs per row as run all at once: a second wave of clusters nearly doubles the call's latency
-            // (with an earlier kernel, 4000 tokens, G = 7, head_dim 128: 74 rows in clusters of four 13.0 us, of three 8.2).  How many clusters fit is asked of the device: all CTAs of a cluster lie
-            // within one GPU processing cluster, which may leave places that no further cluster fits in.
+            // (with an earlier kernel, 4000 tokens, G = 7, head_dim 128: 74 rows in clusters of four 13.0 us, of three
+            // 8.2).  How many clusters fit is asked of the device: all CTAs of a cluster lie within one GPU processing
+            // cluster, which may leave places that no further cluster fits in.
             R = (int)(persistent_ctas / rows_in_call);
             if (R > max_R) R = max_R;
             for (; R > 1; --R) {

@@ -192,9 +192,9 @@ struct UnitCursor {
     }
 };
 
-// What a call's length asks for: kOne, at most a unit per CTA; kMid, the units row by row; kLong, head by head, and the
-// heads that a group's last unit lacks are zeros.
-enum Length : int { kOne, kMid, kLong };
+// What a call's length asks for: kOne, at most a unit per CTA; kMid, the units row by row; kMidLong, so, too, and the heads
+// that a group's last unit lacks are zeros; kLong, zeros, but head by head.
+enum Length : int { kOne, kMid, kMidLong, kLong };
 
 // kSlots: slots that have work, kLength (launch_prefill chooses both); kF32: fp32 output.
 template <int D, int kSlots, bool kF32, Length kLength>
@@ -204,8 +204,8 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                const PrefillArgs a)
 {
     using SM = SmemMap<D>;
-    constexpr bool kRowsFirst = kLength == kMid;
-    constexpr bool kZeros = kLength == kLong;  // (the Q map has a group dimension)
+    constexpr bool kRowsFirst = kLength == kMid || kLength == kMidLong;
+    constexpr bool kZeros = kLength == kMidLong || kLength == kLong;  // (the Q map has a group dimension)
     constexpr int DH = D / 64;  // 64-feature (128-byte) sub-tiles per row
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -1021,10 +1021,15 @@ static pa_status launch_prefill(const pa_prefill_params *p, const void *q, const
     // O take their share: in a loop, 28 / 4 heads, the other order and this, 4001 tokens (8 MB of K and V) 44.7 and 42.2 us,
     // 8192 (17 MB) 93.6 and 90.9, 16100 (33 MB) 193.4 and 193.9, in 256-token blocks 523 and 505; 4 x 16384 tokens, 8 / 8
     // heads (268 MB) 500 and 520; packed prompts of 22 MB 125 and 119, of 95 MB 514 and 522.  The calls beyond are
-    // those that last: what saves power goes with them (it costs calls of one unit per CTA 1.4 %).
+    // those that last, and the zeros that save power go with them (they cost calls of one unit per CTA 1.4 %), and with
+    // calls of more than six rounds of the grid: in a loop, 28 / 4 heads, 16384 tokens 203 -> 201.5 us, in 256-token blocks
+    // 523 -> 518; 4001 tokens, 3.4 rounds, no difference.
     const int64_t kv_bytes = (varlen ? total_tokens : p->batch * p->seq_len) * p->n_kv_heads * p->head_dim * 4;
     const int64_t units = rows * ((G + 2 * slots - 1) / (2 * slots));
-    const Length length = units <= dev.sms ? kOne : kv_bytes <= (int64_t)48 << 20 ? kMid : slots == 2 ? kLong : kOne;
+    const Length length = units <= dev.sms                    ? kOne
+                          : kv_bytes > (int64_t)48 << 20      ? (slots == 2 ? kLong : kOne)
+                          : slots == 2 && units > 6 * dev.sms ? kMidLong
+                                                              : kMid;
 
     // Tensor maps (cached per buffer and shape): a Q box holds the two heads of a tile, K, V and O
     // boxes one head.
@@ -1037,7 +1042,7 @@ static pa_status launch_prefill(const pa_prefill_params *p, const void *q, const
                                   heads, varlen ? 1 : p->batch, box_heads, kBlk, f32 ? 1 : 0, group};
         return get_tensor_map(key, what, m);
     };
-    if (pa_status s = map_of(q, p->n_q_heads, p->q, 2, "q", &tmQ, false, length == kLong ? G : 0)) return s;
+    if (pa_status s = map_of(q, p->n_q_heads, p->q, 2, "q", &tmQ, false, length == kMidLong || length == kLong ? G : 0)) return s;
     if (pa_status s = map_of(k, p->n_kv_heads, p->k, 1, "k", &tmK)) return s;
     if (pa_status s = map_of(v, p->n_kv_heads, p->v, 1, "v", &tmV)) return s;
     if (pa_status s = map_of(o, p->n_q_heads, p->o, 1, "o", &tmO, p->o_dtype == PA_F32)) return s;
@@ -1096,9 +1101,10 @@ static pa_status launch_prefill(const pa_prefill_params *p, const void *q, const
         constexpr bool kF32 = decltype(f32)::value;
         auto go = [&](auto kernel) { return kernel(grid, st, dev.device, tmQ, tmK, tmV, tmO, a); };
         if (slots == 1) return go(length == kMid ? launch_kernel<kD, 1, kF32, kMid> : launch_kernel<kD, 1, kF32, kOne>);
-        return go(length == kMid    ? launch_kernel<kD, 2, kF32, kMid>
-                  : length == kLong ? launch_kernel<kD, 2, kF32, kLong>
-                                    : launch_kernel<kD, 2, kF32, kOne>);
+        return go(length == kMid       ? launch_kernel<kD, 2, kF32, kMid>
+                  : length == kMidLong ? launch_kernel<kD, 2, kF32, kMidLong>
+                  : length == kLong    ? launch_kernel<kD, 2, kF32, kLong>
+                                       : launch_kernel<kD, 2, kF32, kOne>);
     };
     auto launch_of = [&](auto d) { return p->o_dtype == PA_F32 ? launch(d, std::true_type()) : launch(d, std::false_type()); };
     return D == 128 ? launch_of(std::integral_constant<int, 128>()) : launch_of(std::integral_constant<int, 64>());
