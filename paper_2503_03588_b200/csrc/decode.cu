@@ -746,8 +746,9 @@ struct ClusterSmem {
     static constexpr uint32_t kSub = kDecBlock * 128;   // 64 keys x 64 features
     static constexpr uint32_t kTile = kSub * (D / 64);  // one K or V block
     static constexpr uint32_t kStage = 2 * kTile;       // K + V of one key block
-    static constexpr uint32_t kPPitch = 2 * kDecBlock * 2 + 16;  // weights of a head: 128 keys, bf16; the pad spreads the banks
-    static constexpr uint32_t kMax = kMaxGroup * kPPitch;        // (behind the weights) [head][warp] maxima
+    // Weights of a head: 128 keys, bf16; the pad spreads the banks.  Rows 8 .. 15: what that rounding left of them.
+    static constexpr uint32_t kPPitch = 2 * kDecBlock * 2 + 16;
+    static constexpr uint32_t kMax = 2 * kMaxGroup * kPPitch;  // (behind the weights) [head][warp] maxima
     static constexpr uint32_t kSum = kMax + kMaxGroup * kClusterWarps * 4;  // [head][warp] sums
     // What the row's CTAs send to the CTA that merges a head: per sending CTA and head slot, o[D], m, l.
     // R senders x ceil(8 / R) heads of an owner is at most 14 entries (R = 7).
@@ -862,8 +863,8 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     const int k_key = 16 * (wid & 3) + ((lane >> 4) << 3) + (lane & 7), k_ch = (lane >> 3) & 1;
     const uint32_t p_mine = rest + (uint32_t)g * SM::kPPitch + (uint32_t)(16 * wid + 2 * t) * 2u;
     const uint32_t stat_mine = (uint32_t)(g * kClusterWarps + wid) * 4u, stat_row = (uint32_t)(g * kClusterWarps) * 4u;
-    // P as the A operand by ldmatrix: matrices of 8 heads x 8 keys.
-    const uint32_t p_frag = rest + (uint32_t)(lane & 7) * SM::kPPitch + (uint32_t)(lane >> 3) * 16u;
+    // P as the A operand by ldmatrix: 16 rows (the heads, and their weights' remainders) x 16 keys.
+    const uint32_t p_frag = rest + (uint32_t)(lane & 15) * SM::kPPitch + (uint32_t)(lane >> 4) * 16u;
     const int per = stages > 1 ? 2 : 1;  // blocks at a time
     float m_run = -INFINITY, l_run = 0.f;  // of head g: the CTA's maximum, this warp's sum
     float acc[NT][4];
@@ -927,8 +928,17 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         const float alpha = ptx::ex2(m_run - m_new);  // 0 at first
         const float p0 = ptx::ex2(sx[0] - m_new), p1 = ptx::ex2(sx[1] - m_new);
         const float p2 = ptx::ex2(sx[2] - m_new), p3 = ptx::ex2(sx[3] - m_new);
-        ptx::st_shared(p_mine, ptx::cvt_bf16x2(p0, p1));
-        ptx::st_shared(p_mine + 16, ptx::cvt_bf16x2(p2, p3));
+        // A weight is split in two bf16 parts, of which the MMA's rows 8 .. 15, otherwise empty, take the second.  All keys
+        // share one maximum here (in decode_row_kernel each warp's largest weight is 1, exact in bf16), and with the first
+        // part alone the error against 64 bits was 1.2 to 2.5 times that kernel's.
+        const uint32_t h01 = ptx::cvt_bf16x2(p0, p1), h23 = ptx::cvt_bf16x2(p2, p3);
+        ptx::st_shared(p_mine, h01);
+        ptx::st_shared(p_mine + 16, h23);
+        auto left = [](float x, float y, uint32_t h) {
+            return ptx::cvt_bf16x2(x - __uint_as_float(h << 16), y - __uint_as_float(h & 0xffff0000u));
+        };
+        ptx::st_shared(p_mine + kMaxGroup * SM::kPPitch, left(p0, p1, h01));
+        ptx::st_shared(p_mine + kMaxGroup * SM::kPPitch + 16, left(p2, p3, h23));
         float lsum = (p0 + p1) + (p2 + p3);
         lsum += __shfl_xor_sync(0xffffffffu, lsum, 1);
         lsum += __shfl_xor_sync(0xffffffffu, lsum, 2);
@@ -941,6 +951,8 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         for (int e = 0; e < NT; ++e) {
             acc[e][0] *= alpha;
             acc[e][1] *= alpha;
+            acc[e][2] *= alpha;
+            acc[e][3] *= alpha;
         }
 #pragma unroll 1
         for (int x = 0; x < blocks; ++x) {
@@ -948,10 +960,10 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
             wait_bar(bar_vfull(s), (uint32_t)((i0 + x) / stages) & 1, 3);
             __syncwarp();
             const uint32_t sv = smem_base + (uint32_t)s * SM::kStage + SM::kTile;
-            uint32_t pf[4][2], vf[4][2 * NT];
+            uint32_t pf[4][4], vf[4][2 * NT];
 #pragma unroll
-            for (int ks = 0; ks < 4; ks += 2)
-                ptx::ldmatrix_x4(p_frag + (uint32_t)(64 * x + 16 * ks) * 2u, pf[ks][0], pf[ks][1], pf[ks + 1][0], pf[ks + 1][1]);
+            for (int ks = 0; ks < 4; ++ks)
+                ptx::ldmatrix_x4(p_frag + (uint32_t)(64 * x + 16 * ks) * 2u, pf[ks][0], pf[ks][1], pf[ks][2], pf[ks][3]);
             if constexpr (NT == 2) {
                 const int ch = 2 * wid + (lane >> 4);
 #pragma unroll
@@ -990,7 +1002,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
             for (int ks = 0; ks < 4; ++ks)
 #pragma unroll
                 for (int e = 0; e < NT; ++e)
-                    mma_bf16(acc[e], pf[ks][0], 0u, pf[ks][1], 0u, vf[ks][2 * e], vf[ks][2 * e + 1]);
+                    mma_bf16(acc[e], pf[ks][0], pf[ks][1], pf[ks][2], pf[ks][3], vf[ks][2 * e], vf[ks][2 * e + 1]);
         }
         // Once every warp has finished with these blocks, their stages may be loaded again.
         if (i0 + stages < mine) {
@@ -1006,9 +1018,12 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         const uint32_t slot = ((uint32_t)g * inv_R) >> 16, owner = (uint32_t)g - slot * (uint32_t)R;
         const uint32_t dst = ptx::map_shared(rest + SM::kRecv, owner) + ((uint32_t)r * (uint32_t)heads_per_owner + slot) * SM::kRecvRow;
         const uint32_t their_bar = ptx::map_shared(bar_recv, owner);
+        // (An infinite V: 0 x infinity in the remainder's product must not turn the first part's infinity into NaN.)
+        auto both = [](float hi, float lo) { return fabsf(hi) < INFINITY ? hi + lo : hi; };
 #pragma unroll
         for (int e = 0; e < NT; ++e)
-            ptx::st_async_v2(dst + (uint32_t)(wid * (D / 8) + 8 * e + 2 * t) * 4u, acc[e][0], acc[e][1], their_bar);
+            ptx::st_async_v2(dst + (uint32_t)(wid * (D / 8) + 8 * e + 2 * t) * 4u, both(acc[e][0], acc[e][2]),
+                             both(acc[e][1], acc[e][3]), their_bar);
         if (wid == 0 && t == 0) {
             float l = 0.f;
             if (mine > 0) {

@@ -134,6 +134,24 @@ def test_cluster_kernel_edges(pa, oracle, pa_env, Hq, Hkv, D, R, stages):
     compare(o, lse, o_ref, lse_ref, f"R={R} stages={stages}")
 
 
+@pytest.mark.parametrize("Hq,Hkv,D", [(8, 1, 64), (14, 2, 128)])
+def test_cluster_kernel_weights_are_not_rounded(pa, oracle, Hq, Hkv, D):
+    """Error of the fp32 output.  Per weight: two bf16 parts 2^-18, ex2.approx 2^-22, the rounding of an exponent of up to
+    64 2^-18, so 2^-17 and twice that for the quotient; up to 48 accumulations per output at 2^-22 of max |V|: below 2^-14
+    of max |V|.  (One bf16 part: 2^-9 per weight.)  An infinite entry of V stays infinite."""
+    lens = np.array([3000, 1777, 450, 90])
+    q = si.bf16_randn((4, Hq, D), 61)
+    kc, vc = si.bf16_randn((4, 3000, Hkv, D), 62, 3.0), si.bf16_randn((4, 3000, Hkv, D), 63)
+    args = (torch.as_tensor(lens, dtype=torch.int32).cuda(), 5, 1)
+    o, _, _ = pa.pa_decode(q.cuda(), kc.cuda(), vc.cuda(), *args, o_dtype=torch.float32)
+    o_ref, _, _ = oracle.decode(q, kc, vc, lens, 64, 5, 1)
+    worst = np.abs(o.cpu().double().numpy() - np.asarray(o_ref, dtype=np.float64)).max()
+    assert worst <= float(vc.abs().max()) * 2.0 ** -14, worst
+    vc[:, 5] = float("inf")   # (a key of the sink block, in every row)
+    o, _, _ = pa.pa_decode(torch.zeros_like(q).cuda(), kc.cuda(), vc.cuda(), *args, o_dtype=torch.float32)
+    assert (o == float("inf")).all()
+
+
 def test_decode_short_cache_with_wide_window_and_sinks(pa, oracle):
     """A cache of 32 blocks whose window + sink candidates exceed 32: the bound on listed blocks is
     clamped by the row count, the candidate count is not (the library must pick its path by the
