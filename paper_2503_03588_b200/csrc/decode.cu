@@ -736,7 +736,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) decode_row_kernel(const __grid
 // its parts and for nothing else).
 // Bound by that chain of latencies.  Measured in a graph, G = 7, head_dim 128, 4000 tokens, against this split done by
 // decode_row_kernel (keys kept apart by warp up to the end, the warps' outputs merged in shared memory, then all parts
-// behind a barrier of the cluster): 4 rows 3.7 us (5.2), 32 rows 4.9 (6.8), 74 rows 6.8 (8.0), 148 rows 9.1 (10.0).
+// behind a barrier of the cluster): 4 rows 3.8 us (5.2), 32 rows 5.0 (6.8), 74 rows 6.8 (8.0), 148 rows 9.2 (10.0).
 // ------------------------------------------------------------------------------------------
 constexpr int kClusterThreads = 256;
 constexpr int kClusterWarps = kClusterThreads / 32;
@@ -930,7 +930,8 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         const float p2 = ptx::ex2(sx[2] - m_new), p3 = ptx::ex2(sx[3] - m_new);
         // A weight is split in two bf16 parts, of which the MMA's rows 8 .. 15, otherwise empty, take the second.  All keys
         // share one maximum here (in decode_row_kernel each warp's largest weight is 1, exact in bf16), and with the first
-        // part alone the error against 64 bits was 1.2 to 2.5 times that kernel's.
+        // part alone the error against 64 bits was 1.2 to 2.5 times that kernel's (8 x 4 rows, 4000 tokens, relative: 1.0e-3
+        // there, 1.3e-3 with one part, 1.9e-6 with two, for 0 to 0.2 us a call).
         const uint32_t h01 = ptx::cvt_bf16x2(p0, p1), h23 = ptx::cvt_bf16x2(p2, p3);
         ptx::st_shared(p_mine, h01);
         ptx::st_shared(p_mine + 16, h23);
