@@ -1005,9 +1005,10 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
                 for (int e = 0; e < NT; ++e)
                     mma_bf16(acc[e], pf[ks][0], pf[ks][1], pf[ks][2], pf[ks][3], vf[ks][2 * e], vf[ks][2 * e + 1]);
         }
-        // Once every warp has finished with these blocks, their stages may be loaded again.
+        // Once every warp has finished with these blocks, their stages may be loaded again; not if a wait gave up: a barrier
+        // whose phase is not over must not be armed again, nor a stage loaded that copies are still on their way to.
         if (i0 + stages < mine) {
-            __syncthreads();
+            if (__syncthreads_or(*abort_flag)) break;
             if (wid == 0) fetch(i0 + stages, i0 + stages + per);
             __syncwarp();
         }

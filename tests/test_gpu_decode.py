@@ -152,6 +152,37 @@ def test_cluster_kernel_weights_are_not_rounded(pa, oracle, Hq, Hkv, D):
     assert (o == float("inf")).all()
 
 
+@pytest.mark.parametrize("path,R,stages", [("persist", 1, 1), ("cluster", 1, 1), ("cluster", 1, 2), ("cluster", 1, 3)])
+def test_a_wait_that_runs_out_ends_the_kernel(pa, pa_env, path, R, stages):
+    """Rows of up to 28 blocks under a limit of one cycle.  The row kernel's producer waits for a stage that four warps are
+    busy with, long enough to run out; the cluster kernel's waits are seldom longer than what one try of the
+    hardware takes, so that a call may end either way: with PA_ERR_TIMEOUT, or with the right result.  The calls
+    behind it, back at the default limit, are right on the same workspace."""
+    pa_env(PA_DECODE_PATH=path, PA_DECODE_CLUSTER=str(R), PA_DECODE_STAGES=str(stages))
+    rows, max_len, D = 296, 9000, 128
+    q, kc, vc = (si.bf16_randn(s, 55 + i).cuda() for i, s in enumerate([(rows, 7, D)] + [(1, max_len, 1, D)] * 2))
+    kc, vc = kc.repeat(rows, 1, 1, 1), vc.repeat(rows, 1, 1, 1)
+    lens = torch.arange(rows, dtype=torch.int32, device="cuda") * 30 + 100
+    o_ref, lse_ref, ws = pa.pa_decode(q, kc, vc, lens, 20, 1)
+    pa.pa_decode_status(ws)
+    timeouts = 0
+    for _ in range(20):
+        try:
+            pa.pa_set_wait_limit_cycles(1)
+            o, lse, _ = pa.pa_decode(q, kc, vc, lens, 20, 1, workspace=ws)
+            pa.pa_decode_status(ws)
+            assert torch.equal(o, o_ref) and torch.equal(lse, lse_ref)
+        except pa.PaError as err:
+            assert "PA_ERR_TIMEOUT" in str(err) and "wait id" in str(err)
+            timeouts += 1
+        finally:
+            pa.pa_set_wait_limit_cycles(0)
+        o, lse, _ = pa.pa_decode(q, kc, vc, lens, 20, 1, workspace=ws)
+        assert pa.pa_decode_status(ws) == 0
+        assert torch.equal(o, o_ref) and torch.equal(lse, lse_ref)
+    assert path == "cluster" or timeouts > 0
+
+
 def test_decode_short_cache_with_wide_window_and_sinks(pa, oracle):
     """A cache of 32 blocks whose window + sink candidates exceed 32: the bound on listed blocks is
     clamped by the row count, the candidate count is not (the library must pick its path by the
