@@ -152,7 +152,8 @@ def test_cluster_kernel_weights_are_not_rounded(pa, oracle, Hq, Hkv, D):
     assert (o == float("inf")).all()
 
 
-@pytest.mark.parametrize("path,R,stages", [("persist", 1, 1), ("cluster", 1, 1), ("cluster", 1, 2), ("cluster", 1, 3)])
+@pytest.mark.parametrize("path,R,stages", [("persist", 1, 1), ("cluster", 1, 1), ("cluster", 1, 2), ("cluster", 1, 3),
+                                           ("cluster", 2, 3), ("cluster", 3, 1), ("cluster", 8, 2)])
 def test_a_wait_that_runs_out_ends_the_kernel(pa, pa_env, path, R, stages):
     """Rows of up to 28 blocks under a limit of one cycle.  The row kernel's producer waits for a stage that four warps are
     busy with, long enough to run out; the cluster kernel's waits are seldom longer than what one try of the
