@@ -352,11 +352,14 @@ def test_backward_of_a_group_beside_one_that_is_not_finite(pa, D, bad):
         assert torch.allclose(got[:, :, 0], ref[:, :, 0], rtol=1e-4, atol=1e-5)
 
 
+@pytest.mark.parametrize("graph", [False, True])
 @pytest.mark.parametrize("N,Hq,Hkv,D,batch", [(100, 2, 2, 64, 1), (1000, 7, 1, 128, 1), (3000, 8, 2, 64, 2), (9000, 16, 16, 64, 2)])
-def test_backward_calls_back_to_back_on_one_workspace(pa, N, Hq, Hkv, D, batch):
-    """The dQ kernel runs beside the dK / dV kernel and the preparation of the next call may not touch what either reads:
-    two problems in turn on the same workspace and outputs, without a wait in between, from fewer items than SMs to
-    chunks of full size, whose dK and dV are cleared by a kernel of their own."""
+def test_backward_calls_back_to_back_on_one_workspace(pa, N, Hq, Hkv, D, batch, graph):
+    """The dQ kernel runs beside the dK / dV kernel, and the preparation of the next call, which may start beside both (the
+    first two sizes: one round of items), may not touch what either reads: two problems in turn on the same workspace
+    with nothing in between, issued one by one and from a graph, where no launch lets a gap open, from fewer items
+    than SMs to chunks of full size, whose dK and dV are cleared by a kernel of their own."""
+    turns = 8
     rp, ci = pa.pa_build_layout(N, 64, 5, 1)
     problems = []
     for seed in (2100, 2200):
@@ -365,14 +368,23 @@ def test_backward_calls_back_to_back_on_one_workspace(pa, N, Hq, Hkv, D, batch):
         *alone, ws = pa.pa_prefill_backward(Q, K, V, o, lse, dO, rp, ci)
         torch.cuda.synchronize()
         problems.append((Q, K, V, o, lse, dO, alone))
-    out = [torch.empty_like(x) for x in problems[0][6]]
-    got = []
-    for turn in range(6):
-        Q, K, V, o, lse, dO, _ = problems[turn % 2]
-        pa.pa_prefill_backward(Q, K, V, o, lse, dO, rp, ci, dq=out[0], dk=out[1], dv=out[2], workspace=ws)
-        got.append([x.clone() for x in out])
+    outs = [[torch.full_like(x, float("nan")) for x in problems[0][6]] for _ in range(turns)]
+
+    def issue():
+        for turn, (dq, dk, dv) in enumerate(outs):
+            Q, K, V, o, lse, dO, _ = problems[turn % 2]
+            pa.pa_prefill_backward(Q, K, V, o, lse, dO, rp, ci, dq=dq, dk=dk, dv=dv, workspace=ws)
+
+    torch.cuda.synchronize()
+    if graph:
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            issue()
+        g.replay()
+    else:
+        issue()
     pa.pa_prefill_status(ws)
-    for turn, g in enumerate(got):
-        for x, ref in zip(g, problems[turn % 2][6]):
+    for turn, got in enumerate(outs):
+        for x, ref in zip(got, problems[turn % 2][6]):
             # (parts of dK and dV are added up in no fixed order: fp32 sums of at most some thousand terms)
             assert (x - ref).abs().max() <= 1e-5 * ref.abs().max()
