@@ -74,9 +74,10 @@ def test_groups_that_leave_the_second_slot_idle(pa, oracle, G, D):
 @pytest.mark.parametrize("G", [3, 4, 5, 7, 8])
 def test_large_groups_with_few_units(pa, oracle, G, D):
     """Calls whose units of two heads find an SM each run larger groups with one slot, longer ones with two: lengths on both
-    sides of the line for 148 SMs, two KV heads, a ragged last block, the padding head of odd groups."""
+    sides of the line, two KV heads, a ragged last block, the padding head of odd groups."""
     Hkv, pairs = 2, (G + 1) // 2
-    most = 148 // (Hkv * pairs)   # query blocks up to which there is one slot
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    most = sms // (Hkv * pairs)   # query blocks up to which there is one slot
     for blocks in (1, 3, most, most + 1):
         N = 64 * blocks - 5
         Q = si.bf16_randn((1, N, G * Hkv, D), 1400 + G)
@@ -103,6 +104,40 @@ def test_orders_of_units_agree(pa, N, batch, Hkv, G):
     pa.pa_prefill_status(ws)
     assert torch.equal(o, o2[:, :, :G * Hkv]) and torch.equal(lse, lse2[:, :G * Hkv])
     assert (o2[:, :, G * Hkv:] == 0).all()
+
+
+@pytest.mark.parametrize("Hkv", [6, 24])
+@pytest.mark.parametrize("G,D", [(3, 64), (4, 64), (7, 64), (3, 128), (5, 128)])
+def test_long_calls_of_strided_queries(pa, G, D, Hkv):
+    """Calls of many rounds may read Q through a map with a group dimension, with K and V that fit in L2 (6 KV heads) and
+    that do not (24): views of Q with other orders of token and head, with unused heads between, and expanded over the
+    batch give what a call per KV head gives, which has too few units for that map; fp32 and bf16 output, ragged
+    last block."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    sub = (G + 3) // 4
+    nqb = max(sms // sub + 1, (48 << 20) // (24 * D * 4 * 64) + 1)   # more than six rounds; the 24 heads exceed 48 MB
+    N = 64 * nqb - 9
+    assert nqb * 6 * sub > 6 * sms and N * 6 * D * 4 <= 48 << 20 < N * 24 * D * 4 and nqb * sub <= 6 * sms
+    rp, ci = pa.pa_build_layout(N, 64, 2, 1)
+    wide = si.bf16_randn((1, N, G * Hkv + 2, D), 1710 + G).cuda()
+    q = wide[:, :, 1:-1]
+    k, v = (si.bf16_randn((1, N, Hkv, D), 1720 + x).cuda() for x in range(2))
+    by_token = q.transpose(1, 2).contiguous().transpose(1, 2)   # heads outermost in memory
+    for o_dtype in (torch.float32, torch.bfloat16):
+        o_ref, lse_ref = (torch.cat(x, dim=d) for x, d in zip(zip(*[
+            pa.pa_prefill(q[:, :, G * h:G * h + G].contiguous(), k[:, :, h:h + 1].contiguous(), v[:, :, h:h + 1].contiguous(),
+                          rp, ci, o_dtype=o_dtype)[:2] for h in range(Hkv)]), (2, 1)))
+        for x in (q, q.contiguous(), by_token):
+            o, lse, ws = pa.pa_prefill(x, k, v, rp, ci, o_dtype=o_dtype)
+            pa.pa_prefill_status(ws)
+            assert torch.equal(o, o_ref) and torch.equal(lse, lse_ref), (x.stride(), o_dtype)
+        if Hkv == 6:   # (one sequence of queries for two of keys and values)
+            kk, vv = torch.cat([k, v]), torch.cat([v, k])
+            o, lse, ws = pa.pa_prefill(q.expand(2, -1, -1, -1), kk, vv, rp, ci, o_dtype=o_dtype)
+            pa.pa_prefill_status(ws)
+            assert torch.equal(o[:1], o_ref) and torch.equal(lse[:1], lse_ref)
+            o2, lse2, _ = pa.pa_prefill(q.contiguous(), v, k, rp, ci, o_dtype=o_dtype)
+            assert torch.equal(o[1:], o2) and torch.equal(lse[1:], lse2)
 
 
 def test_peaky_logits_fp32_output_and_custom_scale(pa, oracle):
