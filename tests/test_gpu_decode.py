@@ -104,9 +104,8 @@ def test_decode_full_size_workload(pa, oracle):
                                  {"PA_DECODE_PATH": "persist", "PA_DECODE_CLUSTER": "4", "PA_DECODE_STAGES": "2"},
                                  {"PA_DECODE_PATH": "persist", "PA_DECODE_CLUSTER": "8", "PA_DECODE_STAGES": "6"}])
 def test_decode_paths(pa, oracle, pa_env, env):
-    """The split-K pair, the single-launch cluster form of the row kernel and its persistent form
-    (partials + combine, or direct output with one chunk per row) at several chunk counts and ring
-    depths give the same row of Eq. (1)."""
+    """The split-K pair, the cluster kernel and the row kernel (partials + combine, or direct output
+    with one chunk per row) at several chunk counts and ring depths give the same row of Eq. (1)."""
     pa_env(**env)
     batch, max_len, Hq, Hkv, D = 4, 9000, 28, 4, 128
     q = si.bf16_randn((batch, Hq, D), 31)
