@@ -366,6 +366,9 @@ __device__ __forceinline__ int32_t row_block_candidate(int32_t row, int32_t W, i
 }
 
 // kParts: rows come in R chunks; else R = 1, known to the compiler (one block of 128 features, 16 rows: 3.6 us against 3.8).
+// Registers are what 128 features are short of (168 a thread, two CTAs of five warps per SM).  With the next item's Q in
+// registers of its own throughout, and the diagonal block found by its index, this form spilled 104 bytes: 28 / 4 heads, 9000
+// tokens, 150 rows 13.0 us, 296 rows 17.0, 512 rows 33.5; so 36 bytes, 11.7, 16.4 and 32.8.
 template <int D, bool kParts>
 __global__ void __launch_bounds__(kRowThreads, 2) decode_row_kernel(const __grid_constant__ CUtensorMap tmK,
                                                                     const __grid_constant__ CUtensorMap tmV,
@@ -416,7 +419,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) decode_row_kernel(const __grid
     // Item it -> (row of the call, chunk); a row -> (sequence, KV head).
     struct Item {
         int32_t b, hk, r;        // sequence, KV head, chunk
-        int32_t row, last_keys;  // the query's block row; keys of the diagonal block
+        int32_t last_keys;       // keys of the diagonal block
         int32_t cand;            // this lane's candidate key block or -1
         int32_t rank;            // its number among the candidates that exist (lane order)
         int32_t page;            // (paged cache) its page
@@ -435,9 +438,8 @@ __global__ void __launch_bounds__(kRowThreads, 2) decode_row_kernel(const __grid
         const int64_t len = len32;
         const bool valid = len >= 1 && len <= a.max_len;
         const int64_t p = len - 1;
-        w.row = valid ? (int32_t)(p / kDecBlock) : 0;
         w.last_keys = (int32_t)(p % kDecBlock) + 1;
-        w.cand = valid ? row_block_candidate(w.row, a.W, a.S, lane) : -1;
+        w.cand = valid ? row_block_candidate((int32_t)(p / kDecBlock), a.W, a.S, lane) : -1;
         w.page = 0;
         if (a.table && w.cand >= 0) w.page = a.table[(int64_t)w.b * a.table_stride + w.cand];
         w.have = __ballot_sync(0xffffffffu, w.cand >= 0);
@@ -494,17 +496,17 @@ __global__ void __launch_bounds__(kRowThreads, 2) decode_row_kernel(const __grid
         // + lane % 8, chunk + lane / 16.  A 16-byte chunk c of row `key` sits at c ^ (key % 8).
         const int k_key = 16 * wid + ((lane >> 4) << 3) + (lane & 7), k_ch = (lane >> 3) & 1;
         const int v_key = 16 * wid + (((lane >> 3) & 1) << 3) + (lane & 7), v_ch = lane >> 4;
-        // Q fragments: head g is row g of the 16-row A operand (rows 8..15 are zero).  The next
-        // item's are requested while the current item is worked on.
-        uint32_t qn[D / 16][2];
+        // Q fragments: head g is row g of the 16-row A operand (rows 8..15 are zero).  The next item's are requested
+        // behind the last product with the current item's, into the same registers.
+        uint32_t qa[D / 16][2];
         auto load_q = [&](uint32_t it) {
             const bool in = it < n_items && g < G;
             const int32_t rowid = in ? (int32_t)(it / (uint32_t)R) : 0;  // = b Hkv + hk, and its heads start at rowid G
             const __nv_bfloat16 *qb = a.q + ((int64_t)rowid * G + g) * D;
 #pragma unroll
             for (int ks = 0; ks < D / 16; ++ks) {
-                qn[ks][0] = in ? ld4(qb + 16 * ks + 2 * t) : 0u;
-                qn[ks][1] = in ? ld4(qb + 16 * ks + 8 + 2 * t) : 0u;
+                qa[ks][0] = in ? ld4(qb + 16 * ks + 2 * t) : 0u;
+                qa[ks][1] = in ? ld4(qb + 16 * ks + 8 + 2 * t) : 0u;
             }
         };
         load_q(it0);
@@ -514,13 +516,6 @@ __global__ void __launch_bounds__(kRowThreads, 2) decode_row_kernel(const __grid
         for (uint32_t it = it0; it < n_items && ok; it += it_step) {
             const Item w = make_item(it, len_next);
             len_next = item_len(it + it_step);
-            uint32_t qa[D / 16][2];
-#pragma unroll
-            for (int ks = 0; ks < D / 16; ++ks) {
-                qa[ks][0] = qn[ks][0];
-                qa[ks][1] = qn[ks][1];
-            }
-            load_q(it + it_step);
             float m_run = -INFINITY, l_run = 0.f;
             float acc[D / 8][4];
 #pragma unroll
@@ -529,8 +524,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) decode_row_kernel(const __grid
             for (int i = 0; i < w.mine && ok; ++i, ++ci) {
                 const int s = (int)(ci % (uint32_t)stages);
                 const uint32_t parity = (ci / (uint32_t)stages) & 1;
-                const int32_t jblk = __shfl_sync(0xffffffffu, w.cand, lane_of(w, i));
-                const int n_keys = jblk == w.row ? w.last_keys : kDecBlock;
+                const int n_keys = w.r == 0 && i == 0 ? w.last_keys : kDecBlock;  // (the diagonal block is lane 0's)
                 const uint32_t sk = smem_base + (uint32_t)s * SM::kStage, sv = sk + SM::kTile;
                 ok = ptx::mbar_wait_bounded(bar_kfull(s), parity, abort_flag, a.status, 2, a.wait_cycles, (int)PA_ERR_TIMEOUT);
                 ok = __all_sync(0xffffffffu, ok);
@@ -618,6 +612,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) decode_row_kernel(const __grid
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive(bar_empty(s));  // this warp has finished with the stage
             }
+            load_q(it + it_step);
 
             // ---- the four warps' partials are merged with the log-sum-exp rule, each warp taking a
             // quarter of the features (four of the 8-feature tiles): a thread passes on the tiles it
