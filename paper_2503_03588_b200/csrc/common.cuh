@@ -29,8 +29,8 @@ pa_status current_sm100_device(DeviceInfo *out);
 
 // One-time per-device set-up steps (kernel attributes) are keyed by these slots.
 enum DeviceOnce : int {
-    ONCE_PREFILL_ATTR = 0,  // (32: length, head_dim, slots, output type)
-    ONCE_DECODE_ATTR = ONCE_PREFILL_ATTR + 32,
+    ONCE_PREFILL_ATTR = 0,  // (40: order of the units, head_dim, slots, output type)
+    ONCE_DECODE_ATTR = ONCE_PREFILL_ATTR + 40,
     ONCE_BACKWARD_ATTR, ONCE_BACKWARD_ATTR_64, ONCE_BACKWARD_TC_ATTR, ONCE_BACKWARD_TC_ATTR_64,
     ONCE_COUNT
 };

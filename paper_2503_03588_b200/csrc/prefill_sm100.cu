@@ -138,20 +138,49 @@ __device__ __forceinline__ uint32_t divmod(uint32_t u, uint32_t d, uint32_t inv,
     return q;
 }
 
+// The order of the units, of which a group's heads come fastest.
+//   kHeads      then query block (long rows first), KV head, batch entry: the CTAs work on one KV head at a time, whose K and
+//               V (67 MB at 128K tokens) stay in L2.
+//   kRows       then KV head, batch entry, query block (long rows first): the units get shorter and shorter, so that the
+//               CTAs, which take them in turn, end together.
+//   kPlaces     packed sequences of unequal lengths: then KV head, place.  Sequence b has the places from
+//               floor(cu_seqlens[b] / 64) + b on, one for each of its query blocks (long rows first) and at most one more.
+//   kRowsZeros, kHeadsZeros   the same orders, and the heads that a group's last unit lacks are zeros.
+enum Order : int { kHeads, kRows, kPlaces, kRowsZeros, kHeadsZeros };
+template <Order kOrder>
+constexpr bool kByRows = kOrder == kRows || kOrder == kPlaces || kOrder == kRowsZeros;
+
 // Unit index -> coordinates (the unit count fits in 30 bits; checked on the host).
-template <bool kRowsFirst>
+template <Order kOrder>
 __device__ __forceinline__ Unit decode_unit(const PrefillArgs &a, uint32_t u)
 {
     Unit r;
     uint32_t rem;
-    // Order: a group's heads fastest, then
-    //   kRowsFirst: KV head, batch entry, query block (long rows first): the units get shorter and shorter, so that the
-    //               CTAs, which take them in turn, end together;
-    //   else:       query block, KV head, batch entry: the CTAs work on one KV head at a time, whose K and V (67 MB at
-    //               128K tokens) stay in L2.
     u = divmod(u, (uint32_t)a.nsub, a.inv_nsub, rem);
     r.sub = (int32_t)rem;
-    if (kRowsFirst) {
+    if constexpr (kOrder == kPlaces) {
+        u = divmod(u, (uint32_t)a.Hkv, a.inv_Hkv, rem);
+        r.hk = (int32_t)rem;
+        int32_t b = 0;  // the sequence: the last one whose places do not begin behind u
+        for (int32_t end = a.batch; end - b > 1;) {
+            const int32_t mid = (b + end) >> 1;
+            if (a.cu_seqlens[mid] / kBlk + mid <= (int32_t)u) b = mid;
+            else end = mid;
+        }
+        r.b = b;
+        r.bt = 0;
+        r.tok0 = a.cu_seqlens[b];
+        r.len = a.cu_seqlens[b + 1] - r.tok0;
+        const int32_t rows = min((r.len + kBlk - 1) / kBlk, a.nqb), row = rows - 1 - ((int32_t)u - r.tok0 / kBlk - b);
+        if (row < 0 || row >= rows) {  // a place too many: no token of it exists
+            r.i = r.len = r.rs = r.n = 0;
+            return r;
+        }
+        r.i = row;
+        r.rs = a.row_ptr[row];
+        r.n = a.row_ptr[row + 1] - r.rs;
+        return r;
+    } else if constexpr (kByRows<kOrder>) {
         u = divmod(u, (uint32_t)a.Hkv, a.inv_Hkv, rem);
         r.hk = (int32_t)rem;
         u = divmod(u, (uint32_t)a.batch, a.inv_batch, rem);
@@ -178,7 +207,7 @@ __device__ __forceinline__ Unit decode_unit(const PrefillArgs &a, uint32_t u)
     return r;
 }
 
-// The units of a CTA: number k is the one at the CTA's place in round k of the grid; with kRowsFirst from the front in even
+// The units of a CTA: number k is the one at the CTA's place in round k of the grid; with rows first from the front in even
 // rounds and from the back in odd ones, since in every round the first places have the longer rows.
 template <bool kRowsFirst>
 struct UnitCursor {
@@ -192,20 +221,16 @@ struct UnitCursor {
     }
 };
 
-// What a call's length asks for: kOne, at most a unit per CTA; kMid, the units row by row; kMidLong, so, too, and the heads
-// that a group's last unit lacks are zeros; kLong, zeros, but head by head.
-enum Length : int { kOne, kMid, kMidLong, kLong };
-
-// kSlots: slots that have work, kLength (launch_prefill chooses both); kF32: fp32 output.
-template <int D, int kSlots, bool kF32, Length kLength>
+// kSlots: slots that have work, kOrder (launch_prefill chooses both); kF32: fp32 output.
+template <int D, int kSlots, bool kF32, Order kOrder>
 __global__ void __launch_bounds__(kThreads, 1)
 prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO,
                const PrefillArgs a)
 {
     using SM = SmemMap<D>;
-    constexpr bool kRowsFirst = kLength == kMid || kLength == kMidLong;
-    constexpr bool kZeros = kLength == kMidLong || kLength == kLong;  // (the Q map has a group dimension)
+    constexpr bool kRowsFirst = kByRows<kOrder>;
+    constexpr bool kZeros = kOrder == kRowsZeros || kOrder == kHeadsZeros;  // (the Q map has a group dimension)
     constexpr int DH = D / 64;  // 64-feature (128-byte) sub-tiles per row
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -285,7 +310,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             UnitCursor<kRowsFirst> cur;
             auto next_unit = [&](Unit &w, int32_t &j0) {
                 for (; cur.u < (uint32_t)a.n_units; cur.advance()) {
-                    w = decode_unit<kRowsFirst>(a, cur.u);
+                    w = decode_unit<kOrder>(a, cur.u);
                     if (w.n > 0) {
                         j0 = a.col_idx[w.rs];
                         break;
@@ -415,7 +440,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                                       (acc || kk > 0) ? 1u : 0u);
             };
             auto unit_blocks = [&](uint32_t u) {
-                return __shfl_sync(0xffffffffu, u < (uint32_t)a.n_units ? decode_unit<kRowsFirst>(a, u).n : 0, 0);
+                return __shfl_sync(0xffffffffu, u < (uint32_t)a.n_units ? decode_unit<kOrder>(a, u).n : 0, 0);
             };
             // Next non-empty unit after u.  Its block count `n` is already loaded (`ahead`); the
             // count after that is requested now, so no unit boundary waits for a load.
@@ -519,7 +544,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         // extent two units ahead, the row's last block index (needs the extent) one unit ahead.
         auto fetch_unit = [&](uint32_t u) {
             Unit r = {};
-            if (u < (uint32_t)a.n_units) r = decode_unit<kRowsFirst>(a, u);
+            if (u < (uint32_t)a.n_units) r = decode_unit<kOrder>(a, u);
             return r;
         };
         auto fetch_lastcol = [&](const Unit &r) { return r.n > 0 ? a.col_idx[r.rs + r.n - 1] : -1; };
@@ -737,7 +762,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         uint32_t ul = 0, ns = 0;  // units and staged slots so far
         bool ok = true;
         for (UnitCursor<kRowsFirst> cur; cur.u < (uint32_t)a.n_units && ok; cur.advance()) {
-            const Unit w = decode_unit<kRowsFirst>(a, cur.u);
+            const Unit w = decode_unit<kOrder>(a, cur.u);
             const int64_t tok = (int64_t)w.i * kBlk + qrow;
             // The unit's Q buffer is no longer read once its last P V has completed (every S of
             // the unit was issued before it); its output is staged there.
@@ -971,17 +996,17 @@ namespace pa {
 
 // The launch behind pa_prefill (cu_seqlens null) and pa_prefill_varlen (packed sequences:
 // p->seq_len is the longest one, tokens run over [0, total_tokens)).
-template <int D, int kSlots, bool kF32, Length kLength>
+template <int D, int kSlots, bool kF32, Order kOrder>
 static pa_status launch_kernel(unsigned grid, cudaStream_t st, int device, const CUtensorMap &tmQ, const CUtensorMap &tmK,
                                const CUtensorMap &tmV, const CUtensorMap &tmO, const PrefillArgs &a)
 {
-    constexpr DeviceOnce once = (DeviceOnce)(ONCE_PREFILL_ATTR + 8 * (int)kLength + 4 * (D == 64) + 2 * (kSlots == 1) + kF32);
+    constexpr DeviceOnce once = (DeviceOnce)(ONCE_PREFILL_ATTR + 8 * (int)kOrder + 4 * (D == 64) + 2 * (kSlots == 1) + kF32);
     if (pa_status s = device_once(device, once, [] {
-            return cudaFuncSetAttribute(prefill_kernel<D, kSlots, kF32, kLength>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            return cudaFuncSetAttribute(prefill_kernel<D, kSlots, kF32, kOrder>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)SmemMap<D>::kAlloc);
         }))
         return s;
-    PA_CUDA_OK(launch_pdl(prefill_kernel<D, kSlots, kF32, kLength>, dim3(grid), kThreads, SmemMap<D>::kAlloc, st, tmQ, tmK, tmV, tmO, a));
+    PA_CUDA_OK(launch_pdl(prefill_kernel<D, kSlots, kF32, kOrder>, dim3(grid), kThreads, SmemMap<D>::kAlloc, st, tmQ, tmK, tmV, tmO, a));
     return PA_OK;
 }
 
@@ -1020,16 +1045,26 @@ static pa_status launch_prefill(const pa_prefill_params *p, const void *q, const
     // The order that balances the CTAs is taken where K and V of all heads may stay in L2 together, of whose 126 MB Q and
     // O take their share: in a loop, 28 / 4 heads, the other order and this, 4001 tokens (8 MB of K and V) 44.7 and 42.2 us,
     // 8192 (17 MB) 93.6 and 90.9, 16100 (33 MB) 193.4 and 193.9, in 256-token blocks 523 and 505; 4 x 16384 tokens, 8 / 8
-    // heads (268 MB) 500 and 520; packed prompts of 22 MB 125 and 119, of 95 MB 514 and 522.  The calls beyond are
-    // those that last, and the zeros that save power go with them (they cost calls of one unit per CTA 1.4 %), and with
-    // calls of more than six rounds of the grid: in a loop, 28 / 4 heads, 16384 tokens 203 -> 201.5 us, in 256-token blocks
-    // 523 -> 518; 4001 tokens, 3.4 rounds, no difference.
+    // heads (268 MB) 500 and 520; packed prompts of 95 MB 514 and 522.  The calls beyond are those that last, and the
+    // zeros that save power go with them (they cost calls of one unit per CTA 1.4 %), and with calls of more than six
+    // rounds of the grid: in a loop, 28 / 4 heads, 16384 tokens 203 -> 201.5 us, in 256-token blocks 523 -> 518; 4001 tokens,
+    // 3.4 rounds, no difference.
+    // Packed sequences go by places where their mean length is below three quarters of the longest.  With a unit for every
+    // query block of the longest one, those that do not exist fall on the same CTAs again and again when a row's units
+    // and the grid have a divisor in common.  In a loop, head by head, row by row and by places: 12 sequences of 140 to 814
+    // tokens, 28 / 4 heads 45.2, 61.3 and 42.7 us; 5 of 112 to 3735, 14 / 2 heads 54.3, 63.1 and 54.9; 12 of up to 1875, 8 / 2
+    // heads of 64 features 34.0, 43.8 and 28.4.  Of sequences that hardly differ the rows balance better, since places count
+    // down from each sequence's own longest row: 11 of up to 896 tokens, mean 0.68 of that, 28 / 4 heads 54.4, 50.0 and 54.2.
     const int64_t kv_bytes = (varlen ? total_tokens : p->batch * p->seq_len) * p->n_kv_heads * p->head_dim * 4;
-    const int64_t units = rows * ((G + 2 * slots - 1) / (2 * slots));
-    const Length length = units <= dev.sms                    ? kOne
-                          : kv_bytes > (int64_t)48 << 20      ? (slots == 2 ? kLong : kOne)
-                          : slots == 2 && units > 6 * dev.sms ? kMidLong
-                                                              : kMid;
+    const int64_t subs = (G + 2 * slots - 1) / (2 * slots);
+    const bool many = rows * subs > dev.sms, in_l2 = kv_bytes <= (int64_t)48 << 20;
+    const bool places = many && in_l2 && varlen && total_tokens * 4 < (int64_t)p->batch * p->seq_len * 3;
+    const int64_t units = (places ? (total_tokens / kBlk + p->batch) * p->n_kv_heads : rows) * subs;
+    const Order order = !many                               ? kHeads
+                        : !in_l2                            ? (slots == 2 ? kHeadsZeros : kHeads)
+                        : places                            ? kPlaces
+                        : slots == 2 && units > 6 * dev.sms ? kRowsZeros
+                                                            : kRows;
 
     // Tensor maps (cached per buffer and shape): a Q box holds the two heads of a tile, K, V and O
     // boxes one head.
@@ -1042,7 +1077,7 @@ static pa_status launch_prefill(const pa_prefill_params *p, const void *q, const
                                   heads, varlen ? 1 : p->batch, box_heads, kBlk, f32 ? 1 : 0, group};
         return get_tensor_map(key, what, m);
     };
-    if (pa_status s = map_of(q, p->n_q_heads, p->q, 2, "q", &tmQ, false, length == kMidLong || length == kLong ? G : 0)) return s;
+    if (pa_status s = map_of(q, p->n_q_heads, p->q, 2, "q", &tmQ, false, order == kRowsZeros || order == kHeadsZeros ? G : 0)) return s;
     if (pa_status s = map_of(k, p->n_kv_heads, p->k, 1, "k", &tmK)) return s;
     if (pa_status s = map_of(v, p->n_kv_heads, p->v, 1, "v", &tmV)) return s;
     if (pa_status s = map_of(o, p->n_q_heads, p->o, 1, "o", &tmO, p->o_dtype == PA_F32)) return s;
@@ -1062,7 +1097,7 @@ static pa_status launch_prefill(const pa_prefill_params *p, const void *q, const
     a.nqb = (int32_t)nqb;
     a.batch = p->batch; a.Hq = p->n_q_heads; a.Hkv = p->n_kv_heads;
     a.G = G;
-    a.nsub = (a.G + 2 * slots - 1) / (2 * slots);
+    a.nsub = (int32_t)subs;
     a.n_units = units;
     auto inv32 = [](int32_t d) { return d == 1 ? 0xffffffffu : (uint32_t)((1ull << 32) / (uint64_t)d); };
     a.inv_nsub = inv32(a.nsub); a.inv_Hkv = inv32(a.Hkv); a.inv_nqb = inv32(a.nqb); a.inv_batch = inv32(a.batch);
@@ -1100,11 +1135,15 @@ static pa_status launch_prefill(const pa_prefill_params *p, const void *q, const
         constexpr int kD = decltype(d)::value;
         constexpr bool kF32 = decltype(f32)::value;
         auto go = [&](auto kernel) { return kernel(grid, st, dev.device, tmQ, tmK, tmV, tmO, a); };
-        if (slots == 1) return go(length == kMid ? launch_kernel<kD, 1, kF32, kMid> : launch_kernel<kD, 1, kF32, kOne>);
-        return go(length == kMid       ? launch_kernel<kD, 2, kF32, kMid>
-                  : length == kMidLong ? launch_kernel<kD, 2, kF32, kMidLong>
-                  : length == kLong    ? launch_kernel<kD, 2, kF32, kLong>
-                                       : launch_kernel<kD, 2, kF32, kOne>);
+        if (slots == 1)
+            return go(order == kRows     ? launch_kernel<kD, 1, kF32, kRows>
+                      : order == kPlaces ? launch_kernel<kD, 1, kF32, kPlaces>
+                                         : launch_kernel<kD, 1, kF32, kHeads>);
+        return go(order == kRows         ? launch_kernel<kD, 2, kF32, kRows>
+                  : order == kPlaces     ? launch_kernel<kD, 2, kF32, kPlaces>
+                  : order == kRowsZeros  ? launch_kernel<kD, 2, kF32, kRowsZeros>
+                  : order == kHeadsZeros ? launch_kernel<kD, 2, kF32, kHeadsZeros>
+                                         : launch_kernel<kD, 2, kF32, kHeads>);
     };
     auto launch_of = [&](auto d) { return p->o_dtype == PA_F32 ? launch(d, std::true_type()) : launch(d, std::false_type()); };
     return D == 128 ? launch_of(std::integral_constant<int, 128>()) : launch_of(std::integral_constant<int, 64>());

@@ -389,6 +389,40 @@ def test_variable_length_batch_equals_one_call_per_sequence(pa):
         assert torch.equal(o1[0], o[a:e]) and torch.equal(lse1[0], lse[:, a:e])
 
 
+@pytest.mark.parametrize("o_dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("lens,seq_len,Hq,Hkv,D", [([3000, 130, 0, 64, 1, 4096, 777, 65], 4096, 28, 4, 128),
+                                                   ([0, 2000, 64, 128, 640, 0, 0], 2000, 4, 4, 64),
+                                                   ([100, 900, 320] * 4, 5000, 8, 2, 64),     # seq_len: a bound
+                                                   ([2000] + [40] * 20, 1000, 8, 2, 128),     # no output beyond seq_len
+                                                   ([1500], 9000, 8, 8, 64), ([33] * 300 + [2500], 2500, 10, 2, 64),
+                                                   ([640, 1280, 64, 64, 320], 1280, 16, 8, 128)])
+def test_packed_sequences_of_unequal_lengths(pa, lens, seq_len, Hq, Hkv, D, o_dtype):
+    """Units by places along the token axis: empty sequences at both ends, whole blocks, a bound for the longest length on
+    either side, many short ones; one and two slots.  Bit for bit a call per sequence; nothing else is written."""
+    W, S = 3, 1
+    cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    total, nqb = int(cu[-1]), (seq_len + 63) // 64
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert nqb * len(lens) * Hkv > sms and 4 * total < 3 * len(lens) * seq_len   # (what takes the call there)
+    Q, K, V = (si.bf16_randn((total, h, D), 830 + i).cuda() for i, h in enumerate((Hq, Hkv, Hkv)))
+    rp, ci = pa.pa_build_layout(seq_len, 64, W, S)
+    o_all = torch.full((total + 256, Hq, D), 7.0, dtype=o_dtype, device="cuda")
+    lse_all = torch.full((Hq * total + 256,), 7.0, device="cuda")
+    o, lse = o_all[128:-128], lse_all[128:-128].view(Hq, total)
+    ws = pa.pa_prefill_varlen(Q, K, V, torch.as_tensor(cu).cuda(), seq_len, rp, ci, o=o, lse=lse, o_dtype=o_dtype)[2]
+    pa.pa_prefill_status(ws)
+    for edge in (o_all[:128], o_all[-128:], lse_all[:128], lse_all[-128:]):
+        assert bool((edge == 7.0).all())
+    for b, n in enumerate(lens):
+        if n == 0:
+            continue
+        a, m = int(cu[b]), min(n, 64 * nqb)
+        rp1, ci1 = pa.pa_build_layout(n, 64, W, S)
+        o1, lse1, _ = pa.pa_prefill(*(x[None, a:a + n] for x in (Q, K, V)), rp1, ci1, o_dtype=o_dtype)
+        assert torch.equal(o1[0, :m], o[a:a + m]) and torch.equal(lse1[0, :, :m], lse[:, a:a + m]), (b, n)
+        assert bool((o[a + m:a + n] == 7.0).all()) and bool((lse[:, a + m:a + n] == 7.0).all())
+
+
 def test_rows_the_layout_leaves_empty(pa, oracle):
     """A caller's CSR may list nothing for a query block: its rows get O = 0 and LSE = -inf, the
     other rows are untouched by it (oracle: the dense token mask that the CSR stands for)."""
