@@ -1045,10 +1045,13 @@ static pa_status launch_prefill(const pa_prefill_params *p, const void *q, const
     // The order that balances the CTAs is taken where K and V of all heads may stay in L2 together, of whose 126 MB Q and
     // O take their share: in a loop, 28 / 4 heads, the other order and this, 4001 tokens (8 MB of K and V) 44.7 and 42.2 us,
     // 8192 (17 MB) 93.6 and 90.9, 16100 (33 MB) 193.4 and 193.9, in 256-token blocks 523 and 505; 4 x 16384 tokens, 8 / 8
-    // heads (268 MB) 500 and 520; packed prompts of 95 MB 514 and 522.  The calls beyond are those that last, and the
-    // zeros that save power go with them (they cost calls of one unit per CTA 1.4 %), and with calls of more than six
-    // rounds of the grid: in a loop, 28 / 4 heads, 16384 tokens 203 -> 201.5 us, in 256-token blocks 523 -> 518; 4001 tokens,
-    // 3.4 rounds, no difference.
+    // heads (268 MB) 500 and 520; packed prompts of 95 MB 514 and 522.
+    // Zeros for the missing heads of a group save power, which the calls beyond, those that last, have none to spare of: in
+    // a loop, 40000 tokens, 4 KV heads of 128 features, groups of 3, 5, 6 and 7 267 -> 259 us, 509 -> 484, 517 -> 497 and
+    // 519 -> 512; of 64 features (60000 tokens) 0.2 %, in a burst up to 1.4 %.  Of the calls below, those of more than six
+    // rounds and 128 features gain: groups of 3, 5, 6 and 7, 16000 tokens 97.6 -> 95.3, 185 -> 179.7, 188.3 -> 184.6 and
+    // 193 -> 191.3, 28 / 4 heads in 256-token blocks, 9000 tokens 254.8 -> 250.1.  With 64 features they lose (30000 tokens,
+    // groups of 3 to 7 1.0 to 1.4 %), with one unit per CTA 1.4 %, and at 3.4 rounds nothing is gained.
     // Packed sequences go by places where their mean length is below three quarters of the longest.  With a unit for every
     // query block of the longest one, those that do not exist fall on the same CTAs again and again when a row's units
     // and the grid have a divisor in common.  In a loop, head by head, row by row and by places: 12 sequences of 140 to 814
@@ -1060,10 +1063,11 @@ static pa_status launch_prefill(const pa_prefill_params *p, const void *q, const
     const bool many = rows * subs > dev.sms, in_l2 = kv_bytes <= (int64_t)48 << 20;
     const bool places = many && in_l2 && varlen && total_tokens * 4 < (int64_t)p->batch * p->seq_len * 3;
     const int64_t units = (places ? (total_tokens / kBlk + p->batch) * p->n_kv_heads : rows) * subs;
+    const bool zeros = slots == 2 && G % 4 != 0 && p->head_dim == 128;
     const Order order = !many                               ? kHeads
                         : !in_l2                            ? (slots == 2 ? kHeadsZeros : kHeads)
                         : places                            ? kPlaces
-                        : slots == 2 && units > 6 * dev.sms ? kRowsZeros
+                        : zeros && units > 6 * dev.sms      ? kRowsZeros
                                                             : kRows;
 
     // Tensor maps (cached per buffer and shape): a Q box holds the two heads of a tile, K, V and O
@@ -1139,9 +1143,10 @@ static pa_status launch_prefill(const pa_prefill_params *p, const void *q, const
             return go(order == kRows     ? launch_kernel<kD, 1, kF32, kRows>
                       : order == kPlaces ? launch_kernel<kD, 1, kF32, kPlaces>
                                          : launch_kernel<kD, 1, kF32, kHeads>);
+        if constexpr (kD == 128)
+            if (order == kRowsZeros) return go(launch_kernel<kD, 2, kF32, kRowsZeros>);
         return go(order == kRows         ? launch_kernel<kD, 2, kF32, kRows>
                   : order == kPlaces     ? launch_kernel<kD, 2, kF32, kPlaces>
-                  : order == kRowsZeros  ? launch_kernel<kD, 2, kF32, kRowsZeros>
                   : order == kHeadsZeros ? launch_kernel<kD, 2, kF32, kHeadsZeros>
                                          : launch_kernel<kD, 2, kF32, kHeads>);
     };
