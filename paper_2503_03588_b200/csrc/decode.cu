@@ -1001,10 +1001,11 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
                     mma_bf16(acc[e], pf[ks][0], pf[ks][1], pf[ks][2], pf[ks][3], vf[ks][2 * e], vf[ks][2 * e + 1]);
         }
         // Once every warp has finished with these blocks, their stages may be loaded again; not if a wait gave up: a barrier
-        // whose phase is not over must not be armed again, nor a stage loaded that copies are still on their way to.
+        // whose phase is not over must not be armed again, nor a stage loaded that copies are still on their way to.  (The
+        // flag is up for good then, and what waits are left give up at their next look at it.)
         if (i0 + stages < mine) {
-            if (__syncthreads_or(*abort_flag)) break;
-            if (wid == 0) fetch(i0 + stages, i0 + stages + per);
+            __syncthreads();
+            if (wid == 0 && !*abort_flag) fetch(i0 + stages, i0 + stages + per);
             __syncwarp();
         }
     }
@@ -1066,16 +1067,15 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
             if (d == 0) a.lse[(int64_t)rowid * G + h] = any ? (m + log2f(l)) * 0.6931471805599453f : -INFINITY;
         }
     }
-    __syncthreads();  // (the flag is final: no wait of this CTA is left)
     if (*abort_flag) {
-        // A wait gave up, so peers may still be on their way to push parts into this CTA's shared memory, which lasts until
-        // each of them has ended or come here, too (the barrier waits for the threads that have not exited; a CTA none of
-        // whose waits gave up has all its parts and leaves at once).  Then a bounded time for copies and stores that are
-        // under way.
+        // A wait gave up, so peers may still be on their way to push parts into this CTA's shared memory, which lasts as long
+        // as one of its threads.  Those that know stay until every peer has ended or come here, too (the barrier waits for
+        // the threads that have not exited; a CTA none of whose waits gave up has all its parts and leaves at once).  Then
+        // a bounded time for copies and stores that are under way.
         ptx::cluster_arrive();
         ptx::cluster_wait();
         const long long t0 = clock64();
-        while (tid == 0 && clock64() - t0 < 2000000ll) {
+        while (clock64() - t0 < 2000000ll) {
         }
     }
 }
