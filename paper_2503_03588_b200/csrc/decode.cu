@@ -1398,11 +1398,17 @@ static pa_status launch_decode(const DecodeShape &p, const void *q, const void *
         // Started early, clusters take places as the CTAs of the kernel before leave them, one by one, and what is left
         // in between may be of no use to a cluster until more have ended.  A call that needs nearly all places starts
         // on the empty device instead, about 1 us later.  Where that begins to pay was measured for each size, early
-        // and late in us (4000 tokens, G = 7, head_dim 128; 148 SMs): clusters of three 8.0 and 8.0 at 88 rows, 9.2 and
-        // 8.0 at 90; of four and five (20000 tokens, G = 8) 7.2 and 7.8 at 70, 8.5 and 7.8 at 71, 7.7 and 7.8 at 55, 8.8 and
-        // 7.8 at 56; of six to eight never clearly: 5.7 and 6.4 at 45, 5.8 and 6.2 at 37, 5.6 and 6.2 at 33.  Pairs fit
+        // and late in us (148 SMs: 93 clusters of three fit, 71 of four, 56 of five).  Clusters of three, 128 features, G = 7,
+        // 4000 tokens: 7.4 and 8.0 at 87 rows, 8.2 and 8.0 at 88, 9.4 and 8.0 at 90 (G = 8, 30000 tokens: 7.8 and 8.9 at 90, 9.4 and
+        // 8.9 at 93); 64 features, G = 4: 5.4 and 6.4 at 90, 6.1 and 6.4 at 92, 6.7 and 6.4 at 93.  Of four and five 6.8 and 7.7 at
+        // 70, 8.1 and 7.7 at 71, 5.8 and 6.3 at 55, 6.3 and 6.3 at 56 (64 features 5.6 and 6.3 at 71, 5.7 and 5.2 at 56).  Of six to
+        // eight never clearly: 5.4 and 6.2 at 45, 6.2 and 5.9 at 37, 6.1 and 5.9 at 33.  A row of one head is merged by one of its
+        // CTAs, the others leave before it, which spoils more places: of three 7.9 and 7.1 at 85, 8.9 and 7.1 at 88 (64
+        // features 6.6 and 6.8, 8.5 and 6.8), of five 5.8 and 5.7 at 50, 6.9 and 5.7 at 51 (7.2 and 6.2, 7.6 and 6.2).  Pairs fit
         // in any order.
-        const bool full = R == 3 ? rows_in_call * 20 > fit * 19 : R <= 5 && rows_in_call == fit;
+        const bool full = a.G == 1 && (R == 3 || R == 5) ? rows_in_call * 100 > (int64_t)fit * 91
+                          : R == 3 && p.head_dim == 128  ? rows_in_call * 20 > (int64_t)fit * 19
+                                                         : R <= 5 && rows_in_call == fit;
         const bool early = !(cluster && R > 2 && fit > 0 && full);
 
         // Tensor maps over the cache: (feature, token, head, batch or page), one 64 x 64 box per copy.
