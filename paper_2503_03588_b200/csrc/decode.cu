@@ -1035,7 +1035,15 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     }
 
     // ---- Heads r, r + R, ...: D threads a head, a thread one feature.
-    if (heads_here > 0 && ptx::mbar_wait_bounded_cluster(bar_recv, 0, abort_flag, a.status, 4, a.wait_cycles, (int)PA_ERR_TIMEOUT)) {
+    if (heads_here > 0 &&
+        !ptx::mbar_wait_bounded_cluster(bar_recv, 0, abort_flag, a.status, 4, a.wait_cycles, (int)PA_ERR_TIMEOUT)) {
+        // This CTA's shared memory has to last until every peer's part is in it.  A peer is there after at most two waits for
+        // each of its at most 16 blocks, so this is over before its own limit is.  (A second barrier of the cluster would do,
+        // but its mere presence cost 0.1 us a call.)
+        const long long t0 = clock64(), most = 40 * (a.wait_cycles + 2000000ll);
+        while (!ptx::mbar_try_wait_cluster(bar_recv, 0) && clock64() - t0 < most) {
+        }
+    } else if (heads_here > 0) {
         const int d = tid % D;
         for (int slot = tid / D; slot < heads_here; slot += kClusterThreads / D) {
             const int h = r + slot * R;
@@ -1067,13 +1075,10 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
             if (d == 0) a.lse[(int64_t)rowid * G + h] = any ? (m + log2f(l)) * 0.6931471805599453f : -INFINITY;
         }
     }
-    if (*abort_flag) {
-        // A wait gave up, so peers may still be on their way to push parts into this CTA's shared memory, which lasts as long
-        // as one of its threads.  Those that know stay until every peer has ended or come here, too (the barrier waits for
-        // the threads that have not exited; a CTA none of whose waits gave up has all its parts and leaves at once).  Then
-        // a bounded time for copies and stores that are under way.
-        ptx::cluster_arrive();
-        ptx::cluster_wait();
+    if (*abort_flag && tid == 0) {
+        // A wait gave up: leave copies that may still be in flight a bounded time to land before the CTA's shared memory is
+        // handed to another CTA.  (Thread 0 waits for every V block itself and meets the other warps behind every K block,
+        // so it has seen the flag unless all copies have landed.)
         const long long t0 = clock64();
         while (clock64() - t0 < 2000000ll) {
         }
