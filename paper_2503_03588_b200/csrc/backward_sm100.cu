@@ -603,8 +603,9 @@ dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUten
 // it is computed: with the lookup (a halving search, ten dependent loads) in the producer's way and the output in
 // that of the compute warps, every item began with some 8000 clk in which the tensor cores stood still, against
 // 10000 to 30000 of work.
-// Measured, 28 / 4 heads: the whole backward pass at 4K tokens 154 us (160 with items one after the other), at 32K
-// 1430 us at full clocks (1488); 64 features, 16 / 4 heads, 2 x 8K tokens: 234 us (269).
+// Measured before the dQ kernel ran beside it, 28 / 4 heads: the whole backward pass at 4K tokens 154 us (160 with items one
+// after the other), at 32K 1430 us at full clocks (1488); 64 features, 16 / 4 heads, 2 x 8K tokens: 234 us (269).  With it
+// beside: 152, 1370 and 228 us.
 template <int D>
 struct DkvCfg {
     static constexpr int kDH = D / 64;

@@ -70,7 +70,10 @@ long long wait_limit_cycles();
 // Launch attribute under which a kernel may start while the kernel before it in the stream still runs
 // (programmatic dependent launch).  Such a kernel touches no global memory before pdl_wait(), which returns when
 // everything ahead of it in the stream has completed; what it does before that (barriers, tensor memory, the
-// launch itself) is hidden behind the other kernel's last microseconds.
+// launch itself) is hidden behind the other kernel's last microseconds.  One kernel breaks that rule: dq_kernel works beside
+// dkv_kernel, the launch before it.  That one lets it start only behind its own pdl_wait() and a store that dq_kernel
+// acquires (so that the preparation's results are there), neither writes what the other reads or writes, and
+// dq_kernel ends behind pdl_wait() (so that whoever waits for it waits for both).
 // Behind it, plain loads only: __ldg and ld.global.nc are for data that nobody writes while the kernel runs, which here
 // includes the time before the wait, and the compiler may move them across it.
 inline cudaLaunchAttribute pdl_attribute()

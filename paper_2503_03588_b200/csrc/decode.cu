@@ -345,7 +345,7 @@ struct RowSmem {
 // The row's block set, one candidate per lane (the order does not matter for Eq. (1), so the set
 // is not sorted): window distances 0 .. w-1, then the power-of-two distances >= w that do not
 // land on a sink block, then the sink blocks outside the window.  Returns this lane's key block
-// or -1.  The host takes the row kernel only when window + powers + sinks fit the 32 lanes.
+// or -1.  The host takes the cluster and row kernels only when window + powers + sinks fit the 32 lanes.
 __device__ __forceinline__ int32_t row_block_candidate(int32_t row, int32_t W, int32_t S, int lane)
 {
     const int32_t w_eff = W > 1 ? W : 1;
@@ -1093,7 +1093,7 @@ __global__ void decode_block_list_kernel(int64_t len, int32_t W, int32_t S, int3
     *count = (int32_t)row.n;
 }
 
-// One warp: the row kernel's own enumeration, compacted in lane order.
+// One warp: the enumeration of the cluster and row kernels, compacted in lane order.
 __global__ void decode_row_block_set_kernel(int64_t len, int32_t W, int32_t S, int32_t *out, int32_t *count,
                                             int32_t capacity)
 {
@@ -1150,7 +1150,7 @@ kv_append_kernel(const __nv_bfloat16 *k_new, const __nv_bfloat16 *v_new, __nv_bf
 
 // Window distances + power-of-two distances beyond the window + sink blocks that a row below
 // n_rows can have, before any of them coincide or fall off the sequence start: the number of
-// candidate slots the row kernel enumerates (one per lane, so it needs this to be <= 32).
+// candidate slots the cluster and row kernels enumerate (one per lane, so it needs this to be <= 32).
 static int64_t row_candidate_slots(int64_t n_rows, int32_t W, int32_t S)
 {
     const int64_t w = W > 1 ? W : 1;
@@ -1265,7 +1265,7 @@ static cudaLaunchConfig_t row_launch_config(unsigned grid, unsigned threads, int
     return cfg;
 }
 
-// How many clusters of R CTAs of the row kernel the device holds at once.  Asked once per device and kind of launch.
+// How many clusters of R CTAs of the cluster kernel the device holds at once.  Asked once per device and kind of launch.
 static pa_status resident_clusters(int device, int head_dim, int stages, int R, int *out)
 {
     static std::mutex mu;
@@ -1341,7 +1341,7 @@ static pa_status launch_decode(const DecodeShape &p, const void *q, const void *
     a.fixed_chunks = 0;
     a.R = 1;
     a.items = 0;
-    // Rows whose block set fits one warp's lanes take the row kernel.
+    // Rows whose block set fits one warp's lanes take the cluster or the row kernel.
     if (!takes_split_k(p)) {
         const int64_t rows_in_call = (int64_t)a.batch * a.Hkv;
         const int max_R = a.chunks < kRowMaxCluster ? a.chunks : kRowMaxCluster;
